@@ -46,22 +46,22 @@ def listed():
         # Token-by-token decoding (block length 1): eight experts per layer, launches and latency.
         _case("block of 1 token", "block", 2048, 64, 8, 1024, 1, layers=8),
         # The paper's regime: block length 16, the block's tokens activating a third of the experts.
-        _case("block of 16, shared", "block", 2048, 64, 8, 1024, 16, layers=8, tokens_like="shared"),
+        _case("block of 16 shared", "block", 2048, 64, 8, 1024, 16, layers=8, tokens_like="shared"),
         # The 16-layer stack on a 32-token block with every expert resident, in both store formats.
         _case("block of 32", "block", 2048, 64, 8, 1024, 32, layers=16),
-        _case("block of 32, fp8", "block", 2048, 64, 8, 1024, 32, layers=16, fp8=True),
+        _case("block of 32 fp8", "block", 2048, 64, 8, 1024, 32, layers=16, fp8=True),
         # Small-batch serving: four blocks of 64 tokens on the 128-expert stack.
         _case("batch of 256", "block", 2048, 128, 8, 768, 256, layers=8),
         # Eight blocks of 32 from fp8 stores, some sequences already finished (a ragged count).
-        _case("batch of 250, fp8", "block", 2048, 64, 8, 1024, 250, layers=8, fp8=True),
+        _case("batch of 250 fp8", "block", 2048, 64, 8, 1024, 250, layers=8, fp8=True),
         # Thirty-two blocks of 32, ragged: between the weight stream and the tensor cores.
         _case("batch of 1000", "block", 2048, 64, 8, 1024, 1000, layers=4),
         # One layer over a large batch with a skewed gate (the many-token configuration).
         _case("step of 4096 tokens", "step", 4096, 64, 8, 1536, 4096, tokens_like="zipf"),
         # A cache of 40 % on unrelated tokens: the host link carries three fifths of the experts.
-        _case("block of 32, 40 % resident", "block", 2048, 64, 8, 1024, 32, layers=4, iters=2, residency=0.4),
+        _case("block of 32 at 40 % residency", "block", 2048, 64, 8, 1024, 32, layers=4, iters=2, residency=0.4),
         # The paper's setting end to end: 40 % resident, similar tokens, adaptive sizing, host buffers.
-        _case("block of 32, shared, 40 %", "block", 2048, 64, 8, 1024, 32, layers=8, iters=4, tokens_like="shared",
+        _case("block of 32 shared at 40 % residency", "block", 2048, 64, 8, 1024, 32, layers=8, iters=4, tokens_like="shared",
               residency=0.4, host=True),
     ]
 
