@@ -56,6 +56,26 @@ self_check_kernel(const int32_t* __restrict__ ids, const int32_t* __restrict__ c
   }
 }
 
+__global__ void __launch_bounds__(256)
+scatter_check_kernel(const int32_t* __restrict__ ids, const int32_t* __restrict__ counts,
+                     const int32_t* __restrict__ assignment, int cap, int T, int E, int K, uint32_t* __restrict__ status) {
+  const int n = T * K;
+  const int tid = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+  for (int r = tid; r < E * cap; r += step) {
+    const int e = r / cap, i = r - e * cap;
+    if (i == 0 && (counts[e] < 0 || counts[e] > cap)) report(status, OLED_CHECK_OFFSETS, e);
+    if (i >= counts[e]) continue;
+    const int a = assignment[r];
+    if (a < 0 || a >= n) {
+      report(status, OLED_CHECK_PERM_RANGE, r);
+      continue;
+    }
+    if (ids[a] != e) report(status, OLED_CHECK_ROW_EXPERT, r);
+    for (int i2 = 0; i2 < i; ++i2)
+      if (assignment[e * cap + i2] == a) report(status, OLED_CHECK_INVERSE, r);
+  }
+}
+
 __global__ void guard_check_kernel(GuardList guards, uint32_t* __restrict__ status) {
   const int b = blockIdx.x;
   if (b >= guards.n) return;
@@ -85,6 +105,12 @@ void launch_self_check(cudaStream_t st, const int32_t* ids, const int32_t* count
   const int n = T * K;
   const int blocks = std::max(1, std::min(148, (std::max(n, E) + 255) / 256));
   self_check_kernel<<<blocks, 256, 0, st>>>(ids, counts, offsets, perm, pos, T, E, K, status);
+}
+
+void launch_scatter_check(cudaStream_t st, const int32_t* ids, const int32_t* counts, const int32_t* assignment, int cap,
+                          int T, int E, int K, uint32_t* status) {
+  const int blocks = std::max(1, std::min(148, (E * cap + 255) / 256));
+  scatter_check_kernel<<<blocks, 256, 0, st>>>(ids, counts, assignment, cap, T, E, K, status);
 }
 
 void launch_guard_check(cudaStream_t st, const GuardList& guards, uint32_t* status) {

@@ -31,7 +31,7 @@ combine_kernel(const float* __restrict__ y, const float* __restrict__ gate,
   __shared__ int s_r[OLED_MAX_TOPK];
   if (threadIdx.x < K) {
     s_g[threadIdx.x] = gate[(size_t)t * K + threadIdx.x];
-    s_r[threadIdx.x] = pos[(size_t)t * K + threadIdx.x];
+    s_r[threadIdx.x] = pos != nullptr ? pos[(size_t)t * K + threadIdx.x] : t * K + (int)threadIdx.x;
   }
   __syncthreads();
   for (int h = h_begin + threadIdx.x * 4; h < h_end; h += blockDim.x * 4) {
@@ -104,7 +104,7 @@ combine_bf16_wide_kernel(const uint16_t* __restrict__ y, const float* __restrict
   __shared__ int s_r[OLED_MAX_TOPK];
   if (threadIdx.x < K) {
     s_g[threadIdx.x] = gate[(size_t)t * K + threadIdx.x];
-    s_r[threadIdx.x] = pos[(size_t)t * K + threadIdx.x];
+    s_r[threadIdx.x] = pos != nullptr ? pos[(size_t)t * K + threadIdx.x] : t * K + (int)threadIdx.x;
   }
   __syncthreads();
   for (int h = threadIdx.x * 8; h < H; h += blockDim.x * 8) {

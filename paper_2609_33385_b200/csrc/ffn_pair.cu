@@ -196,7 +196,7 @@ constexpr int kRowSlots = 3;
 template <int KIND>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
 ffn_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_act,
-                const __grid_constant__ FfnGroup grp, const int32_t* __restrict__ offsets, void* __restrict__ out_ptr,
+                const __grid_constant__ FfnGroup grp, const __grid_constant__ FfnRows rows, void* __restrict__ out_ptr,
                 int H, int I, int out_bf16, uint32_t* __restrict__ status, uint32_t* __restrict__ work_counter,
                 StepTimeline* timeline, int timeline_slot, const __grid_constant__ RouteReport report,
                 const __grid_constant__ PairSecond sec, const __grid_constant__ PairTokens tok) {
@@ -242,9 +242,8 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant_
   if (threadIdx.x == 0) timeline_start(timeline, timeline_slot);
   for (int g = threadIdx.x; g < grp.n; g += kPairThreads) {
     const int e = grp.expert[g];
-    const int s = offsets[e];
-    ctl->row_start[g] = s;
-    ctl->count[g] = offsets[e + 1] - s;
+    ctl->row_start[g] = rows.first(e);
+    ctl->count[g] = rows.count(e);
   }
   __syncthreads();
   if (warp == 0) {  // exclusive scan of the experts' token-tile counts, 32 experts at a time
@@ -612,10 +611,13 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant_
               p[128] = *reinterpret_cast<const uint16_t*>(&b1);
             }
         } else {
-          float* p = reinterpret_cast<float*>(out_y) + (size_t)(it.row0 + c) * H + col;
+          // (few-token steps only: in a scattered one the output goes to the row's assignment)
+          float* const y0 = reinterpret_cast<float*>(out_y) + col;
 #pragma unroll
-          for (int j = 0; j < 16; ++j, p += H)
+          for (int j = 0; j < 16; ++j)
             if (whole || c + j < it.valid) {
+              const int r = it.row0 + c + j;
+              float* const p = y0 + (size_t)(rows.assignment != nullptr ? __ldg(rows.assignment + r) : r) * H;
               p[0] = __uint_as_float(ra[j]);
               p[128] = __uint_as_float(rb[j]);
             }
@@ -655,7 +657,7 @@ bool ffn_pair_usable(const FfnTcMaps& maps, int n_box, int H, int I) {
   return !maps.fp8 && n_box == kPairN && I % 256 == 0 && H % 512 == 0;
 }
 
-int launch_ffn_pair(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp, int kind, const int32_t* offsets,
+int launch_ffn_pair(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp, int kind, const FfnRows& rows,
                     uint16_t* hbuf, float* y, int y_bf16, int H, int I, int n_sms, uint32_t* status,
                     uint32_t* work_counter, StepTimeline* timeline, int timeline_slot, const RouteReport& report,
                     uint32_t* done) {
@@ -684,14 +686,14 @@ int launch_ffn_pair(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp,
   if (gathers && tok.ready == nullptr) return OLED_ERR_INVALID_ARG;
   if (kind == 3) {
     if (done == nullptr) return OLED_ERR_INVALID_ARG;
-    err = launch_pdl(ffn_pair_kernel<3>, dim3(grid), dim3(kPairThreads), kPairSmem, st, maps.w13, maps.xp[3], grp, offsets,
+    err = launch_pdl(ffn_pair_kernel<3>, dim3(grid), dim3(kPairThreads), kPairSmem, st, maps.w13, maps.xp[3], grp, rows,
                      (void*)hbuf, H, I, y_bf16, status, work_counter, timeline, timeline_slot, report, sec, tok);
   } else if (kind == 1)
-    err = launch_pdl(ffn_pair_kernel<1>, dim3(grid), dim3(kPairThreads), kPairSmem, st, maps.w13, maps.xp[3], grp, offsets,
+    err = launch_pdl(ffn_pair_kernel<1>, dim3(grid), dim3(kPairThreads), kPairSmem, st, maps.w13, maps.xp[3], grp, rows,
                      (void*)hbuf, H, I, 0, status, work_counter, timeline, timeline_slot, report, sec, tok);
   else
     err = launch_pdl(ffn_pair_kernel<2>, dim3(grid), dim3(kPairThreads), kPairSmem, st, maps.w2, maps.hbuf[3], grp,
-                     offsets, (void*)y, H, I, y_bf16, status, work_counter, timeline, timeline_slot, RouteReport{}, sec, tok);
+                     rows, (void*)y, H, I, y_bf16, status, work_counter, timeline, timeline_slot, RouteReport{}, sec, tok);
   return err == cudaSuccess ? OLED_OK : OLED_ERR_CUDA;
 }
 

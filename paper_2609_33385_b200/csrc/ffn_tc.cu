@@ -11,11 +11,11 @@
 // 256.  Weights are addressed through the expert->slot table: one 3-D tensor map covers the
 // whole slot pool and the slot number is a TMA coordinate.
 //
-// KIND 1 has a second form for small token tiles (N <= 32), "stacked": 64 gate rows and the 64 up
-// rows of the same intermediate features share ONE 128-row MMA tile (lanes 0-63 gate, 64-127 up),
-// so an item is half as large and twice as many items exist - with ~4 tokens per expert the
-// kernel is a weight stream, and finer items are what keeps all 148 SMs streaming to the end of
-// the launch.  The up values cross to the gate rows' warps through shared memory.
+// Token tiles of at most 32 rows, the few-token regime, have a kernel of their own (ffn_few.cu); here
+// are tiles of 64 to 256 rows and, for any tile, the fp8 form that widens the codes.  The latter keeps a
+// second form of KIND 1 for tiles of at most 32 rows, "stacked": 64 gate rows and the 64 up
+// rows of the same intermediate features share ONE 128-row MMA tile (lanes 0-63 gate, 64-127 up);
+// the up values cross to the gate rows' warps through shared memory.
 //
 // In the many-token regime (N tile 256) both kernels work on two 128-row weight tiles that share
 // one token tile (gate+up, or two row blocks of Wd): 64 KB of operands per 128x2x256x64 MACs.
@@ -32,8 +32,7 @@
 // warp 16 lane 0 TMA producer, warp 17 lane 0 MMA issuer (warp 17 also owns the TMEM allocation),
 // warps 18-21 widen fp8 weight tiles (fp8 expert stores only, idle otherwise).
 //
-// fp8 expert stores (e4m3 codes + one fp32 scale per weight row), token tiles of 64 and 128 rows
-// (FP8 = 1, "widening"): a pipeline stage is a load
+// fp8 expert stores (e4m3 codes + one fp32 scale per weight row), widening: a pipeline stage is a load
 // slot in shared memory - the code tile of a k-block (64 bytes per weight row, half the bytes in
 // flight of the bf16 form) next to its token tile - plus 32 (64) columns of TENSOR memory.
 // Groups of four converter warps, one per TMEM lane quarter, read the codes, widen them to bf16
@@ -43,25 +42,6 @@
 // never touch shared memory.  The accumulators keep their place in front of the weight stages,
 // which is why the fp8 form stops at token tiles of 128.  The epilogue multiplies each output
 // row by its scale - the rows of a weight tile are the accumulator's lanes.
-//
-// fp8 expert stores, token tiles of at most 32 rows (FP8 = 2, "direct"): the widening form above
-// is bound by the thread that issues the MMAs - an M = 128 instruction consumes 128 weight rows x
-// 16 k whatever the element size, so half the bytes are not half the instructions.  Here the
-// MMAs are kind::f8f6f4 (K = 32 per instruction) and read the e4m3 code tile as the TMA laid it
-// down: a k-block is 128 rows x 128 k, the same 16 KB and the same four instructions as a bf16
-// k-block of 64.  An MMA takes both operands in the same 8-bit kind, so the token rows enter as
-// e4m3 too: every row, scaled by a power of two that brings its largest magnitude into
-// [128, 256), is the sum of two e4m3 terms (fp8_split.h; exact for every element within 2^-14 of
-// the row's maximum, which is as exact as bf16 tokens get next to an fp32 accumulator).  The
-// terms are made once per step and operand - by the gathering permutation kernel for the input
-// rows, by split_rows_kernel between the two projections for the intermediate rows, whose
-// largest magnitudes the gate/up epilogue collects with atomicMax - and loaded as the B tile
-// [term 1 rows | term 2 rows], N = 2 n_box; the epilogue adds the two accumulators (D1 + D2/16)
-// and undoes the row's scale.  No converter warps and no proxy fences in the streaming loop:
-// a form that split the tokens inside the kernel was bound by the fence between the converters'
-// shared-memory writes and the MMA's reads (one per stage, each waiting for the copies in flight).
-// The TMA thread issues one copy for the code tile (a 4-D map whose box takes the 64 gate and
-// the 64 up rows at once) and one for both term tiles per k-block.
 //
 // Every mbarrier wait is bounded: on a timeout the CTA raises a flag in the status word, gives
 // in-flight copies time to land, frees its TMEM and returns.
@@ -73,8 +53,8 @@
 #include <algorithm>
 #include <cstddef>
 #include <cstdlib>
+#include <type_traits>
 
-#include "fp8_split.h"
 #include "kernels.h"
 #include "sm100_ptx.h"
 
@@ -132,20 +112,11 @@ constexpr uint32_t kCtlBytes = (sizeof(SharedCtl) + 1023u) & ~1023u;
 
 struct Item {
   int slot, m0, row0, valid;
-  int kind;  // 1: gate/up (+SwiGLU), 2: down projection
-  int g;     // index of the expert in the launch's group
 };
-// The second half of a FUSED launch's work list (KIND 3): items [n1, n1 + n2) are the down-
-// projection items of the same experts and token tiles as the gate/up items [0, n1).
-struct SecondPhase {
-  int n1;            // number of first-phase items (INT_MAX: no second phase)
-  int m_tiles, m_rows;
-};
-// A role's position in the expert list: items arrive in ascending order within a phase, so the
-// search for an item's expert only moves forward; it restarts with the second phase.
+// A role's position in the expert list: items arrive in ascending order, so the search for an
+// item's expert only moves forward.
 struct ItemCursor {
   int g = 0;
-  int phase2 = 0;
 };
 // Items (expert, token tile, weight tile) are handed out DYNAMICALLY: after its first item (its own
 // CTA number) the producer thread of a CTA draws item numbers from a counter in global memory
@@ -163,78 +134,42 @@ __device__ __forceinline__ int take_item(SharedCtl* ctl, int seq, volatile int* 
   mbar_arrive(smem_u32(&ctl->item_empty[slot]));
   return item;
 }
-__device__ __forceinline__ void decode_item(const SharedCtl* ctl, const FfnGroup& grp, int item, int kind1, int m_tiles,
-                                            int m_rows, int n_box, const SecondPhase& second, ItemCursor& cur,
-                                            Item& it) {
-  it.kind = kind1;
-  if (item >= second.n1) {
-    item -= second.n1;
-    m_tiles = second.m_tiles;
-    m_rows = second.m_rows;
-    it.kind = 2;
-    if (!cur.phase2) {
-      cur.phase2 = 1;
-      cur.g = 0;
-    }
-  }
+__device__ __forceinline__ void decode_item(const SharedCtl* ctl, const FfnGroup& grp, int item, int m_tiles, int m_rows,
+                                            int n_box, ItemCursor& cur, Item& it) {
   const int q = item / m_tiles;
   const int m = item - q * m_tiles;
   int g = cur.g;
   while (ctl->tile_prefix[g + 1] <= q) ++g;
   cur.g = g;
   const int nt = q - ctl->tile_prefix[g];
-  it.g = g;
   it.slot = grp.slot[g];
   it.m0 = m * m_rows;
   it.row0 = ctl->row_start[g] + nt * n_box;
   it.valid = min(n_box, ctl->count[g] - nt * n_box);
 }
 
-// What a FUSED launch (KIND 3) needs on top: the down projection's tensor maps, its output and
-// the completion counters.
-struct FusedSecond {
-  CUtensorMap tm_w2;    // down-projection weights
-  CUtensorMap tm_act2;  // intermediate rows (hbuf)
-  void* out2;           // y
-  uint32_t* done;       // per expert of the group: epilogue warps that have stored gate/up rows; ZERO at start
-};
-
 // DUAL: two accumulators per item - gate and up (KIND 1, always), or two row blocks of Wd
 // (KIND 2 with the 256-token tile).
-// FP8: the slot pool holds fp8 expert blobs (tm_w is a byte map over the e4m3 codes).
-// KIND 3 (bf16 stores, token tiles of at most 32 rows): the gate/up items in their stacked form,
-// then the down-projection items of the same experts, in ONE launch.  A down item reads the
-// intermediate rows that the gate/up items of its expert wrote, so its producer waits (bounded)
-// until the expert's counter in `done` shows that all of them have been stored; items are handed
-// out in order, gate/up first, so that wait is over long before it is reached except in launches
-// with few items per SM - which is where this form pays: the two-kernel form leaves every SM that
-// runs out of gate/up items idle until the last gate/up item of the whole launch is done, this
-// one lets it go on with the down projection of experts that are already complete.
-template <int KIND, bool DUAL, int FP8>
+// WIDEN: the slot pool holds fp8 expert blobs (tm_w is a byte map over the e4m3 codes); the MMA's
+// weight operand comes from tensor memory.
+template <int KIND, bool DUAL, bool WIDEN>
 __global__ void __launch_bounds__(kThreads, 1)
 ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_act,
-              const __grid_constant__ FfnGroup grp, const int32_t* __restrict__ offsets,
+              const __grid_constant__ FfnGroup grp, const __grid_constant__ FfnRows rows,
               void* __restrict__ out_ptr, int H, int I, int n_stages, int k_atoms, int early_start, int out_bf16,
               const uint8_t* __restrict__ pool, unsigned long long slot_bytes,
               uint32_t* __restrict__ status, uint32_t* __restrict__ work_counter, StepTimeline* timeline,
-              int timeline_slot, const __grid_constant__ RouteReport report,
-              const __grid_constant__ FusedSecond fs, const uint32_t* __restrict__ amax_in,
-              uint32_t* __restrict__ amax_out) {
+              int timeline_slot, const __grid_constant__ RouteReport report) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   SharedCtl* ctl = reinterpret_cast<SharedCtl*>(smem_raw);
   const uint32_t tiles_base = (smem_u32(smem_raw) + kCtlBytes + 1023u) & ~1023u;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n_box = grp.n_box;
-  constexpr bool fused = KIND == 3;
-  static_assert(!(fused && (DUAL || FP8)), "the fused form exists for bf16 stores and single tiles only");
-  constexpr bool WIDEN = FP8 == 1;   // fp8 stores, codes widened to bf16 by converter warps
-  constexpr bool DIRECT = FP8 == 2;  // fp8 stores, codes read by the MMA as they are (see the header comment)
-  static_assert(!(DIRECT && DUAL), "the direct fp8 form exists for single 128-row tiles only");
-  constexpr int kK = DIRECT ? 128 : kBlockK;  // k-values of a k-block (one 128-byte swizzle atom of weights)
-  constexpr int kind1 = fused ? 1 : KIND;  // kind of the launch's first-phase (or only) items
+  static_assert(DUAL || WIDEN || KIND == 2, "gate/up tiles of bf16 stores have two accumulators");
+  constexpr int kK = kBlockK;  // k-values of a k-block (one 128-byte swizzle atom of weights)
   constexpr bool dual = DUAL;
-  constexpr bool stacked = (KIND == 1 && !DUAL) || fused;  // gate/up items: 64 gate + 64 up rows in one 128-row tile
+  constexpr bool stacked = KIND == 1 && !DUAL;  // gate/up items: 64 gate + 64 up rows in one 128-row tile
   constexpr uint32_t a_bytes = (dual ? 2u : 1u) * kATile;
   const uint32_t b_bytes = (uint32_t)n_box * 128u;
   // bf16 stores: a stage (shared memory) holds the weight tile(s) and the token tile of a k-block.
@@ -244,19 +179,15 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
   // A stage spans k_atoms (1 or 2) k-blocks of 64, laid out one after the other, each as
   // described above: small token tiles take two, which halves the waits and commits per byte on
   // the serial path of the MMA thread.
-  // direct fp8 form: a stage is the code tile of a k-block of 128 (16 KB) and the two e4m3 term
-  // tiles of the tokens (2 n_box rows of 128 bytes, term 2 behind term 1) - the MMA's B operand.
   constexpr uint32_t raw_bytes = WIDEN ? a_bytes / 2 : 0u;
-  const uint32_t atom_bytes = DIRECT ? kATile + 2u * b_bytes
-                              : WIDEN ? raw_bytes + b_bytes : a_bytes + b_bytes;  // one k-block in shared memory
+  const uint32_t atom_bytes = (WIDEN ? raw_bytes : a_bytes) + b_bytes;  // one k-block in shared memory
   const uint32_t stage_bytes = (uint32_t)k_atoms * atom_bytes;
   constexpr uint32_t atom_cols = dual ? 64u : 32u;  // 64 k-values of one (two) 128-row tile(s), two per column
   const uint32_t a_cols = (uint32_t)k_atoms * atom_cols;
-  const int k_blocks1 = (kind1 == 1 ? H : I) / (kK * k_atoms);  // stages per (first-phase) item
-  const int k_blocks2 = I / (kK * k_atoms);                    // stages per down item of a fused launch
+  const int k_blocks = (KIND == 1 ? H : I) / (kK * k_atoms);  // stages per item
   constexpr int m_rows = (KIND == 2 && dual) ? 2 * kBlockM : stacked ? kBlockM / 2 : kBlockM;  // output features per item
-  const int m_tiles = (kind1 == 1 ? I : H) / m_rows;
-  const int acc_cols = (dual || DIRECT ? 2 : 1) * n_box;  // (direct fp8 form: one accumulator per token term)
+  const int m_tiles = (KIND == 1 ? I : H) / m_rows;
+  const int acc_cols = (dual ? 2 : 1) * n_box;
   const int a_total = WIDEN ? n_stages * (int)a_cols : 0;
   const int acc_stages = (2 * acc_cols + a_total <= 512) ? 2 : 1;
   const uint32_t a_col0 = (uint32_t)(acc_stages * acc_cols);  // first column of the weight stages
@@ -310,10 +241,6 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
   if (warp == kProducerWarp && lane == 0) {  // the two tensor maps, ahead of the first copy
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tm_w)) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tm_act)) : "memory");
-    if (fused) {
-      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&fs.tm_w2)) : "memory");
-      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&fs.tm_act2)) : "memory");
-    }
   }
   if (warp == kMmaWarp) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -334,9 +261,8 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
   if (threadIdx.x == 0) timeline_start(timeline, timeline_slot);
   for (int g = threadIdx.x; g < grp.n; g += kThreads) {
     const int e = grp.expert[g];
-    const int s = offsets[e];
-    ctl->row_start[g] = s;
-    ctl->count[g] = offsets[e + 1] - s;
+    ctl->row_start[g] = rows.first(e);
+    ctl->count[g] = rows.count(e);
   }
   __syncthreads();
   if (warp == 0) {  // exclusive scan of the experts' token-tile counts, 32 experts at a time
@@ -366,13 +292,7 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
   constexpr uint32_t nap_epi = WIDEN ? OLED_NAP_EPI : 0u, nap_load = WIDEN ? OLED_NAP_LOAD : 0u,
                      nap_conv = WIDEN ? OLED_NAP_CONV : 0u;
   const uint32_t tmem_base = ctl->tmem_base;
-  SecondPhase second;
-  second.n1 = fused ? ctl->n_tiles_total * m_tiles : 0x7fffffff;
-  second.m_rows = kBlockM;
-  second.m_tiles = H / kBlockM;
-  const int total_items = ctl->n_tiles_total * m_tiles + (fused ? ctl->n_tiles_total * second.m_tiles : 0);
-  // KIND 3: epilogue warps that store intermediate rows per gate/up item, times the items of one token tile
-  const uint32_t done_per_tile = (uint32_t)(m_tiles * (epi_warps / 2));
+  const int total_items = ctl->n_tiles_total * m_tiles;
   volatile int* abort_flag = &ctl->abort;
 
   if (KIND != 2 && blockIdx.x == 0 && warp == kProducerWarp && lane != 0) {
@@ -384,7 +304,7 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     // ------------------------------------------------------------ TMA producer
     // bf16 stores: weight rows and token tile of a k-block go to one operand stage; fp8 stores:
     // code rows and token tile go to one load slot
-    int stage = 0, ready_g = -1;
+    int stage = 0;
     ItemCursor cur;
     uint32_t phase = 0;
     bool ok = true;
@@ -407,12 +327,8 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
       mbar_arrive(smem_u32(&ctl->item_full[ring_slot]));
       if (none) break;
       Item it;
-      decode_item(ctl, grp, item, kind1, m_tiles, m_rows, n_box, second, cur, it);
+      decode_item(ctl, grp, item, m_tiles, m_rows, n_box, cur, it);
       item = next;
-      const bool down_of_fused = fused && it.kind == 2;
-      const CUtensorMap* map_w = down_of_fused ? &fs.tm_w2 : &tm_w;
-      const CUtensorMap* map_act = down_of_fused ? &fs.tm_act2 : &tm_act;
-      const int k_blocks = down_of_fused ? k_blocks2 : k_blocks1;
       constexpr uint32_t w_tile = WIDEN ? kATile / 2 : kATile;  // bytes of 128 weight rows of a k-block
       auto load_weights = [&](int st, int kb) {
         const uint32_t bar = smem_u32(WIDEN ? &ctl->slot_full[st] : &ctl->full[st]);
@@ -420,19 +336,15 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
         for (int atom = 0; atom < k_atoms; ++atom) {
           const uint32_t w_addr = tiles_base + (uint32_t)st * stage_bytes + (uint32_t)atom * atom_bytes;
           const int k0 = (kb * k_atoms + atom) * kK;
-          if (DIRECT && stacked && it.kind == 1) {
-            // one copy: the map is over [slot][gate | up][row][k], the box takes 64 rows of either
-            // half (the copy instructions are the serial cost of this thread, see rings_for)
-            tma_load_4d(map_w, w_addr, bar, k0, it.m0, 0, it.slot);
-          } else if (stacked && it.kind == 1) {  // the map has 64-row boxes here
-            tma_load_3d(map_w, w_addr, bar, k0, it.m0, it.slot);                  // 64 gate rows
-            tma_load_3d(map_w, w_addr + w_tile / 2, bar, k0, I + it.m0, it.slot);  // 64 up rows
-          } else if (it.kind == 1) {
-            tma_load_3d(map_w, w_addr, bar, k0, it.m0, it.slot);               // gate rows
-            tma_load_3d(map_w, w_addr + w_tile, bar, k0, I + it.m0, it.slot);  // up rows
+          if (stacked) {  // the map has 64-row boxes here
+            tma_load_3d(&tm_w, w_addr, bar, k0, it.m0, it.slot);                  // 64 gate rows
+            tma_load_3d(&tm_w, w_addr + w_tile / 2, bar, k0, I + it.m0, it.slot);  // 64 up rows
+          } else if (KIND == 1) {
+            tma_load_3d(&tm_w, w_addr, bar, k0, it.m0, it.slot);               // gate rows
+            tma_load_3d(&tm_w, w_addr + w_tile, bar, k0, I + it.m0, it.slot);  // up rows
           } else {
-            tma_load_3d(map_w, w_addr, bar, k0, it.m0, it.slot);               // down rows
-            if (dual) tma_load_3d(map_w, w_addr + w_tile, bar, k0, it.m0 + kBlockM, it.slot);
+            tma_load_3d(&tm_w, w_addr, bar, k0, it.m0, it.slot);               // down rows
+            if (dual) tma_load_3d(&tm_w, w_addr + w_tile, bar, k0, it.m0 + kBlockM, it.slot);
           }
         }
       };
@@ -442,11 +354,7 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
           const uint32_t t_addr =
               tiles_base + (uint32_t)st * stage_bytes + (uint32_t)atom * atom_bytes + (WIDEN ? raw_bytes : a_bytes);
           const int k0 = (kb * k_atoms + atom) * kK;
-          if (DIRECT) {  // (the map is over [term][row][k], the box takes both terms)
-            tma_load_3d(map_act, t_addr, bar, k0, it.row0, 0);
-          } else {
-            tma_load_2d(map_act, t_addr, bar, k0, it.row0);
-          }
+          tma_load_2d(&tm_act, t_addr, bar, k0, it.row0);
         }
       };
       int kb = 0;
@@ -459,58 +367,6 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
         kb = pre;
         if (pre == n_stages) phase ^= 1u;
         else stage = pre;
-      }
-      if (down_of_fused) {
-        // The intermediate rows of every token tile of this expert must be in memory.  If they are
-        // not yet (launches with few items per SM), the weights of as many stages as the ring
-        // holds go first, then the wait, then those stages' token tiles.
-        const uint32_t* flag = fs.done + it.g;
-        const uint32_t target = done_per_tile * (uint32_t)(ctl->tile_prefix[it.g + 1] - ctl->tile_prefix[it.g]);
-        uint32_t seen = target;  // (an expert seen complete stays complete: no second look)
-        if (it.g != ready_g) asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(flag) : "memory");
-        int pre = 0;
-        const int stage0 = stage;
-        if (seen < target) {
-          pre = min(n_stages, k_blocks);
-          for (int i = 0; i < pre && ok; ++i) {
-            if (!mbar_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, abort_flag, status, nap_load)) {
-              ok = false;
-              break;
-            }
-            load_weights(stage, i);
-            if (++stage == ring) {
-              stage = 0;
-              phase ^= 1u;
-            }
-          }
-          unsigned long long t0 = 0;
-          for (uint32_t spin = 0; ok; ++spin) {
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(flag) : "memory");
-            if (seen >= target) break;
-            if ((spin & 255u) == 255u) {
-              if (*abort_flag) ok = false;
-              const unsigned long long now = globaltimer();
-              if (t0 == 0) t0 = now;
-              if (now - t0 > kWaitLimitNs) {
-                *abort_flag = 1;
-                atomicExch(status, (uint32_t)kStatusWaitTimeout);
-                ok = false;
-              }
-            }
-          }
-          if (!ok) break;
-        }
-        ready_g = it.g;
-        // the rows were written through the generic proxy; the loads below read through the async proxy
-        asm volatile("fence.proxy.async;" ::: "memory");
-        if (pre > 0) {
-          int st = stage0;
-          for (int i = 0; i < pre; ++i) {
-            load_tokens(st, i);
-            if (++st == ring) st = 0;
-          }
-          kb = pre;
-        }
       }
       for (; kb < k_blocks; ++kb) {
         if (!mbar_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, abort_flag, status, nap_load)) {
@@ -549,14 +405,13 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
       const int item = take_item(ctl, local, abort_flag, status, 0u);
       if (item < 0) break;
       Item it;
-      decode_item(ctl, grp, item, kind1, m_tiles, m_rows, n_box, second, cur, it);
-      const int k_blocks = (fused && it.kind == 2) ? k_blocks2 : k_blocks1;
+      decode_item(ctl, grp, item, m_tiles, m_rows, n_box, cur, it);
       const int acc = local % acc_stages;
       const uint32_t acc_phase = (uint32_t)(local / acc_stages) & 1u;
       if (!mbar_wait(smem_u32(&ctl->tmem_empty[acc]), acc_phase ^ 1u, abort_flag, status)) break;
       tc_fence_after();
       const int n_mma = max(16, (it.valid + 15) & ~15);
-      const uint32_t idesc = DIRECT ? make_idesc_e4m3(2 * n_box) : make_idesc(n_mma);
+      const uint32_t idesc = make_idesc(n_mma);
       const uint32_t d0 = tmem_base + (uint32_t)(acc * acc_cols);
       for (int kb = 0; kb < k_blocks; ++kb) {
         // (fp8 stores: the converters arrive on full[] only after the stage's slot has landed)
@@ -570,9 +425,7 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
 #pragma unroll
           for (int k = 0; k < kBlockK / 16; ++k) {  // 32 bytes along K = 2 address units
             const uint32_t accum = k != 0 ? 1u : first;
-            if (DIRECT) {
-              tc_mma_e4m3_lo(d0, a_lo + k * 2, b_lo + k * 2, desc_hi, idesc, accum);
-            } else if (WIDEN) {
+            if (WIDEN) {
               tc_mma_ts_lo(d0, a_tmem + k * 8, b_lo + k * 2, desc_hi, idesc, accum);
               if (dual) tc_mma_ts_lo(d0 + (uint32_t)n_box, a_tmem + 32 + k * 8, b_lo + k * 2, desc_hi, idesc, accum);
             } else {
@@ -614,7 +467,6 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     int stage = group, mine = group;
     uint32_t phase = 0;
     bool live = true;
-    const int k_blocks = k_blocks1;
     for (int seq = 0; live; ++seq) {
       int item = 0;
       if (lane == 0) item = take_item(ctl, seq, abort_flag, status, nap_conv);
@@ -675,8 +527,7 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
       item = __shfl_sync(0xffffffffu, item, 0);
       if (item < 0) break;
       Item it;
-      decode_item(ctl, grp, item, kind1, m_tiles, m_rows, n_box, second, cur, it);
-      const bool gate_up_item = it.kind == 1;  // (always true for KIND 1, never for KIND 2)
+      decode_item(ctl, grp, item, m_tiles, m_rows, n_box, cur, it);
       const int acc = local % acc_stages;
       const uint32_t acc_phase = (uint32_t)(local / acc_stages) & 1u;
       // one lane polls (keeps issue slots free for the producer and MMA threads); the outcome is
@@ -691,10 +542,10 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
       const int n_mma = max(16, (it.valid + 15) & ~15);
       const int col = it.m0 + quarter * 32 + lane;  // output feature owned by this thread
       // fp8 stores: one fp32 scale per weight row behind the codes: s_gate[I] | s_up[I] | s_down[H]
-      const float* sc = FP8 ? reinterpret_cast<const float*>(pool + (size_t)it.slot * slot_bytes + (size_t)3 * H * I)
+      const float* sc = WIDEN ? reinterpret_cast<const float*>(pool + (size_t)it.slot * slot_bytes + (size_t)3 * H * I)
                             : nullptr;
       float s0 = 1.0f, s1 = 1.0f;
-      if (FP8) {
+      if (WIDEN) {
         if (stacked) {
           const int f = it.m0 + (quarter & 1) * 32 + lane;
           s0 = quarter >= 2 ? sc[I + f] : sc[f];  // this thread's row: an up row or a gate row
@@ -709,18 +560,7 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
       for (int c = half * 16; c < n_mma; c += 16 * (epi_warps / 4 > 0 ? epi_warps / 4 : 1)) {
         uint32_t ra[16];
         tmem_ld16(t_row + (uint32_t)c, ra);
-        if (DIRECT) {
-          // the two terms' accumulators: D = (D1 + D2 / 16) / row scale of the token
-          uint32_t rt[16];
-          tmem_ld16(t_row + (uint32_t)(n_box + c), rt);
-          tmem_ld_wait();
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const float inv = c + j < it.valid ? token_scale_inverse(amax_in[it.row0 + c + j]) : 0.0f;
-            ra[j] = __float_as_uint(__fmaf_rn(__uint_as_float(rt[j]), 0.0625f, __uint_as_float(ra[j])) * inv);
-          }
-        }
-        if (stacked && gate_up_item) {
+        if (stacked) {
           // lanes 0-63 hold silu's argument (gate rows), lanes 64-127 the up rows of the same
           // features: warps 2,3 hand their chunk to warps 0,1 through a double-buffered slot
           tmem_ld_wait();
@@ -758,28 +598,14 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
             }
             mbar_arrive(smem_u32(&ctl->x_empty[buf][half]));
             uint16_t* hb = reinterpret_cast<uint16_t*>(out_ptr);
-            uint32_t mag[16];  // direct fp8 form: magnitudes of the stored values (bf16 bit patterns)
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
-              mag[j] = 0u;
               if (c + j < it.valid) {
                 const float a = __uint_as_float(ra[j]) * s0;
                 const float hm = __fdividef(a, 1.0f + __expf(-a)) * u[j];
                 const __nv_bfloat16 b = __float2bfloat16_rn(hm);
                 hb[(size_t)(it.row0 + c + j) * I + it.m0 + xrow] = *reinterpret_cast<const uint16_t*>(&b);
-                mag[j] = (uint32_t)(*reinterpret_cast<const uint16_t*>(&b) & 0x7fffu);
               }
-            }
-            if (DIRECT) {
-              // the rows' largest magnitudes, for the down projection's token scaling: the warp's
-              // 32 features of token c + j are reduced, lane j raises the row's word
-              uint32_t top = 0u;
-#pragma unroll
-              for (int j = 0; j < 16; ++j) {
-                const uint32_t m = __reduce_max_sync(0xffffffffu, mag[j]);
-                if (lane == j) top = m;
-              }
-              if (lane < 16 && c + lane < it.valid && top != 0u) atomicMax(amax_out + it.row0 + c + lane, top << 16);
             }
           }
         } else if (KIND == 1) {
@@ -798,16 +624,18 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
             }
           }
         } else {
-          void* const out_y = fused ? fs.out2 : out_ptr;
-          float* y = reinterpret_cast<float*>(out_y);
-          uint16_t* yb = reinterpret_cast<uint16_t*>(out_y);  // many-token steps keep y in bf16
+          float* y = reinterpret_cast<float*>(out_ptr);
+          uint16_t* yb = reinterpret_cast<uint16_t*>(out_ptr);  // many-token steps keep y in bf16
           uint32_t rb[16];
           if (dual) tmem_ld16(t_row + (uint32_t)(n_box + c), rb);
+          // (scattered steps: lane j looks up where row c + j's output belongs)
+          int dst = it.row0 + c + (lane & 15);
+          if (rows.assignment != nullptr && c + (lane & 15) < it.valid) dst = __ldg(rows.assignment + dst);
           tmem_ld_wait();
 #pragma unroll
-          for (int j = 0; j < 16; ++j)
+          for (int j = 0; j < 16; ++j) {
+            const size_t o = (size_t)__shfl_sync(0xffffffffu, dst, j) * H + col;
             if (c + j < it.valid) {
-              const size_t o = (size_t)(it.row0 + c + j) * H + col;
               if (out_bf16) {
                 const __nv_bfloat16 b0 = __float2bfloat16_rn(__uint_as_float(ra[j]) * s0);
                 yb[o] = *reinterpret_cast<const uint16_t*>(&b0);
@@ -820,17 +648,10 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
                 if (dual) y[o + kBlockM] = __uint_as_float(rb[j]) * s1;
               }
             }
+          }
         }
       }
       if (!alive) break;
-      if (fused && gate_up_item && quarter < 2) {
-        // this warp's intermediate rows of the item are stored: make them visible device-wide,
-        // then count the warp in (the down items of this expert wait for the full count)
-        __threadfence();
-        asm volatile("fence.proxy.async;" ::: "memory");
-        __syncwarp();
-        if (lane == 0) atomicAdd(fs.done + it.g, 1u);
-      }
       tc_fence_before();
       mbar_arrive(smem_u32(&ctl->tmem_empty[acc]));
     }
@@ -853,35 +674,6 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
   if (threadIdx.x == 0) timeline_end(timeline, timeline_slot);
 }
 
-// fp8 direct form, between the two projections: the intermediate rows of the group's experts
-// (bf16, written by the gate/up epilogue together with every row's largest magnitude) as two e4m3
-// terms per element.  Four CTAs per expert of the group (a quarter of the columns each); a warp
-// takes a row at a time.
-__global__ void __launch_bounds__(256)
-split_rows_kernel(const __grid_constant__ FfnGroup grp, const int32_t* __restrict__ offsets,
-                  const uint16_t* __restrict__ hbuf, const uint32_t* __restrict__ amax_mid,
-                  uint8_t* __restrict__ terms_mid, int I, int rows_total) {
-  griddep_launch_dependents();
-  griddep_wait();
-  const int e = grp.expert[blockIdx.x];
-  const int first = offsets[e], last = offsets[e + 1];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int r = first + warp; r < last; r += 8) {
-    const float scale = token_scale(amax_mid[r]);
-    const uint4* src = reinterpret_cast<const uint4*>(hbuf + (size_t)r * I);
-    uint2* out1 = reinterpret_cast<uint2*>(terms_mid + (size_t)r * I);
-    uint2* out2 = reinterpret_cast<uint2*>(terms_mid + ((size_t)rows_total + r) * I);
-    for (int c = lane + 32 * (int)blockIdx.y; c < I / 8; c += 32 * (int)gridDim.y) {
-      const uint4 v = src[c];
-      uint2 t1, t2;
-      split_bf16x4(v.x, v.y, scale, t1.x, t2.x);
-      split_bf16x4(v.z, v.w, scale, t1.y, t2.y);
-      out1[c] = t1;
-      out2[c] = t2;
-    }
-  }
-}
-
 // ---------------------------------------------------------------- host side
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*,
@@ -900,8 +692,9 @@ EncodeTiledFn get_encode_fn() {
   return fn;
 }
 
-bool encode(CUtensorMap* m, int rank, const void* base, const cuuint64_t* dims, const cuuint64_t* strides,
-            const cuuint32_t* box, bool bytes = false, bool bytes_swizzle_128 = false) {
+}  // namespace
+bool encode_tensor_map(CUtensorMap* m, int rank, const void* base, const cuuint64_t* dims, const cuuint64_t* strides,
+                       const cuuint32_t* box, bool bytes, bool narrow) {
   EncodeTiledFn fn = get_encode_fn();
   if (!fn) return false;
   cuuint32_t estr[5] = {1, 1, 1, 1, 1};
@@ -912,9 +705,10 @@ bool encode(CUtensorMap* m, int rank, const void* base, const cuuint64_t* dims, 
   // in the 128-byte-swizzled layout again
   return fn(m, bytes ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank,
             const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-            bytes && !bytes_swizzle_128 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, promo,
+            narrow ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, promo,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
+namespace {
 
 struct Rings {
   int stages;     // pipeline stages
@@ -931,23 +725,20 @@ int epi_warps_for(int kind, int out_bf16, int n_box) {
 // (eleven measured slower).  fp8 stores: a stage is a load slot in shared memory plus columns of
 // tensor memory behind the accumulators (two accumulator stages if at least two weight stages
 // still fit); the depth is a multiple of the number of converter groups (see the kernel).
-// k_dim2: the second contraction length of a fused launch (0 otherwise).
-// fp8: 0 = bf16 stores, 1 = fp8 stores widened by converter warps, 2 = fp8 stores read directly.
-Rings rings_for(int kind, bool dual, int n_box, int out_bf16, int fp8, int k_dim, int k_dim2 = 0) {
+Rings rings_for(int kind, bool dual, int n_box, int out_bf16, bool fp8, int k_dim) {
   const uint32_t a = (dual ? 2u : 1u) * kATile, b = (uint32_t)n_box * 128u;
   const uint32_t avail = kSmemMax - kCtlBytes - 1024u;
-  const uint32_t atom = fp8 == 2 ? kATile + 2u * b : fp8 ? a / 2 + b : a + b;  // one k-block in shared memory
-  int kblocks = (int)std::min<uint32_t>((uint32_t)(fp8 == 2 ? kMaxStages : fp8 ? 2 * kMaxStages : 10), avail / atom);
-  if (fp8 == 1) {
+  const uint32_t atom = (fp8 ? a / 2 : a) + b;  // one k-block in shared memory
+  int kblocks = (int)std::min<uint32_t>((uint32_t)(fp8 ? 2 * kMaxStages : 10), avail / atom);
+  if (fp8) {
     const int acc_cols = (dual ? 2 : 1) * n_box, a_cols = dual ? 64 : 32;
     const int free_cols = 512 - 2 * acc_cols >= 2 * a_cols ? 512 - 2 * acc_cols : 512 - acc_cols;
     kblocks = std::min(kblocks, free_cols / a_cols);
   }
   Rings r;
-  const int kk = fp8 == 2 ? 128 : kBlockK;  // k-values of a k-block
-  r.k_atoms = (!dual && kblocks >= 8 && (k_dim / kk) % 2 == 0 && (k_dim2 / kk) % 2 == 0) ? 2 : 1;
+  r.k_atoms = (!dual && kblocks >= 8 && (k_dim / kBlockK) % 2 == 0) ? 2 : 1;
   r.stages = std::min(kblocks / r.k_atoms, kMaxStages);
-  if (fp8 == 1) {
+  if (fp8) {
     const int groups = std::min(2, 1 + (kEpiWarps - epi_warps_for(kind, out_bf16, n_box)) / 4);
     if (r.stages >= groups) r.stages -= r.stages % groups;
   }
@@ -955,42 +746,25 @@ Rings rings_for(int kind, bool dual, int n_box, int out_bf16, int fp8, int k_dim
   return r;
 }
 
-template <int KIND, bool DUAL, int FP8>
+template <int KIND, bool DUAL, bool WIDEN>
 bool set_smem_attr() {
-  return cudaFuncSetAttribute(ffn_tc_kernel<KIND, DUAL, FP8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  return cudaFuncSetAttribute(ffn_tc_kernel<KIND, DUAL, WIDEN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)kSmemMax) == cudaSuccess;
 }
 
-template <int KIND, bool DUAL>
-void launch_variant(int fp8, int grid, cudaStream_t st, const CUtensorMap& tw, const CUtensorMap& ta,
-                    const FfnGroup& grp, const int32_t* offsets, void* out, int H, int I, int out_bf16,
-                    const uint8_t* pool, size_t slot_bytes, uint32_t* status, uint32_t* work_counter,
-                    uint32_t smem_of_predecessor, bool early_allowed, StepTimeline* timeline, int timeline_slot,
-                    const RouteReport& report, const FusedSecond& fs = FusedSecond{}, const uint32_t* amax_in = nullptr,
-                    uint32_t* amax_out = nullptr) {
-  const Rings r = rings_for(KIND, DUAL, grp.n_box, out_bf16, fp8, KIND == 2 ? I : H, KIND == 3 ? I : 0);
+template <int KIND, bool DUAL, bool WIDEN>
+void launch_variant(int grid, cudaStream_t st, const CUtensorMap& tw, const CUtensorMap& ta, const FfnGroup& grp,
+                    const FfnRows& rows, void* out, int H, int I, int out_bf16, const uint8_t* pool, size_t slot_bytes,
+                    uint32_t* status, uint32_t* work_counter, uint32_t smem_of_predecessor, bool early_allowed,
+                    StepTimeline* timeline, int timeline_slot, const RouteReport& report) {
+  const Rings r = rings_for(KIND, DUAL, grp.n_box, out_bf16, WIDEN, KIND == 2 ? I : H);
   // KIND 2 may start ahead of its dependency wait only where the caller vouches for the ordering
   // (early_allowed, see launch_ffn_tc) AND one of its CTAs and one of the KIND 1 kernel before it
   // cannot share an SM, so that it gets an SM only when a KIND 1 CTA has left it
   const int early = (KIND == 2 && early_allowed && smem_of_predecessor + r.smem > 228u * 1024u) ? 1 : 0;
-  if constexpr (KIND == 3) {
-    launch_pdl(ffn_tc_kernel<3, false, 0>, dim3(grid), dim3(kThreads), r.smem, st, tw, ta, grp, offsets, out, H, I,
-               r.stages, r.k_atoms, 0, out_bf16, pool, (unsigned long long)slot_bytes, status, work_counter, timeline,
-               timeline_slot, report, fs, amax_in, amax_out);
-  } else if (fp8 == 2) {
-    if constexpr (!DUAL)
-      launch_pdl(ffn_tc_kernel<KIND, false, 2>, dim3(grid), dim3(kThreads), r.smem, st, tw, ta, grp, offsets, out, H,
-                 I, r.stages, r.k_atoms, early, out_bf16, pool, (unsigned long long)slot_bytes, status, work_counter,
-                 timeline, timeline_slot, report, fs, amax_in, amax_out);
-  } else if (fp8) {
-    launch_pdl(ffn_tc_kernel<KIND, DUAL, 1>, dim3(grid), dim3(kThreads), r.smem, st, tw, ta, grp, offsets, out, H,
-               I, r.stages, r.k_atoms, early, out_bf16, pool, (unsigned long long)slot_bytes, status, work_counter, timeline,
-               timeline_slot, report, fs, amax_in, amax_out);
-  } else {
-    launch_pdl(ffn_tc_kernel<KIND, DUAL, 0>, dim3(grid), dim3(kThreads), r.smem, st, tw, ta, grp, offsets, out, H,
-               I, r.stages, r.k_atoms, early, out_bf16, pool, (unsigned long long)slot_bytes, status, work_counter, timeline,
-               timeline_slot, report, fs, amax_in, amax_out);
-  }
+  launch_pdl(ffn_tc_kernel<KIND, DUAL, WIDEN>, dim3(grid), dim3(kThreads), r.smem, st, tw, ta, grp, rows, out, H, I,
+             r.stages, r.k_atoms, early, out_bf16, pool, (unsigned long long)slot_bytes, status, work_counter, timeline,
+             timeline_slot, report);
 }
 
 }  // namespace
@@ -1008,14 +782,14 @@ int ffn_tc_setup(FfnTcMaps* maps, const uint8_t* pool, size_t slot_bytes, int n_
     const cuuint64_t strides[2] = {(cuuint64_t)H * esz, (cuuint64_t)slot_bytes};
     const cuuint32_t box[3] = {kBlockK, kBlockM, 1};
     const cuuint32_t box_half[3] = {kBlockK, kBlockM / 2, 1};  // stacked gate/up tiles
-    if (!encode(&maps->w13, 3, pool, dims, strides, box, fp8)) return OLED_ERR_CUDA;
-    if (!encode(&maps->w13_half, 3, pool, dims, strides, box_half, fp8)) return OLED_ERR_CUDA;
+    if (!encode_tensor_map(&maps->w13, 3, pool, dims, strides, box, fp8, fp8)) return OLED_ERR_CUDA;
+    if (!encode_tensor_map(&maps->w13_half, 3, pool, dims, strides, box_half, fp8, fp8)) return OLED_ERR_CUDA;
   }
   {
     const cuuint64_t dims[3] = {(cuuint64_t)I, (cuuint64_t)H, (cuuint64_t)n_slots};
     const cuuint64_t strides[2] = {(cuuint64_t)I * esz, (cuuint64_t)slot_bytes};
     const cuuint32_t box[3] = {kBlockK, kBlockM, 1};
-    if (!encode(&maps->w2, 3, pool + (size_t)2 * I * H * esz, dims, strides, box, fp8)) return OLED_ERR_CUDA;
+    if (!encode_tensor_map(&maps->w2, 3, pool + (size_t)2 * I * H * esz, dims, strides, box, fp8, fp8)) return OLED_ERR_CUDA;
   }
   // fp8 stores: maps for the form whose MMAs read the codes themselves - k-blocks of 128 bytes
   maps->e4m3_direct = fp8 && H % 128 == 0 && I % 128 == 0 && split != nullptr && split->complete() && split->rows == rows;
@@ -1024,36 +798,32 @@ int ffn_tc_setup(FfnTcMaps* maps, const uint8_t* pool, size_t slot_bytes, int n_
       const cuuint32_t tbox[3] = {128, (cuuint32_t)(16 << i), 2};
       const cuuint64_t dims_in[3] = {(cuuint64_t)H, (cuuint64_t)rows, 2}, dims_mid[3] = {(cuuint64_t)I, (cuuint64_t)rows, 2};
       const cuuint64_t str_in[2] = {(cuuint64_t)H, (cuuint64_t)rows * H}, str_mid[2] = {(cuuint64_t)I, (cuuint64_t)rows * I};
-      if (!encode(&maps->xp_terms[i], 3, split->terms_in, dims_in, str_in, tbox, true, true)) return OLED_ERR_CUDA;
-      if (!encode(&maps->hbuf_terms[i], 3, split->terms_mid, dims_mid, str_mid, tbox, true, true)) return OLED_ERR_CUDA;
+      if (!encode_tensor_map(&maps->xp_terms[i], 3, split->terms_in, dims_in, str_in, tbox, true)) return OLED_ERR_CUDA;
+      if (!encode_tensor_map(&maps->hbuf_terms[i], 3, split->terms_mid, dims_mid, str_mid, tbox, true)) return OLED_ERR_CUDA;
     }
-    const cuuint32_t box_half[4] = {128, kBlockM / 2, 2, 1}, box[3] = {128, kBlockM, 1};
-    const cuuint64_t dims13[4] = {(cuuint64_t)H, (cuuint64_t)I, 2, (cuuint64_t)n_slots};
-    const cuuint64_t strides13[3] = {(cuuint64_t)H, (cuuint64_t)I * H, (cuuint64_t)slot_bytes};
+    const cuuint32_t box[3] = {128, kBlockM, 1};
     const cuuint64_t dims2[3] = {(cuuint64_t)I, (cuuint64_t)H, (cuuint64_t)n_slots};
     const cuuint64_t strides2[2] = {(cuuint64_t)I, (cuuint64_t)slot_bytes};
-    if (!encode(&maps->w13_half_e4m3, 4, pool, dims13, strides13, box_half, true, true)) return OLED_ERR_CUDA;
-    if (!encode(&maps->w2_e4m3, 3, pool + (size_t)2 * I * H, dims2, strides2, box, true, true)) return OLED_ERR_CUDA;
+    if (!encode_tensor_map(&maps->w2_e4m3, 3, pool + (size_t)2 * I * H, dims2, strides2, box, true)) return OLED_ERR_CUDA;
   }
+  if (const int rc = ffn_few_setup(maps, pool, slot_bytes, n_slots, H, I, fp8); rc != OLED_OK) return rc;
   for (int i = 0; i < 5; ++i) {
     const cuuint32_t box[2] = {kBlockK, (cuuint32_t)(16 << i)};
     {
       const cuuint64_t dims[2] = {(cuuint64_t)H, (cuuint64_t)rows};
       const cuuint64_t strides[1] = {(cuuint64_t)H * 2};
-      if (!encode(&maps->xp[i], 2, xp, dims, strides, box)) return OLED_ERR_CUDA;
+      if (!encode_tensor_map(&maps->xp[i], 2, xp, dims, strides, box)) return OLED_ERR_CUDA;
     }
     {
       const cuuint64_t dims[2] = {(cuuint64_t)I, (cuuint64_t)rows};
       const cuuint64_t strides[1] = {(cuuint64_t)I * 2};
-      if (!encode(&maps->hbuf[i], 2, hbuf, dims, strides, box)) return OLED_ERR_CUDA;
+      if (!encode_tensor_map(&maps->hbuf[i], 2, hbuf, dims, strides, box)) return OLED_ERR_CUDA;
     }
   }
   static bool attr_done = false;
   if (!attr_done) {
-    if (!set_smem_attr<1, true, 0>() || !set_smem_attr<1, false, 0>() || !set_smem_attr<2, true, 0>() ||
-        !set_smem_attr<2, false, 0>() || !set_smem_attr<1, true, 1>() || !set_smem_attr<1, false, 1>() ||
-        !set_smem_attr<2, true, 1>() || !set_smem_attr<2, false, 1>() || !set_smem_attr<3, false, 0>() ||
-        !set_smem_attr<1, false, 2>() || !set_smem_attr<2, false, 2>())
+    if (!set_smem_attr<1, true, false>() || !set_smem_attr<2, true, false>() || !set_smem_attr<2, false, false>() ||
+        !set_smem_attr<1, true, true>() || !set_smem_attr<1, false, true>() || !set_smem_attr<2, false, true>())
       return OLED_ERR_CUDA;
     attr_done = true;
   }
@@ -1067,27 +837,28 @@ static int box_index(int max_count, int cap) {
 }
 
 int launch_ffn_tc(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp_in, int max_count, int kind,
-                  const int32_t* host_counts, const int32_t* offsets, uint16_t* hbuf, float* y, int y_bf16, int H, int I,
+                  const int32_t* host_counts, const FfnRows& rows, uint16_t* hbuf, float* y, int y_bf16, int H, int I,
                   int n_sms, uint32_t* status, uint32_t* work_counter, bool behind_event_wait, StepTimeline* timeline,
                   int timeline_slot, const RouteReport& report_in, uint32_t* done, const TokenSplit* split) {
   const RouteReport report = kind != 2 ? report_in : RouteReport{};
   if (grp_in.n <= 0 || max_count <= 0) return OLED_OK;
   FfnGroup grp = grp_in;
   const bool fp8 = maps.fp8;
-  grp.pad = 0;
   // N <= 128 keeps the accumulators double-buffered in TMEM; more tokens per expert than that
   // take N = 256 with two weight tiles per item (all 512 TMEM columns, one accumulator stage).
   // (fp8 stores stop at N = 128: the widened weights need tensor-memory columns of their own)
   const int ib = box_index(max_count, fp8 ? 128 : 256);
   grp.n_box = 16 << ib;
-  // fp8 stores, token tiles of at most 32 rows, row magnitudes at hand: the MMAs read the codes
-  // themselves (mode 2); otherwise converter warps widen them to bf16 (mode 1)
+  // fp8 stores, token tiles of at most 32 rows, the rows' terms at hand: the MMAs read the codes
+  // themselves (ffn_few.cu); otherwise converter warps widen them to bf16
   const bool direct = fp8 && maps.e4m3_direct && grp.n_box <= 32 && split != nullptr && split->complete();
-  const int mode = direct ? 2 : fp8 ? 1 : 0;
+  if (direct || (!fp8 && grp.n_box <= 32))
+    return launch_ffn_few(st, maps, grp, ib, kind, host_counts, rows, hbuf, y, H, I, n_sms, status, work_counter,
+                          behind_event_wait, timeline, timeline_slot, report, done, split);
   // many-token tiles: the CTA-pair kernel, unless its cluster launch has failed before on this
   // device (the one-CTA form below computes the same)
   if (maps.use_pairs && !g_pairs_refused && ffn_pair_usable(maps, grp.n_box, H, I)) {
-    if (launch_ffn_pair(st, maps, grp, kind, offsets, hbuf, y, y_bf16, H, I, n_sms, status, work_counter, timeline,
+    if (launch_ffn_pair(st, maps, grp, kind, rows, hbuf, y, y_bf16, H, I, n_sms, status, work_counter, timeline,
                         timeline_slot, report, done) == OLED_OK)
       return OLED_OK;
     cudaGetLastError();  // (a refused launch enqueues nothing)
@@ -1101,11 +872,11 @@ int launch_ffn_tc(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp_in
   if (kind == 3 && grp.n_box > 32) {
     // (only reached when the pair launch was refused: the two launches of the one-CTA form, the
     // work counter cleared in stream order between them)
-    int rc = launch_ffn_tc(st, maps, grp_in, max_count, 1, host_counts, offsets, hbuf, y, y_bf16, H, I, n_sms, status,
+    int rc = launch_ffn_tc(st, maps, grp_in, max_count, 1, host_counts, rows, hbuf, y, y_bf16, H, I, n_sms, status,
                            work_counter, behind_event_wait, timeline, timeline_slot, report_in, done, split);
     if (rc != OLED_OK) return rc;
     if (cudaMemsetAsync(work_counter, 0, sizeof(uint32_t), st) != cudaSuccess) return OLED_ERR_CUDA;
-    return launch_ffn_tc(st, maps, grp_in, max_count, 2, host_counts, offsets, hbuf, y, y_bf16, H, I, n_sms, status,
+    return launch_ffn_tc(st, maps, grp_in, max_count, 2, host_counts, rows, hbuf, y, y_bf16, H, I, n_sms, status,
                          work_counter, false, timeline, timeline_slot, report_in, done, split);
   }
   // one CTA per SM, fewer if the group has fewer (weight tile, token tile) items than SMs
@@ -1122,40 +893,25 @@ int launch_ffn_tc(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp_in
   // CTA then gets an SM only after a KIND 1 CTA, which waited for the permutation, has left it),
   // or the launch pair sits behind an event wait, which completes everything enqueued before it.
   const bool early_allowed = kind == 2 && (behind_event_wait || host_counts == nullptr);
-  const uint32_t smem1 = kind == 2 ? rings_for(1, !stacked1, grp.n_box, 0, mode, H).smem : 0u;
-  if (kind == 3) {
-    if (fp8 || !stacked1 || done == nullptr) return OLED_ERR_INVALID_ARG;  // callers ask ffn_tc_can_fuse() first
-    FusedSecond fs;
-    fs.tm_w2 = maps.w2;
-    fs.tm_act2 = maps.hbuf[ib];
-    fs.out2 = y;
-    fs.done = done;
-    launch_variant<3, false>(0, grid_for(I / (kBlockM / 2) + H / kBlockM), st, maps.w13_half, maps.xp[ib], grp, offsets,
-                             hbuf, H, I, 0, maps.pool, maps.slot_bytes, status, work_counter, 0u, false, timeline,
-                             timeline_slot, report, fs);
-  } else if (kind == 1 && stacked1) {
-    launch_variant<1, false>(mode, grid_for(I / (kBlockM / 2)), st, direct ? maps.w13_half_e4m3 : maps.w13_half,
-                             direct ? maps.xp_terms[ib] : maps.xp[ib], grp, offsets, hbuf, H, I, 0, maps.pool,
-                             maps.slot_bytes, status, work_counter, smem1, early_allowed, timeline, timeline_slot, report,
-                             FusedSecond{}, direct ? split->amax_in : nullptr, direct ? split->amax_mid : nullptr);
-  } else if (kind == 1) {
-    launch_variant<1, true>(mode, grid_for(I / kBlockM), st, maps.w13, maps.xp[ib], grp, offsets, hbuf, H, I, 0,
-                            maps.pool, maps.slot_bytes, status, work_counter, smem1, early_allowed, timeline, timeline_slot, report);
-  } else {
-    const bool dual = grp.n_box == 256;
-    if (dual)
-      launch_variant<2, true>(mode, grid_for(H / (2 * kBlockM)), st, maps.w2, maps.hbuf[ib], grp, offsets, y, H, I,
-                              y_bf16, maps.pool, maps.slot_bytes, status, work_counter, smem1, early_allowed, timeline, timeline_slot, report);
-    else {
-      if (direct)  // the intermediate rows as e4m3 terms, now that their magnitudes are complete
-        launch_pdl(split_rows_kernel, dim3(grp.n, 4), dim3(256), 0, st, grp, offsets, (const uint16_t*)hbuf,
-                   (const uint32_t*)split->amax_mid, split->terms_mid, I, split->rows);
-      launch_variant<2, false>(mode, grid_for(H / kBlockM), st, direct ? maps.w2_e4m3 : maps.w2,
-                               direct ? maps.hbuf_terms[ib] : maps.hbuf[ib], grp, offsets, y, H, I, y_bf16, maps.pool,
-                               maps.slot_bytes, status, work_counter, smem1, early_allowed, timeline, timeline_slot,
-                               report, FusedSecond{}, direct ? split->amax_mid : nullptr, nullptr);
-    }
-  }
+  const uint32_t smem1 = kind == 2 ? rings_for(1, !stacked1, grp.n_box, 0, fp8, H).smem : 0u;
+  if (kind == 3) return OLED_ERR_INVALID_ARG;  // callers ask ffn_tc_can_fuse() / ffn_pair_can_fuse() first
+  const bool dual2 = grp.n_box == 256;
+  auto go = [&](auto kind_c, auto dual_c, auto widen_c, int m_tiles, const CUtensorMap& tw, const CUtensorMap& ta, void* out,
+                int out_bf16) {
+    launch_variant<decltype(kind_c)::value, decltype(dual_c)::value, decltype(widen_c)::value>(
+        grid_for(m_tiles), st, tw, ta, grp, rows, out, H, I, out_bf16, maps.pool, maps.slot_bytes, status, work_counter,
+        smem1, early_allowed, timeline, timeline_slot, report);
+  };
+  using std::false_type;
+  using std::true_type;
+  constexpr std::integral_constant<int, 1> k1{};
+  constexpr std::integral_constant<int, 2> k2{};
+  if (kind == 1 && stacked1) go(k1, false_type{}, true_type{}, I / (kBlockM / 2), maps.w13_half, maps.xp[ib], hbuf, 0);
+  else if (kind == 1 && fp8) go(k1, true_type{}, true_type{}, I / kBlockM, maps.w13, maps.xp[ib], hbuf, 0);
+  else if (kind == 1) go(k1, true_type{}, false_type{}, I / kBlockM, maps.w13, maps.xp[ib], hbuf, 0);
+  else if (dual2) go(k2, true_type{}, false_type{}, H / (2 * kBlockM), maps.w2, maps.hbuf[ib], y, y_bf16);
+  else if (fp8) go(k2, false_type{}, true_type{}, H / kBlockM, maps.w2, maps.hbuf[ib], y, y_bf16);
+  else go(k2, false_type{}, false_type{}, H / kBlockM, maps.w2, maps.hbuf[ib], y, y_bf16);
   return cudaGetLastError() == cudaSuccess ? OLED_OK : OLED_ERR_CUDA;
 }
 

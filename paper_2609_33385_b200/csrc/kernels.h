@@ -74,7 +74,7 @@ struct FfnGroup {
   int32_t n;
   int32_t n_box;  // token rows per TMA box / MMA N tile of this launch
   int32_t withhold_loads;  // test aid: the producer issues nothing, the consumers' waits run out
-  int32_t pad;             // tuning aid: cap on the fp8 converter groups (0 = default)
+  int32_t n_guess;         // experts at the head of the list expected to have tokens (few-token form; 0: no guess)
   uint16_t expert[OLED_MAX_EXPERTS];
   uint16_t slot[OLED_MAX_EXPERTS];
 };
@@ -137,7 +137,7 @@ void launch_report(cudaStream_t st, const RouteReport& rep);  // the one-CTA ker
 struct CombinePrev {
   const float* y = nullptr;        // [T*K,H] fp32 per-assignment outputs of the previous layer
   const float* gate = nullptr;     // [T,K]   its gate scores
-  const int32_t* pos = nullptr;    // [T*K]   its inverse permutation
+  const int32_t* pos = nullptr;    // [T*K]   its inverse permutation (nullptr: y is in assignment order)
   const uint16_t* x = nullptr;     // [T,H]   its input
   uint16_t* out = nullptr;         // [T,H]   its MoE output
   uint16_t* x_next = nullptr;      // [T,H]   its input plus its output
@@ -149,16 +149,12 @@ struct CombinePrev {
 // counts every expert's assignments per segment of seg_tokens consecutive tokens, so that the
 // permutation kernel can work on the segments in parallel.
 constexpr int kPermuteSegments = 16;
-void launch_route(cudaStream_t st, const uint16_t* x, const uint16_t* w_router, const float* bias,
-                  const float* conf, int T, int H, int E, int K, float* logits, int32_t* ids,
-                  float* gate, int32_t* counts, unsigned long long* scores, const CombinePrev& prev,
-                  StepTimeline* timeline, int32_t* seg_counts = nullptr, int seg_tokens = 0);
-bool route_can_take_combine(int T);  // does the gate kernel of a T-token step carry out a CombinePrev?
 // fp8 expert stores, direct form: the two token operands of a step's expert FFN - the gathered
 // input rows and the intermediate rows - as sums of two e4m3 terms each, after scaling every row
 // by a power of two taken from its largest magnitude (fp8_split.h).  The magnitudes are kept as the
 // bit pattern of a non-negative fp32, so that an unsigned integer maximum orders them.
-//   amax_in, terms_in:   written by the gathering permutation kernel, which also zeroes amax_mid
+//   amax_in, terms_in:   written by the gate kernel of a scattered step (or the gathering
+//                        permutation kernel), which also zeroes amax_mid
 //   amax_mid:            raised with atomicMax by the gate/up epilogue
 //   terms_mid:           written by the split kernel between the two projections
 struct TokenSplit {
@@ -168,6 +164,42 @@ struct TokenSplit {
   uint8_t* terms_mid = nullptr;  // [2][rows][I]
   int rows = 0;                  // rows of the buffers above (tokens x top-k of the context)
   bool complete() const { return amax_in && amax_mid && terms_in && terms_mid && rows > 0; }
+};
+// Few-token steps: the gate kernel itself brings the token rows to their experts, so that no
+// permutation kernel stands between it and the expert FFN.  Expert e owns the rows e * cap ..
+// e * cap + counts[e] - 1 of the row buffers (cap >= tokens of the step), in the order its count was
+// raised by the tokens: no result depends on that order, because a row of the FFN never meets
+// another, and its output goes to y[assignment], which `assignment` names.
+struct ScatterRows {
+  int cap = 0;                     // 0: the step sorts its rows with the permutation kernel instead
+  int dense = 0;                   // steps of at most kDenseTokens tokens: xp holds the rows once, in token order,
+                                   // and the FFN multiplies every expert with all of them (ffn_few.cu)
+  int32_t* assignment = nullptr;   // [E * cap] row -> t * K + j
+  uint16_t* xp = nullptr;          // [E * cap][H] copies of the token rows
+  TokenSplit split;                // fp8 stores, direct form: the rows' e4m3 terms and magnitudes as well
+};
+void launch_route(cudaStream_t st, const uint16_t* x, const uint16_t* w_router, const float* bias,
+                  const float* conf, int T, int H, int E, int K, float* logits, int32_t* ids,
+                  float* gate, int32_t* counts, unsigned long long* scores, const CombinePrev& prev,
+                  StepTimeline* timeline, int32_t* seg_counts = nullptr, int seg_tokens = 0,
+                  const ScatterRows& scatter = ScatterRows{});
+// Does the gate kernel of a T-token step carry out a CombinePrev and a ScatterRows?
+bool route_can_take_combine(int T);
+constexpr int kDenseTokens = 32;
+// Where the FFN finds an expert's token rows: offsets[e] .. offsets[e + 1] - 1 (sorted steps), or
+// e * cap .. e * cap + counts[e] - 1 (scattered steps, offsets == nullptr; the output of row r then
+// goes to y[assignment[r]]).
+struct FfnRows {
+  const int32_t* offsets = nullptr;
+  const int32_t* counts = nullptr;
+  const int32_t* assignment = nullptr;
+  int cap = 0;
+  int K = 1, E = 0;
+  int dense = 0;  // the input rows are stored once, in token order (ScatterRows::dense)
+#ifdef __CUDACC__
+  __device__ __forceinline__ int first(int e) const { return offsets ? offsets[e] : e * cap; }
+  __device__ __forceinline__ int count(int e) const { return offsets ? offsets[e + 1] - offsets[e] : counts[e]; }
+#endif
 };
 // Offsets (exclusive scan), stable permutation by expert and its inverse.  With xp != nullptr the
 // kernel also gathers the token rows (xp[r,:] = x[perm[r]/K,:]); meant for small steps.
@@ -194,7 +226,8 @@ void launch_l2_prefetch(cudaStream_t st, const uint8_t* pool, size_t slot_bytes,
                         size_t bytes_per_slot);
 
 // ---- combine.cu -----------------------------------------------------------------------
-// out[t,:] = bf16( sum_j gate[t,j] * y[pos[t*K+j],:] ), j ascending, fp32 accumulation.  With
+// out[t,:] = bf16( sum_j gate[t,j] * y[pos[t*K+j],:] ), j ascending, fp32 accumulation (pos ==
+// nullptr: y is in assignment order, row t*K+j).  With
 // x_next != nullptr also x_next[t,:] = bf16(x[t,:] + out[t,:]) (the residual between layers).
 // zero_words != nullptr: CTA 0 also clears n_zero_words 32-bit words there (the step's control
 // block, ready for the next step's atomics).
@@ -211,13 +244,14 @@ void launch_ffn_simple(cudaStream_t st, const FfnGroup& grp, const uint8_t* pool
 
 // ---- ffn_tc.cu (tcgen05 / TMEM / TMA) ------------------------------------------------------
 struct FfnTcMaps {
-  CUtensorMap w13_half_e4m3;  // fp8 stores: [slots][2][I][H] bytes, box {128,64,2,1}, 128-byte swizzle
+  CUtensorMap w13_few;        // gate/up rows of 64 features as four groups of 16 gate and 16 up rows (ffn_few.cu)
+  CUtensorMap w13_few_e4m3;   // the same over e4m3 codes
   CUtensorMap w2_e4m3;        // fp8 stores: [slots][H][I] bytes, box {128,128,1}, 128-byte swizzle
   CUtensorMap xp_terms[2];    // [2][rows][H] bytes (TokenSplit::terms_in), box {128, 16<<i, 2}
   CUtensorMap hbuf_terms[2];  // [2][rows][I] bytes (TokenSplit::terms_mid), box {128, 16<<i, 2}
   bool e4m3_direct = false;   // the maps above exist (fp8 stores, H and I multiples of 128, term buffers given)
   CUtensorMap w13;       // [slots][2I][H] bf16, box {64,128,1}
-  CUtensorMap w13_half;  // the same, box {64,64,1}
+  CUtensorMap w13_half;  // fp8 stores, widening form: the same, box {64,64,1}
   CUtensorMap w2;        // [slots][H][I]  bf16, box {64,128,1}
   CUtensorMap xp[5];     // [rows][H] bf16, box {64, 16<<i}
   CUtensorMap hbuf[5];   // [rows][I] bf16, box {64, 16<<i}
@@ -254,7 +288,7 @@ int ffn_tc_setup(FfnTcMaps* maps, const uint8_t* pool, size_t slot_bytes, int n_
 // at most 32 rows take the form whose MMAs read the experts' e4m3 codes as they are; a kind 2
 // launch is then preceded by the split kernel (ffn_tc_launches tells how many launches a call makes).
 int launch_ffn_tc(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp, int max_count, int kind,
-                  const int32_t* host_counts, const int32_t* offsets, uint16_t* hbuf, float* y, int y_bf16, int H,
+                  const int32_t* host_counts, const FfnRows& rows, uint16_t* hbuf, float* y, int y_bf16, int H,
                   int I, int n_sms, uint32_t* status, uint32_t* work_counter, bool behind_event_wait,
                   StepTimeline* timeline, int timeline_slot, const RouteReport& report, uint32_t* done = nullptr,
                   const TokenSplit* split = nullptr);
@@ -271,15 +305,29 @@ bool ffn_pair_can_fuse(const FfnTcMaps& maps, int max_count, int H, int I);  // 
 // intermediate a multiple of 256 and hidden a multiple of 512); kinds 1 and 2 as above, kind 3 both
 // in one launch (`done`: one ZERO word per expert of the group).
 bool ffn_pair_usable(const FfnTcMaps& maps, int n_box, int H, int I);
-int launch_ffn_pair(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp, int kind, const int32_t* offsets,
+int launch_ffn_pair(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp, int kind, const FfnRows& rows,
                     uint16_t* hbuf, float* y, int y_bf16, int H, int I, int n_sms, uint32_t* status,
                     uint32_t* work_counter, StepTimeline* timeline, int timeline_slot, const RouteReport& report,
                     uint32_t* done = nullptr);
 constexpr int kFfnWorkCounters = 8;  // FFN launches of one layer execution: 3 groups x 2 kinds, rounded up
 
+// A tensor map over bf16 elements (bytes: over bytes) with the 128-byte swizzle (narrow: the 64-byte one).
+bool encode_tensor_map(CUtensorMap* m, int rank, const void* base, const cuuint64_t* dims, const cuuint64_t* strides,
+                       const cuuint32_t* box, bool bytes = false, bool narrow = false);
+// ---- ffn_few.cu: token tiles of at most 32 rows (bf16 stores, or fp8 stores with the token terms at
+// hand).  Kinds as above; kind 2 of fp8 stores is preceded by the split kernel.
+int ffn_few_setup(FfnTcMaps* maps, const uint8_t* pool, size_t slot_bytes, int n_slots, int H, int I, bool fp8);
+int launch_ffn_few(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp, int box_index, int kind,
+                   const int32_t* host_counts, const FfnRows& rows, uint16_t* hbuf, float* y, int H, int I, int n_sms,
+                   uint32_t* status, uint32_t* work_counter, bool behind_event_wait, StepTimeline* timeline,
+                   int timeline_slot, const RouteReport& report, uint32_t* done, const TokenSplit* split);
+
 // Self-check (check.cu): invariants of the routing and the permutation, guard words.
 void launch_self_check(cudaStream_t st, const int32_t* ids, const int32_t* counts, const int32_t* offsets,
                        const int32_t* perm, const int32_t* pos, int T, int E, int K, uint32_t* status);
+// The same for a scattered step: every row of every expert names one assignment routed to it, none twice.
+void launch_scatter_check(cudaStream_t st, const int32_t* ids, const int32_t* counts, const int32_t* assignment, int cap,
+                          int T, int E, int K, uint32_t* status);
 void launch_guard_check(cudaStream_t st, const GuardList& guards, uint32_t* status);
 void launch_guard_fill(cudaStream_t st, const GuardList& guards);
 void launch_corrupt_perm(cudaStream_t st, int32_t* perm, int n);  // test aid

@@ -78,14 +78,18 @@ struct oled_ctx {
     uint16_t* x_next = nullptr;
     uint32_t* ctrl = nullptr;      // the control block that step used (to be cleared)
   } pending;
-  int fuse_ffn = 1;            // OLED_OPT_FUSE_FFN: 0 never, 1 where few items per SM are expected, 2 wherever possible
+  int fuse_ffn = 1;            // OLED_OPT_FUSE_FFN: 0 never, 1 or 2 wherever that form exists
   bool fuse_combine = true;    // stack iterations of few-token steps: a layer's combine runs inside the
                                // next layer's gate kernel (OLED_OPT_FUSE_COMBINE)
   int32_t* d_offsets = nullptr;// [E+1]
   int32_t* d_perm = nullptr;   // [T*k]
   int32_t* d_pos = nullptr;    // [T*k]
-  uint16_t* d_xp = nullptr;    // [T*k,H]
-  uint16_t* d_hbuf = nullptr;  // [T*k,I]
+  size_t row_buf = 0;          // rows of xp and hbuf: T*k, or more where scattered steps need it (kScatterRows)
+  int32_t* d_assignment = nullptr;  // [row_buf] scattered steps: row -> assignment
+  ScatterRows scatter;         // the current step's (cap == 0: it sorts its rows)
+  bool perm_stale = false;     // the last step was scattered: offsets, perm and pos are made when asked for
+  uint16_t* d_xp = nullptr;    // [row_buf,H]
+  uint16_t* d_hbuf = nullptr;  // [row_buf,I]
   TokenSplit split;            // fp8 stores: the FFN's token operands as e4m3 terms (see TokenSplit)
   const TokenSplit* step_split = nullptr;  // &split in steps whose permutation kernel fills it
   float* d_y = nullptr;        // [T*k,H]
@@ -202,6 +206,33 @@ int check_status(oled_ctx* ctx) {
   return OLED_OK;
 }
 
+// The most token rows a scattered step may spread over its experts' regions (experts x tokens, a
+// region has room for every token of the step): 64 experts x 512 tokens.  Beyond it the buffers
+// would outgrow what the step saves.
+constexpr size_t kScatterRows = 32768;
+// A scattered step's rows per expert region.
+inline size_t scatter_cap(size_t T) { return (T + 15) / 16 * 16; }
+
+// offsets, perm and pos of the last step, where it was a scattered one (parity aids only).
+int make_perm(oled_ctx* ctx) {
+  if (!ctx->perm_stale) return OLED_OK;
+  const int E = ctx->shape.n_experts, K = ctx->shape.top_k;
+  int32_t* tmp = nullptr;
+  OLED_CUDA(ctx, cudaMalloc(reinterpret_cast<void**>(&tmp), (size_t)E * sizeof(int32_t)));
+  cudaError_t err = cudaMemcpyAsync(tmp, ctx->host_counts.data(), (size_t)E * sizeof(int32_t), cudaMemcpyHostToDevice,
+                                    ctx->stream);
+  if (err == cudaSuccess) {
+    launch_permute(ctx->stream, ctx->d_ids, tmp, ctx->last_tokens, E, K, ctx->d_offsets, ctx->d_perm, ctx->d_pos, nullptr,
+                   nullptr, ctx->shape.hidden, nullptr);
+    err = cudaStreamSynchronize(ctx->stream);
+  }
+  cudaFree(tmp);
+  OLED_CUDA(ctx, err);
+  ctx->launches += 1;
+  ctx->perm_stale = false;
+  return OLED_OK;
+}
+
 // Carries out a combine that was left to the next layer's gate kernel and never got one.
 int flush_pending_combine(oled_ctx* ctx) {
   if (!ctx->pending.valid) return OLED_OK;
@@ -243,6 +274,7 @@ void free_ctx(oled_ctx* ctx) {
   cudaFree(ctx->d_perm);
   cudaFree(ctx->d_pos_buf[0]);
   cudaFree(ctx->d_pos_buf[1]);
+  cudaFree(ctx->d_assignment);
   cudaFree(ctx->d_xp);
   cudaFree(ctx->d_hbuf);
   cudaFree(ctx->split.amax_in);
@@ -362,15 +394,14 @@ void prof_add_ffn(oled_ctx* ctx, uint64_t n, uint64_t rows, bool fused) {
 
 // The FFN launches over one group: gate/up and down projection, or ONE fused launch where that
 // form exists (bf16 stores, token tiles of at most 32 rows, no event to wait for between the two
-// projections) and few items per SM are expected (expected_experts: how many of the group's
-// experts are expected to have tokens).  host_counts == nullptr: the per-expert counts are not
-// known on the host yet (the group is the resident set and experts without tokens cost nothing).
+// projections).  host_counts == nullptr: the per-expert counts are not known on the host yet (the
+// group is the resident set and experts without tokens cost nothing).
 // before_down: an event the down projection (and nothing before it) has to wait for, or null.
 // behind_event_wait: the caller has just enqueued a cudaStreamWaitEvent on the stream.
 // report: the step's report to the host, sent by the first launch (the plain-FMA bring-up path
 // and an empty group send it from a kernel of its own).
 int run_ffn_launches(oled_ctx* ctx, const FfnGroup& grp, int max_count, const int32_t* host_counts,
-                     cudaEvent_t before_down, bool behind_event_wait, int expected_experts, bool* fused_out,
+                     cudaEvent_t before_down, bool behind_event_wait, bool* fused_out,
                      const RouteReport& report = RouteReport{}) {
   if (fused_out) *fused_out = false;
   if ((grp.n <= 0 || max_count <= 0 || ctx->ffn_impl == 1) && report.host_scores != nullptr) {
@@ -382,21 +413,22 @@ int run_ffn_launches(oled_ctx* ctx, const FfnGroup& grp, int max_count, const in
   // (no gathered copy of the token rows exists: every launch of the step takes the token tile of 256
   // rows, whatever its experts' counts, and gathers its own rows)
   if (ctx->maps.token_source.perm != nullptr) max_count = std::max(max_count, 129);
+  // (every launch of a dense step multiplies with all of the step's rows)
+  if (ctx->scatter.dense && max_count > 0) max_count = ctx->last_tokens;
   if (ctx->ffn_impl == 1) {
     if (before_down) OLED_CUDA(ctx, cudaStreamWaitEvent(ctx->stream, before_down, 0));
     launch_ffn_simple(ctx->stream, grp, ctx->pool, ctx->slot_bytes, ctx->d_offsets, ctx->d_xp, ctx->d_hbuf,
                       ctx->d_y, H, I);
     ctx->launches += 2;
   } else {
-    // With many items per SM the two-kernel form is a little faster (the down projection's early
-    // start hides the boundary; measured 125 against 129 us for 63 experts); with few, the SMs
-    // that run out of gate/up items would idle until the whole gate/up launch has finished.
-    const bool few_items = (long long)expected_experts * (I / 64) < 4ll * ctx->n_sms;
+    // Token tiles of at most 32 rows, bf16 stores: one launch.  SMs that run out of gate/up items go on with
+    // the down projection of experts that are complete (per layer: 8 experts 35 against 39 us as two launches,
+    // 20 experts 52 against 56, 63 and 128 experts 133 and 217 us either way).
     // Many-token tiles on CTA pairs: always one launch (a boundary between cluster kernels is a full stop).
     const bool fuse_pairs = before_down == nullptr && ctx->fuse_ffn != 0 && ffn_pair_can_fuse(ctx->maps, max_count, H, I);
     const bool fuse = fuse_pairs ||
                       (before_down == nullptr && !ctx->y_bf16 && ffn_tc_can_fuse(ctx->maps, max_count) &&
-                       (ctx->fuse_ffn == 2 || (ctx->fuse_ffn == 1 && few_items)));
+                       ctx->fuse_ffn != 0);
     for (int kind = fuse ? 3 : 1; kind <= (fuse ? 3 : 2); ++kind) {
       if (kind == 2 && before_down) OLED_CUDA(ctx, cudaStreamWaitEvent(ctx->stream, before_down, 0));
       ProfScope ps(ctx, kind == 3 ? OLED_KERNEL_FFN_FUSED : kind == 1 ? OLED_KERNEL_FFN_GATE_UP : OLED_KERNEL_FFN_DOWN, 0, 0);
@@ -414,8 +446,18 @@ int run_ffn_launches(oled_ctx* ctx, const FfnGroup& grp, int max_count, const in
       }
       ctx->maps.token_source.ready = ready;
       ctx->work_next += 1;
-      const int rc = launch_ffn_tc(ctx->stream, ctx->maps, grp, max_count, kind, host_counts, ctx->d_offsets,
-                                   ctx->d_hbuf, ctx->d_y, ctx->y_bf16 ? 1 : 0, H, I, ctx->n_sms, ctx->d_status, work,
+      FfnRows rows;
+      if (ctx->scatter.cap > 0) {
+        rows.counts = ctx->d_counts;
+        rows.assignment = ctx->d_assignment;
+        rows.cap = ctx->scatter.cap;
+        rows.dense = ctx->scatter.dense;
+        rows.K = ctx->shape.top_k;
+        rows.E = ctx->shape.n_experts;
+      } else {
+        rows.offsets = ctx->d_offsets;
+      }
+      const int rc = launch_ffn_tc(ctx->stream, ctx->maps, grp, max_count, kind, host_counts, rows, ctx->d_hbuf, ctx->d_y, ctx->y_bf16 ? 1 : 0, H, I, ctx->n_sms, ctx->d_status, work,
                                    behind_event_wait || (kind == 2 && before_down != nullptr),
                                    ctx->timeline_on ? ctx->d_timeline + ctx->last_layer : nullptr, 3 + li, report, done,
                                    ctx->step_split);
@@ -436,7 +478,7 @@ int run_ffn_group(oled_ctx* ctx, LayerData& L, const std::vector<int32_t>& exper
   grp.n = (int32_t)(end - begin);
   grp.n_box = 16;
   grp.withhold_loads = ctx->withhold_loads;
-  grp.pad = 0;
+  grp.n_guess = 0;
   int max_count = 0;
   uint64_t rows = 0;
   for (size_t i = begin; i < end; ++i) {
@@ -447,7 +489,7 @@ int run_ffn_group(oled_ctx* ctx, LayerData& L, const std::vector<int32_t>& exper
     rows += (uint64_t)counts[e];
   }
   bool fused = false;
-  const int rc = run_ffn_launches(ctx, grp, max_count, counts, before_down, behind_event_wait, grp.n, &fused);
+  const int rc = run_ffn_launches(ctx, grp, max_count, counts, before_down, behind_event_wait, &fused);
   prof_add_ffn(ctx, (uint64_t)grp.n, rows, fused);
   return rc;
 }
@@ -568,6 +610,7 @@ int oled_create(const oled_model_shape* shape, const int32_t* cache_capacity, vo
   const size_t T = (size_t)s.max_tokens, E = (size_t)s.n_experts, K = (size_t)s.top_k;
   const size_t H = (size_t)s.hidden, I = (size_t)s.intermediate;
   ctx->ready_words = T * K / 256 + E;
+  ctx->row_buf = std::max(T * K, std::min(kScatterRows, E * scatter_cap(std::min(T, std::max<size_t>(1, 4096 / K)))));
   ctx->ctrl_bytes = E * (sizeof(unsigned long long) + sizeof(int32_t)) + kFfnWorkCounters * sizeof(uint32_t) +
                     (size_t)kFfnWorkCounters * (E + ctx->ready_words) * sizeof(uint32_t) +
                     (size_t)kPermuteSegments * E * sizeof(int32_t);
@@ -586,14 +629,15 @@ int oled_create(const oled_model_shape* shape, const int32_t* cache_capacity, vo
   if ((rc = dev_alloc_guarded(ctx, &ctx->d_pos_buf[0], T * K)) != OLED_OK) return fail(rc);
   if ((rc = dev_alloc_guarded(ctx, &ctx->d_pos_buf[1], T * K)) != OLED_OK) return fail(rc);
   ctx->d_pos = ctx->d_pos_buf[0];
-  if ((rc = dev_alloc_guarded(ctx, &ctx->d_xp, T * K * H)) != OLED_OK) return fail(rc);
-  if ((rc = dev_alloc_guarded(ctx, &ctx->d_hbuf, T * K * I)) != OLED_OK) return fail(rc);
+  if ((rc = dev_alloc_guarded(ctx, &ctx->d_xp, ctx->row_buf * H)) != OLED_OK) return fail(rc);
+  if ((rc = dev_alloc_guarded(ctx, &ctx->d_hbuf, ctx->row_buf * I)) != OLED_OK) return fail(rc);
+  if ((rc = dev_alloc(ctx, &ctx->d_assignment, ctx->row_buf)) != OLED_OK) return fail(rc);
   if (s.expert_format == OLED_EXPERTS_FP8 && H % 128 == 0 && I % 128 == 0) {
-    if ((rc = dev_alloc(ctx, &ctx->split.amax_in, T * K)) != OLED_OK) return fail(rc);
-    if ((rc = dev_alloc(ctx, &ctx->split.amax_mid, T * K)) != OLED_OK) return fail(rc);
-    if ((rc = dev_alloc(ctx, &ctx->split.terms_in, 2 * T * K * H)) != OLED_OK) return fail(rc);
-    if ((rc = dev_alloc(ctx, &ctx->split.terms_mid, 2 * T * K * I)) != OLED_OK) return fail(rc);
-    ctx->split.rows = (int)(T * K);
+    if ((rc = dev_alloc(ctx, &ctx->split.amax_in, ctx->row_buf)) != OLED_OK) return fail(rc);
+    if ((rc = dev_alloc(ctx, &ctx->split.amax_mid, ctx->row_buf)) != OLED_OK) return fail(rc);
+    if ((rc = dev_alloc(ctx, &ctx->split.terms_in, 2 * ctx->row_buf * H)) != OLED_OK) return fail(rc);
+    if ((rc = dev_alloc(ctx, &ctx->split.terms_mid, 2 * ctx->row_buf * I)) != OLED_OK) return fail(rc);
+    ctx->split.rows = (int)ctx->row_buf;
   }
   if ((rc = dev_alloc_guarded(ctx, &ctx->d_y, T * K * H)) != OLED_OK) return fail(rc);
   if ((rc = dev_alloc(ctx, &ctx->d_status, kStatusWords)) != OLED_OK) return fail(rc);
@@ -618,13 +662,13 @@ int oled_create(const oled_model_shape* shape, const int32_t* cache_capacity, vo
   ctx->host_counts.assign(E, 0);
   launch_guard_fill(ctx->stream, ctx->guards);
   if (cudaMemcpy(ctx->d_status, ctx->h_status, kStatusWords * sizeof(uint32_t), cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemset(ctx->d_xp, 0, T * K * H * 2) != cudaSuccess ||
-      cudaMemset(ctx->d_hbuf, 0, T * K * I * 2) != cudaSuccess ||
+      cudaMemset(ctx->d_xp, 0, ctx->row_buf * H * 2) != cudaSuccess ||
+      cudaMemset(ctx->d_hbuf, 0, ctx->row_buf * I * 2) != cudaSuccess ||
       cudaMemset(ctx->d_y, 0, T * K * H * 4) != cudaSuccess)
     return fail(OLED_ERR_CUDA);
   rc = ffn_tc_setup(&ctx->maps, ctx->pool, ctx->slot_bytes, ctx->n_slots, s.hidden, s.intermediate,
                     s.expert_format == OLED_EXPERTS_FP8, ctx->d_xp,
-                    ctx->d_hbuf, (int)(T * K), ctx->split.complete() ? &ctx->split : nullptr);
+                    ctx->d_hbuf, (int)ctx->row_buf, ctx->split.complete() ? &ctx->split : nullptr);
   if (rc != OLED_OK) return fail(rc);
   if (cudaDeviceSynchronize() != cudaSuccess) return fail(OLED_ERR_CUDA);
   *out_ctx = ctx;
@@ -741,10 +785,31 @@ static int step_impl(oled_ctx* ctx, int32_t layer, const void* hidden, const flo
     const int rcp = flush_pending_combine(ctx);
     if (rcp != OLED_OK) return rcp;
   }
+  // few-token steps: the gate kernel scatters the token rows to their experts itself; the permutation
+  // kernel runs where a region per expert would be too large, for the plain-FMA path and its test aid
+  const bool few = (size_t)T * K <= 4096;
+  ctx->scatter = ScatterRows{};
+  ctx->perm_stale = false;
+  ctx->step_split = nullptr;
+  if (few && route_can_take_combine(T) && (size_t)E * scatter_cap(T) <= ctx->row_buf && ctx->ffn_impl == 0 &&
+      !ctx->corrupt_perm) {
+    ctx->scatter.cap = (int)scatter_cap(T);
+    ctx->scatter.assignment = ctx->d_assignment;
+    ctx->scatter.xp = ctx->d_xp;
+    if (ctx->fp8_direct && ctx->split.complete()) {
+      ctx->scatter.split = ctx->split;
+      ctx->step_split = &ctx->split;
+    }
+    // at most 32 tokens: one copy of the rows serves every expert (the FFN form that can use it takes
+    // every launch of such a step, unless fp8 codes are to be widened)
+    ctx->scatter.dense = T <= kDenseTokens && (ctx->shape.expert_format != OLED_EXPERTS_FP8 || ctx->step_split) ? 1 : 0;
+    ctx->perm_stale = true;
+  }
+  const bool scattered = ctx->scatter.cap > 0;
   {
     NvtxRange nv(ctx, "oled.step.1_gate_topk_scores");
     ProfScope ps(ctx, OLED_KERNEL_ROUTE,
-                 ((uint64_t)T * H + (uint64_t)E * H) * 2 + (uint64_t)T * K * 8 +
+                 ((uint64_t)T * H + (uint64_t)E * H) * 2 + (uint64_t)T * K * 8 + (scattered ? (uint64_t)T * K * H * 2 : 0) +
                      (fuse_prev ? (uint64_t)T * K * H * 4 + (uint64_t)T * H * 6 : 0),
                  2ull * T * H * E + (fuse_prev ? 2ull * T * K * H : 0));
     CombinePrev prev;
@@ -761,9 +826,10 @@ static int step_impl(oled_ctx* ctx, int32_t layer, const void* hidden, const flo
       ctx->pending.valid = false;
     }
     launch_route(st, static_cast<const uint16_t*>(hidden), L.w_router, L.bias, confidences, T, H, E, K,
-                 ctx->d_logits, ctx->d_ids, ctx->d_gate, ctx->d_counts, ctx->d_scores, prev, tl, seg_counts, seg_tokens);
+                 ctx->d_logits, ctx->d_ids, ctx->d_gate, ctx->d_counts, ctx->d_scores, prev, tl, seg_counts, seg_tokens,
+                 ctx->scatter);
   }
-  const bool fuse_gather = (size_t)T * K <= 4096;  // few rows per expert: one CTA per expert copies them
+  const bool fuse_gather = few;  // few rows per expert: the permutation kernel, where one runs, copies them
   // Many rows per expert (every FFN launch of the step on CTA pairs, token tiles of 256 rows): no
   // gather kernel, each gate/up launch copies its experts' token rows while its first items run.
   const bool gather_in_ffn = !fuse_gather && ctx->gather_in_ffn && ctx->ffn_impl == 0 &&
@@ -775,7 +841,7 @@ static int step_impl(oled_ctx* ctx, int32_t layer, const void* hidden, const flo
   else
     ffn_tc_clear_token_source(&ctx->maps);
   NvtxRange nv_perm(ctx, "oled.step.2_permutation_counts");
-  {
+  if (!scattered) {
     ProfScope ps(ctx, OLED_KERNEL_PERMUTE, (uint64_t)T * K * 12 + (fuse_gather ? (uint64_t)T * K * H * 4 : 0), 0);
     // (fp8 stores: a gathering permutation kernel also leaves the rows' magnitudes for the FFN)
     ctx->step_split = fuse_gather && ctx->fp8_direct && ctx->split.complete() ? &ctx->split : nullptr;
@@ -787,11 +853,18 @@ static int step_impl(oled_ctx* ctx, int32_t layer, const void* hidden, const flo
     ProfScope ps(ctx, OLED_KERNEL_GATHER, (uint64_t)T * K * H * 4, 0);
     launch_gather(st, static_cast<const uint16_t*>(hidden), ctx->d_perm, T, H, K, ctx->d_xp);
   }
-  ctx->launches += fuse_gather || gather_in_ffn ? 2 : 3;
+  ctx->launches += scattered ? 1 : fuse_gather || gather_in_ffn ? 2 : 3;
   nv_perm.end();
   if (ctx->corrupt_perm) {
     launch_corrupt_perm(st, ctx->d_perm, T * K);
     ctx->launches += 1;
+  }
+  if (ctx->self_check && scattered) {
+    launch_permute(st, ctx->d_ids, ctx->d_counts, T, E, K, ctx->d_offsets, ctx->d_perm, ctx->d_pos, nullptr, nullptr, H,
+                   nullptr);
+    ctx->perm_stale = false;
+    launch_scatter_check(st, ctx->d_ids, ctx->d_counts, ctx->d_assignment, ctx->scatter.cap, T, E, K, ctx->d_status);
+    ctx->launches += 2;
   }
   if (ctx->self_check) {
     launch_self_check(st, ctx->d_ids, ctx->d_counts, ctx->d_offsets, ctx->d_perm, ctx->d_pos, T, E, K, ctx->d_status);
@@ -808,26 +881,29 @@ static int step_impl(oled_ctx* ctx, int32_t layer, const void* hidden, const flo
     grp.n = 0;
     grp.n_box = 16;
     grp.withhold_loads = ctx->withhold_loads;
-    grp.pad = 0;
-    for (int32_t e = 0; e < E; ++e)
-      if (L.cache.resident[e] && L.cache.slot_of[e] >= 0) {
-        grp.expert[grp.n] = (uint16_t)e;
-        grp.slot[grp.n] = (uint16_t)L.cache.slot_of[e];
-        ++grp.n;
+    // those the layer activated at its previous execution come first (adjacent iterations activate mostly
+    // the same experts, Sec. 3.3): their weights are loaded before the gate has decided
+    for (int pass = 0; pass < 2; ++pass) {
+      for (int32_t e = 0; e < E; ++e) {
+        const bool before = !L.last_counts.empty() && L.last_counts[e] > 0;
+        if (before == (pass == 0) && L.cache.resident[e] && L.cache.slot_of[e] >= 0) {
+          grp.expert[grp.n] = (uint16_t)e;
+          grp.slot[grp.n] = (uint16_t)L.cache.slot_of[e];
+          ++grp.n;
+        }
       }
+      if (pass == 0) grp.n_guess = grp.n;
+    }
     // token tile of this launch (the counts are not known on the host yet): twice the mean load
     // per expert, but at least 32 rows - an expert that received more rows than the tile holds
     // has its weights streamed once per tile, and in a block of 32 tokens whose routing is
     // concentrated on few experts (the regime the paper reports) counts of 17..32 are common
     const int mean_load = (int)(((size_t)T * K + E - 1) / E);
-    // (how many of the residents will have tokens is not known yet: the layer's previous
-    // execution is the estimate - adjacent iterations activate mostly the same experts, Sec. 3.3)
-    const int expected = std::min<int>(grp.n, L.last_active >= 0 ? L.last_active : E);
     // (direct fp8 form: its token operand is two rows per token and a third of a stage at 32, so
     // where the layer's previous execution gave no expert more than 16 rows the tile is 16)
     const int floor_rows = ctx->step_split != nullptr && L.last_max_count >= 0 && L.last_max_count <= 16 ? 16 : 32;
     const int rc0 = run_ffn_launches(ctx, grp, std::min(T, std::max(floor_rows, 2 * mean_load)), nullptr, nullptr, false,
-                                     expected, &ctx->hit_fused, rep);
+                                     &ctx->hit_fused, rep);
     if (rc0 != OLED_OK) return rc0;
   }
 
@@ -926,7 +1002,7 @@ static int step_impl(oled_ctx* ctx, int32_t layer, const void* hidden, const flo
     ctx->pending.valid = true;
     ctx->pending.T = T;
     ctx->pending.gate = ctx->d_gate;
-    ctx->pending.pos = ctx->d_pos;
+    ctx->pending.pos = scattered ? nullptr : ctx->d_pos;
     ctx->pending.x = static_cast<const uint16_t*>(hidden);
     ctx->pending.out = static_cast<uint16_t*>(out);
     ctx->pending.x_next = static_cast<uint16_t*>(x_next);
@@ -936,7 +1012,7 @@ static int step_impl(oled_ctx* ctx, int32_t layer, const void* hidden, const flo
     {
       ProfScope ps(ctx, OLED_KERNEL_COMBINE, (uint64_t)T * K * H * (ctx->y_bf16 ? 2 : 4) + (uint64_t)T * H * 2,
                    2ull * T * K * H);
-      launch_combine(st, ctx->d_y, ctx->y_bf16 ? 1 : 0, ctx->d_gate, ctx->d_pos, T, H, K, static_cast<uint16_t*>(out),
+      launch_combine(st, ctx->d_y, ctx->y_bf16 ? 1 : 0, ctx->d_gate, scattered ? nullptr : ctx->d_pos, T, H, K, static_cast<uint16_t*>(out),
                      static_cast<const uint16_t*>(hidden), static_cast<uint16_t*>(x_next),
                      reinterpret_cast<uint32_t*>(ctx->d_scores), (int)(ctx->ctrl_bytes / 4), tl);
     }
@@ -1006,6 +1082,9 @@ int oled_denoise_step_host(oled_ctx* ctx, int32_t layer, const void* host_hidden
 // kernel.  A prefetch only: what the gate then decides changes nothing but the hit rate in L2.
 static int prefetch_next_layer(oled_ctx* ctx, int32_t next) {
   if (!ctx->l2_prefetch || ctx->ffn_impl != 0) return OLED_OK;
+  // (few-token steps: the FFN kernel itself loads on a guess, and a prefetch between two layers costs the
+  // early launch of the next gate kernel: 2158 against 2138 us for 16 layers of 63 experts)
+  if (ctx->scatter.cap > 0 && ctx->l2_prefetch != 2) return OLED_OK;
   const LayerData& N = ctx->layers[next];
   if (N.last_misses != 0 || (int32_t)N.last_counts.size() != ctx->shape.n_experts) return OLED_OK;
   constexpr size_t kPrefetchBytes = 64u << 20;  // about what the HBM delivers during gate + permutation (32-96 MB measured alike, more costs)
@@ -1125,6 +1204,8 @@ int oled_debug_last(oled_ctx* ctx, int32_t layer, int32_t* ids, float* gate, int
   if (rc != OLED_OK && rc != OLED_ERR_TIMEOUT) return rc;
   const size_t n = (size_t)ctx->last_tokens * ctx->shape.top_k, E = (size_t)ctx->shape.n_experts;
   if (n > 0) {
+    const int rcp = perm ? make_perm(ctx) : OLED_OK;
+    if (rcp != OLED_OK) return rcp;
     if (ids) OLED_CUDA(ctx, cudaMemcpy(ids, ctx->d_ids, n * sizeof(int32_t), cudaMemcpyDeviceToHost));
     if (gate) OLED_CUDA(ctx, cudaMemcpy(gate, ctx->d_gate, n * sizeof(float), cudaMemcpyDeviceToHost));
     if (perm) OLED_CUDA(ctx, cudaMemcpy(perm, ctx->d_perm, n * sizeof(int32_t), cudaMemcpyDeviceToHost));
@@ -1146,6 +1227,8 @@ int oled_debug_perm(oled_ctx* ctx, int32_t layer, int32_t* offsets, int32_t* pos
   if (rc != OLED_OK && rc != OLED_ERR_TIMEOUT) return rc;
   const size_t n = (size_t)ctx->last_tokens * ctx->shape.top_k, E = (size_t)ctx->shape.n_experts;
   if (n > 0) {
+    const int rcp = make_perm(ctx);
+    if (rcp != OLED_OK) return rcp;
     if (offsets) OLED_CUDA(ctx, cudaMemcpy(offsets, ctx->d_offsets, (E + 1) * sizeof(int32_t), cudaMemcpyDeviceToHost));
     if (pos) OLED_CUDA(ctx, cudaMemcpy(pos, ctx->d_pos, n * sizeof(int32_t), cudaMemcpyDeviceToHost));
   } else if (offsets) {

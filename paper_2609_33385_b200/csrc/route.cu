@@ -113,7 +113,7 @@ __device__ __forceinline__ void combine_rows(const CombinePrev& p, int t0, int n
   // the small operands of all rows first (one round trip), then row after row
   for (int i = threadIdx.x; i < n_rows * K; i += blockDim.x) {
     s_g_all[i] = p.gate[(size_t)t0 * K + i];
-    s_r_all[i] = p.pos[(size_t)t0 * K + i];
+    s_r_all[i] = p.pos != nullptr ? p.pos[(size_t)t0 * K + i] : t0 * K + i;
   }
   __syncthreads();
   for (int row = 0; row < n_rows; ++row) {
@@ -177,7 +177,8 @@ route_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ wr,
              const float* __restrict__ bias, const float* __restrict__ conf, int T, int H, int E,
              int K, float* __restrict__ logits_out, int32_t* __restrict__ ids,
              float* __restrict__ gate, int32_t* __restrict__ counts,
-             unsigned long long* __restrict__ scores, CombinePrev prev, StepTimeline* timeline) {
+             unsigned long long* __restrict__ scores, CombinePrev prev, StepTimeline* timeline,
+             const __grid_constant__ ScatterRows scatter) {
   extern __shared__ __align__(16) uint8_t s_dyn[];
   float* s_logits = reinterpret_cast<float*>(s_dyn);                       // [TT][E]
   constexpr bool staged = TT <= 4;
@@ -188,6 +189,7 @@ route_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ wr,
   __shared__ float s_sel_logit[kST][OLED_MAX_TOPK];
   __shared__ float s_g[kST * OLED_MAX_TOPK];
   __shared__ int s_r[kST * OLED_MAX_TOPK];
+  __shared__ uint32_t s_amax[kST];  // fp8 stores: the rows' largest magnitudes (bf16 bits)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t0 = blockIdx.x * TT;
   griddep_launch_dependents();
@@ -218,7 +220,19 @@ route_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ wr,
       for (int c = threadIdx.x; c < my_tokens * (H / 8); c += blockDim.x)
         reinterpret_cast<uint4*>(s_x)[c] = reinterpret_cast<const uint4*>(x + (size_t)t0 * H)[c];
     }
+    if (threadIdx.x < kST) s_amax[threadIdx.x] = 0u;
     __syncthreads();
+    if (scatter.split.amax_in != nullptr)
+      for (int a = 0; a < my_tokens; ++a) {
+        uint32_t big = 0u;
+        for (int c = threadIdx.x; c < H / 8; c += blockDim.x) {
+          const uint4 v = reinterpret_cast<const uint4*>(s_x + (size_t)a * H)[c];
+          big = __vmaxu2(__vmaxu2(big, __vmaxu2(v.x & 0x7fff7fffu, v.y & 0x7fff7fffu)),
+                         __vmaxu2(v.z & 0x7fff7fffu, v.w & 0x7fff7fffu));
+        }
+        big = __reduce_max_sync(0xffffffffu, max(big & 0xffffu, big >> 16));
+        if (lane == 0 && big != 0u) atomicMax(&s_amax[a], big);
+      }
   }
 
   for (int eb = warp * kEPerWarp; eb < E; eb += kRouteWarps * kEPerWarp) {
@@ -291,7 +305,22 @@ route_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ wr,
       }
     }
     __syncthreads();
-    for (int a = warp; a < my_tokens; a += kRouteWarps) {
+    // scattered steps: every assignment of the CTA's tokens takes a row of its expert (the last warps
+    // turn the selected logits into gate scores meanwhile)
+    if (scatter.cap > 0) {
+      for (int i = threadIdx.x; i < my_tokens * K; i += blockDim.x) {
+        const int a = i / K, e = s_sel_id[a][i - a * K];
+        const int row = e * scatter.cap + atomicAdd(&counts[e], 1);
+        s_r[i] = row;
+        scatter.assignment[row] = t0 * K + i;
+        if (scatter.split.amax_in != nullptr) {
+          // (dense steps: the input rows are the tokens', the intermediate rows the first T * K)
+          scatter.split.amax_in[scatter.dense ? t0 + a : row] = s_amax[a] << 16;
+          scatter.split.amax_mid[scatter.dense ? t0 * K + i : row] = 0u;
+        }
+      }
+    }
+    for (int a = kRouteWarps - 1 - warp; a < my_tokens; a += kRouteWarps) {
       const int t = t0 + a;
       const int my_id = lane < K ? s_sel_id[a][lane] : 0;
       const float my_logit = lane < K ? s_sel_logit[a][lane] : 0.0f;
@@ -303,8 +332,30 @@ route_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ wr,
         const float g = __fdiv_rn(z, sum);
         ids[(size_t)t * K + lane] = my_id;
         gate[(size_t)t * K + lane] = g;
-        atomicAdd(&counts[my_id], 1);
+        if (scatter.cap == 0) atomicAdd(&counts[my_id], 1);
         atomicAdd(&scores[my_id], score_quantum(g, conf[t]));
+      }
+    }
+    if (scatter.cap > 0) {
+      __syncthreads();  // the rows of all assignments are known
+      const int vec_per_row = H / 8, total = my_tokens * vec_per_row;
+      for (int i = threadIdx.x; i < total; i += blockDim.x) {
+        const int a = i / vec_per_row, c = i - a * vec_per_row;
+        const uint4 v = reinterpret_cast<const uint4*>(s_x)[i];
+        uint2 t1 = make_uint2(0u, 0u), t2 = t1;
+        if (scatter.split.amax_in != nullptr) {
+          const float scale = token_scale(s_amax[a] << 16);
+          split_bf16x4(v.x, v.y, scale, t1.x, t2.x);
+          split_bf16x4(v.z, v.w, scale, t1.y, t2.y);
+        }
+        for (int j = 0; j < (scatter.dense ? 1 : K); ++j) {
+          const size_t row = scatter.dense ? (size_t)(t0 + a) : (size_t)s_r[a * K + j];
+          reinterpret_cast<uint4*>(scatter.xp)[row * vec_per_row + c] = v;
+          if (scatter.split.amax_in != nullptr) {
+            reinterpret_cast<uint2*>(scatter.split.terms_in)[row * vec_per_row + c] = t1;
+            reinterpret_cast<uint2*>(scatter.split.terms_in)[((size_t)scatter.split.rows + row) * vec_per_row + c] = t2;
+          }
+        }
       }
     }
   } else {
@@ -687,7 +738,7 @@ bool route_can_take_combine(int T) { return T <= kRouteSmallMax; }
 void launch_route(cudaStream_t st, const uint16_t* x, const uint16_t* w_router, const float* bias,
                   const float* conf, int T, int H, int E, int K, float* logits, int32_t* ids,
                   float* gate, int32_t* counts, unsigned long long* scores, const CombinePrev& prev,
-                  StepTimeline* timeline, int32_t* seg_counts, int seg_tokens) {
+                  StepTimeline* timeline, int32_t* seg_counts, int seg_tokens, const ScatterRows& scatter) {
   if (T <= kRouteSmallMax) {
     constexpr int W = 16;
     static bool attr_done = false;
@@ -701,13 +752,13 @@ void launch_route(cudaStream_t st, const uint16_t* x, const uint16_t* w_router, 
     auto smem = [&](int tt) { return ((((size_t)tt * E * sizeof(float)) + 15) & ~(size_t)15) + (size_t)tt * H * 2; };
     if (T <= 148)
       launch_pdl(route_kernel<1, W, 4, 4>, dim3(T), dim3(W * 32), smem(1), st, x, w_router, bias, conf, T, H, E, K,
-                 logits, ids, gate, counts, scores, prev, timeline);
+                 logits, ids, gate, counts, scores, prev, timeline, scatter);
     else if (T <= 296)  // (four tokens per CTA measured slower at 256 tokens x 128 experts: 33 against 20 us)
       launch_pdl(route_kernel<2, W, 4, 4>, dim3((T + 1) / 2), dim3(W * 32), smem(2), st, x, w_router, bias, conf, T, H,
-                 E, K, logits, ids, gate, counts, scores, prev, timeline);
+                 E, K, logits, ids, gate, counts, scores, prev, timeline, scatter);
     else
       launch_pdl(route_kernel<4, W, 2, 4>, dim3((T + 3) / 4), dim3(W * 32), smem(4), st, x, w_router, bias, conf, T, H,
-                 E, K, logits, ids, gate, counts, scores, prev, timeline);
+                 E, K, logits, ids, gate, counts, scores, prev, timeline, scatter);
   } else {
     // (re-tilings of the plain kernel - more tokens or experts per warp, more warps per CTA, deeper
     // unrolling - were all slower at 4096 tokens x 64 experts x 4096)

@@ -843,3 +843,28 @@ def test_one_launch_and_two_launch_ffn_forms_agree_bit_for_bit():
             run.close()
     for a, b in zip(outs[0], outs[2]):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("fp8", [False, True], ids=["bf16", "fp8"])
+@pytest.mark.parametrize("n_experts,top_k,hidden,inter", [(20, 3, 512, 384), (6, 6, 256, 128), (512, 2, 256, 128)])
+def test_few_token_steps_at_the_edges_of_their_forms(n_experts, top_k, hidden, inter, fp8):
+    """Steps of 1..32 tokens (every expert multiplies with the step's rows as they are), beyond (rows
+    copied to their experts' regions; 512 experts x 65 tokens: too many, sorted rows), token tiles of 16 and
+    32, weights loaded on the guess that the previous execution's experts return - right for a repeated
+    input, wrong for the next one, where a run of nearly equal tokens leaves most experts without any."""
+    from paper_2609_33385_b200.runner import bits_to_dev
+    w = synth.tiny(n_layers=1, n_experts=n_experts, top_k=top_k, hidden=hidden, intermediate=inter)
+    run = _runner(w, capacity=[n_experts], max_tokens=65, fp8=fp8)
+    ora = _oracle_for(run, [n_experts])
+    try:
+        for rep, n in enumerate((65, 32, 32, 17, 16, 1, 31, 33, 2, 64)):
+            h_bits, conf = synth.flat_tokens(w, n, 200 + rep // 2)
+            if rep % 3 == 1:
+                h_bits[:] = h_bits[0]
+            x, c = bits_to_dev(h_bits, run.device), torch.from_numpy(conf).to(run.device)
+            out = torch.empty((n, w.hidden), dtype=torch.bfloat16, device=run.device)
+            run.step(0, x, c, out)
+            _check_step(run, 0, n, out, ora.denoise_step(0, h_bits, conf))
+        _check_stats(run, ora)
+    finally:
+        run.close()
