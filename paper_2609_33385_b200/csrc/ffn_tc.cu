@@ -791,22 +791,8 @@ int ffn_tc_setup(FfnTcMaps* maps, const uint8_t* pool, size_t slot_bytes, int n_
     const cuuint32_t box[3] = {kBlockK, kBlockM, 1};
     if (!encode_tensor_map(&maps->w2, 3, pool + (size_t)2 * I * H * esz, dims, strides, box, fp8, fp8)) return OLED_ERR_CUDA;
   }
-  // fp8 stores: maps for the form whose MMAs read the codes themselves - k-blocks of 128 bytes
-  maps->e4m3_direct = fp8 && H % 128 == 0 && I % 128 == 0 && split != nullptr && split->complete() && split->rows == rows;
-  if (maps->e4m3_direct) {
-    for (int i = 0; i < 2; ++i) {
-      const cuuint32_t tbox[3] = {128, (cuuint32_t)(16 << i), 2};
-      const cuuint64_t dims_in[3] = {(cuuint64_t)H, (cuuint64_t)rows, 2}, dims_mid[3] = {(cuuint64_t)I, (cuuint64_t)rows, 2};
-      const cuuint64_t str_in[2] = {(cuuint64_t)H, (cuuint64_t)rows * H}, str_mid[2] = {(cuuint64_t)I, (cuuint64_t)rows * I};
-      if (!encode_tensor_map(&maps->xp_terms[i], 3, split->terms_in, dims_in, str_in, tbox, true)) return OLED_ERR_CUDA;
-      if (!encode_tensor_map(&maps->hbuf_terms[i], 3, split->terms_mid, dims_mid, str_mid, tbox, true)) return OLED_ERR_CUDA;
-    }
-    const cuuint32_t box[3] = {128, kBlockM, 1};
-    const cuuint64_t dims2[3] = {(cuuint64_t)I, (cuuint64_t)H, (cuuint64_t)n_slots};
-    const cuuint64_t strides2[2] = {(cuuint64_t)I, (cuuint64_t)slot_bytes};
-    if (!encode_tensor_map(&maps->w2_e4m3, 3, pool + (size_t)2 * I * H, dims2, strides2, box, true)) return OLED_ERR_CUDA;
-  }
-  if (const int rc = ffn_few_setup(maps, pool, slot_bytes, n_slots, H, I, fp8); rc != OLED_OK) return rc;
+  if (!fp8 || (split != nullptr && split->complete() && split->rows == rows))
+    if (const int rc = ffn_few_setup(maps, pool, slot_bytes, n_slots, H, I, fp8, xp, hbuf, rows, split); rc != OLED_OK) return rc;
   for (int i = 0; i < 5; ++i) {
     const cuuint32_t box[2] = {kBlockK, (cuuint32_t)(16 << i)};
     {
@@ -836,6 +822,15 @@ static int box_index(int max_count, int cap) {
   return i;
 }
 
+// Token tiles of at most kFewMaxRows rows go to ffn_few.cu (4 layers of 64 experts, us, against the two-accumulator
+// tiles here: 300 tokens 635 / 707, 512 tokens 701 / 773; beyond 128 rows the operand traffic of its single weight
+// tile costs more than it saves: 1000 tokens 1035 against 926 on CTA pairs).  Of fp8 stores every tile does, provided
+// the rows' e4m3 terms are at hand (8 layers of 250 tokens: 907 / 1459); otherwise converter warps widen the codes.
+static bool few_form(const FfnTcMaps& maps, int max_count, const TokenSplit* split) {
+  if (!maps.few) return false;
+  return maps.fp8 ? split != nullptr && split->complete() : max_count <= kFewMaxRows;
+}
+
 int launch_ffn_tc(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp_in, int max_count, int kind,
                   const int32_t* host_counts, const FfnRows& rows, uint16_t* hbuf, float* y, int y_bf16, int H, int I,
                   int n_sms, uint32_t* status, uint32_t* work_counter, bool behind_event_wait, StepTimeline* timeline,
@@ -849,12 +844,9 @@ int launch_ffn_tc(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp_in
   // (fp8 stores stop at N = 128: the widened weights need tensor-memory columns of their own)
   const int ib = box_index(max_count, fp8 ? 128 : 256);
   grp.n_box = 16 << ib;
-  // fp8 stores, token tiles of at most 32 rows, the rows' terms at hand: the MMAs read the codes
-  // themselves (ffn_few.cu); otherwise converter warps widen them to bf16
-  const bool direct = fp8 && maps.e4m3_direct && grp.n_box <= 32 && split != nullptr && split->complete();
-  if (direct || (!fp8 && grp.n_box <= 32))
-    return launch_ffn_few(st, maps, grp, ib, kind, host_counts, rows, hbuf, y, H, I, n_sms, status, work_counter,
-                          behind_event_wait, timeline, timeline_slot, report, done, split);
+  if (few_form(maps, max_count, split))
+    return launch_ffn_few(st, maps, grp, max_count, kind, host_counts, rows, hbuf, y, y_bf16, H, I, n_sms, status,
+                          work_counter, behind_event_wait, timeline, timeline_slot, report, done, split);
   // many-token tiles: the CTA-pair kernel, unless its cluster launch has failed before on this
   // device (the one-CTA form below computes the same)
   if (maps.use_pairs && !g_pairs_refused && ffn_pair_usable(maps, grp.n_box, H, I)) {
@@ -929,16 +921,13 @@ void ffn_tc_set_token_source(FfnTcMaps* maps, const uint16_t* x, int T, const in
 void ffn_tc_clear_token_source(FfnTcMaps* maps) { maps->token_source.perm = nullptr; }
 
 int ffn_tc_launches(const FfnTcMaps& maps, int max_count, int kind, const TokenSplit* split) {
-  const bool direct = maps.fp8 && maps.e4m3_direct && (16 << box_index(max_count, 128)) <= 32 && split != nullptr &&
-                      split->complete();
-  return kind == 2 && direct ? 2 : 1;
+  return kind == 2 && maps.fp8 && few_form(maps, max_count, split) ? 2 : 1;
 }
 
-bool ffn_tc_can_fuse(const FfnTcMaps& maps, int max_count) {
-  return !maps.fp8 && (16 << box_index(max_count, 256)) <= 32;
-}
+bool ffn_tc_can_fuse(const FfnTcMaps& maps, int max_count) { return !maps.fp8 && few_form(maps, max_count, nullptr); }
 bool ffn_pair_can_fuse(const FfnTcMaps& maps, int max_count, int H, int I) {
-  return maps.use_pairs && !g_pairs_refused && ffn_pair_usable(maps, 16 << box_index(max_count, maps.fp8 ? 128 : 256), H, I);
+  return !few_form(maps, max_count, nullptr) && maps.use_pairs && !g_pairs_refused &&
+         ffn_pair_usable(maps, 16 << box_index(max_count, maps.fp8 ? 128 : 256), H, I);
 }
 
 }  // namespace oled

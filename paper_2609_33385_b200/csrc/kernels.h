@@ -244,12 +244,8 @@ void launch_ffn_simple(cudaStream_t st, const FfnGroup& grp, const uint8_t* pool
 
 // ---- ffn_tc.cu (tcgen05 / TMEM / TMA) ------------------------------------------------------
 struct FfnTcMaps {
-  CUtensorMap w13_few;        // gate/up rows of 64 features as four groups of 16 gate and 16 up rows (ffn_few.cu)
-  CUtensorMap w13_few_e4m3;   // the same over e4m3 codes
-  CUtensorMap w2_e4m3;        // fp8 stores: [slots][H][I] bytes, box {128,128,1}, 128-byte swizzle
-  CUtensorMap xp_terms[2];    // [2][rows][H] bytes (TokenSplit::terms_in), box {128, 16<<i, 2}
-  CUtensorMap hbuf_terms[2];  // [2][rows][I] bytes (TokenSplit::terms_mid), box {128, 16<<i, 2}
-  bool e4m3_direct = false;   // the maps above exist (fp8 stores, H and I multiples of 128, term buffers given)
+  CUtensorMap few_w1, few_w2, few_x[3], few_h[3];  // the maps of ffn_few.cu (fp8 stores: over codes and token terms)
+  bool few = false;                                // ... exist
   CUtensorMap w13;       // [slots][2I][H] bf16, box {64,128,1}
   CUtensorMap w13_half;  // fp8 stores, widening form: the same, box {64,64,1}
   CUtensorMap w2;        // [slots][H][I]  bf16, box {64,128,1}
@@ -314,11 +310,13 @@ constexpr int kFfnWorkCounters = 8;  // FFN launches of one layer execution: 3 g
 // A tensor map over bf16 elements (bytes: over bytes) with the 128-byte swizzle (narrow: the 64-byte one).
 bool encode_tensor_map(CUtensorMap* m, int rank, const void* base, const cuuint64_t* dims, const cuuint64_t* strides,
                        const cuuint32_t* box, bool bytes = false, bool narrow = false);
-// ---- ffn_few.cu: token tiles of at most 32 rows (bf16 stores, or fp8 stores with the token terms at
-// hand).  Kinds as above; kind 2 of fp8 stores is preceded by the split kernel.
-int ffn_few_setup(FfnTcMaps* maps, const uint8_t* pool, size_t slot_bytes, int n_slots, int H, int I, bool fp8);
-int launch_ffn_few(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp, int box_index, int kind,
-                   const int32_t* host_counts, const FfnRows& rows, uint16_t* hbuf, float* y, int H, int I, int n_sms,
+// ---- ffn_few.cu: token tiles of at most kFewMaxRows rows (bf16 stores, or fp8 stores with the token
+// terms at hand).  Kinds as above; kind 2 of fp8 stores is preceded by the split kernel.
+constexpr int kFewMaxRows = 128;  // the largest token tile of ffn_few.cu
+int ffn_few_setup(FfnTcMaps* maps, const uint8_t* pool, size_t slot_bytes, int n_slots, int H, int I, bool fp8,
+                  const uint16_t* xp, const uint16_t* hbuf, int rows, const TokenSplit* split);
+int launch_ffn_few(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp, int max_count, int kind,
+                   const int32_t* host_counts, const FfnRows& rows, uint16_t* hbuf, float* y, int y_bf16, int H, int I, int n_sms,
                    uint32_t* status, uint32_t* work_counter, bool behind_event_wait, StepTimeline* timeline,
                    int timeline_slot, const RouteReport& report, uint32_t* done, const TokenSplit* split);
 

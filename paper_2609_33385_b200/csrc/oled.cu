@@ -447,13 +447,13 @@ int run_ffn_launches(oled_ctx* ctx, const FfnGroup& grp, int max_count, const in
       ctx->maps.token_source.ready = ready;
       ctx->work_next += 1;
       FfnRows rows;
+      rows.E = ctx->shape.n_experts;
       if (ctx->scatter.cap > 0) {
         rows.counts = ctx->d_counts;
         rows.assignment = ctx->d_assignment;
         rows.cap = ctx->scatter.cap;
         rows.dense = ctx->scatter.dense;
         rows.K = ctx->shape.top_k;
-        rows.E = ctx->shape.n_experts;
       } else {
         rows.offsets = ctx->d_offsets;
       }
@@ -894,15 +894,13 @@ static int step_impl(oled_ctx* ctx, int32_t layer, const void* hidden, const flo
       }
       if (pass == 0) grp.n_guess = grp.n;
     }
-    // token tile of this launch (the counts are not known on the host yet): twice the mean load
-    // per expert, but at least 32 rows - an expert that received more rows than the tile holds
-    // has its weights streamed once per tile, and in a block of 32 tokens whose routing is
-    // concentrated on few experts (the regime the paper reports) counts of 17..32 are common
+    // Token tile of this launch (the counts are not known on the host yet): the most rows an expert received at
+    // the layer's previous execution and an eighth, at most twice the mean load per expert (a few heavily loaded
+    // experts take several tiles).  An expert that receives more rows than the tile holds has its weights
+    // streamed once per tile, a tile that is too large costs pipeline stages.
     const int mean_load = (int)(((size_t)T * K + E - 1) / E);
-    // (direct fp8 form: its token operand is two rows per token and a third of a stage at 32, so
-    // where the layer's previous execution gave no expert more than 16 rows the tile is 16)
-    const int floor_rows = ctx->step_split != nullptr && L.last_max_count >= 0 && L.last_max_count <= 16 ? 16 : 32;
-    const int rc0 = run_ffn_launches(ctx, grp, std::min(T, std::max(floor_rows, 2 * mean_load)), nullptr, nullptr, false,
+    const int seen = L.last_max_count >= 0 ? L.last_max_count + (L.last_max_count + 7) / 8 : T;
+    const int rc0 = run_ffn_launches(ctx, grp, std::min(T, std::min(seen, std::max(32, 2 * mean_load))), nullptr, nullptr, false,
                                      &ctx->hit_fused, rep);
     if (rc0 != OLED_OK) return rc0;
   }

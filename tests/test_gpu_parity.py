@@ -868,3 +868,24 @@ def test_few_token_steps_at_the_edges_of_their_forms(n_experts, top_k, hidden, i
         _check_stats(run, ora)
     finally:
         run.close()
+
+
+@pytest.mark.parametrize("fp8", [False, True], ids=["bf16", "fp8"])
+@pytest.mark.parametrize("n_experts,top_k,counts", [(4, 1, (150, 200, 260, 520)), (10, 4, (120, 130, 250)), (512, 8, (600,))])
+def test_token_tiles_between_16_and_128_rows(n_experts, top_k, counts, fp8):
+    """Items of 48, 64, 96 and 128 token rows and several tiles per expert, with the tile taken from the previous
+    execution's counts; 512 experts x 600 tokens: small tiles in a many-token step (bf16 outputs per assignment)."""
+    from paper_2609_33385_b200.runner import bits_to_dev
+    w = synth.tiny(n_layers=1, n_experts=n_experts, top_k=top_k, hidden=256, intermediate=128)
+    run = _runner(w, capacity=[n_experts], max_tokens=max(counts), fp8=fp8)
+    ora = _oracle_for(run, [n_experts])
+    try:
+        for rep, n in enumerate(counts + counts[:1]):
+            h_bits, conf = synth.flat_tokens(w, n, 300 + rep)
+            x, c = bits_to_dev(h_bits, run.device), torch.from_numpy(conf).to(run.device)
+            out = torch.empty((n, w.hidden), dtype=torch.bfloat16, device=run.device)
+            run.step(0, x, c, out)
+            _check_step(run, 0, n, out, ora.denoise_step(0, h_bits, conf))
+        _check_stats(run, ora)
+    finally:
+        run.close()
