@@ -72,6 +72,14 @@ __device__ __forceinline__ void tma_load_3d(const CUtensorMap* map, uint32_t dst
       ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
       : "memory");
 }
+// The same with an L2 cache policy.
+__device__ __forceinline__ void tma_load_3d_hint(const CUtensorMap* map, uint32_t dst, uint32_t bar, int c0, int c1,
+                                                 int c2, uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4, %5}], [%2], %6;"
+      ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "l"(policy)
+      : "memory");
+}
 __device__ __forceinline__ void tma_load_4d(const CUtensorMap* map, uint32_t dst, uint32_t bar, int c0,
                                             int c1, int c2, int c3) {
   asm volatile(
