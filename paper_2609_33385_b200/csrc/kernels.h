@@ -184,7 +184,7 @@ void launch_route(cudaStream_t st, const uint16_t* x, const uint16_t* w_router, 
                   StepTimeline* timeline, int32_t* seg_counts = nullptr, int seg_tokens = 0,
                   const ScatterRows& scatter = ScatterRows{});
 // Does the gate kernel of a T-token step carry out a CombinePrev and a ScatterRows?
-bool route_can_take_combine(int T);
+bool route_staged(int T, int K);
 constexpr int kDenseTokens = 32;
 // Where the FFN finds an expert's token rows: offsets[e] .. offsets[e + 1] - 1 (sorted steps), or
 // e * cap .. e * cap + counts[e] - 1 (scattered steps, offsets == nullptr; the output of row r then

@@ -746,7 +746,9 @@ static int step_impl(oled_ctx* ctx, int32_t layer, const void* hidden, const flo
     return OLED_OK;
   }
 
-  pdl_set_step((size_t)T * K <= 4096);
+  // (4 layers, 64 experts x 2048, dependent launch off / on: 600 tokens 814 / 781 us, 1000 tokens 908 / 867; 2 layers of
+  // 2048 tokens 677 / 668; at 4096 tokens no difference beyond the noise)
+  pdl_set_step((size_t)T * K <= 16384);
   // per-assignment outputs y: fp32 for small steps; bf16 once y's traffic matters (the rounding
   // adds at most 2^-9 relative per term, far inside the output tolerance)
   ctx->y_bf16 = ctx->ffn_impl == 0 && (size_t)T * K > 4096;
@@ -772,14 +774,14 @@ static int step_impl(oled_ctx* ctx, int32_t layer, const void* hidden, const flo
   }
   // many-token steps: the gate kernel counts every expert's assignments per segment of the token
   // range, and the permutation kernel then scans the segments in parallel
-  int32_t* const seg_counts = (size_t)T * K > 4096 && !route_can_take_combine(T) ? ctx->d_seg : nullptr;
+  int32_t* const seg_counts = (size_t)T * K > 4096 && !route_staged(T, K) ? ctx->d_seg : nullptr;
   const int seg_tokens = ((T + kPermuteSegments - 1) / kPermuteSegments + 3) / 4 * 4;
   // the current step's gate-score and inverse-permutation buffers (the previous step's stay
   // intact for a combine that has been left to this step's gate kernel)
   ctx->buf_sel ^= 1;
   ctx->d_gate = ctx->d_gate_buf[ctx->buf_sel];
   ctx->d_pos = ctx->d_pos_buf[ctx->buf_sel];
-  const bool fuse_prev = ctx->pending.valid && ctx->pending.T == T && route_can_take_combine(T) &&
+  const bool fuse_prev = ctx->pending.valid && ctx->pending.T == T && route_staged(T, K) &&
                          ctx->pending.x_next == static_cast<const uint16_t*>(hidden);
   if (ctx->pending.valid && !fuse_prev) {
     const int rcp = flush_pending_combine(ctx);
@@ -791,7 +793,7 @@ static int step_impl(oled_ctx* ctx, int32_t layer, const void* hidden, const flo
   ctx->scatter = ScatterRows{};
   ctx->perm_stale = false;
   ctx->step_split = nullptr;
-  if (few && route_can_take_combine(T) && (size_t)E * scatter_cap(T) <= ctx->row_buf && ctx->ffn_impl == 0 &&
+  if (few && route_staged(T, K) && (size_t)E * scatter_cap(T) <= ctx->row_buf && ctx->ffn_impl == 0 &&
       !ctx->corrupt_perm) {
     ctx->scatter.cap = (int)scatter_cap(T);
     ctx->scatter.assignment = ctx->d_assignment;
@@ -835,6 +837,10 @@ static int step_impl(oled_ctx* ctx, int32_t layer, const void* hidden, const flo
   const bool gather_in_ffn = !fuse_gather && ctx->gather_in_ffn && ctx->ffn_impl == 0 &&
                              std::min<size_t>(T, 2 * (((size_t)T * K + E - 1) / E)) > 128 &&
                              (reinterpret_cast<uintptr_t>(hidden) & 15u) == 0 &&  // (bulk copies of whole rows)
+                             // (a row's copy - loads, stores, fence and count on one thread - takes as long as 4 M
+                             // elements of an expert matrix take the tensor cores; measured with / without: 2 layers
+                             // of 2048 tokens, H x I 2 M: 875 / 654 us, one of 4096 tokens, 6 M: 1372 / 1418 us)
+                             (size_t)H * ctx->shape.intermediate >= (size_t)4 << 20 &&
                              ffn_tc_token_source_usable(ctx->maps, H, ctx->shape.intermediate);
   if (gather_in_ffn)
     ffn_tc_set_token_source(&ctx->maps, static_cast<const uint16_t*>(hidden), T, ctx->d_perm, K, ctx->d_xp);
@@ -994,7 +1000,7 @@ static int step_impl(oled_ctx* ctx, int32_t layer, const void* hidden, const flo
   nv_ffn_miss.end();
   NvtxRange nv_comb(ctx, "oled.step.4_combine");
   // 5. combine - or, inside a stack iteration of few-token steps, left to the next layer's gate kernel
-  const bool defer = defer_combine && ctx->fuse_combine && route_can_take_combine(T) && x_next != nullptr &&
+  const bool defer = defer_combine && ctx->fuse_combine && route_staged(T, K) && x_next != nullptr &&
                      !ctx->y_bf16 && !ctx->self_check && ctx->ffn_impl == 0;
   if (defer) {
     ctx->pending.valid = true;
