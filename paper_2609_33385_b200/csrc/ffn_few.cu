@@ -38,7 +38,7 @@
 // fp8 expert stores (FP8): the MMAs are kind::f8f6f4 and read the e4m3 codes as they are; the token operand
 // is two e4m3 terms per row (fp8_split.h), the epilogue adds the two accumulators (D1 + D2 / 16), undoes the
 // row's power-of-two scale and applies the weight row's scale.  The input rows' terms come from the gate
-// kernel, those of the intermediate rows from split_rows_kernel between the two projections.  (An M = 128
+// kernel, those of the intermediate rows from four more warps per CTA (KIND 3) or from split_rows_kernel.  (An M = 128
 // instruction consumes 128 weight rows x 32 bytes whatever the element size; widening the codes to bf16 first
 // makes the thread that issues the MMAs the bound: 8 layers of 250 tokens 1459 us, now 907.)
 //
@@ -59,7 +59,8 @@ namespace {
 
 constexpr int kFewEpiWarps = 8;
 constexpr int kFewWeightWarp = kFewEpiWarps, kFewTokenWarp = kFewEpiWarps + 1, kFewMmaWarp = kFewEpiWarps + 2;
-constexpr int kFewThreads = (kFewEpiWarps + 3) * 32;
+constexpr int kFewSplitWarp = kFewEpiWarps + 3, kFewSplitWarps = 4;  // fp8 stores, KIND 3
+constexpr int few_threads(int kind, bool fp8) { return (kFewEpiWarps + 3 + (kind == 3 && fp8 ? kFewSplitWarps : 0)) * 32; }
 constexpr uint32_t kFewWTile = 128 * 128;  // a k-block of weights: 128 rows of 128 bytes (64 bf16 or 128 e4m3)
 constexpr int kFewMaxStages = 12;
 constexpr int kFewRing = 8;
@@ -110,11 +111,11 @@ struct FewArgs {
   int early;           // KIND 2: everything but hbuf is known to be older than this kernel's predecessor
   const uint8_t* pool;
   unsigned long long slot_bytes;
-  const uint32_t* amax_act;  // fp8: magnitudes of the token operand's rows (kind 1: input, kind 2: intermediate)
-  uint32_t* amax_out;        // fp8, kind 1: raised by the epilogue
+  TokenSplit split;          // fp8: the token operands' terms and magnitudes (amax_mid is raised by the gate/up epilogue)
   uint32_t* status;
   uint32_t* work_counter;    // zero at the start
-  uint32_t* done;            // KIND 3: per expert of the group, zero at the start
+  uint32_t* done;            // KIND 3: per expert of the group, zero at the start: epilogue warps that have stored its rows
+  uint32_t* split_done;      // KIND 3, fp8: the same for its intermediate rows whose terms have been stored
   StepTimeline* timeline;
   int timeline_slot;
   RouteReport report;
@@ -137,8 +138,31 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatil
   return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status)) != 0;
 }
 
+// One intermediate row (bf16, its largest magnitude final) as two e4m3 terms per element; thread `rank` of `n`.
+__device__ __forceinline__ void split_row(const uint16_t* hbuf, const TokenSplit& split, int row, int I, int rank, int n) {
+  const float scale = token_scale(__ldcg(split.amax_mid + row));
+  const uint4* src = reinterpret_cast<const uint4*>(hbuf + (size_t)row * I);
+  uint2* out1 = reinterpret_cast<uint2*>(split.terms_mid + (size_t)row * I);
+  uint2* out2 = reinterpret_cast<uint2*>(split.terms_mid + ((size_t)split.rows + row) * I);
+  for (int c0 = rank; c0 < I / 8; c0 += 4 * n) {  // (four loads in flight)
+    uint4 v[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (c0 + i * n < I / 8) v[i] = __ldcg(src + c0 + i * n);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (c0 + i * n < I / 8) {
+        uint2 t1, t2;
+        split_bf16x4(v[i].x, v[i].y, scale, t1.x, t2.x);
+        split_bf16x4(v[i].z, v[i].w, scale, t1.y, t2.y);
+        out1[c0 + i * n] = t1;
+        out2[c0 + i * n] = t2;
+      }
+  }
+}
+
 template <int KIND, bool FP8>
-__global__ void __launch_bounds__(kFewThreads, 1)
+__global__ void __launch_bounds__(few_threads(KIND, FP8), 1)
 ffn_few_kernel(const __grid_constant__ FewArgs p) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   FewCtl* ctl = reinterpret_cast<FewCtl*>(smem_raw);
@@ -147,7 +171,6 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
   const FfnGroup& grp = p.grp;
   const int n_box = grp.n_box, H = p.H, I = p.I;
   constexpr bool fused = KIND == 3;
-  static_assert(!(fused && FP8), "fp8 stores need the split kernel between the two projections");
   constexpr int kK = FP8 ? 128 : 64;  // k-values of a k-block
   const bool dense = p.rows.dense != 0;
   constexpr uint32_t kRowBytes = FP8 ? 256u : 128u;  // of a token row in a k-block (fp8: two terms)
@@ -232,6 +255,26 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
   const uint32_t tmem_base = ctl->tmem_base;
   // KIND 3: epilogue warps that store intermediate rows per gate/up item, times the items of a token tile
   const uint32_t done_per_tile = (uint32_t)(m_tiles1 * epi_warps);
+  auto done_target = [&](int g) { return done_per_tile * (uint32_t)(ctl->tile_prefix[g + 1] - ctl->tile_prefix[g]); };
+  // (a whole warp) waits until a counter in global memory has reached `target`
+  auto wait_count = [&](const uint32_t* counter, uint32_t target, uint32_t sleep_ns) {
+    unsigned long long t0 = 0;
+    for (uint32_t spin = 0;; ++spin) {
+      uint32_t seen;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(counter) : "memory");
+      if (__all_sync(0xffffffffu, seen >= target)) return true;
+      if (sleep_ns) __nanosleep(sleep_ns);
+      if ((spin & 255u) == 255u) {
+        const unsigned long long now = globaltimer();
+        if (t0 == 0) t0 = now;
+        if (now - t0 > kWaitLimitNs) {
+          *abort_flag = 1;
+          atomicExch(p.status, (uint32_t)kStatusWaitTimeout);
+        }
+        if (__any_sync(0xffffffffu, *abort_flag != 0)) return false;
+      }
+    }
+  };
   auto wait_table = [&]() { return warp_wait(smem_u32(&ctl->table), 0u, abort_flag, p.status); };
 
   if (warp == kFewWeightWarp) {
@@ -354,27 +397,8 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
         if (down) k_blocks = k_blocks2;
         row0 = dense && !down ? 0 : (loaded ? e * p.rows.cap : first_row(e)) + nt * n_box;
         if (fused && down && g != ready_g) {
-          // the intermediate rows of every token tile of this expert must be in memory
-          const uint32_t* flag = p.done + g;
-          const uint32_t target = done_per_tile * (uint32_t)(ctl->tile_prefix[g + 1] - ctl->tile_prefix[g]);
-          unsigned long long t0 = 0;
-          for (uint32_t spin = 0;; ++spin) {
-            uint32_t seen;
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(flag) : "memory");
-            if (__all_sync(0xffffffffu, seen >= target)) break;
-            if ((spin & 255u) == 255u) {
-              const unsigned long long now = globaltimer();
-              if (t0 == 0) t0 = now;
-              if (now - t0 > kWaitLimitNs) {
-                *abort_flag = 1;
-                atomicExch(p.status, (uint32_t)kStatusWaitTimeout);
-              }
-              if (__any_sync(0xffffffffu, *abort_flag != 0)) {
-                ok = false;
-                break;
-              }
-            }
-          }
+          // the intermediate rows of every token tile of this expert (fp8: their terms) must be in memory
+          ok = FP8 ? wait_count(p.split_done + g, (uint32_t)ctl->count[e], 0u) : wait_count(p.done + g, done_target(g), 0u);
           if (!ok) break;
           ready_g = g;
           // the rows were written through the generic proxy; the loads below read through the async proxy
@@ -464,6 +488,28 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
           stage = 0;
           phase ^= 1u;
         }
+      }
+    }
+  } else if (FP8 && fused && warp >= kFewSplitWarp) {
+    // ------------------------------------------------------------ terms of the intermediate rows (fp8, one launch)
+    // CTA b looks after expert b mod n of the group, together with the other CTAs of that number: as soon as all
+    // of its gate/up items are stored, the rows' magnitudes are final and the rows become two e4m3 terms each.  All
+    // gate/up items are handed out before the first down item, so that is over long before most down items need
+    // it, and the weight stream runs on.  (As a kernel between two launches it cost 8 of 80 us per layer of 32 tokens.)
+    if (wait_table() && !grp.withhold_loads) {
+      const int owners = max(1, (int)gridDim.x / grp.n);  // CTAs per expert
+      for (int g = (int)blockIdx.x % grp.n, part = (int)blockIdx.x / grp.n; g < grp.n && part < owners; g += (int)gridDim.x) {
+        const int e = grp.expert[g], count = ctl->count[e], row0 = first_row(e);
+        const int w = part * kFewSplitWarps + warp - kFewSplitWarp;
+        if (w >= count) continue;  // (no row of this expert is this warp's)
+        if (!wait_count(p.done + g, done_target(g), 500u)) break;
+        uint32_t mine = 0;
+        for (int r = w; r < count; r += owners * kFewSplitWarps, ++mine)
+          split_row(p.hbuf, p.split, row0 + r, I, lane, 32);
+        __threadfence();
+        asm volatile("fence.proxy.async;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) atomicAdd(p.split_done + g, mine);
       }
     }
   } else {
@@ -575,7 +621,7 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
             dst = __ldcg(p.rows.assignment + e * p.rows.cap + nt * n_box + my_col);
           }
         }
-        if (FP8) inv = row >= 0 ? token_scale_inverse(__ldcg(p.amax_act + (dense && !down ? my_col : row))) : 0.0f;
+        if (FP8) inv = row >= 0 ? token_scale_inverse(__ldcg(down ? p.split.amax_mid + row : p.split.amax_in + (dense ? my_col : row))) : 0.0f;
       };
       // fp8 stores: one fp32 scale per weight row behind the codes (s_gate[I] | s_up[I] | s_down[H])
       float s0 = 1.0f;
@@ -588,7 +634,10 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
       int c = (warp >> 2) * 16;
       int row = -1, dst = 0;
       float inv = 0.0f;
-      if (c < n) columns(c, row, dst, inv);  // (looked up while the MMAs still run)
+      // looked up while the MMAs still run - but the magnitudes of intermediate rows that this launch itself makes
+      // are final only once the item's MMAs are through
+      const bool ahead = !(FP8 && fused && down);
+      if (c < n && ahead) columns(c, row, dst, inv);
       int ready = 0;
       if (lane == 0) ready = mbar_wait(smem_u32(&ctl->tmem_full[acc]), acc_phase, abort_flag, p.status) ? 1 : 0;
       ready = __shfl_sync(0xffffffffu, ready, 0);
@@ -603,7 +652,7 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
           const int col0 = FP8 ? 2 * (c & ~(box - 1)) + (c & (box - 1)) : c;
           const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * acc_cols + col0);
           tmem_ld16(t_row, ra);
-          if (!first) columns(c, row, dst, inv);
+          if (!first || !ahead) columns(c, row, dst, inv);
           if (FP8) {  // D = (D1 + D2 / 16) / row scale of the token
             uint32_t rt[16];
             tmem_ld16(t_row + (uint32_t)box, rt);
@@ -657,7 +706,7 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
             const uint32_t top = max(mag[0], __shfl_xor_sync(0xffffffffu, mag[0], 1));
             // lane bits 3, 2, 1 = bits 2, 1, 0 of the column within the half
             const int r = __shfl_sync(0xffffffffu, row, (up_half ? 8 : 0) + ((lane >> 1) & 7));
-            if ((lane & 1) == 0 && r >= 0 && top != 0u) atomicMax(p.amax_out + r, top << 16);
+            if ((lane & 1) == 0 && r >= 0 && top != 0u) atomicMax(p.split.amax_mid + r, top << 16);
           }
         } else if (c < valid) {
           const size_t col = (size_t)(m * 128 + quarter * 32 + lane);
@@ -695,14 +744,13 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
   if (threadIdx.x == 0) timeline_end(p.timeline, p.timeline_slot);
 }
 
-// fp8 stores, between the two projections: the intermediate rows of the group's experts (bf16,
+// fp8 stores, between the two projections as two launches: the intermediate rows of the group's experts (bf16,
 // written by the gate/up epilogue together with every row's largest magnitude) as two e4m3 terms
 // per element.  Four CTAs per expert of the group (a quarter of the columns each); a warp takes a
 // row at a time.
 __global__ void __launch_bounds__(256)
 split_rows_kernel(const __grid_constant__ FfnGroup grp, const __grid_constant__ FfnRows rows,
-                  const uint16_t* __restrict__ hbuf, const uint32_t* __restrict__ amax_mid,
-                  uint8_t* __restrict__ terms_mid, int I, int rows_total) {
+                  const uint16_t* __restrict__ hbuf, const __grid_constant__ TokenSplit split, int I) {
   griddep_launch_dependents();
   griddep_wait();
   const int e = grp.expert[blockIdx.x];
@@ -714,20 +762,8 @@ split_rows_kernel(const __grid_constant__ FfnGroup grp, const __grid_constant__ 
     for (int i = lane; i < e; i += 32) first += rows.counts[i];
     first = __reduce_add_sync(0xffffffffu, first);
   }
-  for (int r = first + warp; r < first + count; r += 8) {
-    const float scale = token_scale(amax_mid[r]);
-    const uint4* src = reinterpret_cast<const uint4*>(hbuf + (size_t)r * I);
-    uint2* out1 = reinterpret_cast<uint2*>(terms_mid + (size_t)r * I);
-    uint2* out2 = reinterpret_cast<uint2*>(terms_mid + ((size_t)rows_total + r) * I);
-    for (int c = lane + 32 * (int)blockIdx.y; c < I / 8; c += 32 * (int)gridDim.y) {
-      const uint4 v = src[c];
-      uint2 t1, t2;
-      split_bf16x4(v.x, v.y, scale, t1.x, t2.x);
-      split_bf16x4(v.z, v.w, scale, t1.y, t2.y);
-      out1[c] = t1;
-      out2[c] = t2;
-    }
-  }
+  for (int r = first + warp; r < first + count; r += 8)
+    split_row(hbuf, split, r, I, lane + 32 * (int)blockIdx.y, 32 * (int)gridDim.y);
 }
 
 // Stage shape and count: two k-blocks per stage where at least four such stages fit and both contractions
@@ -784,6 +820,7 @@ int ffn_few_setup(FfnTcMaps* maps, const uint8_t* pool, size_t slot_bytes, int n
            cudaFuncSetAttribute(ffn_few_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFewSmemMax) == cudaSuccess &&
            cudaFuncSetAttribute(ffn_few_kernel<3, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFewSmemMax) == cudaSuccess &&
            cudaFuncSetAttribute(ffn_few_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFewSmemMax) == cudaSuccess &&
+           cudaFuncSetAttribute(ffn_few_kernel<3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFewSmemMax) == cudaSuccess &&
            cudaFuncSetAttribute(ffn_few_kernel<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFewSmemMax) == cudaSuccess;
   }();
   return attr_ok ? OLED_OK : OLED_ERR_CUDA;
@@ -792,9 +829,10 @@ int ffn_few_setup(FfnTcMaps* maps, const uint8_t* pool, size_t slot_bytes, int n
 int launch_ffn_few(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& group, int max_count, int kind,
                    const int32_t* host_counts, const FfnRows& rows, uint16_t* hbuf, float* y, int y_bf16, int H, int I, int n_sms,
                    uint32_t* status, uint32_t* work_counter, bool behind_event_wait, StepTimeline* timeline,
-                   int timeline_slot, const RouteReport& report, uint32_t* done, const TokenSplit* split) {
+                   int timeline_slot, const RouteReport& report, uint32_t* done, const TokenSplit* split,
+                   uint32_t* split_done) {
   const bool fp8 = maps.fp8;
-  if (kind == 3 && (fp8 || done == nullptr)) return OLED_ERR_INVALID_ARG;  // callers ask ffn_tc_can_fuse() first
+  if (kind == 3 && (done == nullptr || (fp8 && split_done == nullptr))) return OLED_ERR_INVALID_ARG;  // callers ask ffn_tc_can_fuse() first
   FewArgs a;
   a.tm_w1 = maps.few_w1;
   a.tm_w2 = maps.few_w2;
@@ -824,11 +862,11 @@ int launch_ffn_few(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& group
   a.early = kind == 2 && (behind_event_wait || host_counts == nullptr) && 2 * r.smem > 228u * 1024u ? 1 : 0;
   a.pool = maps.pool;
   a.slot_bytes = (unsigned long long)maps.slot_bytes;
-  a.amax_act = !fp8 ? nullptr : kind == 2 ? split->amax_mid : split->amax_in;
-  a.amax_out = fp8 && kind == 1 ? split->amax_mid : nullptr;
+  if (fp8) a.split = *split;
   a.status = status;
   a.work_counter = work_counter;
   a.done = done;
+  a.split_done = split_done;
   a.timeline = timeline;
   a.timeline_slot = timeline_slot;
   a.report = report;
@@ -841,11 +879,10 @@ int launch_ffn_few(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& group
   }
   if (kind == 2 && fp8)  // the intermediate rows as e4m3 terms, now that their magnitudes are complete
     launch_pdl(split_rows_kernel, dim3(grp.n, 4), dim3(256), 0, st, grp, rows, (const uint16_t*)hbuf,
-               (const uint32_t*)split->amax_mid, split->terms_mid, I, split->rows);
-  if (fp8) launch_pdl(kind == 2 ? ffn_few_kernel<2, true> : ffn_few_kernel<1, true>, dim3(grid), dim3(kFewThreads), r.smem, st, a);
-  else
-    launch_pdl(kind == 3 ? ffn_few_kernel<3, false> : kind == 2 ? ffn_few_kernel<2, false> : ffn_few_kernel<1, false>,
-               dim3(grid), dim3(kFewThreads), r.smem, st, a);
+               *split, I);
+  launch_pdl(fp8 ? (kind == 3 ? ffn_few_kernel<3, true> : kind == 2 ? ffn_few_kernel<2, true> : ffn_few_kernel<1, true>)
+                 : (kind == 3 ? ffn_few_kernel<3, false> : kind == 2 ? ffn_few_kernel<2, false> : ffn_few_kernel<1, false>),
+             dim3(grid), dim3(few_threads(kind, fp8)), r.smem, st, a);
   return cudaGetLastError() == cudaSuccess ? OLED_OK : OLED_ERR_CUDA;
 }
 

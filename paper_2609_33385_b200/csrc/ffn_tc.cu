@@ -834,7 +834,7 @@ static bool few_form(const FfnTcMaps& maps, int max_count, const TokenSplit* spl
 int launch_ffn_tc(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp_in, int max_count, int kind,
                   const int32_t* host_counts, const FfnRows& rows, uint16_t* hbuf, float* y, int y_bf16, int H, int I,
                   int n_sms, uint32_t* status, uint32_t* work_counter, bool behind_event_wait, StepTimeline* timeline,
-                  int timeline_slot, const RouteReport& report_in, uint32_t* done, const TokenSplit* split) {
+                  int timeline_slot, const RouteReport& report_in, uint32_t* done, const TokenSplit* split, uint32_t* split_done) {
   const RouteReport report = kind != 2 ? report_in : RouteReport{};
   if (grp_in.n <= 0 || max_count <= 0) return OLED_OK;
   FfnGroup grp = grp_in;
@@ -846,7 +846,7 @@ int launch_ffn_tc(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp_in
   grp.n_box = 16 << ib;
   if (few_form(maps, max_count, split))
     return launch_ffn_few(st, maps, grp, max_count, kind, host_counts, rows, hbuf, y, y_bf16, H, I, n_sms, status,
-                          work_counter, behind_event_wait, timeline, timeline_slot, report, done, split);
+                          work_counter, behind_event_wait, timeline, timeline_slot, report, done, split, split_done);
   // many-token tiles: the CTA-pair kernel, unless its cluster launch has failed before on this
   // device (the one-CTA form below computes the same)
   if (maps.use_pairs && !g_pairs_refused && ffn_pair_usable(maps, grp.n_box, H, I)) {
@@ -924,7 +924,7 @@ int ffn_tc_launches(const FfnTcMaps& maps, int max_count, int kind, const TokenS
   return kind == 2 && maps.fp8 && few_form(maps, max_count, split) ? 2 : 1;
 }
 
-bool ffn_tc_can_fuse(const FfnTcMaps& maps, int max_count) { return !maps.fp8 && few_form(maps, max_count, nullptr); }
+bool ffn_tc_can_fuse(const FfnTcMaps& maps, int max_count, const TokenSplit* split) { return few_form(maps, max_count, split); }
 bool ffn_pair_can_fuse(const FfnTcMaps& maps, int max_count, int H, int I) {
   return !few_form(maps, max_count, nullptr) && maps.use_pairs && !g_pairs_refused &&
          ffn_pair_usable(maps, 16 << box_index(max_count, maps.fp8 ? 128 : 256), H, I);

@@ -287,7 +287,7 @@ int launch_ffn_tc(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp, i
                   const int32_t* host_counts, const FfnRows& rows, uint16_t* hbuf, float* y, int y_bf16, int H,
                   int I, int n_sms, uint32_t* status, uint32_t* work_counter, bool behind_event_wait,
                   StepTimeline* timeline, int timeline_slot, const RouteReport& report, uint32_t* done = nullptr,
-                  const TokenSplit* split = nullptr);
+                  const TokenSplit* split = nullptr, uint32_t* split_done = nullptr);
 int ffn_tc_launches(const FfnTcMaps& maps, int max_count, int kind, const TokenSplit* split);
 // No gathered copy of the step's token rows exists: every FFN launch until
 // ffn_tc_clear_token_source must be one the CTA-pair kernel takes (token tile 256), and each gets
@@ -295,7 +295,7 @@ int ffn_tc_launches(const FfnTcMaps& maps, int max_count, int kind, const TokenS
 bool ffn_tc_token_source_usable(const FfnTcMaps& maps, int H, int I);
 void ffn_tc_set_token_source(FfnTcMaps* maps, const uint16_t* x, int T, const int32_t* perm, int K, uint16_t* xp);
 void ffn_tc_clear_token_source(FfnTcMaps* maps);
-bool ffn_tc_can_fuse(const FfnTcMaps& maps, int max_count);
+bool ffn_tc_can_fuse(const FfnTcMaps& maps, int max_count, const TokenSplit* split);
 bool ffn_pair_can_fuse(const FfnTcMaps& maps, int max_count, int H, int I);  // kind 3 on CTA pairs
 // ---- ffn_pair.cu: the many-token form on CTA pairs (bf16 stores, token tiles of 256 rows,
 // intermediate a multiple of 256 and hidden a multiple of 512); kinds 1 and 2 as above, kind 3 both
@@ -318,7 +318,8 @@ int ffn_few_setup(FfnTcMaps* maps, const uint8_t* pool, size_t slot_bytes, int n
 int launch_ffn_few(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp, int max_count, int kind,
                    const int32_t* host_counts, const FfnRows& rows, uint16_t* hbuf, float* y, int y_bf16, int H, int I, int n_sms,
                    uint32_t* status, uint32_t* work_counter, bool behind_event_wait, StepTimeline* timeline,
-                   int timeline_slot, const RouteReport& report, uint32_t* done, const TokenSplit* split);
+                   int timeline_slot, const RouteReport& report, uint32_t* done, const TokenSplit* split,
+                   uint32_t* split_done);
 
 // Self-check (check.cu): invariants of the routing and the permutation, guard words.
 void launch_self_check(cudaStream_t st, const int32_t* ids, const int32_t* counts, const int32_t* offsets,

@@ -427,7 +427,7 @@ int run_ffn_launches(oled_ctx* ctx, const FfnGroup& grp, int max_count, const in
     // Many-token tiles on CTA pairs: always one launch (a boundary between cluster kernels is a full stop).
     const bool fuse_pairs = before_down == nullptr && ctx->fuse_ffn != 0 && ffn_pair_can_fuse(ctx->maps, max_count, H, I);
     const bool fuse = fuse_pairs ||
-                      (before_down == nullptr && !ctx->y_bf16 && ffn_tc_can_fuse(ctx->maps, max_count) &&
+                      (before_down == nullptr && ffn_tc_can_fuse(ctx->maps, max_count, ctx->step_split) &&
                        ctx->fuse_ffn != 0);
     for (int kind = fuse ? 3 : 1; kind <= (fuse ? 3 : 2); ++kind) {
       if (kind == 2 && before_down) OLED_CUDA(ctx, cudaStreamWaitEvent(ctx->stream, before_down, 0));
@@ -460,7 +460,7 @@ int run_ffn_launches(oled_ctx* ctx, const FfnGroup& grp, int max_count, const in
       const int rc = launch_ffn_tc(ctx->stream, ctx->maps, grp, max_count, kind, host_counts, rows, ctx->d_hbuf, ctx->d_y, ctx->y_bf16 ? 1 : 0, H, I, ctx->n_sms, ctx->d_status, work,
                                    behind_event_wait || (kind == 2 && before_down != nullptr),
                                    ctx->timeline_on ? ctx->d_timeline + ctx->last_layer : nullptr, 3 + li, report, done,
-                                   ctx->step_split);
+                                   ctx->step_split, ready);
       if (rc != OLED_OK) return rc;
       ctx->launches += ffn_tc_launches(ctx->maps, max_count, kind, ctx->step_split);
     }
