@@ -401,8 +401,10 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
           ok = FP8 ? wait_count(p.split_done + g, (uint32_t)ctl->count[e], 0u) : wait_count(p.done + g, done_target(g), 0u);
           if (!ok) break;
           ready_g = g;
-          // the rows were written through the generic proxy; the loads below read through the async proxy
-          asm volatile("fence.proxy.async;" ::: "memory");
+          // The rows were written through the generic proxy, the loads below read through the async proxy: the one
+          // proxy fence between the two stands here.  (On the writers' side as well, and for all state spaces, it
+          // waited for the CTA's copies in flight: 6000 to 12800 cycles per item.)
+          asm volatile("fence.proxy.async.global;" ::: "memory");
         }
       }
       const CUtensorMap* const maps = down ? p.tm_h : p.tm_x;
@@ -506,10 +508,8 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
         uint32_t mine = 0;
         for (int r = w; r < count; r += owners * kFewSplitWarps, ++mine)
           split_row(p.hbuf, p.split, row0 + r, I, lane, 32);
-        __threadfence();
-        asm volatile("fence.proxy.async;" ::: "memory");
         __syncwarp();
-        if (lane == 0) atomicAdd(p.split_done + g, mine);
+        if (lane == 0) red_release_add(p.split_done + g, mine);
       }
     }
   } else {
@@ -577,6 +577,16 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
     const bool live = warp < epi_warps && wait_table();
     const int quarter = warp & 3;  // this warp's lanes; its columns: every epi_warps / 4-th chunk of 16
     if (early) griddep_wait();  // (the rows' magnitudes below are products of the predecessor)
+    // (one launch) The expert whose intermediate rows this warp has stored last.  The warp is counted in - the down items
+    // of the expert wait for the full count - only when the next item's operands have been looked up: the release
+    // waits until the stores are visible, up to 5 us while the stream saturates the memory, and most of that lies
+    // under the lookups then.  (The next item has been published long before, so nothing waits on this.)
+    int stored_g = -1;
+    auto count_stored = [&]() {
+      __syncwarp();
+      if (stored_g >= 0 && lane == 0) red_release_add(p.done + stored_g, 1u);
+      stored_g = -1;
+    };
     int local = 0;
     for (int seq = 0; live; ++seq) {
       int code = kItemAbort, m = 0;
@@ -638,6 +648,7 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
       // are final only once the item's MMAs are through
       const bool ahead = !(FP8 && fused && down);
       if (c < n && ahead) columns(c, row, dst, inv);
+      count_stored();
       int ready = 0;
       if (lane == 0) ready = mbar_wait(smem_u32(&ctl->tmem_full[acc]), acc_phase, abort_flag, p.status) ? 1 : 0;
       ready = __shfl_sync(0xffffffffu, ready, 0);
@@ -720,15 +731,9 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
           }
         }
       }
-      if (fused && !down) {
-        // this warp's intermediate rows of the item are stored: visible device-wide, then the warp is counted in
-        // (the down items of this expert wait for the full count)
-        __threadfence();
-        asm volatile("fence.proxy.async;" ::: "memory");
-        __syncwarp();
-        if (lane == 0) atomicAdd(p.done + g, 1u);
-      }
+      if (fused && !down) stored_g = g;
     }
+    count_stored();
   }
 
   // ---- teardown.  Every way out passes the dependency wait, so that no kernel of a step completes before
@@ -768,14 +773,14 @@ split_rows_kernel(const __grid_constant__ FfnGroup grp, const __grid_constant__ 
 
 // Stage shape and count: two k-blocks per stage where at least four such stages fit and both contractions
 // have an even number of them (half the waits and commits on the MMA thread); ten bf16 k-blocks in flight
-// at most (eleven measured slower), twelve of e4m3 codes.
+// at most (eleven measured slower), eight of e4m3 codes (16 tokens, 8 layers: 557 us, with ten 569).
 struct FewRings {
   int stages, k_atoms;
   uint32_t smem;
 };
 FewRings few_rings(int n_box, bool fp8, int H, int I) {
   const uint32_t atom = kFewWTile + (uint32_t)n_box * 128u * (fp8 ? 2u : 1u);
-  const int kblocks = (int)std::min<uint32_t>(fp8 ? 12u : 10u, (kFewSmemMax - kFewCtlBytes - 1024u) / atom);
+  const int kblocks = (int)std::min<uint32_t>(fp8 ? 8u : 10u, (kFewSmemMax - kFewCtlBytes - 1024u) / atom);
   const int kk = fp8 ? 128 : 64;
   FewRings r;
   r.k_atoms = kblocks >= 8 && (H / kk) % 2 == 0 && (I / kk) % 2 == 0 ? 2 : 1;

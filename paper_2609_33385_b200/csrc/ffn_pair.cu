@@ -348,8 +348,9 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant_
         }
         if (!ok) break;
         ready_g = wait_key;
-        // (the intermediate rows were written through the generic proxy; the copies below read through the async proxy)
-        asm volatile("fence.proxy.async;" ::: "memory");
+        // (the intermediate rows were written through the generic proxy; the copies below read through the async proxy.
+        // This is the only proxy fence between the two; on the writers' side it would wait for the CTA's copies in flight)
+        asm volatile("fence.proxy.async.global;" ::: "memory");
       }
       const int n_mma = max(32, (it.valid + 31) & ~31);
       const int my_row0 = it.row0 + (int)rank * (n_mma >> 1);  // this CTA's half of the tile's token rows
@@ -423,9 +424,8 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant_
         }
       };
       auto count_chunk = [&](int n) {  // chunk n is in global memory: visible device-wide, then counted
-        asm volatile("fence.proxy.async;" ::: "memory");
-        __threadfence();
-        atomicAdd(tok.ready + ctl->row_tile[n & 7], 1u);
+        asm volatile("fence.proxy.async.global;" ::: "memory");
+        red_release_add(tok.ready + ctl->row_tile[n & 7], 1u);
       };
       while (issued < kRowSlots - 1 && g < grp.n) issue();
       int n = 0;
@@ -533,11 +533,8 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant_
             for (int j = 0; j < 8; ++j)
               if (i0 + 32 * j < n16) dst[i0 + 32 * j] = v[j];
           }
-          // visible device-wide and to the async proxy of the items' copies, then counted
-          __threadfence();
-          asm volatile("fence.proxy.async;" ::: "memory");
           __syncwarp();
-          if (lane == 0) atomicAdd(tok.ready + ctl->tile_prefix[g] + r / kPairN, chunks);
+          if (lane == 0) red_release_add(tok.ready + ctl->tile_prefix[g] + r / kPairN, chunks);
         }
         before += ctl->count[g];
       }
@@ -629,12 +626,9 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant_
         if (lane == 0) mbar_arrive_cluster(tmem_empty_on_first);
       }
       if (fused && it.kind == 1) {
-        // this warp's intermediate rows of the item are stored: visible device-wide (and to the
-        // async proxy of the down items' copies), then counted
-        __threadfence();
-        asm volatile("fence.proxy.async;" ::: "memory");
+        // this warp's intermediate rows of the item are stored: counted once they are visible device-wide
         __syncwarp();
-        if (lane == 0) atomicAdd(sec.done + it.g, 1u);
+        if (lane == 0) red_release_add(sec.done + it.g, 1u);
       }
     }
   }
