@@ -43,7 +43,8 @@
 // makes the thread that issues the MMAs the bound: 8 layers of 250 tokens 1459 us, now 907.)
 //
 // Warp roles: warps 0-7 the work table, then the epilogue (lane quarter = warp mod 4, interleaved 16-column
-// chunks), warp 8 weights, warp 9 token rows, warp 10 MMA issue.  Every wait is bounded as in ffn_tc.cu.
+// chunks), warp 8 weights, warp 9 token rows, warp 10 MMA issue; in one
+// launch warp 11 counts stored items, and with fp8 stores warps 12-15 make the intermediate rows' terms.  Every wait is bounded as in ffn_tc.cu.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -59,8 +60,9 @@ namespace {
 
 constexpr int kFewEpiWarps = 8;
 constexpr int kFewWeightWarp = kFewEpiWarps, kFewTokenWarp = kFewEpiWarps + 1, kFewMmaWarp = kFewEpiWarps + 2;
-constexpr int kFewSplitWarp = kFewEpiWarps + 3, kFewSplitWarps = 4;  // fp8 stores, KIND 3
-constexpr int few_threads(int kind, bool fp8) { return (kFewEpiWarps + 3 + (kind == 3 && fp8 ? kFewSplitWarps : 0)) * 32; }
+constexpr int kFewCountWarp = kFewEpiWarps + 3;                           // KIND 3
+constexpr int kFewSplitWarp = kFewEpiWarps + 4, kFewSplitWarps = 4;       // KIND 3, fp8 stores
+constexpr int few_threads(int kind, bool fp8) { return (kFewEpiWarps + 3 + (kind != 3 ? 0 : fp8 ? 1 + kFewSplitWarps : 1)) * 32; }
 constexpr uint32_t kFewWTile = 128 * 128;  // a k-block of weights: 128 rows of 128 bytes (64 bf16 or 128 e4m3)
 constexpr int kFewMaxStages = 12;
 constexpr int kFewRing = 8;
@@ -71,6 +73,7 @@ struct __align__(16) FewCtl {
   unsigned long long empty[kFewMaxStages];
   unsigned long long item_full[kFewRing];
   unsigned long long item_empty[kFewRing];
+  unsigned long long item_stored[kFewRing];  // (one launch) the epilogue warps have stored the item's rows
   unsigned long long tmem_full[2];
   unsigned long long tmem_empty[2];
   unsigned long long table;   // the work table below is complete
@@ -114,7 +117,7 @@ struct FewArgs {
   TokenSplit split;          // fp8: the token operands' terms and magnitudes (amax_mid is raised by the gate/up epilogue)
   uint32_t* status;
   uint32_t* work_counter;    // zero at the start
-  uint32_t* done;            // KIND 3: per expert of the group, zero at the start: epilogue warps that have stored its rows
+  uint32_t* done;            // KIND 3: per expert of the group, zero at the start: its gate/up items that have been stored
   uint32_t* split_done;      // KIND 3, fp8: the same for its intermediate rows whose terms have been stored
   StepTimeline* timeline;
   int timeline_slot;
@@ -224,7 +227,9 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
       }
       for (int s = 0; s < kFewRing; ++s) {
         mbar_init(smem_u32(&ctl->item_full[s]), 1);
-        mbar_init(smem_u32(&ctl->item_empty[s]), 2u + (uint32_t)epi_warps);  // token warp, MMA warp, epilogue warps
+        // token warp, MMA warp, epilogue warps, counting warp
+        mbar_init(smem_u32(&ctl->item_empty[s]), (fused ? 3u : 2u) + (uint32_t)epi_warps);
+        mbar_init(smem_u32(&ctl->item_stored[s]), (uint32_t)epi_warps);
       }
       for (int a = 0; a < 2; ++a) {
         mbar_init(smem_u32(&ctl->tmem_full[a]), 1);
@@ -253,9 +258,7 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = ctl->tmem_base;
-  // KIND 3: epilogue warps that store intermediate rows per gate/up item, times the items of a token tile
-  const uint32_t done_per_tile = (uint32_t)(m_tiles1 * epi_warps);
-  auto done_target = [&](int g) { return done_per_tile * (uint32_t)(ctl->tile_prefix[g + 1] - ctl->tile_prefix[g]); };
+  auto done_target = [&](int g) { return (uint32_t)m_tiles1 * (uint32_t)(ctl->tile_prefix[g + 1] - ctl->tile_prefix[g]); };
   // (a whole warp) waits until a counter in global memory has reached `target`
   auto wait_count = [&](const uint32_t* counter, uint32_t target, uint32_t sleep_ns) {
     unsigned long long t0 = 0;
@@ -492,6 +495,22 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
         }
       }
     }
+  } else if (fused && warp == kFewCountWarp) {
+    // ------------------------------------------------------------ counts stored gate/up items (one launch)
+    // The down items of an expert wait until all of its gate/up items are counted.  The count is a release: it waits
+    // until the stores before it are visible device-wide, 2 to 5 us while the stream saturates the memory, so a warp
+    // of its own waits and not the epilogue.
+    for (int seq = 0;; ++seq) {
+      const int slot = seq % kFewRing;
+      const uint32_t parity = (uint32_t)(seq / kFewRing) & 1u;
+      if (!warp_wait(smem_u32(&ctl->item_full[slot]), parity, abort_flag, p.status)) break;
+      const int code = __shfl_sync(0xffffffffu, *reinterpret_cast<volatile int*>(&ctl->item_ring[slot]), 0);
+      if (code == kItemNone) break;
+      if (!warp_wait(smem_u32(&ctl->item_stored[slot]), parity, abort_flag, p.status)) break;
+      if (lane == 0 && code != kItemDrop && !((code >> 9) & 1)) red_release_add(p.done + (code & 511), 1u);
+      // (handed back only now: the barrier above is not used again before this warp has seen its phase)
+      if (lane == 0) mbar_arrive(smem_u32(&ctl->item_empty[slot]));
+    }
   } else if (FP8 && fused && warp >= kFewSplitWarp) {
     // ------------------------------------------------------------ terms of the intermediate rows (fp8, one launch)
     // CTA b looks after expert b mod n of the group, together with the other CTAs of that number: as soon as all
@@ -577,16 +596,6 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
     const bool live = warp < epi_warps && wait_table();
     const int quarter = warp & 3;  // this warp's lanes; its columns: every epi_warps / 4-th chunk of 16
     if (early) griddep_wait();  // (the rows' magnitudes below are products of the predecessor)
-    // (one launch) The expert whose intermediate rows this warp has stored last.  The warp is counted in - the down items
-    // of the expert wait for the full count - only when the next item's operands have been looked up: the release
-    // waits until the stores are visible, up to 5 us while the stream saturates the memory, and most of that lies
-    // under the lookups then.  (The next item has been published long before, so nothing waits on this.)
-    int stored_g = -1;
-    auto count_stored = [&]() {
-      __syncwarp();
-      if (stored_g >= 0 && lane == 0) red_release_add(p.done + stored_g, 1u);
-      stored_g = -1;
-    };
     int local = 0;
     for (int seq = 0; live; ++seq) {
       int code = kItemAbort, m = 0;
@@ -600,7 +609,10 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
       }
       code = __shfl_sync(0xffffffffu, code, 0);
       m = __shfl_sync(0xffffffffu, m, 0);
-      if (code == kItemDrop) continue;
+      if (code == kItemDrop) {
+        if (fused && lane == 0) mbar_arrive(smem_u32(&ctl->item_stored[seq % kFewRing]));
+        continue;
+      }
       if (code < 0) break;
       const int g = code & 511, nt = code >> 11;
       const bool down = KIND == 2 || (fused && ((code >> 9) & 1));
@@ -648,7 +660,6 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
       // are final only once the item's MMAs are through
       const bool ahead = !(FP8 && fused && down);
       if (c < n && ahead) columns(c, row, dst, inv);
-      count_stored();
       int ready = 0;
       if (lane == 0) ready = mbar_wait(smem_u32(&ctl->tmem_full[acc]), acc_phase, abort_flag, p.status) ? 1 : 0;
       ready = __shfl_sync(0xffffffffu, ready, 0);
@@ -731,9 +742,11 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
           }
         }
       }
-      if (fused && !down) stored_g = g;
+      if (fused) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&ctl->item_stored[seq % kFewRing]));
+      }
     }
-    count_stored();
   }
 
   // ---- teardown.  Every way out passes the dependency wait, so that no kernel of a step completes before
