@@ -341,10 +341,10 @@ int oled_last_cuda_error(oled_ctx* ctx);
 /* Routing of one step without any allocation.  The paper has no counterpart: this exists for
  * hosts that cannot let a library allocate device memory - a server that gives all of it to its
  * own arena at start-up, or a decode loop that cannot afford the device-wide synchronisation
- * hidden in cudaMalloc/cudaFree.  It runs the same gate, top-k, gate-score and permutation
- * kernels as oled_denoise_step(), needs no context, and keeps its scratch (gate logits, inverse
- * permutation, reuse-score accumulators; about 0.55 MB) in a fixed array inside the library
- * image, which every GPU that loads the library holds until the process exits.
+ * hidden in cudaMalloc/cudaFree.  It runs the same gate, top-k and gate-score arithmetic as
+ * oled_denoise_step() and the same stable permutation in one kernel, needs no context, and its only scratch is a
+ * word per call out of a fixed array of 1024 inside the library image, which every GPU that loads the
+ * library holds until the process exits.
  *   hidden [n_tokens,hidden_dim] bf16, w_router [n_experts,hidden_dim] bf16, bias fp32[n_experts]
  *   or NULL, confidences fp32[n_tokens]: device, read only.
  *   ids int32[n_tokens*top_k], gate fp32[n_tokens*top_k], counts int32[n_experts],
@@ -358,10 +358,9 @@ int oled_last_cuda_error(oled_ctx* ctx);
  * thread has run no step; either way the results are the same.
  * The work is enqueued on cuda_stream.  The first call on a device looks up the array's device
  * address (one-time set-up under a lock); make that first call before any stream capture.
- * All calls share the one array, which still holds the previous call's data: the accumulators
- * are cleared on the stream at the start of every call, and two calls whose work overlaps on
- * the GPU (different streams, no ordering between them) race on it.  Calls cudaMemsetAsync and
- * kernel launches only: no cudaMalloc, cudaFree or allocating library routine. */
+ * The words are taken in turn: calls may overlap on the GPU as long as no more than 1024 do.  (A captured call
+ * keeps its word: replays of one graph must not overlap each other.)  One kernel launch (two memsets if
+ * n_tokens is 0): no cudaMalloc, cudaFree or allocating library routine. */
 #define OLED_NOALLOC_MAX_TOKENS 256
 int oled_route_noalloc(const void* hidden, const void* w_router, const float* bias,
                        const float* confidences, int32_t n_tokens, int32_t hidden_dim,

@@ -181,6 +181,69 @@ __device__ __forceinline__ void combine_rows(const CombinePrev& p, int t0, int n
   }
 }
 
+// What the allocation-free routing entry point adds to the gate kernel: the counts, offsets and the stable
+// permutation, made by the CTA that finishes last.  ticket: a ZERO word, zero again afterwards.
+struct RouteFinish {
+  unsigned int* ticket = nullptr;
+  int32_t* offsets = nullptr;
+  int32_t* perm = nullptr;
+};
+// counts[E], offsets[E + 1] and the stable permutation by expert of n assignments, by one CTA of WARPS warps (E at most
+// one expert per thread).  Every warp counts the experts of a contiguous part of the list, the counts are scanned over
+// (expert, warp), and every warp hands out its part's rows in order.  s_hist: [WARPS][E].
+template <int WARPS>
+__device__ __forceinline__ void sort_assignments(const int32_t* ids, int n, int E, int32_t* __restrict__ counts,
+                                                 int32_t* __restrict__ offsets, int32_t* __restrict__ perm, int* s_hist) {
+  static_assert(WARPS * 32 >= OLED_MAX_EXPERTS, "a thread per expert");
+  __shared__ int s_warp[WARPS];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int i = threadIdx.x; i < WARPS * E; i += WARPS * 32) s_hist[i] = 0;
+  __syncthreads();
+  const int part = (n + WARPS * 32 - 1) / (WARPS * 32) * 32, first = warp * part, last = min(n, first + part);
+  int* const hist = s_hist + warp * E;
+  for (int i0 = first; i0 < last; i0 += 32) {
+    const int id = i0 + lane < last ? __ldcg(ids + i0 + lane) : -1;
+    const uint32_t same = __match_any_sync(0xffffffffu, id);
+    if (id >= 0 && lane == __ffs((int)same) - 1) hist[id] += __popc(same);
+    __syncwarp();
+  }
+  __syncthreads();
+  const int e = threadIdx.x;
+  int total = 0;
+  if (e < E)
+    for (int w = 0; w < WARPS; ++w) {
+      const int c = s_hist[w * E + e];
+      s_hist[w * E + e] = total;
+      total += c;
+    }
+  int incl = total;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int o = __shfl_up_sync(0xffffffffu, incl, d);
+    if (lane >= d) incl += o;
+  }
+  if (lane == 31) s_warp[warp] = incl;
+  __syncthreads();
+  int before = incl - total;
+  for (int w = 0; w < warp; ++w) before += s_warp[w];
+  if (e < E) {
+    counts[e] = total;
+    offsets[e] = before;
+    if (e == E - 1) offsets[E] = before + total;
+    for (int w = 0; w < WARPS; ++w) s_hist[w * E + e] += before;
+  }
+  __syncthreads();
+  for (int i0 = first; i0 < last; i0 += 32) {
+    const int id = i0 + lane < last ? __ldcg(ids + i0 + lane) : -1;
+    const uint32_t same = __match_any_sync(0xffffffffu, id);
+    const int rank = __popc(same & ((1u << lane) - 1u));
+    if (id >= 0) perm[hist[id] + rank] = i0 + lane;
+    __syncwarp();
+    if (id >= 0 && rank == 0) hist[id] += __popc(same);
+    __syncwarp();
+  }
+}
+
 // TT tokens per CTA, WARPS warps; each warp owns kEPerWarp experts per pass and all TT tokens.  Small
 // blocks use TT = 1 with 16 warps (one pass covers 64 experts) and keep several 256-wide
 // chunks of loads in flight; the chain order of every logit is the same in all variants.
@@ -200,7 +263,7 @@ route_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ wr,
              int K, float* __restrict__ logits_out, int32_t* __restrict__ ids,
              float* __restrict__ gate, int32_t* __restrict__ counts,
              unsigned long long* __restrict__ scores, CombinePrev prev, StepTimeline* timeline,
-             const __grid_constant__ ScatterRows scatter) {
+             const __grid_constant__ ScatterRows scatter, const __grid_constant__ RouteFinish finish) {
   extern __shared__ __align__(16) uint8_t s_dyn[];
   float* s_logits = reinterpret_cast<float*>(s_dyn);                       // [TT][E]
   constexpr bool staged = TT <= 4;
@@ -373,8 +436,10 @@ route_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ wr,
         const float g = __fdiv_rn(z, sum);
         ids[(size_t)t * K + lane] = my_id;
         gate[(size_t)t * K + lane] = g;
-        if (scatter.cap == 0) atomicAdd(&counts[my_id], 1);
-        atomicAdd(&scores[my_id], score_quantum(g, s_conf[a]));
+        if (finish.ticket == nullptr) {
+          if (scatter.cap == 0) atomicAdd(&counts[my_id], 1);
+          atomicAdd(&scores[my_id], score_quantum(g, s_conf[a]));
+        }
       }
     }
     if (scatter.cap > 0 && dense_rows == nullptr) {  // (dense rows of bf16 stores have been stored already)
@@ -405,6 +470,25 @@ route_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ wr,
       const int t = t0 + a;
       if (t >= T) continue;
       route_token_tail(s_logits + a * E, t, lane, E, K, conf, ids, gate, counts, scores);
+    }
+  }
+  if (finish.ticket != nullptr) {
+    // routing without a step: the last CTA to get here sorts the assignments (the ids of the others are visible to it:
+    // every CTA's stores precede its ticket)
+    __shared__ int s_last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      __threadfence();
+      s_last = atomicAdd(finish.ticket, 1u) == gridDim.x - 1 ? 1 : 0;
+    }
+    __syncthreads();
+    if (s_last) {
+      if (threadIdx.x == 0) {
+        __threadfence();
+        *finish.ticket = 0u;  // ready for a later call
+      }
+      __syncthreads();
+      sort_assignments<WARPS>(ids, T * K, E, counts, finish.offsets, finish.perm, reinterpret_cast<int*>(s_dyn));
     }
   }
   if (threadIdx.x == 0) timeline_end(timeline, 0);
@@ -776,6 +860,21 @@ bool pdl_enabled() { return g_pdl_allowed.load() && g_pdl_step; }
 // The staged gate kernel takes few-token steps, where it brings the rows to their experts and may carry out a
 // combine; beyond two tokens per SM it re-reads the router matrix too often (64 experts x 2048, 1000 tokens: 35 us
 // against 16 in the many-token kernel), so it stays there only for what the other does not do.
+constexpr int kStagedWarps = 16;
+static size_t staged_smem(int tt, int H, int E) {  // logits, rows, keys
+  return ((((size_t)tt * E * sizeof(float)) + 15) & ~(size_t)15) + (size_t)tt * H * 2 + (size_t)tt * ((E + 3) & ~3) * 4;
+}
+static bool staged_attributes() {  // the staged rows: up to 4 x 16 K elements
+  static const bool ok = [] {
+    const bool done =
+        cudaFuncSetAttribute(route_kernel<1, kStagedWarps, 4, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024) == cudaSuccess &&
+        cudaFuncSetAttribute(route_kernel<2, kStagedWarps, 4, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024) == cudaSuccess &&
+        cudaFuncSetAttribute(route_kernel<4, kStagedWarps, 2, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024) == cudaSuccess;
+    if (!done) cudaGetLastError();
+    return done;
+  }();
+  return ok;
+}
 bool route_staged(int T, int K) { return T <= 296 || (T <= 1024 && (size_t)T * K <= 4096); }
 
 void launch_route(cudaStream_t st, const uint16_t* x, const uint16_t* w_router, const float* bias,
@@ -783,27 +882,18 @@ void launch_route(cudaStream_t st, const uint16_t* x, const uint16_t* w_router, 
                   float* gate, int32_t* counts, unsigned long long* scores, const CombinePrev& prev,
                   StepTimeline* timeline, int32_t* seg_counts, int seg_tokens, const ScatterRows& scatter) {
   if (route_staged(T, K)) {
-    constexpr int W = 16;
-    static bool attr_done = false;
-    if (!attr_done) {  // the staged rows: up to 4 x 16 K elements
-      cudaFuncSetAttribute(route_kernel<1, W, 4, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
-      cudaFuncSetAttribute(route_kernel<2, W, 4, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
-      cudaFuncSetAttribute(route_kernel<4, W, 2, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
-      cudaGetLastError();
-      attr_done = true;
-    }
-    auto smem = [&](int tt) {
-      return ((((size_t)tt * E * sizeof(float)) + 15) & ~(size_t)15) + (size_t)tt * H * 2 + (size_t)tt * ((E + 3) & ~3) * 4;
-    };
+    constexpr int W = kStagedWarps;
+    staged_attributes();
+    auto smem = [&](int tt) { return staged_smem(tt, H, E); };
     if (T <= 148)
       launch_pdl(route_kernel<1, W, 4, 4>, dim3(T), dim3(W * 32), smem(1), st, x, w_router, bias, conf, T, H, E, K,
-                 logits, ids, gate, counts, scores, prev, timeline, scatter);
+                 logits, ids, gate, counts, scores, prev, timeline, scatter, RouteFinish{});
     else if (T <= 296)  // (four tokens per CTA measured slower at 256 tokens x 128 experts: 33 against 20 us)
       launch_pdl(route_kernel<2, W, 4, 4>, dim3((T + 1) / 2), dim3(W * 32), smem(2), st, x, w_router, bias, conf, T, H,
-                 E, K, logits, ids, gate, counts, scores, prev, timeline, scatter);
+                 E, K, logits, ids, gate, counts, scores, prev, timeline, scatter, RouteFinish{});
     else
       launch_pdl(route_kernel<4, W, 2, 4>, dim3((T + 3) / 4), dim3(W * 32), smem(4), st, x, w_router, bias, conf, T, H,
-                 E, K, logits, ids, gate, counts, scores, prev, timeline, scatter);
+                 E, K, logits, ids, gate, counts, scores, prev, timeline, scatter, RouteFinish{});
   } else {
     // (re-tilings of the plain kernel - more tokens or experts per warp, more warps per CTA, deeper
     // unrolling - were all slower at 4096 tokens x 64 experts x 4096)
@@ -886,39 +976,54 @@ void launch_gather(cudaStream_t st, const uint16_t* x, const int32_t* perm, int 
 // device memory to its own arena at start-up, or a latency-critical decode loop in which the
 // implicit device-wide synchronisation of cudaMalloc / cudaFree is not acceptable.  For them
 // this entry point runs the gate, top-k, gate scores and the token->expert permutation of one
-// step with its scratch (gate logits, inverse permutation, reuse-score accumulators) in a
-// fixed array that is part of the loaded module, so nothing is allocated or freed.
+// step in one launch, without logits or scores in memory: its only scratch is a word per call, by which the CTA that
+// finishes last knows that it does (it then sorts the assignments).  The words are a fixed array in the
+// loaded module, taken in turn, so nothing is allocated or freed.  (As three memsets, the gate kernel and the permutation
+// kernel a call of 32 tokens took 16 us, nearly all of it on the host.)
 namespace oled {
 namespace {
 
-constexpr size_t kNaScoreBytes = (size_t)OLED_MAX_EXPERTS * sizeof(unsigned long long);
-constexpr size_t kNaPosBytes = (size_t)OLED_NOALLOC_MAX_TOKENS * OLED_MAX_TOPK * sizeof(int32_t);
-constexpr size_t kNaLogitBytes = (size_t)OLED_NOALLOC_MAX_TOKENS * OLED_MAX_EXPERTS * sizeof(float);
-constexpr size_t kNaScratchBytes = kNaScoreBytes + kNaPosBytes + kNaLogitBytes;
-
-// Lives in every GPU that loads the library until the process exits (about 0.55 MB).
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kNaScratchBytes];
+// Lives in every GPU that loads the library until the process exits; all words are zero between calls.
+constexpr unsigned int kNaTickets = 1024;
+static __device__ unsigned int g_noalloc_tickets[kNaTickets];
 
 constexpr int kNaMaxDevices = 64;
 std::mutex g_na_mutex;
-void* g_na_ptr[kNaMaxDevices] = {};
+unsigned int* g_na_ptr[kNaMaxDevices] = {};
+std::atomic<unsigned int> g_na_next{0};
 
-// In host code g_noalloc_scratch is only a handle for the symbol, not an address a kernel can
+// In host code the array is only a handle for the symbol, not an address a kernel can
 // use: the device address is looked up once per device, with that device current.
-int noalloc_scratch_ptr(unsigned char** out) {
+int noalloc_ticket(unsigned int** out) {
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kNaMaxDevices) return OLED_ERR_CUDA;
   std::lock_guard<std::mutex> lock(g_na_mutex);
   if (g_na_ptr[dev] == nullptr) {
     void* p = nullptr;
-    if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess || p == nullptr) {
+    if (cudaGetSymbolAddress(&p, g_noalloc_tickets) != cudaSuccess || p == nullptr) {
       cudaGetLastError();
       return OLED_ERR_CUDA;
     }
-    g_na_ptr[dev] = p;
+    g_na_ptr[dev] = static_cast<unsigned int*>(p);
   }
-  *out = static_cast<unsigned char*>(g_na_ptr[dev]);
+  *out = g_na_ptr[dev] + g_na_next.fetch_add(1u) % kNaTickets;
   return OLED_OK;
+}
+
+void launch_route_alone(cudaStream_t st, const uint16_t* x, const uint16_t* w_router, const float* bias, const float* conf,
+                        int T, int H, int E, int K, int32_t* ids, float* gate, int32_t* counts, const RouteFinish& finish) {
+  const size_t sort_bytes = (size_t)kStagedWarps * E * sizeof(int);
+  if (T <= 148) {
+    const size_t smem = std::max(staged_smem(1, H, E), sort_bytes);
+    launch_pdl(route_kernel<1, kStagedWarps, 4, 4>, dim3(T), dim3(kStagedWarps * 32), smem, st, x, w_router, bias, conf, T, H, E,
+               K, (float*)nullptr, ids, gate, counts, (unsigned long long*)nullptr, CombinePrev{}, (StepTimeline*)nullptr,
+               ScatterRows{}, finish);
+  } else {
+    const size_t smem = std::max(staged_smem(2, H, E), sort_bytes);
+    launch_pdl(route_kernel<2, kStagedWarps, 4, 4>, dim3((T + 1) / 2), dim3(kStagedWarps * 32), smem, st, x, w_router, bias,
+               conf, T, H, E, K, (float*)nullptr, ids, gate, counts, (unsigned long long*)nullptr, CombinePrev{},
+               (StepTimeline*)nullptr, ScatterRows{}, finish);
+  }
 }
 
 }  // namespace
@@ -942,25 +1047,22 @@ extern "C" int oled_route_noalloc(const void* hidden, const void* w_router, cons
         off(gate, 4) || off(counts, 4) || off(offsets, 4) || off(perm, 4))
       return OLED_ERR_INVALID_ARG;
   }
-  unsigned char* scratch = nullptr;
-  const int rc = noalloc_scratch_ptr(&scratch);
-  if (rc != OLED_OK) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  unsigned long long* scores = reinterpret_cast<unsigned long long*>(scratch);
-  int32_t* pos = reinterpret_cast<int32_t*>(scratch + kNaScoreBytes);
-  float* logits = reinterpret_cast<float*>(scratch + kNaScoreBytes + kNaPosBytes);
-  // the array keeps the previous call's contents: the accumulators must start at zero
-  if (cudaMemsetAsync(scores, 0, (size_t)n_experts * sizeof(unsigned long long), st) != cudaSuccess ||
-      cudaMemsetAsync(counts, 0, (size_t)n_experts * sizeof(int32_t), st) != cudaSuccess ||
-      cudaMemsetAsync(offsets, 0, (size_t)(n_experts + 1) * sizeof(int32_t), st) != cudaSuccess) {
-    cudaGetLastError();
-    return OLED_ERR_CUDA;
+  if (n_tokens == 0) {
+    if (cudaMemsetAsync(counts, 0, (size_t)n_experts * sizeof(int32_t), st) != cudaSuccess ||
+        cudaMemsetAsync(offsets, 0, (size_t)(n_experts + 1) * sizeof(int32_t), st) != cudaSuccess) {
+      cudaGetLastError();
+      return OLED_ERR_CUDA;
+    }
+    return OLED_OK;
   }
-  if (n_tokens == 0) return OLED_OK;
-  launch_route(st, static_cast<const uint16_t*>(hidden), static_cast<const uint16_t*>(w_router), bias,
-               confidences, n_tokens, hidden_dim, n_experts, top_k, logits, ids, gate, counts, scores,
-               CombinePrev{}, nullptr);
-  launch_permute(st, ids, counts, n_tokens, n_experts, top_k, offsets, perm, pos, nullptr, nullptr, hidden_dim,
-                 nullptr);
+  RouteFinish finish;
+  const int rc = noalloc_ticket(&finish.ticket);
+  if (rc != OLED_OK) return rc;
+  if (!staged_attributes()) return OLED_ERR_CUDA;
+  finish.offsets = offsets;
+  finish.perm = perm;
+  launch_route_alone(st, static_cast<const uint16_t*>(hidden), static_cast<const uint16_t*>(w_router), bias, confidences,
+                     n_tokens, hidden_dim, n_experts, top_k, ids, gate, counts, finish);
   return cudaGetLastError() == cudaSuccess ? OLED_OK : OLED_ERR_CUDA;
 }

@@ -889,3 +889,34 @@ def test_token_tiles_between_16_and_128_rows(n_experts, top_k, counts, fp8):
         _check_stats(run, ora)
     finally:
         run.close()
+
+
+@pytest.mark.parametrize("n_experts,top_k,hidden", [(8, 3, 512), (64, 8, 2048), (512, 32, 256), (33, 1, 256)])
+def test_routing_alone_at_the_edges_of_its_range(n_experts, top_k, hidden):
+    """oled_route_noalloc from 1 to 256 tokens (one and two tokens per CTA, parts of the assignment list of one warp and
+    of many), with a bias: ids, gate scores, counts, offsets and the stable order equal the oracle's bit for bit."""
+    from oracle import moe_layer as oracle_moe
+    from paper_2609_33385_b200 import binding
+    from paper_2609_33385_b200.runner import bits_to_dev
+    dev = torch.device("cuda:0")
+    w = synth.tiny(n_layers=1, n_experts=n_experts, top_k=top_k, hidden=hidden, zipf_bias=0.3)
+    wr_bits, bias = synth.router_weights(w, 0)
+    wr, b = bits_to_dev(wr_bits, dev), torch.from_numpy(bias).to(dev)
+    stream = torch.cuda.current_stream(dev).cuda_stream
+    for n in (256, 1, 148, 149, 33, 255):
+        h_bits, conf = synth.flat_tokens(w, n, 400)
+        x, c = bits_to_dev(h_bits, dev), torch.from_numpy(conf).to(dev)
+        ids, perm = (torch.full((n * top_k,), -1, dtype=torch.int32, device=dev) for _ in range(2))
+        gate = torch.zeros(n * top_k, device=dev)
+        counts, offsets = (torch.full((m,), -1, dtype=torch.int32, device=dev) for m in (n_experts, n_experts + 1))
+        rc = binding.route_noalloc(x.data_ptr(), wr.data_ptr(), b.data_ptr(), c.data_ptr(), n, hidden, n_experts, top_k, stream,
+                                   ids.data_ptr(), gate.data_ptr(), counts.data_ptr(), offsets.data_ptr(), perm.data_ptr())
+        assert rc == binding.OLED_OK, binding.strerror(rc)
+        torch.cuda.synchronize(dev)
+        logits = oracle_moe.gate_logits(oracle_moe.bf16_to_f32(h_bits), oracle_moe.bf16_to_f32(wr_bits), bias)
+        o_ids, o_gate = oracle_moe.topk_route(logits, top_k)
+        o_counts, o_offsets, o_perm, _ = oracle_moe.permutation(o_ids, n_experts)
+        assert np.array_equal(ids.cpu().numpy().reshape(n, top_k), o_ids)
+        assert np.array_equal(gate.cpu().numpy().view(np.uint32).reshape(n, top_k), o_gate.view(np.uint32))
+        assert np.array_equal(counts.cpu().numpy(), o_counts) and np.array_equal(offsets.cpu().numpy(), o_offsets)
+        assert np.array_equal(perm.cpu().numpy(), o_perm)
