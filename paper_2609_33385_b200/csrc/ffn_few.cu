@@ -136,11 +136,6 @@ __device__ __forceinline__ void few_prefetch_w1(const CUtensorMap* map, int k, i
                : "memory");
 }
 
-// mbar_wait by a whole warp with one outcome for all lanes.
-__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, uint32_t* status) {
-  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status)) != 0;
-}
-
 // One intermediate row (bf16, its largest magnitude final) as two e4m3 terms per element; thread `rank` of `n`.
 __device__ __forceinline__ void split_row(const uint16_t* hbuf, const TokenSplit& split, int row, int I, int rank, int n) {
   const float scale = token_scale(__ldcg(split.amax_mid + row));

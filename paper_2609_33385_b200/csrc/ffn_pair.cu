@@ -14,7 +14,7 @@
 //           epilogue hbuf[n, f] = bf16(silu(D_gate) * D_up)
 //   KIND 2: output rows c0 + 256 r .. + 255 for CTA r (two row blocks of Wd), epilogue y[n, c] = D
 // No TMA multicast: every CTA loads what lies in its own shared memory.
-// 19 warps per CTA: 16 epilogue warps, the TMA thread's, the MMA thread's, and one whose first thread
+// 11 warps per CTA: 8 epilogue warps, the TMA thread's, the MMA thread's, and one whose first thread
 // gathers token rows when the launch is asked to (PairTokens below); its lanes are idle otherwise.
 //
 // Protocol per pipeline stage (barriers at the same shared-memory offsets in both CTAs):
@@ -44,7 +44,7 @@
 namespace oled {
 namespace {
 
-constexpr int kPairEpiWarps = 16;
+constexpr int kPairEpiWarps = 8;
 constexpr int kPairProducerWarp = kPairEpiWarps;
 constexpr int kPairMmaWarp = kPairEpiWarps + 1;
 constexpr int kPairGatherWarp = kPairEpiWarps + 2;
@@ -160,11 +160,15 @@ __device__ __forceinline__ int take_pair_item(PairCtl* ctl, int seq, volatile in
   return *reinterpret_cast<volatile int*>(&ctl->item_ring[slot]);
 }
 
+// Token rows and intermediate rows, boxes of 16, 32, 64 and 128 rows: each CTA copies the smallest that holds its half
+// of the tile's rows.
+struct PairActs {
+  CUtensorMap x[4], h[4];
+};
 // What a FUSED launch (KIND 3) needs on top: the down projection's tensor maps, its output and the
 // completion counters (one ZERO word per expert of the group).
 struct PairSecond {
   CUtensorMap tm_w2;    // down-projection weights
-  CUtensorMap tm_act2;  // intermediate rows (hbuf)
   void* out2;           // y
   uint32_t* done;       // per expert: epilogue warps (of either CTA) that have stored gate/up rows
 };
@@ -195,9 +199,9 @@ constexpr int kRowSlots = 3;
 // over long before it is reached except at the switch of phases.
 template <int KIND>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
-ffn_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_act,
+ffn_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ PairActs acts,
                 const __grid_constant__ FfnGroup grp, const __grid_constant__ FfnRows rows, void* __restrict__ out_ptr,
-                int H, int I, int out_bf16, uint32_t* __restrict__ status, uint32_t* __restrict__ work_counter,
+                int H, int I, int out_bf16, int weights_once, uint32_t* __restrict__ status, uint32_t* __restrict__ work_counter,
                 StepTimeline* timeline, int timeline_slot, const __grid_constant__ RouteReport report,
                 const __grid_constant__ PairSecond sec, const __grid_constant__ PairTokens tok) {
   constexpr bool fused = KIND == 3;
@@ -226,11 +230,7 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant_
   }
   if (warp == kPairProducerWarp && lane == 0) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tm_w)) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tm_act)) : "memory");
-    if (fused) {
-      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&sec.tm_w2)) : "memory");
-      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&sec.tm_act2)) : "memory");
-    }
+    if (fused) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&sec.tm_w2)) : "memory");
   }
   if (warp == kPairMmaWarp) {  // all 512 columns, allocated by the same warp of both CTAs
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl->tmem_base)),
@@ -287,38 +287,46 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant_
   const uint32_t full_on_first = map_to_cta(smem_u32(&ctl->full[0]), 0);         // cluster-wide addresses
   const uint32_t tmem_empty_on_first = map_to_cta(smem_u32(&ctl->tmem_empty), 0);
 
-  if (KIND != 2 && blockIdx.x == 0 && warp == kPairProducerWarp && lane != 0) publish_report(report, lane - 1, 31);
+  if (KIND != 2 && blockIdx.x == 0 && warp == kPairGatherWarp && lane != 0) publish_report(report, lane - 1, 31);
 
-  if (warp == kPairProducerWarp && lane == 0) {
-    // ------------------------------------------------------------ TMA producer (one per CTA)
+  if (warp == kPairProducerWarp) {
+    // ------------------------------------------------------------ TMA producer (one warp per CTA, an elected lane copies)
     int stage = 0, ready_g = -1;
     PairCursor cur;
     uint32_t phase = 0;
     bool ok = true;
+    // Where every expert has one token tile its weights are read once and leave L2 first, so that what the layers hand on
+    // survives (4 layers of 1000 tokens 847 us, with it 809); with several tiles they are read again (one layer of 4096
+    // tokens 1345 us, with it 1510).
+    uint64_t policy;
+    if (weights_once) asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+    else asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(policy));
     int next_item = pair;  // (first CTA) the pair's first item is its own number
     // (with loads withheld - the test of the bounded waits - nothing is published either: every
     // other role of both CTAs runs into the limit of its wait for the first item)
     for (int seq = 0; ok && !(grp.withhold_loads && rank == 0); ++seq) {
-      int item;
+      int item, drawn = 0;
       if (rank == 0) {
         item = next_item < total_items ? next_item : -1;
-        // the following item's number is fetched now: the atomic's latency lies under this item's copies
-        if (item >= 0) next_item = (int)atomicAdd(work_counter, 1u) + n_pairs;
-        const int slot = seq % kPairRing;
-        *reinterpret_cast<volatile int*>(&ctl->item_ring[slot]) = item;
-        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(map_to_cta(smem_u32(&ctl->item_ring[slot]), 1)), "r"(item)
-                     : "memory");
-        mbar_arrive_cluster(map_to_cta(smem_u32(&ctl->item_full[slot]), 0));
-        mbar_arrive_cluster(map_to_cta(smem_u32(&ctl->item_full[slot]), 1));
+        if (lane == 0) {
+          // the following item's number is fetched now: the atomic's latency lies under this item's copies
+          if (item >= 0) drawn = (int)atomicAdd(work_counter, 1u) + n_pairs;
+          const int slot = seq % kPairRing;
+          *reinterpret_cast<volatile int*>(&ctl->item_ring[slot]) = item;
+          asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(map_to_cta(smem_u32(&ctl->item_ring[slot]), 1)), "r"(item)
+                       : "memory");
+          mbar_arrive_cluster(map_to_cta(smem_u32(&ctl->item_full[slot]), 0));
+          mbar_arrive_cluster(map_to_cta(smem_u32(&ctl->item_full[slot]), 1));
+        }
+        __syncwarp();
       } else {
-        item = take_pair_item(ctl, seq, abort_flag, status);
+        item = __shfl_sync(0xffffffffu, take_pair_item(ctl, seq, abort_flag, status), 0);
       }
       if (item < 0) break;
       PairItem it;
       pair_decode(ctl, grp, item, plan, cur, it);
       const bool down_of_fused = fused && it.kind == 2;
       const CUtensorMap* map_w = down_of_fused ? &sec.tm_w2 : &tm_w;
-      const CUtensorMap* map_act = down_of_fused ? &sec.tm_act2 : &tm_act;
       const int k_blocks = (it.kind == 1 ? H : I) / kPairK;
       // what the item's token operand waits for: (down items of a fused launch) all intermediate rows of
       // the expert stored by its gate/up items; (gate/up items of a launch that gathers) the tile's token
@@ -334,16 +342,15 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant_
         for (uint32_t spin = 0; ok; ++spin) {
           uint32_t seen;
           asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(counter) : "memory");
-          if (seen >= target) break;
+          if (__all_sync(0xffffffffu, seen >= target)) break;
           if ((spin & 255u) == 255u) {
-            if (*abort_flag) ok = false;
             const unsigned long long now = globaltimer();
             if (t0 == 0) t0 = now;
             if (now - t0 > kWaitLimitNs) {
               *abort_flag = 1;
               atomicExch(status, (uint32_t)kStatusWaitTimeout);
-              ok = false;
             }
+            if (__any_sync(0xffffffffu, *abort_flag != 0)) ok = false;
           }
         }
         if (!ok) break;
@@ -352,31 +359,34 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant_
         // This is the only proxy fence between the two; on the writers' side it would wait for the CTA's copies in flight)
         asm volatile("fence.proxy.async.global;" ::: "memory");
       }
-      const int n_mma = max(32, (it.valid + 31) & ~31);
-      const int my_row0 = it.row0 + (int)rank * (n_mma >> 1);  // this CTA's half of the tile's token rows
+      const int half = max(32, (it.valid + 31) & ~31) >> 1;  // token rows this CTA holds for the pair's MMAs
+      const int box = half <= 16 ? 0 : half <= 32 ? 1 : half <= 64 ? 2 : 3;
+      const CUtensorMap* const map_act = (it.kind == 1 ? acts.x : acts.h) + box;
+      const uint32_t pair_bytes = 2u * (2u * kPairATile + (16u << box) * 128u);  // a stage's, both CTAs
+      const int my_row0 = it.row0 + (int)rank * half;
       const int my_m0 = it.m0 + (int)rank * (it.kind == 1 ? 128 : 256);
+      const int second_row = it.kind == 1 ? I + my_m0 : my_m0 + 128;  // gate and up rows, or two row blocks of Wd
       for (int kb = 0; kb < k_blocks; ++kb) {
-        if (!mbar_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, abort_flag, status)) {
+        if (!warp_wait(smem_u32(&ctl->empty[stage]), phase ^ 1u, abort_flag, status)) {
           ok = false;
           break;
         }
-        const uint32_t bar = full_on_first + (uint32_t)stage * 8u;
-        if (rank == 0) mbar_expect_tx(smem_u32(&ctl->full[stage]), 2u * kPairStage);
-        const uint32_t base = tiles_base + (uint32_t)stage * kPairStage;
-        const int k0 = kb * kPairK;
-        if (it.kind == 1) {
-          tma_load_3d_pair(map_w, base, bar, k0, my_m0, it.slot);                   // gate rows
-          tma_load_3d_pair(map_w, base + kPairATile, bar, k0, I + my_m0, it.slot);  // up rows
-        } else {
-          tma_load_3d_pair(map_w, base, bar, k0, my_m0, it.slot);
-          tma_load_3d_pair(map_w, base + kPairATile, bar, k0, my_m0 + 128, it.slot);
+        if (elect_one()) {
+          const uint32_t bar = full_on_first + (uint32_t)stage * 8u;
+          if (rank == 0) mbar_expect_tx(smem_u32(&ctl->full[stage]), pair_bytes);
+          const uint32_t base = tiles_base + (uint32_t)stage * kPairStage;
+          const int k0 = kb * kPairK;
+          tma_load_3d_pair(map_w, base, bar, k0, my_m0, it.slot, policy);
+          tma_load_3d_pair(map_w, base + kPairATile, bar, k0, second_row, it.slot, policy);
+          tma_load_2d_pair(map_act, base + 2 * kPairATile, bar, k0, my_row0);
         }
-        tma_load_2d_pair(map_act, base + 2 * kPairATile, bar, k0, my_row0);
+        __syncwarp();
         if (++stage == kPairStages) {
           stage = 0;
           phase ^= 1u;
         }
       }
+      next_item = __shfl_sync(0xffffffffu, drawn, 0);
     }
     if (!ok) {  // let copies already issued land before the CTA's shared memory is released
       const unsigned long long t0 = globaltimer();
@@ -458,52 +468,59 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant_
         }
       }
     }
-  } else if (warp == kPairMmaWarp && lane == 0 && rank == 0) {
+  } else if (warp == kPairMmaWarp && rank == 0) {
     // ------------------------------------------------------------ MMA issuer (first CTA only)
-    int stage = 0, local = 0;
+    // The whole warp runs the loop and one elected lane issues, which keeps the descriptors in uniform registers
+    // (ffn_few.cu): a single lane in a divergent branch took 540 cycles for the eight instructions of a k-block, more than
+    // they last for token tiles of fewer than 136 rows.
+    int stage = 0;
     PairCursor cur;
     uint32_t phase = 0;
     bool ok = true;
-    const uint32_t desc_hi = (uint32_t)(make_smem_desc(0) >> 32);
-    const uint32_t a_lo0 = (uint32_t)make_smem_desc(tiles_base);
-    const uint32_t b_lo0 = (uint32_t)make_smem_desc(tiles_base + 2 * kPairATile);
-    const uint32_t ring_step = kPairStage >> 4;
-    uint32_t a_lo = a_lo0, b_lo = b_lo0;
-    for (; ok; ++local) {
-      const int item = take_pair_item(ctl, local, abort_flag, status);
+    const uint64_t a_desc0 = make_smem_desc(tiles_base), b_desc0 = make_smem_desc(tiles_base + 2 * kPairATile);
+    constexpr uint32_t kStageStep = kPairStage >> 4, kTileStep = kPairATile >> 4;  // descriptor addresses count 16 bytes
+    const uint32_t d0 = __shfl_sync(0xffffffffu, tmem_base, 0);
+    for (int local = 0; ok; ++local) {
+      const int item = __shfl_sync(0xffffffffu, take_pair_item(ctl, local, abort_flag, status), 0);
       if (item < 0) break;
       PairItem it;
       pair_decode(ctl, grp, item, plan, cur, it);
       const int k_blocks = (it.kind == 1 ? H : I) / kPairK;
       // one accumulator stage: both CTAs' epilogues must have drained the previous item
-      if (!mbar_wait(smem_u32(&ctl->tmem_empty), ((uint32_t)local & 1u) ^ 1u, abort_flag, status)) break;
+      if (!warp_wait(smem_u32(&ctl->tmem_empty), ((uint32_t)local & 1u) ^ 1u, abort_flag, status)) break;
       tc_fence_after();
-      const int n_mma = max(32, (it.valid + 31) & ~31);
-      const uint32_t idesc = make_idesc_pair(n_mma);
+      const uint32_t idesc = __shfl_sync(0xffffffffu, make_idesc_pair(max(32, (it.valid + 31) & ~31)), 0);
       for (int kb = 0; kb < k_blocks; ++kb) {
-        if (!mbar_wait(smem_u32(&ctl->full[stage]), phase, abort_flag, status)) {
+        if (!warp_wait(smem_u32(&ctl->full[stage]), phase, abort_flag, status)) {
           ok = false;
           break;
         }
         tc_fence_after();
+        if (elect_one()) {
+          const uint64_t a0 = a_desc0 + (uint64_t)((uint32_t)stage * kStageStep);
+          const uint64_t b0 = b_desc0 + (uint64_t)((uint32_t)stage * kStageStep);
+          // 32 bytes along K = 2 address units
+          if (kb == 0) {
+            tc_mma_pair<false>(d0, a0, b0, idesc);
+            tc_mma_pair<false>(d0 + (uint32_t)kPairN, a0 + kTileStep, b0, idesc);
+          } else {
+            tc_mma_pair<true>(d0, a0, b0, idesc);
+            tc_mma_pair<true>(d0 + (uint32_t)kPairN, a0 + kTileStep, b0, idesc);
+          }
 #pragma unroll
-        for (int k = 0; k < kPairK / 16; ++k) {  // 32 bytes along K = 2 address units
-          const uint32_t accum = (kb | k) != 0 ? 1u : 0u;
-          tc_mma_pair_lo(tmem_base, a_lo + k * 2, b_lo + k * 2, desc_hi, idesc, accum);
-          tc_mma_pair_lo(tmem_base + (uint32_t)kPairN, a_lo + (kPairATile >> 4) + k * 2, b_lo + k * 2, desc_hi, idesc,
-                         accum);
+          for (int k = 1; k < kPairK / 16; ++k) {
+            tc_mma_pair<true>(d0, a0 + k * 2, b0 + k * 2, idesc);
+            tc_mma_pair<true>(d0 + (uint32_t)kPairN, a0 + kTileStep + k * 2, b0 + k * 2, idesc);
+          }
+          tc_commit_pair(smem_u32(&ctl->empty[stage]), 3u);
+          if (kb + 1 == k_blocks) tc_commit_pair(smem_u32(&ctl->tmem_full), 3u);
         }
-        tc_commit_pair(smem_u32(&ctl->empty[stage]), 3u);
-        a_lo += ring_step;
-        b_lo += ring_step;
+        __syncwarp();
         if (++stage == kPairStages) {
           stage = 0;
           phase ^= 1u;
-          a_lo = a_lo0;
-          b_lo = b_lo0;
         }
       }
-      if (ok) tc_commit_pair(smem_u32(&ctl->tmem_full), 3u);
     }
   } else if (warp < kPairEpiWarps) {
     // ------------------------------------------------------------ epilogue (both CTAs)
@@ -558,72 +575,99 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant_
       const int n_mma = max(32, (it.valid + 31) & ~31);
       const int col = it.m0 + (int)rank * (it.kind == 1 ? 128 : 256) + quarter * 32 + lane;  // feature / output row of this thread
       void* const out_y = fused ? sec.out2 : out_ptr;
-      // The warp's chunks, one in registers while the next one's TMEM loads are in flight; the
-      // accumulators are handed back as soon as the LAST chunk has been read - its arithmetic and
-      // stores run while the MMAs of the next item already write the columns.
-      constexpr int kStep = 16 * (kPairEpiWarps / 4);
-      uint32_t na[16], nb[16];
-      int c = part * 16;
-      if (c < n_mma) {
-        tmem_ld16(t_row + (uint32_t)c, na);
-        tmem_ld16(t_row + (uint32_t)(kPairN + c), nb);
-      }
-      bool released = false;
-      for (; c < n_mma; c += kStep) {
-        uint32_t ra[16], rb[16];
-        tmem_ld_wait();
+      // The warp's chunks (four at most: chunk ci is columns 16 * (4 ci + part) ..).  The accumulators are handed back
+      // as soon as the LAST chunk has been read, so what stands before that is kept short: the results
+      // stay in registers as packed bf16 and are stored afterwards, while the MMAs of the next item already write
+      // the columns.  (With every chunk stored before the next was read the MMAs waited 8000 cycles per item, 16 % of a
+      // launch of 4096 tokens; 16 epilogue warps had no registers for it, eight do: 2 layers of 2048 tokens 668 us, now 647.)
+      constexpr int kStep = 16 * (kPairEpiWarps / 4), kChunks = kPairN / kStep;
+      auto release = [&]() {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(tmem_empty_on_first);
+      };
+      const int c0 = part * 16;
+      if (it.kind == 1 || out_bf16) {
+        const bool gate_up = it.kind == 1;
+        uint32_t ra[16], rb[16], held[kChunks - 1][16];  // (gate/up: the first eight words of a chunk)
+        auto pack = [&](uint32_t* out) {
+          if (gate_up) {
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          ra[j] = na[j];
-          rb[j] = nb[j];
-        }
-        if (c + kStep < n_mma) {
-          tmem_ld16(t_row + (uint32_t)(c + kStep), na);
-          tmem_ld16(t_row + (uint32_t)(kPairN + c + kStep), nb);
-        } else {
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive_cluster(tmem_empty_on_first);
-          released = true;
-        }
-        const bool whole = c + 16 <= it.valid;  // no ragged end inside this chunk
-        if (it.kind == 1) {
-          uint16_t* p = reinterpret_cast<uint16_t*>(out_ptr) + (size_t)(it.row0 + c) * I + col;
-#pragma unroll
-          for (int j = 0; j < 16; ++j, p += I)
-            if (whole || c + j < it.valid) {
-              const float a = __uint_as_float(ra[j]);
-              const float hm = __fdividef(a, 1.0f + __expf(-a)) * __uint_as_float(rb[j]);
-              const __nv_bfloat16 b = __float2bfloat16_rn(hm);
-              *p = *reinterpret_cast<const uint16_t*>(&b);
+            for (int j = 0; j < 16; j += 2) {
+              const float a0 = __uint_as_float(ra[j]), a1 = __uint_as_float(ra[j + 1]);
+              const __nv_bfloat162 h =
+                  __floats2bfloat162_rn(__fdividef(a0, 1.0f + __expf(-a0)) * __uint_as_float(rb[j]),
+                                        __fdividef(a1, 1.0f + __expf(-a1)) * __uint_as_float(rb[j + 1]));
+              out[j / 2] = *reinterpret_cast<const uint32_t*>(&h);
             }
-        } else if (out_bf16) {  // many-token steps keep y in bf16
-          uint16_t* p = reinterpret_cast<uint16_t*>(out_y) + (size_t)(it.row0 + c) * H + col;
+          } else {
 #pragma unroll
-          for (int j = 0; j < 16; ++j, p += H)
-            if (whole || c + j < it.valid) {
-              const __nv_bfloat16 b0 = __float2bfloat16_rn(__uint_as_float(ra[j]));
-              const __nv_bfloat16 b1 = __float2bfloat16_rn(__uint_as_float(rb[j]));
-              p[0] = *reinterpret_cast<const uint16_t*>(&b0);
-              p[128] = *reinterpret_cast<const uint16_t*>(&b1);
+            for (int j = 0; j < 16; ++j) {  // row j: this thread's two outputs (128 columns apart)
+              const __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(ra[j]), __uint_as_float(rb[j]));
+              out[j] = *reinterpret_cast<const uint32_t*>(&h);
             }
-        } else {
-          // (few-token steps only: in a scattered one the output goes to the row's assignment)
+          }
+        };
+        auto store = [&](int c, const uint32_t* packed) {
+          const bool whole = c + 16 <= it.valid;  // no ragged end inside this chunk
+          if (gate_up) {
+            uint16_t* p = reinterpret_cast<uint16_t*>(out_ptr) + (size_t)(it.row0 + c) * I + col;
+#pragma unroll
+            for (int j = 0; j < 16; ++j, p += I)
+              if (whole || c + j < it.valid) *p = (uint16_t)(packed[j / 2] >> (16 * (j & 1)));
+          } else {  // many-token steps keep y in bf16
+            uint16_t* p = reinterpret_cast<uint16_t*>(out_y) + (size_t)(it.row0 + c) * H + col;
+#pragma unroll
+            for (int j = 0; j < 16; ++j, p += H)
+              if (whole || c + j < it.valid) {
+                p[0] = (uint16_t)packed[j];
+                p[128] = (uint16_t)(packed[j] >> 16);
+              }
+          }
+        };
+        auto load = [&](int c) {
+          tmem_ld16(t_row + (uint32_t)c, ra);
+          tmem_ld16(t_row + (uint32_t)(kPairN + c), rb);
+        };
+        if (c0 < n_mma) load(c0);
+        else release();  // (a warp without a chunk in this item)
+#pragma unroll
+        for (int ci = 0; ci < kChunks; ++ci) {
+          const int c = c0 + ci * kStep;
+          if (c >= n_mma) break;
+          tmem_ld_wait();
+          if (c + kStep >= n_mma) release();
+          if (ci + 1 < kChunks) {
+            pack(held[ci < kChunks - 1 ? ci : 0]);
+            if (c + kStep < n_mma) load(c + kStep);
+          } else {
+            uint32_t last[16];
+            pack(last);
+            store(c, last);
+          }
+        }
+#pragma unroll
+        for (int ci = 0; ci + 1 < kChunks; ++ci)
+          if (c0 + ci * kStep < n_mma) store(c0 + ci * kStep, held[ci]);
+      } else {  // (few-token steps: fp32 outputs)
+        if (c0 >= n_mma) release();
+        for (int c = c0; c < n_mma; c += kStep) {
+          uint32_t ra[16], rb[16];
+          tmem_ld16(t_row + (uint32_t)c, ra);
+          tmem_ld16(t_row + (uint32_t)(kPairN + c), rb);
+          tmem_ld_wait();
+          if (c + kStep >= n_mma) release();
+          // (in a scattered step the output goes to the row's assignment)
           float* const y0 = reinterpret_cast<float*>(out_y) + col;
 #pragma unroll
           for (int j = 0; j < 16; ++j)
-            if (whole || c + j < it.valid) {
+            if (c + j < it.valid) {
               const int r = it.row0 + c + j;
               float* const p = y0 + (size_t)(rows.assignment != nullptr ? __ldg(rows.assignment + r) : r) * H;
               p[0] = __uint_as_float(ra[j]);
               p[128] = __uint_as_float(rb[j]);
             }
         }
-      }
-      if (!released) {  // (a warp without a chunk in this item)
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(tmem_empty_on_first);
       }
       if (fused && it.kind == 1) {
         // this warp's intermediate rows of the item are stored: counted once they are visible device-wide
@@ -652,7 +696,7 @@ bool ffn_pair_usable(const FfnTcMaps& maps, int n_box, int H, int I) {
 }
 
 int launch_ffn_pair(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp, int kind, const FfnRows& rows,
-                    uint16_t* hbuf, float* y, int y_bf16, int H, int I, int n_sms, uint32_t* status,
+                    uint16_t* hbuf, float* y, int y_bf16, int weights_once, int H, int I, int n_sms, uint32_t* status,
                     uint32_t* work_counter, StepTimeline* timeline, int timeline_slot, const RouteReport& report,
                     uint32_t* done) {
   static bool attr_done = false;
@@ -665,9 +709,13 @@ int launch_ffn_pair(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp,
   }
   const int grid = 2 * (n_sms / 2);  // one CTA per SM, in pairs
   cudaError_t err;
+  PairActs acts;
+  for (int i = 0; i < 4; ++i) {
+    acts.x[i] = maps.xp[i];
+    acts.h[i] = maps.hbuf[i];
+  }
   PairSecond sec;
   sec.tm_w2 = maps.w2;
-  sec.tm_act2 = maps.hbuf[3];
   sec.out2 = y;
   sec.done = done;
   PairTokens tok;
@@ -680,14 +728,14 @@ int launch_ffn_pair(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp,
   if (gathers && tok.ready == nullptr) return OLED_ERR_INVALID_ARG;
   if (kind == 3) {
     if (done == nullptr) return OLED_ERR_INVALID_ARG;
-    err = launch_pdl(ffn_pair_kernel<3>, dim3(grid), dim3(kPairThreads), kPairSmem, st, maps.w13, maps.xp[3], grp, rows,
-                     (void*)hbuf, H, I, y_bf16, status, work_counter, timeline, timeline_slot, report, sec, tok);
+    err = launch_pdl(ffn_pair_kernel<3>, dim3(grid), dim3(kPairThreads), kPairSmem, st, maps.w13, acts, grp, rows,
+                     (void*)hbuf, H, I, y_bf16, weights_once, status, work_counter, timeline, timeline_slot, report, sec, tok);
   } else if (kind == 1)
-    err = launch_pdl(ffn_pair_kernel<1>, dim3(grid), dim3(kPairThreads), kPairSmem, st, maps.w13, maps.xp[3], grp, rows,
-                     (void*)hbuf, H, I, 0, status, work_counter, timeline, timeline_slot, report, sec, tok);
+    err = launch_pdl(ffn_pair_kernel<1>, dim3(grid), dim3(kPairThreads), kPairSmem, st, maps.w13, acts, grp, rows,
+                     (void*)hbuf, H, I, 0, weights_once, status, work_counter, timeline, timeline_slot, report, sec, tok);
   else
-    err = launch_pdl(ffn_pair_kernel<2>, dim3(grid), dim3(kPairThreads), kPairSmem, st, maps.w2, maps.hbuf[3], grp,
-                     rows, (void*)y, H, I, y_bf16, status, work_counter, timeline, timeline_slot, RouteReport{}, sec, tok);
+    err = launch_pdl(ffn_pair_kernel<2>, dim3(grid), dim3(kPairThreads), kPairSmem, st, maps.w2, acts, grp,
+                     rows, (void*)y, H, I, y_bf16, weights_once, status, work_counter, timeline, timeline_slot, RouteReport{}, sec, tok);
   return err == cudaSuccess ? OLED_OK : OLED_ERR_CUDA;
 }
 

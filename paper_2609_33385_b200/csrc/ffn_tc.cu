@@ -850,7 +850,7 @@ int launch_ffn_tc(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp_in
   // many-token tiles: the CTA-pair kernel, unless its cluster launch has failed before on this
   // device (the one-CTA form below computes the same)
   if (maps.use_pairs && !g_pairs_refused && ffn_pair_usable(maps, grp.n_box, H, I)) {
-    if (launch_ffn_pair(st, maps, grp, kind, rows, hbuf, y, y_bf16, H, I, n_sms, status, work_counter, timeline,
+    if (launch_ffn_pair(st, maps, grp, kind, rows, hbuf, y, y_bf16, max_count <= 256 ? 1 : 0, H, I, n_sms, status, work_counter, timeline,
                         timeline_slot, report, done) == OLED_OK)
       return OLED_OK;
     cudaGetLastError();  // (a refused launch enqueues nothing)

@@ -302,7 +302,7 @@ bool ffn_pair_can_fuse(const FfnTcMaps& maps, int max_count, int H, int I);  // 
 // in one launch (`done`: one ZERO word per expert of the group).
 bool ffn_pair_usable(const FfnTcMaps& maps, int n_box, int H, int I);
 int launch_ffn_pair(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp, int kind, const FfnRows& rows,
-                    uint16_t* hbuf, float* y, int y_bf16, int H, int I, int n_sms, uint32_t* status,
+                    uint16_t* hbuf, float* y, int y_bf16, int weights_once, int H, int I, int n_sms, uint32_t* status,
                     uint32_t* work_counter, StepTimeline* timeline, int timeline_slot, const RouteReport& report,
                     uint32_t* done = nullptr);
 constexpr int kFfnWorkCounters = 8;  // FFN launches of one layer execution: 3 groups x 2 kinds, rounded up
