@@ -238,8 +238,11 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
     __syncwarp();
     if (spec && elect_one()) {
       for (int i = 0; i < pre1; ++i) load_weights(i, i, false, spec_m, grp.slot[spec_g]);
-      for (int a = pre1 * p.k_atoms; a < k_blocks1 * p.k_atoms; ++a)
-        few_prefetch_w1(&p.tm_w1, a * kK, spec_m, grp.slot[spec_g], policy);
+      // the rest of the item into L2, for steps whose gate kernel is short (8 layers of 16 similar tokens 362 -> 356 us; with
+      // 250 tokens fp8 it took bandwidth from the gate's own loads, 775 -> 789, with 100 tokens still 523 -> 517)
+      if (p.rows.cap <= 148)
+        for (int a = pre1 * p.k_atoms; a < k_blocks1 * p.k_atoms; ++a)
+          few_prefetch_w1(&p.tm_w1, a * kK, spec_m, grp.slot[spec_g], policy);
     }
     __syncwarp();
   }
@@ -779,7 +782,7 @@ split_rows_kernel(const __grid_constant__ FfnGroup grp, const __grid_constant__ 
     split_row(hbuf, split, r, I, lane + 32 * (int)blockIdx.y, 32 * (int)gridDim.y);
 }
 
-// Stage shape and count: two k-blocks per stage where at least four such stages fit and both contractions
+// Stage shape and count: two k-blocks per stage where at least three such stages fit and both contractions
 // have an even number of them (half the waits and commits on the MMA thread); ten bf16 k-blocks in flight
 // at most (eleven measured slower), eight of e4m3 codes (16 tokens, 8 layers: 557 us, with ten 569).
 struct FewRings {
@@ -791,7 +794,7 @@ FewRings few_rings(int n_box, bool fp8, int H, int I) {
   const int kblocks = (int)std::min<uint32_t>(fp8 ? 8u : 10u, (kFewSmemMax - kFewCtlBytes - 1024u) / atom);
   const int kk = fp8 ? 128 : 64;
   FewRings r;
-  r.k_atoms = kblocks >= 8 && (H / kk) % 2 == 0 && (I / kk) % 2 == 0 ? 2 : 1;
+  r.k_atoms = kblocks >= 6 && (H / kk) % 2 == 0 && (I / kk) % 2 == 0 ? 2 : 1;
   r.stages = std::min(kblocks / r.k_atoms, kFewMaxStages);
   r.smem = kFewCtlBytes + 1024u + (uint32_t)(r.stages * r.k_atoms) * atom;
   return r;

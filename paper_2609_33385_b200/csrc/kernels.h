@@ -203,7 +203,7 @@ struct FfnRows {
 };
 // Offsets (exclusive scan), stable permutation by expert and its inverse.  With xp != nullptr the
 // kernel also gathers the token rows (xp[r,:] = x[perm[r]/K,:]); meant for small steps.
-// seg_counts (launches that do not gather; nullptr: none): the gate kernel's per-segment counts (see
+// seg_counts (many-token steps; nullptr: none): the gate kernel's per-segment counts (see
 // launch_route): kPermuteSegments CTAs per expert then scan one segment of the assignment list each.
 // split (gathering launches only; nullptr: none): the kernel also writes, per sorted row, the
 // largest magnitude of the row it copied and the row's two e4m3 terms, and zeroes amax_mid (see

@@ -831,10 +831,9 @@ static int step_impl(oled_ctx* ctx, int32_t layer, const void* hidden, const flo
                  ctx->d_logits, ctx->d_ids, ctx->d_gate, ctx->d_counts, ctx->d_scores, prev, tl, seg_counts, seg_tokens,
                  ctx->scatter);
   }
-  const bool fuse_gather = few;  // few rows per expert: the permutation kernel, where one runs, copies them
   // Many rows per expert (every FFN launch of the step on CTA pairs, token tiles of 256 rows): no
   // gather kernel, each gate/up launch copies its experts' token rows while its first items run.
-  const bool gather_in_ffn = !fuse_gather && ctx->gather_in_ffn && ctx->ffn_impl == 0 &&
+  const bool gather_in_ffn = !few && ctx->gather_in_ffn && ctx->ffn_impl == 0 &&
                              std::min<size_t>(T, 2 * (((size_t)T * K + E - 1) / E)) > 128 &&
                              (reinterpret_cast<uintptr_t>(hidden) & 15u) == 0 &&  // (bulk copies of whole rows)
                              // (a row's copy - loads, stores, fence and count on one thread - takes as long as 4 M
@@ -842,6 +841,9 @@ static int step_impl(oled_ctx* ctx, int32_t layer, const void* hidden, const flo
                              // of 2048 tokens, H x I 2 M: 875 / 654 us, one of 4096 tokens, 6 M: 1372 / 1418 us)
                              (size_t)H * ctx->shape.intermediate >= (size_t)4 << 20 &&
                              ffn_tc_token_source_usable(ctx->maps, H, ctx->shape.intermediate);
+  // Otherwise the permutation kernel, where one runs, copies the rows (a step without per-segment counts but beyond 4096
+  // assignments leaves that to a gather kernel).
+  const bool fuse_gather = few || (!gather_in_ffn && seg_counts != nullptr);
   if (gather_in_ffn)
     ffn_tc_set_token_source(&ctx->maps, static_cast<const uint16_t*>(hidden), T, ctx->d_perm, K, ctx->d_xp);
   else
@@ -849,8 +851,13 @@ static int step_impl(oled_ctx* ctx, int32_t layer, const void* hidden, const flo
   NvtxRange nv_perm(ctx, "oled.step.2_permutation_counts");
   if (!scattered) {
     ProfScope ps(ctx, OLED_KERNEL_PERMUTE, (uint64_t)T * K * 12 + (fuse_gather ? (uint64_t)T * K * H * 4 : 0), 0);
-    // (fp8 stores: a gathering permutation kernel also leaves the rows' magnitudes for the FFN)
-    ctx->step_split = fuse_gather && ctx->fp8_direct && ctx->split.complete() ? &ctx->split : nullptr;
+    // fp8 stores: a gathering permutation kernel also leaves the rows' terms and magnitudes for the FFN, whose MMAs then
+    // read the codes directly.  In many-token steps only from 1 M elements per expert matrix on: below, the terms of the
+    // intermediate rows take longer than the wider tiles save (direct / widened, us: 64 experts of 2048 x 1024, 2048 tokens
+    // 355 / 515, 4096 tokens 662 / 897; 4096 x 1536, 4096 tokens 1665 / 2505; 128 experts of 2048 x 768, 4096 tokens
+    // 626 / 813; but 16 experts of 512 x 1024, 1500 tokens 94 / 79, 3000 tokens 123 / 106).
+    const bool terms_pay = few || (size_t)H * ctx->shape.intermediate >= (size_t)1 << 20;
+    ctx->step_split = fuse_gather && terms_pay && ctx->fp8_direct && ctx->split.complete() ? &ctx->split : nullptr;
     launch_permute(st, ctx->d_ids, ctx->d_counts, T, E, K, ctx->d_offsets, ctx->d_perm, ctx->d_pos,
                    static_cast<const uint16_t*>(hidden), fuse_gather ? ctx->d_xp : nullptr, H, tl, ctx->step_split,
                    seg_counts, seg_tokens);

@@ -646,7 +646,7 @@ route_many_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ w
 // round trip before the first load), and takes every gridDim.y-th batch of RB rows, so that an
 // expert that received many tokens does not make the step wait for one CTA's chain of batches.
 // Only the CTAs with blockIdx.y == 0 write offsets, perm and pos.
-constexpr int kGatherTokMax = 4096;  // rows of one expert in a step that gathers here (T * K <= 4096)
+constexpr int kGatherTokMax = 4096;  // rows of one expert in a step that gathers here (T * K <= 4096), or in a segment
 // RB: rows a CTA copies at a time.  Two, with eight CTAs per expert, in gathering launches: an
 // expert's handful of rows is then spread over several SMs (with one CTA taking eight rows the
 // step waited 3 us longer whenever an expert had more than eight, and the e4m3 terms of fp8
@@ -660,12 +660,12 @@ permute_kernel(const int32_t* __restrict__ ids, const int32_t* __restrict__ coun
   uint32_t* const amax_in = split.amax_in;
   uint32_t* const amax_mid = split.amax_mid;
   __shared__ int s_red[8];
-  __shared__ int s_base;
+  __shared__ int s_base, s_seg;
   __shared__ int s_tok[kGatherTokMax];
   __shared__ uint32_t s_amax[3][RB];  // per batch of RB rows, three batches in rotation (see the gather loop)
   const int e = blockIdx.x;
-  // segmented launches (no gathering): CTA (e, s) scans segment s of the assignment list only and
-  // starts behind the expert's rows of the earlier segments, whose number the gate kernel counted
+  // segmented launches: CTA (e, s) scans segment s of the assignment list only and starts behind the expert's rows of
+  // the earlier segments, whose number the gate kernel counted
   const bool segmented = seg_counts != nullptr;
   const bool writer = blockIdx.y == 0 || segmented;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -674,6 +674,12 @@ permute_kernel(const int32_t* __restrict__ ids, const int32_t* __restrict__ coun
   griddep_wait();
   if (threadIdx.x == 0) timeline_start(timeline, 1);
   int part = 0;
+  if (segmented && warp == 1) {  // the expert's rows of the earlier segments (requested together: one after the other, 16 of
+                                 // them were most of this kernel's 9 us at 1000 tokens)
+    int s = lane < (int)blockIdx.y ? seg_counts[lane * E + e] : 0;
+    s = __reduce_add_sync(0xffffffffu, s);
+    if (lane == 0) s_seg = s;
+  }
   for (int i = threadIdx.x; i < e; i += blockDim.x) part += counts[i];
 #pragma unroll
   for (int d = 16; d >= 1; d >>= 1) part += __shfl_xor_sync(0xffffffffu, part, d);
@@ -687,10 +693,7 @@ permute_kernel(const int32_t* __restrict__ ids, const int32_t* __restrict__ coun
       offsets[e] = off;
       if (e == E - 1) offsets[E] = off + counts[e];
     }
-    if (segmented) {
-      for (int s = 0; s < (int)blockIdx.y; ++s) off += seg_counts[s * E + e];
-      s_base = off;
-    }
+    if (segmented) s_base = off + s_seg;
   }
   __syncthreads();
   // (a CTA beyond the first of an expert has work only if the expert has a batch of rows for it)
@@ -755,11 +758,13 @@ permute_kernel(const int32_t* __restrict__ ids, const int32_t* __restrict__ coun
   __syncthreads();  // the tokens of this expert's rows are in shared memory
   // eight rows at a time: their token numbers, then their loads, are independent memory
   // operations in flight together (a row-by-row loop is a chain of dependent round trips)
-  const int vec_per_row = H / 8, first = s_base, rows = counts[e];
+  // (segmented launches: all rows of the segment are this CTA's)
+  const int vec_per_row = H / 8, first = s_base, rows = segmented ? seg_counts[blockIdx.y * E + e] : counts[e];
+  const int r_first = segmented ? 0 : (int)blockIdx.y * RB, r_step = segmented ? RB : RB * (int)gridDim.y;
   const uint4* src = reinterpret_cast<const uint4*>(x);
   uint4* dst = reinterpret_cast<uint4*>(xp);
   int batch = 0;
-  for (int r0 = (int)blockIdx.y * RB; r0 < rows; r0 += RB * (int)gridDim.y, ++batch) {
+  for (int r0 = r_first; r0 < rows; r0 += r_step, ++batch) {
     int tok[RB];
 #pragma unroll
     for (int j = 0; j < RB; ++j) tok[j] = r0 + j < rows ? s_tok[r0 + j] : -1;
@@ -935,7 +940,11 @@ void launch_permute(cudaStream_t st, const int32_t* ids, const int32_t* counts, 
                     int32_t* offsets, int32_t* perm, int32_t* pos, const uint16_t* x, uint16_t* xp, int H,
                     StepTimeline* timeline, const TokenSplit* split, const int32_t* seg_counts, int seg_tokens) {
   const TokenSplit sp = xp != nullptr && split != nullptr && split->complete() ? *split : TokenSplit{};
-  if (xp != nullptr) {
+  if (xp != nullptr && seg_counts != nullptr) {
+    // many-token steps: each segment's CTA copies its own rows (1000 tokens: a gather kernel behind this one took 6 us)
+    launch_pdl(permute_kernel<4>, dim3(E, kPermuteSegments), dim3(256), 0, st, ids, counts, T * K, E, offsets, perm, pos, x, xp,
+               H, K, timeline, sp, seg_counts, seg_tokens);
+  } else if (xp != nullptr) {
     // gathering steps: two rows per CTA and batch, eight CTAs per expert (see the kernel) - fewer where
     // eight per expert would not be resident at once (four CTAs fit an SM; 128 experts take four each:
     // 7.2 instead of 8.9 us at 256 tokens, two each 9.5 us)

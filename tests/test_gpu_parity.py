@@ -871,12 +871,14 @@ def test_few_token_steps_at_the_edges_of_their_forms(n_experts, top_k, hidden, i
 
 
 @pytest.mark.parametrize("fp8", [False, True], ids=["bf16", "fp8"])
-@pytest.mark.parametrize("n_experts,top_k,counts", [(4, 1, (150, 200, 260, 520)), (10, 4, (120, 130, 250)), (512, 8, (600,))])
-def test_token_tiles_between_16_and_128_rows(n_experts, top_k, counts, fp8):
+@pytest.mark.parametrize("n_experts,top_k,inter,counts", [(4, 1, 128, (150, 200, 260, 520)), (10, 4, 128, (120, 130, 250)),
+                                                           (512, 8, 128, (600,)), (64, 8, 1024, (250, 400, 512))])
+def test_token_tiles_between_16_and_128_rows(n_experts, top_k, inter, counts, fp8):
     """Items of 48, 64, 96 and 128 token rows and several tiles per expert, with the tile taken from the previous
-    execution's counts; 512 experts x 600 tokens: small tiles in a many-token step (bf16 outputs per assignment)."""
+    execution's counts; 512 experts x 600 tokens: small tiles in a many-token step (bf16 outputs per assignment); 64 experts x 1024: more
+    items than CTAs."""
     from paper_2609_33385_b200.runner import bits_to_dev
-    w = synth.tiny(n_layers=1, n_experts=n_experts, top_k=top_k, hidden=256, intermediate=128)
+    w = synth.tiny(n_layers=1, n_experts=n_experts, top_k=top_k, hidden=256, intermediate=inter)
     run = _runner(w, capacity=[n_experts], max_tokens=max(counts), fp8=fp8)
     ora = _oracle_for(run, [n_experts])
     try:
