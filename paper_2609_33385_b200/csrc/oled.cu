@@ -45,6 +45,7 @@ struct oled_ctx {
   int n_sms = 148;
   size_t slot_bytes = 0;
   int n_slots = 0;
+  uint8_t* device_memory = nullptr;  // everything below that is on the device (DeviceLayout)
   uint8_t* pool = nullptr;
   SlotPool slots;
   std::vector<LayerData> layers;
@@ -87,6 +88,7 @@ struct oled_ctx {
   size_t row_buf = 0;          // rows of xp and hbuf: T*k, or more where scattered steps need it (kScatterRows)
   int32_t* d_assignment = nullptr;  // [row_buf] scattered steps: row -> assignment
   ScatterRows scatter;         // the current step's (cap == 0: it sorts its rows)
+  int32_t* d_counts_copy = nullptr;  // [E] for the parity aids
   bool perm_stale = false;     // the last step was scattered: offsets, perm and pos are made when asked for
   uint16_t* d_xp = nullptr;    // [row_buf,H]
   uint16_t* d_hbuf = nullptr;  // [row_buf,I]
@@ -170,32 +172,41 @@ void select_ctrl(oled_ctx* ctx, int sel) {
   ctx->d_seg = reinterpret_cast<int32_t*>(ctx->d_ready + (size_t)kFfnWorkCounters * ctx->ready_words);
 }
 
-template <typename T>
-int dev_alloc(oled_ctx* ctx, T** p, size_t n) {
-  void* q = nullptr;
-  cudaError_t err = cudaMalloc(&q, std::max<size_t>(n, 1) * sizeof(T));
-  if (err != cudaSuccess) {
-    ctx->last_cuda_error = (int)err;
-    cudaGetLastError();
-    return OLED_ERR_OOM;
+// The context's device memory is one allocation (two dozen of them took 5 to 20 ms of oled_create): the buffers are
+// laid out first, each on a 256-byte boundary, and get their addresses when the whole has been allocated.
+struct DeviceLayout {
+  struct Item {
+    void** p;
+    size_t offset;
+  };
+  std::vector<Item> items;
+  size_t total = 0;
+  template <typename T>
+  void add(T** p, size_t n) {
+    items.push_back({reinterpret_cast<void**>(p), total});
+    total += (std::max<size_t>(n, 1) * sizeof(T) + 255) / 256 * 256;
   }
-  *p = static_cast<T*>(q);
-  return OLED_OK;
-}
-
-// A scratch buffer of n elements followed by guard words (16-byte aligned), which the self-check
-// verifies after every step: a kernel that writes past its buffer shows up there.
-template <typename T>
-int dev_alloc_guarded(oled_ctx* ctx, T** p, size_t n) {
-  const size_t bytes = (std::max<size_t>(n, 1) * sizeof(T) + 15) / 16 * 16;
-  uint8_t* q = nullptr;
-  const int rc = dev_alloc(ctx, &q, bytes + kGuardWords * sizeof(uint32_t));
-  if (rc != OLED_OK) return rc;
-  *p = reinterpret_cast<T*>(q);
-  if (ctx->guards.n < (int)(sizeof(ctx->guards.words) / sizeof(ctx->guards.words[0])))
-    ctx->guards.words[ctx->guards.n++] = reinterpret_cast<uint32_t*>(q + bytes);
-  return OLED_OK;
-}
+  // A scratch buffer of n elements followed by guard words (16-byte aligned), which the self-check
+  // verifies after every step: a kernel that writes past its buffer shows up there.
+  template <typename T>
+  void add_guarded(GuardList& guards, T** p, size_t n) {
+    const size_t bytes = (std::max<size_t>(n, 1) * sizeof(T) + 15) / 16 * 16;
+    uint8_t** q = reinterpret_cast<uint8_t**>(p);
+    add(q, bytes + kGuardWords * sizeof(uint32_t));
+    if (guards.n < (int)(sizeof(guards.words) / sizeof(guards.words[0])))
+      items.push_back({reinterpret_cast<void**>(&guards.words[guards.n++]), items.back().offset + bytes});
+  }
+  int allocate(oled_ctx* ctx) {
+    const cudaError_t err = cudaMalloc(reinterpret_cast<void**>(&ctx->device_memory), std::max<size_t>(total, 1));
+    if (err != cudaSuccess) {
+      ctx->last_cuda_error = (int)err;
+      cudaGetLastError();
+      return OLED_ERR_OOM;
+    }
+    for (const Item& it : items) *it.p = ctx->device_memory + it.offset;
+    return OLED_OK;
+  }
+};
 
 inline bool misaligned(const void* p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) != 0; }
 
@@ -217,17 +228,11 @@ inline size_t scatter_cap(size_t T) { return (T + 15) / 16 * 16; }
 int make_perm(oled_ctx* ctx) {
   if (!ctx->perm_stale) return OLED_OK;
   const int E = ctx->shape.n_experts, K = ctx->shape.top_k;
-  int32_t* tmp = nullptr;
-  OLED_CUDA(ctx, cudaMalloc(reinterpret_cast<void**>(&tmp), (size_t)E * sizeof(int32_t)));
-  cudaError_t err = cudaMemcpyAsync(tmp, ctx->host_counts.data(), (size_t)E * sizeof(int32_t), cudaMemcpyHostToDevice,
-                                    ctx->stream);
-  if (err == cudaSuccess) {
-    launch_permute(ctx->stream, ctx->d_ids, tmp, ctx->last_tokens, E, K, ctx->d_offsets, ctx->d_perm, ctx->d_pos, nullptr,
-                   nullptr, ctx->shape.hidden, nullptr);
-    err = cudaStreamSynchronize(ctx->stream);
-  }
-  cudaFree(tmp);
-  OLED_CUDA(ctx, err);
+  OLED_CUDA(ctx, cudaMemcpyAsync(ctx->d_counts_copy, ctx->host_counts.data(), (size_t)E * sizeof(int32_t),
+                                 cudaMemcpyHostToDevice, ctx->stream));
+  launch_permute(ctx->stream, ctx->d_ids, ctx->d_counts_copy, ctx->last_tokens, E, K, ctx->d_offsets, ctx->d_perm, ctx->d_pos,
+                 nullptr, nullptr, ctx->shape.hidden, nullptr);
+  OLED_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
   ctx->launches += 1;
   ctx->perm_stale = false;
   return OLED_OK;
@@ -260,35 +265,7 @@ int sync_all(oled_ctx* ctx) {
 void free_ctx(oled_ctx* ctx) {
   if (!ctx) return;
   if (ctx->stream || ctx->copy_stream) cudaDeviceSynchronize();
-  for (auto& l : ctx->layers) {
-    cudaFree(l.w_router);
-    cudaFree(l.bias);
-  }
-  cudaFree(ctx->pool);
-  cudaFree(ctx->d_ctrl[0]);
-  cudaFree(ctx->d_logits);
-  cudaFree(ctx->d_ids);
-  cudaFree(ctx->d_gate_buf[0]);
-  cudaFree(ctx->d_gate_buf[1]);
-  cudaFree(ctx->d_offsets);
-  cudaFree(ctx->d_perm);
-  cudaFree(ctx->d_pos_buf[0]);
-  cudaFree(ctx->d_pos_buf[1]);
-  cudaFree(ctx->d_assignment);
-  cudaFree(ctx->d_xp);
-  cudaFree(ctx->d_hbuf);
-  cudaFree(ctx->split.amax_in);
-  cudaFree(ctx->split.amax_mid);
-  cudaFree(ctx->split.terms_in);
-  cudaFree(ctx->split.terms_mid);
-  cudaFree(ctx->d_y);
-  cudaFree(ctx->d_status);
-  cudaFree(ctx->d_timeline);
-  cudaFree(ctx->d_hidden_stage);
-  cudaFree(ctx->d_conf_stage);
-  cudaFree(ctx->d_out_stage);
-  cudaFree(ctx->d_iter[0]);
-  cudaFree(ctx->d_iter[1]);
+  cudaFree(ctx->device_memory);
   if (ctx->h_ctrl) cudaFreeHost(ctx->h_ctrl);
   if (ctx->h_status) cudaFreeHost(ctx->h_status);
   for (auto ev : ctx->fill_events) cudaEventDestroy(ev);
@@ -615,42 +592,45 @@ int oled_create(const oled_model_shape* shape, const int32_t* cache_capacity, vo
                     (size_t)kFfnWorkCounters * (E + ctx->ready_words) * sizeof(uint32_t) +
                     (size_t)kPermuteSegments * E * sizeof(int32_t);
   ctx->ctrl_bytes = (ctx->ctrl_bytes + 15) / 16 * 16;
-  if ((rc = dev_alloc(ctx, &ctx->pool, (size_t)ctx->n_slots * ctx->slot_bytes)) != OLED_OK) return fail(rc);
-  if ((rc = dev_alloc(ctx, &ctx->d_ctrl[0], 2 * ctx->ctrl_bytes)) != OLED_OK) return fail(rc);
-  ctx->d_ctrl[1] = ctx->d_ctrl[0] + ctx->ctrl_bytes;
-  select_ctrl(ctx, 0);
-  if ((rc = dev_alloc_guarded(ctx, &ctx->d_logits, T * E)) != OLED_OK) return fail(rc);
-  if ((rc = dev_alloc_guarded(ctx, &ctx->d_ids, T * K)) != OLED_OK) return fail(rc);
-  if ((rc = dev_alloc_guarded(ctx, &ctx->d_gate_buf[0], T * K)) != OLED_OK) return fail(rc);
-  if ((rc = dev_alloc_guarded(ctx, &ctx->d_gate_buf[1], T * K)) != OLED_OK) return fail(rc);
-  ctx->d_gate = ctx->d_gate_buf[0];
-  if ((rc = dev_alloc_guarded(ctx, &ctx->d_offsets, E + 1)) != OLED_OK) return fail(rc);
-  if ((rc = dev_alloc_guarded(ctx, &ctx->d_perm, T * K)) != OLED_OK) return fail(rc);
-  if ((rc = dev_alloc_guarded(ctx, &ctx->d_pos_buf[0], T * K)) != OLED_OK) return fail(rc);
-  if ((rc = dev_alloc_guarded(ctx, &ctx->d_pos_buf[1], T * K)) != OLED_OK) return fail(rc);
-  ctx->d_pos = ctx->d_pos_buf[0];
-  if ((rc = dev_alloc_guarded(ctx, &ctx->d_xp, ctx->row_buf * H)) != OLED_OK) return fail(rc);
-  if ((rc = dev_alloc_guarded(ctx, &ctx->d_hbuf, ctx->row_buf * I)) != OLED_OK) return fail(rc);
-  if ((rc = dev_alloc(ctx, &ctx->d_assignment, ctx->row_buf)) != OLED_OK) return fail(rc);
+  DeviceLayout mem;
+  mem.add(&ctx->pool, (size_t)ctx->n_slots * ctx->slot_bytes);
+  mem.add(&ctx->d_ctrl[0], 2 * ctx->ctrl_bytes);
+  mem.add_guarded(ctx->guards, &ctx->d_logits, T * E);
+  mem.add_guarded(ctx->guards, &ctx->d_ids, T * K);
+  mem.add_guarded(ctx->guards, &ctx->d_gate_buf[0], T * K);
+  mem.add_guarded(ctx->guards, &ctx->d_gate_buf[1], T * K);
+  mem.add_guarded(ctx->guards, &ctx->d_offsets, E + 1);
+  mem.add_guarded(ctx->guards, &ctx->d_perm, T * K);
+  mem.add_guarded(ctx->guards, &ctx->d_pos_buf[0], T * K);
+  mem.add_guarded(ctx->guards, &ctx->d_pos_buf[1], T * K);
+  mem.add_guarded(ctx->guards, &ctx->d_xp, ctx->row_buf * H);
+  mem.add_guarded(ctx->guards, &ctx->d_hbuf, ctx->row_buf * I);
+  mem.add(&ctx->d_assignment, ctx->row_buf);
   if (s.expert_format == OLED_EXPERTS_FP8 && H % 128 == 0 && I % 128 == 0) {
-    if ((rc = dev_alloc(ctx, &ctx->split.amax_in, ctx->row_buf)) != OLED_OK) return fail(rc);
-    if ((rc = dev_alloc(ctx, &ctx->split.amax_mid, ctx->row_buf)) != OLED_OK) return fail(rc);
-    if ((rc = dev_alloc(ctx, &ctx->split.terms_in, 2 * ctx->row_buf * H)) != OLED_OK) return fail(rc);
-    if ((rc = dev_alloc(ctx, &ctx->split.terms_mid, 2 * ctx->row_buf * I)) != OLED_OK) return fail(rc);
+    mem.add(&ctx->split.amax_in, ctx->row_buf);
+    mem.add(&ctx->split.amax_mid, ctx->row_buf);
+    mem.add(&ctx->split.terms_in, 2 * ctx->row_buf * H);
+    mem.add(&ctx->split.terms_mid, 2 * ctx->row_buf * I);
     ctx->split.rows = (int)ctx->row_buf;
   }
-  if ((rc = dev_alloc_guarded(ctx, &ctx->d_y, T * K * H)) != OLED_OK) return fail(rc);
-  if ((rc = dev_alloc(ctx, &ctx->d_status, kStatusWords)) != OLED_OK) return fail(rc);
-  if ((rc = dev_alloc(ctx, &ctx->d_timeline, (size_t)s.n_layers)) != OLED_OK) return fail(rc);
-  if ((rc = dev_alloc(ctx, &ctx->d_hidden_stage, T * H)) != OLED_OK) return fail(rc);
-  if ((rc = dev_alloc(ctx, &ctx->d_conf_stage, T)) != OLED_OK) return fail(rc);
-  if ((rc = dev_alloc(ctx, &ctx->d_out_stage, T * H)) != OLED_OK) return fail(rc);
-  if ((rc = dev_alloc(ctx, &ctx->d_iter[0], T * H)) != OLED_OK) return fail(rc);
-  if ((rc = dev_alloc(ctx, &ctx->d_iter[1], T * H)) != OLED_OK) return fail(rc);
+  mem.add_guarded(ctx->guards, &ctx->d_y, T * K * H);
+  mem.add(&ctx->d_status, kStatusWords);
+  mem.add(&ctx->d_timeline, (size_t)s.n_layers);
+  mem.add(&ctx->d_hidden_stage, T * H);
+  mem.add(&ctx->d_conf_stage, T);
+  mem.add(&ctx->d_out_stage, T * H);
+  mem.add(&ctx->d_iter[0], T * H);
+  mem.add(&ctx->d_iter[1], T * H);
   for (int l = 0; l < s.n_layers; ++l) {
-    if ((rc = dev_alloc(ctx, &ctx->layers[l].w_router, E * H)) != OLED_OK) return fail(rc);
-    if (s.has_router_bias && (rc = dev_alloc(ctx, &ctx->layers[l].bias, E)) != OLED_OK) return fail(rc);
+    mem.add(&ctx->layers[l].w_router, E * H);
+    if (s.has_router_bias) mem.add(&ctx->layers[l].bias, E);
   }
+  mem.add(&ctx->d_counts_copy, E);
+  if ((rc = mem.allocate(ctx)) != OLED_OK) return fail(rc);
+  ctx->d_ctrl[1] = ctx->d_ctrl[0] + ctx->ctrl_bytes;
+  select_ctrl(ctx, 0);
+  ctx->d_gate = ctx->d_gate_buf[0];
+  ctx->d_pos = ctx->d_pos_buf[0];
   if (cudaMallocHost(reinterpret_cast<void**>(&ctx->h_ctrl), 2 * E * sizeof(unsigned long long)) != cudaSuccess ||
       cudaMallocHost(reinterpret_cast<void**>(&ctx->h_status), kStatusWords * sizeof(uint32_t)) != cudaSuccess)
     return fail(OLED_ERR_OOM);

@@ -108,11 +108,12 @@ inline bool plan_step(LayerCacheState& L, SlotPool& pool, const int32_t* counts,
     else val[e] = L.frequency[e] + (act ? 1 : 0);
   }
   auto value = [&](int32_t e) -> uint64_t { return val[e]; };
-  std::stable_sort(cand.begin(), cand.end(), [&](int32_t a, int32_t b) {
-    const uint64_t va = value(a), vb = value(b);
-    if (va != vb) return va > vb;
-    return a < b;
-  });
+  if (cand.size() > (size_t)L.capacity)  // (otherwise all of them stay)
+    std::stable_sort(cand.begin(), cand.end(), [&](int32_t a, int32_t b) {
+      const uint64_t va = value(a), vb = value(b);
+      if (va != vb) return va > vb;
+      return a < b;
+    });
   const size_t keep = std::min<size_t>(cand.size(), (size_t)L.capacity);
   for (size_t i = 0; i < keep; ++i) plan.after[cand[i]] = 1;
 
