@@ -647,10 +647,11 @@ route_many_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ w
 // expert that received many tokens does not make the step wait for one CTA's chain of batches.
 // Only the CTAs with blockIdx.y == 0 write offsets, perm and pos.
 constexpr int kGatherTokMax = 4096;  // rows of one expert in a step that gathers here (T * K <= 4096), or in a segment
-// RB: rows a CTA copies at a time.  Two, with eight CTAs per expert, in gathering launches: an
+// RB: rows a CTA copies at a time.  Two, with eight CTAs per expert, in gathering launches of few-token steps: an
 // expert's handful of rows is then spread over several SMs (with one CTA taking eight rows the
 // step waited 3 us longer whenever an expert had more than eight, and the e4m3 terms of fp8
-// steps, whose conversions are the long pole, came to 7 us).  (Eight: launches that do not gather.)
+// steps, whose conversions are the long pole, came to 7 us).  Four where a segment's CTA copies its rows.  (Launches that
+// do not gather take the smallest, for its registers: with eight, 152 of them, one CTA fits an SM and 4096 tokens took 18 us.)
 template <int RB>
 __global__ void __launch_bounds__(256)
 permute_kernel(const int32_t* __restrict__ ids, const int32_t* __restrict__ counts, int n, int E,
@@ -954,7 +955,7 @@ void launch_permute(cudaStream_t st, const int32_t* ids, const int32_t* counts, 
                H, K, timeline, sp, (const int32_t*)nullptr, 0);
   }
   else
-    launch_pdl(permute_kernel<8>, dim3(E, seg_counts != nullptr ? kPermuteSegments : 1), dim3(256), 0, st, ids, counts,
+    launch_pdl(permute_kernel<2>, dim3(E, seg_counts != nullptr ? kPermuteSegments : 1), dim3(256), 0, st, ids, counts,
                T * K, E, offsets, perm, pos, x, xp, H, K, timeline, sp, seg_counts, seg_tokens);
 }
 
