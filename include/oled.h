@@ -77,12 +77,11 @@ typedef struct {
  *     fp32 scale per weight row, s_gate[I] | s_up[I] | s_down[H]; a weight is code * scale of its
  *     row.  3*H*I + 4*(2*I+H) bytes, padded to a multiple of 256.  Half the host-link and HBM
  *     traffic per expert (the paper names quantisation as the complementary lever for H2D volume).
- *     Token tiles of at most 32 rows (hidden and intermediate multiples of 128, steps of at most
- *     4096 token-expert assignments): the tensor cores read the codes as they are; a bf16 token
- *     row, scaled by a power of two, enters as the sum of two e4m3 terms, which represents every
- *     element within 2^-14 of the row's largest magnitude exactly (OLED_OPT_FP8_DIRECT).
- *     Otherwise the codes are widened to bf16 on chip (exactly) and the arithmetic is the bf16
- *     path's. */
+ *     The tensor cores read the codes as they are; a bf16 token row, scaled by a power of two, enters
+ *     as the sum of two e4m3 terms, which represents every element within 2^-14 of the row's
+ *     largest magnitude exactly (OLED_OPT_FP8_DIRECT; in steps of more than 4096 token-expert
+ *     assignments where hidden * intermediate is at least 2^20).  Otherwise the codes are widened to
+ *     bf16 on chip (exactly) and the arithmetic is the bf16 path's. */
 #define OLED_EXPERTS_BF16 0
 #define OLED_EXPERTS_FP8 1
 /* Bytes of one expert blob in the given format. */
@@ -231,10 +230,9 @@ int oled_residual_add(oled_ctx* ctx, const void* x, const void* r, void* y, size
  *   layer's combine and residual to the next layer's gate kernel (one kernel boundary and one
  *   reload of the hidden states less per layer).
  * OLED_OPT_FUSE_FFN: 0 = gate/up and down projection of an expert group always as two launches;
- *   1 (default) = as ONE launch where few work items per SM are expected (bf16 stores, token tiles
- *   of at most 32 rows): SMs that run out of gate/up items go on with the down projection of
- *   experts that are complete instead of idling until the whole gate/up launch has ended;
- *   2 = one launch wherever that form exists.
+ *   1 (default) or 2 = as ONE launch wherever that form exists: SMs that run out of gate/up items
+ *   go on with the down projection of experts that are complete instead of idling until the whole
+ *   gate/up launch has ended.
  * OLED_OPT_PDL: programmatic dependent launch between the kernels of a few-token step
  *   (process-wide, not per context). */
 #define OLED_OPT_SPLIT_LAST_FILL 9
@@ -245,8 +243,8 @@ int oled_residual_add(oled_ctx* ctx, const void* x, const void* r, void* y, size
  * when the first one got past its dependency wait and when the last one finished (GPU global
  * timer); read with oled_debug_timeline().  Off by default (a few atomics per CTA). */
 #define OLED_OPT_TIMELINE 13
-/* OLED_OPT_FP8_DIRECT (fp8 expert stores): 1 (default) = token tiles of at most 32 rows take the
- * form whose MMAs read the e4m3 codes directly; 0 = every tile widens the codes to bf16. */
+/* OLED_OPT_FP8_DIRECT (fp8 expert stores): 1 (default) = the form whose MMAs read the e4m3 codes
+ * directly; 0 = every tile widens the codes to bf16. */
 #define OLED_OPT_FP8_DIRECT 14
 /* OLED_OPT_FFN_PAIRS: 1 (default) = many-token steps (token tiles of 256 rows, bf16 stores,
  * intermediate a multiple of 256, hidden a multiple of 512) run the expert FFN on pairs of CTAs
@@ -257,12 +255,14 @@ int oled_residual_add(oled_ctx* ctx, const void* x, const void* r, void* y, size
  * of the first experts its FFN will stream - the residents activated at that previous execution,
  * adjacent iterations activating mostly the same experts (Sec. 3.3) - are called into L2 from
  * the side stream, provided that execution streamed at least 320 MB of experts (shorter streams
- * were measured to lose); 2 = the same without that condition; 0 = off. */
+ * were measured to lose) and the step's FFN does not itself load weights before the gate has
+ * decided (few-token steps do); 2 = without those conditions; 0 = off. */
 #define OLED_OPT_L2_PREFETCH 16
-/* OLED_OPT_GATHER_IN_FFN: 1 (default) = a many-token step whose FFN launches all run on CTA pairs
- * has no gather kernel: each gate/up launch copies its own experts' token rows into sorted order
- * while its first items run (one thread per CTA, bulk copies through shared memory, a counter
- * per expert that the items wait for); 0 = a gather kernel in front, as for every other step. */
+/* OLED_OPT_GATHER_IN_FFN: 1 (default) = in a many-token step whose FFN launches all run on CTA pairs
+ * and whose expert matrices have at least 2^22 elements, each gate/up launch copies its own experts'
+ * token rows into sorted order while its first items run (one thread per CTA, bulk copies through
+ * shared memory, a counter per token tile that the items wait for); 0 = the permutation kernel
+ * copies them, as in every other many-token step. */
 #define OLED_OPT_GATHER_IN_FFN 17
 #define OLED_TIMELINE_SLOTS 12 /* 0 gate, 1 permutation, 2 gather (not recorded),
                                   3..10 the step's FFN launches in order, 11 combine */

@@ -173,7 +173,7 @@ void launch_combine(cudaStream_t st, const float* y, int y_bf16, const float* ga
                     int H, int K, uint16_t* out, const uint16_t* x, uint16_t* x_next,
                     uint32_t* zero_words, int n_zero_words, StepTimeline* timeline) {
   static bool carveout_done = false;
-  if (!carveout_done) {  // keep the FFN kernels' shared-memory carve-out: see gate_cluster.cu
+  if (!carveout_done) {  // keep the FFN kernels' shared-memory carve-out
     cudaFuncSetAttribute(combine_kernel<true, 8>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     cudaFuncSetAttribute(combine_kernel<false, 8>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     cudaGetLastError();

@@ -14,7 +14,7 @@ namespace oled {
 // Every kernel of a step is launched with programmatic stream serialization: it may be scheduled
 // while its predecessor drains, does its data-independent prologue, then blocks in
 // griddep_wait() until the predecessor has completed and its writes are visible.  Every kernel
-// executes griddep_wait() before touching global data, so dependencies hold transitively.
+// executes griddep_wait() before touching what its predecessors write, so dependencies hold transitively.
 #ifdef __CUDACC__
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void griddep_launch_dependents() {
@@ -22,7 +22,7 @@ __device__ __forceinline__ void griddep_launch_dependents() {
 }
 #endif
 bool pdl_enabled();            // attribute on?
-void pdl_set_step(bool on);    // per step and thread: used for small steps only (it costs ~2 % on many-token steps)
+void pdl_set_step(bool on);    // per step and thread: used for steps of up to 16384 assignments
 void pdl_set_allowed(bool on); // process-wide switch (OLED_OPT_PDL)
 
 template <typename... KArgs, typename... Args>
