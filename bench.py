@@ -37,20 +37,21 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 # captured launch).  Traffic grows in proportion to the experts (few-token regime) or token rows
 # (many-token regime) a launch processes, so the ratio scales a capture to any launch.
 NCU_TRAFFIC_RATIO = {
-    # profiles/ffn_tc_kernel_cfg2_full_residency.md: 60 experts x 4 tokens, H 2048, I 1024
-    ("ffn_gate_up", "few_tokens"): (504.42 + 4.48) / 504.9,
-    ("ffn_down", "few_tokens"): (252.23 + 7.01) / 254.4,
-    # the one-launch form runs the same items as those two kernels together
-    ("ffn_fused", "few_tokens"): (504.42 + 4.48 + 252.23 + 7.01) / (504.9 + 254.4),
-    # profiles/ffn_tc_kernel_fp8_cfg2_full_residency.md: the same launch with fp8 stores
-    ("ffn_gate_up", "few_tokens", "fp8"): (261.71 + 4.15) / 270.6,
-    ("ffn_down", "few_tokens", "fp8"): (131.12 + 4.37) / 136.9,
+    # profiles/ffn_few_kernel_64_experts_32_tokens.md: 63 experts x 4 tokens, H 2048, I 1024; the launches of one
+    # projection run the same items
+    ("ffn_fused", "few_tokens"): (793.0 + 2.9) / 792.7,
+    ("ffn_gate_up", "few_tokens"): (793.0 + 2.9) / 792.7,
+    ("ffn_down", "few_tokens"): (793.0 + 2.9) / 792.7,
+    # the same launch with fp8 stores
+    ("ffn_fused", "few_tokens", "fp8"): (397.6 + 3.7) / 396.6,
+    ("ffn_gate_up", "few_tokens", "fp8"): (397.6 + 3.7) / 396.6,
+    ("ffn_down", "few_tokens", "fp8"): (397.6 + 3.7) / 396.6,
     # profiles/ffn_pair_kernel_cfg5_4096_tokens.md: 4096 tokens, H 4096, I 1536
     ("ffn_gate_up", "many_tokens"): (1944.0 + 100.7) / 1979.7,
     ("ffn_down", "many_tokens"): (909.4 + 264.2) / 1174.4,
     # the one-launch form on CTA pairs, which also gathers its token rows (268 MB read and written
     # on top of the projections' algorithmic bytes)
-    ("ffn_fused", "many_tokens"): (3180.0 + 631.6) / 3154.1,
+    ("ffn_fused", "many_tokens"): (3288.9 + 634.0) / 3154.1,
 }
 
 

@@ -40,7 +40,7 @@
 // row's power-of-two scale and applies the weight row's scale.  The input rows' terms come from the gate
 // kernel, those of the intermediate rows from four more warps per CTA (KIND 3) or from split_rows_kernel.  (An M = 128
 // instruction consumes 128 weight rows x 32 bytes whatever the element size; widening the codes to bf16 first
-// makes the thread that issues the MMAs the bound: 8 layers of 250 tokens 1459 us, now 907.)
+// makes the thread that issues the MMAs the bound: 8 layers of 250 tokens 1459 us, now 763.)
 //
 // Warp roles: warps 0-7 the work table, then the epilogue (lane quarter = warp mod 4, interleaved 16-column
 // chunks), warp 8 weights, warp 9 token rows, warp 10 MMA issue; in one

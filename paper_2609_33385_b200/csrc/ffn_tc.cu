@@ -11,8 +11,8 @@
 // 256.  Weights are addressed through the expert->slot table: one 3-D tensor map covers the
 // whole slot pool and the slot number is a TMA coordinate.
 //
-// Token tiles of at most 32 rows, the few-token regime, have a kernel of their own (ffn_few.cu); here
-// are tiles of 64 to 256 rows and, for any tile, the fp8 form that widens the codes.  The latter keeps a
+// Token tiles of at most 128 rows have a kernel of their own (ffn_few.cu, the rule is few_form below); here are
+// tiles of 256 rows and, for tiles of at most 128, the fp8 form that widens the codes.  The latter keeps a
 // second form of KIND 1 for tiles of at most 32 rows, "stacked": 64 gate rows and the 64 up
 // rows of the same intermediate features share ONE 128-row MMA tile (lanes 0-63 gate, 64-127 up);
 // the up values cross to the gate rows' warps through shared memory.
@@ -52,7 +52,6 @@
 
 #include <algorithm>
 #include <cstddef>
-#include <cstdlib>
 #include <type_traits>
 
 #include "kernels.h"
@@ -825,7 +824,7 @@ static int box_index(int max_count, int cap) {
 // Token tiles of at most kFewMaxRows rows go to ffn_few.cu (4 layers of 64 experts, us, against the two-accumulator
 // tiles here: 300 tokens 635 / 707, 512 tokens 701 / 773; beyond 128 rows the operand traffic of its single weight
 // tile costs more than it saves: 1000 tokens 1035 against 926 on CTA pairs).  Of fp8 stores every tile does, provided
-// the rows' e4m3 terms are at hand (8 layers of 250 tokens: 907 / 1459); otherwise converter warps widen the codes.
+// the rows' e4m3 terms are at hand (8 layers of 250 tokens: 763 / 1459); otherwise converter warps widen the codes.
 static bool few_form(const FfnTcMaps& maps, int max_count, const TokenSplit* split) {
   if (!maps.few) return false;
   return maps.fp8 ? split != nullptr && split->complete() : max_count <= kFewMaxRows;
