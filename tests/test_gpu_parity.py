@@ -893,6 +893,26 @@ def test_token_tiles_between_16_and_128_rows(n_experts, top_k, inter, counts, fp
         run.close()
 
 
+@pytest.mark.parametrize("n_experts,top_k,counts", [(16, 16, (297, 1030)), (65, 14, (300, 2072)), (512, 32, (298, 401))])
+def test_gate_sums_of_tokens_in_two_segments(n_experts, top_k, counts):
+    """Many-token gate: a CTA's 8 to 14 tokens lie in one segment of the order or in two, segments are 20 tokens at the
+    least, and tokens and experts end inside a tile; routing, order and reuse scores equal the oracle's."""
+    from paper_2609_33385_b200.runner import bits_to_dev
+    w = synth.tiny(n_layers=1, n_experts=n_experts, top_k=top_k, hidden=256, intermediate=128)
+    run = _runner(w, capacity=[n_experts], max_tokens=max(counts))
+    ora = _oracle_for(run, [n_experts])
+    try:
+        for rep, n in enumerate(counts):
+            h_bits, conf = synth.flat_tokens(w, n, 500 + rep)
+            x, c = bits_to_dev(h_bits, run.device), torch.from_numpy(conf).to(run.device)
+            out = torch.empty((n, w.hidden), dtype=torch.bfloat16, device=run.device)
+            run.step(0, x, c, out)
+            _check_step(run, 0, n, out, ora.denoise_step(0, h_bits, conf))
+        _check_stats(run, ora)
+    finally:
+        run.close()
+
+
 @pytest.mark.parametrize("n_experts,top_k,hidden", [(8, 3, 512), (64, 8, 2048), (512, 32, 256), (33, 1, 256)])
 def test_routing_alone_at_the_edges_of_its_range(n_experts, top_k, hidden):
     """oled_route_noalloc from 1 to 256 tokens (one and two tokens per CTA, parts of the assignment list of one warp and
