@@ -342,9 +342,8 @@ int oled_last_cuda_error(oled_ctx* ctx);
  * hosts that cannot let a library allocate device memory - a server that gives all of it to its
  * own arena at start-up, or a decode loop that cannot afford the device-wide synchronisation
  * hidden in cudaMalloc/cudaFree.  It runs the same gate, top-k and gate-score arithmetic as
- * oled_denoise_step() and the same stable permutation in one kernel, needs no context, and its only scratch is a
- * word per call out of a fixed array of 1024 inside the library image, which every GPU that loads the
- * library holds until the process exits.
+ * oled_denoise_step() and the same stable permutation, needs no context and has no scratch but the arrays
+ * of the call itself.
  *   hidden [n_tokens,hidden_dim] bf16, w_router [n_experts,hidden_dim] bf16, bias fp32[n_experts]
  *   or NULL, confidences fp32[n_tokens]: device, read only.
  *   ids int32[n_tokens*top_k], gate fp32[n_tokens*top_k], counts int32[n_experts],
@@ -354,13 +353,11 @@ int oled_last_cuda_error(oled_ctx* ctx);
  *   other arrays 4-byte aligned; a misaligned pointer is rejected with OLED_ERR_INVALID_ARG before
  *   anything is launched.
  * The launches use programmatic dependent launch when the calling thread's most recent
- * oled_denoise_step() did (steps of at most 4096 token-expert assignments), and by default if the
+ * oled_denoise_step() did (steps of at most 16384 token-expert assignments), and by default if the
  * thread has run no step; either way the results are the same.
- * The work is enqueued on cuda_stream.  The first call on a device looks up the array's device
- * address (one-time set-up under a lock); make that first call before any stream capture.
- * The words are taken in turn: calls may overlap on the GPU as long as no more than 1024 do.  (A captured call
- * keeps its word: replays of one graph must not overlap each other.)  One kernel launch (two memsets if
- * n_tokens is 0): no cudaMalloc, cudaFree or allocating library routine. */
+ * The work is enqueued on cuda_stream.  Calls share nothing: they may overlap on the GPU, be captured and
+ * be replayed in any order, provided that they write different arrays.  Two kernel launches (one for a single
+ * token, two memsets if n_tokens is 0): no cudaMalloc, cudaFree or allocating library routine. */
 #define OLED_NOALLOC_MAX_TOKENS 256
 int oled_route_noalloc(const void* hidden, const void* w_router, const float* bias,
                        const float* confidences, int32_t n_tokens, int32_t hidden_dim,

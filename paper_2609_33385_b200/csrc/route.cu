@@ -15,7 +15,6 @@
 
 #include <algorithm>
 #include <atomic>
-#include <mutex>
 
 #include "kernels.h"
 #include "fp8_split.h"
@@ -178,10 +177,10 @@ __device__ __forceinline__ void combine_rows(const CombinePrev& p, int t0, int n
 }
 
 // What the allocation-free routing entry point adds to the gate kernel: the counts, offsets and the stable
-// permutation, made by the CTA that finishes last.  ticket: a ZERO word, zero again afterwards.
+// permutation, made by the CTA that finishes last.  Which one that is the CTAs find out by counting in offsets[E], the
+// call's own output word: ZERO at the start (several CTAs; one CTA needs no count), overwritten by the sort.
 struct RouteFinish {
-  unsigned int* ticket = nullptr;
-  int32_t* offsets = nullptr;
+  int32_t* offsets = nullptr;  // nullptr: a gate kernel of a step
   int32_t* perm = nullptr;
 };
 // counts[E], offsets[E + 1] and the stable permutation by expert of n assignments, by one CTA of WARPS warps (E at most
@@ -432,7 +431,7 @@ route_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ wr,
         const float g = __fdiv_rn(z, sum);
         ids[(size_t)t * K + lane] = my_id;
         gate[(size_t)t * K + lane] = g;
-        if (finish.ticket == nullptr) {
+        if (finish.offsets == nullptr) {
           if (scatter.cap == 0) atomicAdd(&counts[my_id], 1);
           atomicAdd(&scores[my_id], score_quantum(g, s_conf[a]));
         }
@@ -468,24 +467,18 @@ route_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ wr,
       route_token_tail(s_logits + a * E, t, lane, E, K, conf, ids, gate, counts, scores);
     }
   }
-  if (finish.ticket != nullptr) {
+  if (finish.offsets != nullptr) {
     // routing without a step: the last CTA to get here sorts the assignments (the ids of the others are visible to it:
-    // every CTA's stores precede its ticket)
+    // every CTA's stores precede its count)
     __shared__ int s_last;
     __syncthreads();
     if (threadIdx.x == 0) {
       __threadfence();
-      s_last = atomicAdd(finish.ticket, 1u) == gridDim.x - 1 ? 1 : 0;
+      s_last = gridDim.x == 1 || atomicAdd(finish.offsets + E, 1) == (int)gridDim.x - 1 ? 1 : 0;
+      __threadfence();
     }
     __syncthreads();
-    if (s_last) {
-      if (threadIdx.x == 0) {
-        __threadfence();
-        *finish.ticket = 0u;  // ready for a later call
-      }
-      __syncthreads();
-      sort_assignments<WARPS>(ids, T * K, E, counts, finish.offsets, finish.perm, reinterpret_cast<int*>(s_dyn));
-    }
+    if (s_last) sort_assignments<WARPS>(ids, T * K, E, counts, finish.offsets, finish.perm, reinterpret_cast<int*>(s_dyn));
   }
   if (threadIdx.x == 0) timeline_end(timeline, 0);
 }
@@ -1003,43 +996,24 @@ void launch_gather(cudaStream_t st, const uint16_t* x, const int32_t* perm, int 
 // device memory to its own arena at start-up, or a latency-critical decode loop in which the
 // implicit device-wide synchronisation of cudaMalloc / cudaFree is not acceptable.  For them
 // this entry point runs the gate, top-k, gate scores and the token->expert permutation of one
-// step in one launch, without logits or scores in memory: its only scratch is a word per call, by which the CTA that
-// finishes last knows that it does (it then sorts the assignments).  The words are a fixed array in the
-// loaded module, taken in turn, so nothing is allocated or freed.  (As three memsets, the gate kernel and the permutation
-// kernel a call of 32 tokens took 16 us, nearly all of it on the host.)
+// step without logits or scores in memory.  Its only scratch is the call's own output word offsets[n_experts], by which
+// the CTA that finishes last knows that it does (it then sorts the assignments), so calls share nothing and may overlap
+// or be replayed in any order.  The word is cleared by a kernel of one thread, under which the gate kernel already
+// starts.  (As three memsets, the gate kernel and the permutation kernel a call of 32 tokens took 16 us, nearly all of
+// it on the host.)
 namespace oled {
 namespace {
 
-// Lives in every GPU that loads the library until the process exits; all words are zero between calls.
-constexpr unsigned int kNaTickets = 1024;
-static __device__ unsigned int g_noalloc_tickets[kNaTickets];
-
-constexpr int kNaMaxDevices = 64;
-std::mutex g_na_mutex;
-unsigned int* g_na_ptr[kNaMaxDevices] = {};
-std::atomic<unsigned int> g_na_next{0};
-
-// In host code the array is only a handle for the symbol, not an address a kernel can
-// use: the device address is looked up once per device, with that device current.
-int noalloc_ticket(unsigned int** out) {
-  int dev = -1;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kNaMaxDevices) return OLED_ERR_CUDA;
-  std::lock_guard<std::mutex> lock(g_na_mutex);
-  if (g_na_ptr[dev] == nullptr) {
-    void* p = nullptr;
-    if (cudaGetSymbolAddress(&p, g_noalloc_tickets) != cudaSuccess || p == nullptr) {
-      cudaGetLastError();
-      return OLED_ERR_CUDA;
-    }
-    g_na_ptr[dev] = static_cast<unsigned int*>(p);
-  }
-  *out = g_na_ptr[dev] + g_na_next.fetch_add(1u) % kNaTickets;
-  return OLED_OK;
+__global__ void clear_word_kernel(int32_t* word) {
+  griddep_launch_dependents();
+  griddep_wait();
+  *word = 0;
 }
 
 void launch_route_alone(cudaStream_t st, const uint16_t* x, const uint16_t* w_router, const float* bias, const float* conf,
                         int T, int H, int E, int K, int32_t* ids, float* gate, int32_t* counts, const RouteFinish& finish) {
   const size_t sort_bytes = (size_t)kStagedWarps * E * sizeof(int);
+  if (T > 1) launch_pdl(clear_word_kernel, dim3(1), dim3(1), 0, st, finish.offsets + E);
   if (T <= 148) {
     const size_t smem = std::max(staged_smem(1, H, E), sort_bytes);
     launch_pdl(route_kernel<1, kStagedWarps, 4, 4>, dim3(T), dim3(kStagedWarps * 32), smem, st, x, w_router, bias, conf, T, H, E,
@@ -1084,8 +1058,6 @@ extern "C" int oled_route_noalloc(const void* hidden, const void* w_router, cons
     return OLED_OK;
   }
   RouteFinish finish;
-  const int rc = noalloc_ticket(&finish.ticket);
-  if (rc != OLED_OK) return rc;
   if (!staged_attributes()) return OLED_ERR_CUDA;
   finish.offsets = offsets;
   finish.perm = perm;

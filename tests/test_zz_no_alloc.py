@@ -2,11 +2,12 @@
 
 Some hosts hand all device memory to their own arena, or cannot afford the device-wide
 synchronisation of cudaMalloc inside the decode loop; for them the library offers
-``oled_route_noalloc``, whose scratch is a fixed array inside the library.  This test calls it
-through the C ABI twice in a row, with different inputs (so stale contents of the shared array
+``oled_route_noalloc``, whose only scratch is the call's own output arrays.  The first test calls it
+through the C ABI twice in a row, with different inputs (so stale contents of anything shared
 would show), and checks every output bit for bit against what ``oled_denoise_step`` produced
-for the same inputs and against the CPU oracle's gate, top-k and permutation of the same bits.  It is collected last on purpose: a run that stops at the first failure
-has then already run every other test.
+for the same inputs and against the CPU oracle's gate, top-k and permutation of the same bits; the
+second one overlaps calls on two streams.  They are collected last on purpose: a run that stops at the first
+failure has then already run every other test.
 """
 import numpy as np
 import pytest
@@ -72,3 +73,62 @@ def test_route_noalloc_matches_denoise_step_twice_in_a_row():
         assert rc == binding.ERR_TOO_MANY_TOKENS
     finally:
         run.close()
+
+
+def test_overlapping_and_replayed_calls_share_nothing():
+    """Calls that overlap on two streams, more than 1024 enqueued calls apart or side by side, and calls captured in a
+    graph that is replayed next to live ones: every call's arrays hold what a call by itself gives."""
+    from paper_2609_33385_b200 import binding, build
+    build.build()
+    from paper_2609_33385_b200.runner import bits_to_dev
+    dev = torch.device("cuda:0")
+    h, e, k, n = 512, 16, 3, 64
+    w = synth.tiny(n_layers=1, n_experts=e, top_k=k, hidden=h)
+    wr = bits_to_dev(synth.router_weights(w, 0)[0], dev)
+    h_bits, conf = synth.flat_tokens(w, n, 60)
+    x, c = bits_to_dev(h_bits, dev), torch.from_numpy(conf).to(dev)
+    words = 3 * n * k + e + (e + 1)                       # ids, gate, perm, counts, offsets: one block per call
+    words = (words + 3) // 4 * 4
+    calls = 1100
+    a, b = torch.cuda.Stream(dev), torch.cuda.Stream(dev)
+
+    def call(block, stream):
+        p = block.data_ptr()
+        rc = binding.route_noalloc(x.data_ptr(), wr.data_ptr(), None, c.data_ptr(), n, h, e, k, stream.cuda_stream, p,
+                                   p + 4 * n * k, p + 12 * n * k, p + 12 * n * k + 4 * e, p + 8 * n * k)
+        assert rc == binding.OLED_OK, binding.strerror(rc)
+
+    one = torch.zeros(words, dtype=torch.int32, device=dev)
+    call(one, torch.cuda.current_stream(dev))
+    torch.cuda.synchronize(dev)
+    want = one.clone()
+    assert int(want[3 * n * k:3 * n * k + e].sum()) == n * k
+    for _ in range(3):
+        blocks = torch.full((calls, words), -1, dtype=torch.int32, device=dev)
+        blocks[:, 3 * n * k + e + (e + 1):] = want[3 * n * k + e + (e + 1):]
+        first = torch.full((8, words), -1, dtype=torch.int32, device=dev)
+        first[:, 3 * n * k + e + (e + 1):] = want[3 * n * k + e + (e + 1):]
+        graph = torch.cuda.CUDAGraph()
+        torch.cuda.synchronize(dev)
+        with torch.cuda.graph(graph, stream=a):
+            for i in range(4):
+                call(first[i], a)
+        torch.cuda.synchronize(dev)
+        started = torch.cuda.Event()
+        with torch.cuda.stream(b):
+            torch.cuda._sleep(20_000_000)                 # (about ten milliseconds: the calls below queue up behind it)
+            started.record(b)
+        a.wait_event(started)
+        for i in range(4, 8):                             # these run beside the calls on the other stream
+            call(first[i], a)
+        with torch.cuda.stream(a):
+            graph.replay()
+        for i in range(calls):
+            call(blocks[i], b)
+            if i % 100 == 0:
+                with torch.cuda.stream(a):
+                    graph.replay()
+        torch.cuda.synchronize(dev)
+        del graph
+        assert bool((first == want).all()), "a call beside the others, or a captured one"
+        assert bool((blocks == want).all()), "one of many calls on a stream"
