@@ -21,7 +21,9 @@
  *   - "device" pointers are CUDA device memory of the current device; "host" pointers are
  *     ordinary host memory unless "pinned" is stated.
  *   - bf16 tensors are row-major arrays of 16-bit bfloat16 values.
- *   - One context is used by one host thread at a time.  Work is ordered on the stream given
+ *   - One context is used by one host thread at a time; contexts with streams of their own may be used at
+ *     the same time and share the GPU.  (The many-token FFN on CTA pairs needs all of its CTAs to get an
+ *     SM within 2 s of each other, else the step ends in TIMEOUT; no other kernel does.)  Work is ordered on the stream given
  *     to oled_create(); oled_denoise_step() blocks the host until the gate results of the step
  *     are known (a few hundred bytes are read back to plan the copies), not until the step ends.
  *   - Shape limits: hidden a multiple of 256, at most 16384; intermediate a multiple of 128;

@@ -21,7 +21,14 @@
 // resident experts are not written while they are resident, so these loads depend on nothing.  When the
 // gate is through, the stages only lack their token rows; if the expert was not activated after
 // all they are released unread and the CTA draws another item.
-// Items other than the first are drawn from a counter in global memory.
+// Items other than guesses are drawn from a counter in global memory.
+//
+// One launch (KIND 3) makes no assumption about which of its CTAs run at the same time: kernels of other streams may hold
+// SMs for as long as they like.  Everything a down item waits for is in the hands of a running CTA: counter-drawn
+// gate/up items are all drawn before the first down item is, a guess belongs to its CTA only once that CTA has claimed
+// it after the gate, and before its first down item a CTA looks whether every guess has been claimed and takes over those
+// that have not (after a grace of 10 us; a late owner then drops what it has loaded).  The terms of fp8 rows are
+// handed out the same way.  No gate/up item waits for another CTA.
 //
 // With few experts activated (8 at one token) it is bound by the chain of one CTA's item instead.  Hence the
 // roles: one warp loads weights, one loads token rows (each TMA copy is 120 cycles of its thread; with both on one
@@ -77,10 +84,14 @@ struct __align__(16) FewCtl {
   unsigned long long tmem_full[2];
   unsigned long long tmem_empty[2];
   unsigned long long table;   // the work table below is complete
+  unsigned long long claimed; // (one launch) guess_lost is known
+  unsigned long long looked;  // ... guesses_open is
   uint32_t tmem_base;
   int abort;
   int n_tiles;      // token tiles of the group
   int n_first;      // first-phase (or only) items that are drawn from the counter
+  int guess_lost;   // another CTA has taken this one's guess over: its results are not stored
+  int guesses_open; // some guess has not been claimed yet, after a grace
   int item_ring[kFewRing];                  // an item as the roles see it: expert of the group, kind, token tile
   int item_m[kFewRing];                     // ... and weight tile
   int count[OLED_MAX_EXPERTS];              // per expert: token rows
@@ -90,6 +101,7 @@ struct __align__(16) FewCtl {
 };
 constexpr uint32_t kFewCtlBytes = (sizeof(FewCtl) + 1023u) & ~1023u;
 
+constexpr unsigned long long kGuessGraceNs = 10000;  // for a CTA to claim its guess after the gate's end
 constexpr int kItemNone = -1, kItemAbort = -2, kItemDrop = -3;
 // whole: the item multiplies with n_box rows (dense gate/up items, items loaded on a guess), not the fewest that do
 __device__ __forceinline__ int pack_item(int g, int down, int whole, int nt) { return g | down << 9 | whole << 10 | nt << 11; }
@@ -116,7 +128,8 @@ struct FewArgs {
   unsigned long long slot_bytes;
   TokenSplit split;          // fp8: the token operands' terms and magnitudes (amax_mid is raised by the gate/up epilogue)
   uint32_t* status;
-  uint32_t* work_counter;    // zero at the start
+  uint32_t* work_counter;    // two words, zero at the start: items, and (KIND 3, fp8) rows to split
+  uint32_t* claims;          // KIND 3: per CTA, zero at the start: its guess has been claimed (by itself or another)
   uint32_t* done;            // KIND 3: per expert of the group, zero at the start: its gate/up items that have been stored
   uint32_t* split_done;      // KIND 3, fp8: the same for its intermediate rows whose terms have been stored
   StepTimeline* timeline;
@@ -195,6 +208,7 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
   const bool early = KIND == 2 && p.early != 0;
   const int spec_g = (int)blockIdx.x / m_tiles1, spec_m = (int)blockIdx.x - spec_g * m_tiles1;
   const bool spec = guess && spec_g < p.n_guess && !grp.withhold_loads;
+  const int n_spec = guess ? min((int)gridDim.x, p.n_guess * m_tiles1) : 0;  // CTAs with a guess
   const int pre1 = min(p.n_stages, k_blocks1);  // stages that a first item loaded on a guess fills
   // The weights are read once per layer execution and leave L2 first: what the layers hand on and use again - hidden
   // states, outputs, router matrices - then survives the stream.  (Without it those were HBM reads queued behind the
@@ -231,6 +245,8 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
         mbar_init(smem_u32(&ctl->tmem_empty[a]), (uint32_t)epi_warps);
       }
       mbar_init(smem_u32(&ctl->table), kFewEpiWarps);
+      mbar_init(smem_u32(&ctl->claimed), 1);
+      mbar_init(smem_u32(&ctl->looked), 1);
       ctl->abort = 0;
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -286,7 +302,6 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
     if (!early) griddep_wait();
     if (lane == 0) timeline_start(p.timeline, p.timeline_slot);
     const bool spec_ok = spec && __ldcg(p.rows.counts + grp.expert[spec_g]) > 0;
-    auto draw = [&]() { return __shfl_sync(0xffffffffu, lane == 0 ? (int)atomicAdd(p.work_counter, 1u) : 0, 0); };
     auto publish = [&](int code, int m) {
       const int slot = seq % kFewRing;
       if (!warp_wait(smem_u32(&ctl->item_empty[slot]), ((uint32_t)(seq / kFewRing) & 1u) ^ 1u, abort_flag, p.status))
@@ -311,17 +326,23 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
       }
       return true;
     };
-    // First item: the guess, or (without one) the CTA's own number; later ones from the counter, each number
-    // fetched an item ahead.  (With loads withheld - the test of the bounded waits - nothing is published.)
+    // First item: the guess, or (two launches, without one) the CTA's own number; later ones from the counter, each
+    // number fetched an item ahead.  (With loads withheld - the test of the bounded waits - nothing is published.)
     if (!grp.withhold_loads) {
-      const int counter_base = guess ? 0 : (int)gridDim.x;
-      int item = guess ? draw() : (int)blockIdx.x;
+      const bool drawn_first = guess || fused;
+      const int counter_base = drawn_first ? 0 : (int)gridDim.x;
+      int item = 0;
+      bool guesses_claimed = !(fused && guess);
       if (spec) {
         ok = spec_ok ? publish(pack_item(spec_g, 0, 1, 0), spec_m) : publish(kItemDrop, 0);
+        if (lane == 0) item = (int)atomicAdd(p.work_counter, 1u);  // (in flight under the guess's loads)
         stage = pre1 == p.n_stages ? 0 : pre1;
         phase = pre1 == p.n_stages ? 1u : 0u;
         if (ok && spec_ok) ok = load_item(pre1, k_blocks1, false, spec_m, grp.slot[spec_g]);
+      } else if (lane == 0) {
+        item = drawn_first ? (int)atomicAdd(p.work_counter, 1u) : (int)blockIdx.x;
       }
+      item = __shfl_sync(0xffffffffu, item, 0);
       ok = ok && wait_table();
       const int n_first = ctl->n_first, n_items = n_first + (fused ? ctl->n_tiles * m_tiles2 : 0);
       while (ok) {
@@ -330,6 +351,22 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
         if (item >= n_items) {
           publish(kItemNone, 0);
           break;
+        }
+        if (item >= n_first && !guesses_claimed) {
+          // before the CTA's first down item: every guess that turned out right must have a running CTA
+          if (!(ok = warp_wait(smem_u32(&ctl->looked), 0u, abort_flag, p.status))) break;
+          const bool open = *reinterpret_cast<volatile int*>(&ctl->guesses_open) != 0;
+          for (int c0 = 0; ok && open && c0 < n_spec; c0 += 32) {
+            const int c = c0 + lane;
+            const bool needed = c < n_spec && ctl->count[grp.expert[c / m_tiles1]] > 0;
+            uint32_t mine = __ballot_sync(0xffffffffu, needed && atomicExch(p.claims + c, 1u) == 0u);
+            for (; ok && mine != 0u; mine &= mine - 1u) {
+              const int it = c0 + __ffs((int)mine) - 1, ig = it / m_tiles1, im = it - ig * m_tiles1;
+              ok = publish(pack_item(ig, 0, 1, 0), im) && load_item(0, k_blocks1, false, im, grp.slot[ig]);
+            }
+          }
+          guesses_claimed = true;
+          if (!ok) break;
         }
         if (item < n_first) {
           while (ctl->item_prefix[g1 + 1] <= item) ++g1;
@@ -497,7 +534,34 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
     // ------------------------------------------------------------ counts stored gate/up items (one launch)
     // The down items of an expert wait until all of its gate/up items are counted.  The count is a release: it waits
     // until the stores before it are visible device-wide, 2 to 5 us while the stream saturates the memory, so a warp
-    // of its own waits and not the epilogue.
+    // of its own waits and not the epilogue.  Before that it claims the CTA's guess and looks whether every other one is
+    // claimed: the weight warp, had it to wait for those answers, would not keep the stream going (a look by it before
+    // its first down item cost 0.7 us per layer at one token, 2 us at 32 from fp8 stores).
+    bool lost = false;
+    if (guess) {
+      griddep_wait();
+      if (spec) {
+        uint32_t taken = 0;
+        if (lane == 0) taken = atomicExch(p.claims + blockIdx.x, 1u);
+        lost = __shfl_sync(0xffffffffu, taken, 0) != 0u;
+      }
+      if (lane == 0) {
+        *reinterpret_cast<volatile int*>(&ctl->guess_lost) = lost ? 1 : 0;
+        mbar_arrive(smem_u32(&ctl->claimed));
+      }
+      const unsigned long long t0 = globaltimer();
+      bool open = true, late = false;
+      while (open && !late) {
+        late = __any_sync(0xffffffffu, globaltimer() - t0 > kGuessGraceNs);
+        open = false;
+        for (int c = lane; c < n_spec; c += 32) open |= __ldcg(p.claims + c) == 0u;
+        open = __any_sync(0xffffffffu, open);
+      }
+      if (lane == 0) {
+        *reinterpret_cast<volatile int*>(&ctl->guesses_open) = open ? 1 : 0;
+        mbar_arrive(smem_u32(&ctl->looked));
+      }
+    }
     for (int seq = 0;; ++seq) {
       const int slot = seq % kFewRing;
       const uint32_t parity = (uint32_t)(seq / kFewRing) & 1u;
@@ -505,26 +569,28 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
       const int code = __shfl_sync(0xffffffffu, *reinterpret_cast<volatile int*>(&ctl->item_ring[slot]), 0);
       if (code == kItemNone) break;
       if (!warp_wait(smem_u32(&ctl->item_stored[slot]), parity, abort_flag, p.status)) break;
-      if (lane == 0 && code != kItemDrop && !((code >> 9) & 1)) red_release_add(p.done + (code & 511), 1u);
+      if (lane == 0 && code != kItemDrop && !((code >> 9) & 1) && !(lost && seq == 0)) red_release_add(p.done + (code & 511), 1u);
       // (handed back only now: the barrier above is not used again before this warp has seen its phase)
       if (lane == 0) mbar_arrive(smem_u32(&ctl->item_empty[slot]));
     }
   } else if (FP8 && fused && warp >= kFewSplitWarp) {
     // ------------------------------------------------------------ terms of the intermediate rows (fp8, one launch)
-    // CTA b looks after expert b mod n of the group, together with the other CTAs of that number: as soon as all
-    // of its gate/up items are stored, the rows' magnitudes are final and the rows become two e4m3 terms each.  All
-    // gate/up items are handed out before the first down item, so that is over long before most down items need
-    // it, and the weight stream runs on.  (As a kernel between two launches it cost 8 of 80 us per layer of 32 tokens.)
+    // A task is every `workers`-th row of one expert, and the warps draw them from a counter (a fixed share per CTA
+    // would wait for CTAs that have no SM yet): as soon as all of the expert's gate/up items are stored, the rows'
+    // magnitudes are final and the rows become two e4m3 terms each.  All gate/up items are handed out before the
+    // first down item, so that is over long before most down items need it, and the weight stream runs on.  (As a kernel
+    // between two launches it cost 8 of 80 us per layer of 32 tokens.)
     if (wait_table() && !grp.withhold_loads) {
-      const int owners = max(1, (int)gridDim.x / grp.n);  // CTAs per expert
-      for (int g = (int)blockIdx.x % grp.n, part = (int)blockIdx.x / grp.n; g < grp.n && part < owners; g += (int)gridDim.x) {
+      const int workers = max(1, (int)gridDim.x / grp.n) * kFewSplitWarps;  // warps per expert
+      for (;;) {
+        const int task = __shfl_sync(0xffffffffu, lane == 0 ? (int)atomicAdd(p.work_counter + 1, 1u) : 0, 0);
+        if (task >= grp.n * workers) break;
+        const int w = task / grp.n, g = task - w * grp.n;
         const int e = grp.expert[g], count = ctl->count[e], row0 = first_row(e);
-        const int w = part * kFewSplitWarps + warp - kFewSplitWarp;
-        if (w >= count) continue;  // (no row of this expert is this warp's)
+        if (w >= count) continue;  // (no row of this expert is this task's)
         if (!wait_count(p.done + g, done_target(g), 500u)) break;
         uint32_t mine = 0;
-        for (int r = w; r < count; r += owners * kFewSplitWarps, ++mine)
-          split_row(p.hbuf, p.split, row0 + r, I, lane, 32);
+        for (int r = w; r < count; r += workers, ++mine) split_row(p.hbuf, p.split, row0 + r, I, lane, 32);
         __syncwarp();
         if (lane == 0) red_release_add(p.split_done + g, mine);
       }
@@ -663,6 +729,12 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
       ready = __shfl_sync(0xffffffffu, ready, 0);
       if (!ready) break;
       tc_fence_after();
+      bool lost = false;  // (another CTA computes and stores this guess)
+      if (fused && spec && seq == 0) {
+        if (!warp_wait(smem_u32(&ctl->claimed), 0u, abort_flag, p.status)) break;
+        lost = *reinterpret_cast<volatile int*>(&ctl->guess_lost) != 0;
+        if (lost) row = -1;
+      }
       for (bool first = true; first || c < n; first = false, c += step) {
         const bool last = c + step >= n;
         uint32_t ra[16];
@@ -672,7 +744,10 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
           const int col0 = FP8 ? 2 * (c & ~(box - 1)) + (c & (box - 1)) : c;
           const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * acc_cols + col0);
           tmem_ld16(t_row, ra);
-          if (!first || !ahead) columns(c, row, dst, inv);
+          if (!first || !ahead) {
+            columns(c, row, dst, inv);
+            if (lost) row = -1;
+          }
           if (FP8) {  // D = (D1 + D2 / 16) / row scale of the token
             uint32_t rt[16];
             tmem_ld16(t_row + (uint32_t)box, rt);
@@ -846,9 +921,9 @@ int launch_ffn_few(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& group
                    const int32_t* host_counts, const FfnRows& rows, uint16_t* hbuf, float* y, int y_bf16, int H, int I, int n_sms,
                    uint32_t* status, uint32_t* work_counter, bool behind_event_wait, StepTimeline* timeline,
                    int timeline_slot, const RouteReport& report, uint32_t* done, const TokenSplit* split,
-                   uint32_t* split_done) {
+                   uint32_t* split_done, uint32_t* claims) {
   const bool fp8 = maps.fp8;
-  if (kind == 3 && (done == nullptr || (fp8 && split_done == nullptr))) return OLED_ERR_INVALID_ARG;  // callers ask ffn_tc_can_fuse() first
+  if (kind == 3 && (done == nullptr || claims == nullptr || (fp8 && split_done == nullptr))) return OLED_ERR_INVALID_ARG;  // callers ask ffn_tc_can_fuse() first
   FewArgs a;
   a.tm_w1 = maps.few_w1;
   a.tm_w2 = maps.few_w2;
@@ -883,6 +958,7 @@ int launch_ffn_few(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& group
   a.work_counter = work_counter;
   a.done = done;
   a.split_done = split_done;
+  a.claims = claims;
   a.timeline = timeline;
   a.timeline_slot = timeline_slot;
   a.report = report;

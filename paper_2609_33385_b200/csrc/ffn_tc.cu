@@ -833,7 +833,8 @@ static bool few_form(const FfnTcMaps& maps, int max_count, const TokenSplit* spl
 int launch_ffn_tc(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp_in, int max_count, int kind,
                   const int32_t* host_counts, const FfnRows& rows, uint16_t* hbuf, float* y, int y_bf16, int H, int I,
                   int n_sms, uint32_t* status, uint32_t* work_counter, bool behind_event_wait, StepTimeline* timeline,
-                  int timeline_slot, const RouteReport& report_in, uint32_t* done, const TokenSplit* split, uint32_t* split_done) {
+                  int timeline_slot, const RouteReport& report_in, uint32_t* done, const TokenSplit* split, uint32_t* split_done,
+                  uint32_t* claims) {
   const RouteReport report = kind != 2 ? report_in : RouteReport{};
   if (grp_in.n <= 0 || max_count <= 0) return OLED_OK;
   FfnGroup grp = grp_in;
@@ -845,7 +846,7 @@ int launch_ffn_tc(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp_in
   grp.n_box = 16 << ib;
   if (few_form(maps, max_count, split))
     return launch_ffn_few(st, maps, grp, max_count, kind, host_counts, rows, hbuf, y, y_bf16, H, I, n_sms, status,
-                          work_counter, behind_event_wait, timeline, timeline_slot, report, done, split, split_done);
+                          work_counter, behind_event_wait, timeline, timeline_slot, report, done, split, split_done, claims);
   // many-token tiles: the CTA-pair kernel, unless its cluster launch has failed before on this
   // device (the one-CTA form below computes the same)
   if (maps.use_pairs && !g_pairs_refused && ffn_pair_usable(maps, grp.n_box, H, I)) {

@@ -274,8 +274,9 @@ int ffn_tc_setup(FfnTcMaps* maps, const uint8_t* pool, size_t slot_bytes, int n_
 // kind 1: gate/up + SwiGLU into hbuf; kind 2: down projection into y; kind 3: both in one launch
 // (bf16 stores and token tiles of at most 32 rows only: ask ffn_tc_can_fuse; `done` then points at
 // one ZERO word per expert of the group).  One launch each.
-// work_counter: a device word that is ZERO when the kernel starts; its CTAs draw their work items
-// from it (every launch that can be in flight at the same time needs a word of its own).
+// work_counter: two device words that are ZERO when the kernel starts; its CTAs draw their work items
+// from the first and rows to split from the second (every launch that can be in flight at the same time needs
+// words of its own).  claims (few-token form, one launch): one ZERO word per SM, for the step's one launch with guesses.
 // report (kinds 1 and 3; host_scores == nullptr: none): the kernel's first CTA publishes the step's
 // counts and scores to the host.
 // behind_event_wait: the launch follows a cudaStreamWaitEvent (with, for kind 2, at most its own
@@ -287,7 +288,7 @@ int launch_ffn_tc(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp, i
                   const int32_t* host_counts, const FfnRows& rows, uint16_t* hbuf, float* y, int y_bf16, int H,
                   int I, int n_sms, uint32_t* status, uint32_t* work_counter, bool behind_event_wait,
                   StepTimeline* timeline, int timeline_slot, const RouteReport& report, uint32_t* done = nullptr,
-                  const TokenSplit* split = nullptr, uint32_t* split_done = nullptr);
+                  const TokenSplit* split = nullptr, uint32_t* split_done = nullptr, uint32_t* claims = nullptr);
 int ffn_tc_launches(const FfnTcMaps& maps, int max_count, int kind, const TokenSplit* split);
 // No gathered copy of the step's token rows exists: every FFN launch until
 // ffn_tc_clear_token_source must be one the CTA-pair kernel takes (token tile 256), and each gets
@@ -306,6 +307,7 @@ int launch_ffn_pair(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp,
                     uint32_t* work_counter, StepTimeline* timeline, int timeline_slot, const RouteReport& report,
                     uint32_t* done = nullptr);
 constexpr int kFfnWorkCounters = 8;  // FFN launches of one layer execution: 3 groups x 2 kinds, rounded up
+constexpr int kFfnCounterWords = 2;  // words of each launch's work counter
 
 // A tensor map over bf16 elements (bytes: over bytes) with the 128-byte swizzle (narrow: the 64-byte one).
 bool encode_tensor_map(CUtensorMap* m, int rank, const void* base, const cuuint64_t* dims, const cuuint64_t* strides,
@@ -319,7 +321,7 @@ int launch_ffn_few(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp, 
                    const int32_t* host_counts, const FfnRows& rows, uint16_t* hbuf, float* y, int y_bf16, int H, int I, int n_sms,
                    uint32_t* status, uint32_t* work_counter, bool behind_event_wait, StepTimeline* timeline,
                    int timeline_slot, const RouteReport& report, uint32_t* done, const TokenSplit* split,
-                   uint32_t* split_done);
+                   uint32_t* split_done, uint32_t* claims);
 
 // Self-check (check.cu): invariants of the routing and the permutation, guard words.
 void launch_self_check(cudaStream_t st, const int32_t* ids, const int32_t* counts, const int32_t* offsets,

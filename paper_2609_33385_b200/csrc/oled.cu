@@ -97,6 +97,7 @@ struct oled_ctx {
   float* d_y = nullptr;        // [T*k,H]
   uint32_t* d_status = nullptr;
   uint32_t* d_work = nullptr;         // control block: work-item counters of the step's FFN launches
+  uint32_t* d_claims = nullptr;       // control block: [n_sms] guesses of the step's first FFN launch that a CTA has claimed
   uint32_t* d_done = nullptr;         // control block: [kFfnWorkCounters][E] completion counters of fused FFN launches
   uint32_t* d_ready = nullptr;        // control block: [kFfnWorkCounters][ready_words] row-copy counters of FFN launches that gather
   size_t ready_words = 0;             // token tiles of 256 rows a launch can have: max_tokens * K / 256 + E
@@ -167,7 +168,8 @@ void select_ctrl(oled_ctx* ctx, int sel) {
   ctx->d_scores = reinterpret_cast<unsigned long long*>(b);
   ctx->d_counts = reinterpret_cast<int32_t*>(b + E * sizeof(unsigned long long));
   ctx->d_work = reinterpret_cast<uint32_t*>(b + E * (sizeof(unsigned long long) + sizeof(int32_t)));
-  ctx->d_done = ctx->d_work + kFfnWorkCounters;
+  ctx->d_claims = ctx->d_work + kFfnWorkCounters * kFfnCounterWords;
+  ctx->d_done = ctx->d_claims + ctx->n_sms;
   ctx->d_ready = ctx->d_done + (size_t)kFfnWorkCounters * E;
   ctx->d_seg = reinterpret_cast<int32_t*>(ctx->d_ready + (size_t)kFfnWorkCounters * ctx->ready_words);
 }
@@ -413,11 +415,11 @@ int run_ffn_launches(oled_ctx* ctx, const FfnGroup& grp, int max_count, const in
       // per launch; a layer execution has at most three launch pairs, should there ever be more,
       // used words are cleared in stream order and taken again
       const int li = ctx->work_next % kFfnWorkCounters;
-      uint32_t* work = ctx->d_work + li;
+      uint32_t* work = ctx->d_work + li * kFfnCounterWords;
       uint32_t* done = ctx->d_done + (size_t)li * ctx->shape.n_experts;
       uint32_t* ready = ctx->d_ready + (size_t)li * ctx->ready_words;
       if (ctx->work_next >= kFfnWorkCounters) {
-        OLED_CUDA(ctx, cudaMemsetAsync(work, 0, sizeof(uint32_t), ctx->stream));
+        OLED_CUDA(ctx, cudaMemsetAsync(work, 0, kFfnCounterWords * sizeof(uint32_t), ctx->stream));
         OLED_CUDA(ctx, cudaMemsetAsync(done, 0, (size_t)ctx->shape.n_experts * sizeof(uint32_t), ctx->stream));
         OLED_CUDA(ctx, cudaMemsetAsync(ready, 0, ctx->ready_words * sizeof(uint32_t), ctx->stream));
       }
@@ -437,7 +439,7 @@ int run_ffn_launches(oled_ctx* ctx, const FfnGroup& grp, int max_count, const in
       const int rc = launch_ffn_tc(ctx->stream, ctx->maps, grp, max_count, kind, host_counts, rows, ctx->d_hbuf, ctx->d_y, ctx->y_bf16 ? 1 : 0, H, I, ctx->n_sms, ctx->d_status, work,
                                    behind_event_wait || (kind == 2 && before_down != nullptr),
                                    ctx->timeline_on ? ctx->d_timeline + ctx->last_layer : nullptr, 3 + li, report, done,
-                                   ctx->step_split, ready);
+                                   ctx->step_split, ready, ctx->d_claims);
       if (rc != OLED_OK) return rc;
       ctx->launches += ffn_tc_launches(ctx->maps, max_count, kind, ctx->step_split);
     }
@@ -588,7 +590,7 @@ int oled_create(const oled_model_shape* shape, const int32_t* cache_capacity, vo
   const size_t H = (size_t)s.hidden, I = (size_t)s.intermediate;
   ctx->ready_words = T * K / 256 + E;
   ctx->row_buf = std::max(T * K, std::min(kScatterRows, E * scatter_cap(std::min(T, std::max<size_t>(1, 4096 / K)))));
-  ctx->ctrl_bytes = E * (sizeof(unsigned long long) + sizeof(int32_t)) + kFfnWorkCounters * sizeof(uint32_t) +
+  ctx->ctrl_bytes = E * (sizeof(unsigned long long) + sizeof(int32_t)) + (kFfnWorkCounters * kFfnCounterWords + (size_t)ctx->n_sms) * sizeof(uint32_t) +
                     (size_t)kFfnWorkCounters * (E + ctx->ready_words) * sizeof(uint32_t) +
                     (size_t)kPermuteSegments * E * sizeof(int32_t);
   ctx->ctrl_bytes = (ctx->ctrl_bytes + 15) / 16 * 16;

@@ -942,3 +942,58 @@ def test_routing_alone_at_the_edges_of_its_range(n_experts, top_k, hidden):
         assert np.array_equal(gate.cpu().numpy().view(np.uint32).reshape(n, top_k), o_gate.view(np.uint32))
         assert np.array_equal(counts.cpu().numpy(), o_counts) and np.array_equal(offsets.cpu().numpy(), o_offsets)
         assert np.array_equal(perm.cpu().numpy(), o_perm)
+
+
+@pytest.mark.parametrize("fp8", [False, True], ids=["bf16", "fp8"])
+@pytest.mark.parametrize("n", [20, 40])
+def test_contexts_on_streams_of_their_own_run_side_by_side(n, fp8):
+    """Two contexts, each with a stream (of different priority) and a host thread of its own, next to matrix
+    products on a third stream: the SMs a one-launch expert FFN gets, and when, are then up to the others.  No wait runs out
+    and every iteration's output is, bit for bit, the one the context computes by itself; there are more gate/up
+    items (24 experts x 8 weight tiles) than SMs, and half of the iterations meet other tokens than the one before."""
+    import threading
+    from paper_2609_33385_b200.runner import bits_to_dev
+    w = synth.tiny(n_layers=4, n_experts=24, top_k=4, hidden=512, intermediate=512)
+    iters, dev = 40, torch.device("cuda:0")
+    a = torch.randn((4096, 4096), device=dev).to(torch.bfloat16)
+    streams = [torch.cuda.Stream(dev, priority=0), torch.cuda.Stream(dev, priority=-1)]
+    runs, inputs, alone, beside, errors = [], [], [], [], []
+    try:
+        for i, st in enumerate(streams):
+            with torch.cuda.stream(st):
+                runs.append(_runner(w, capacity=[24] * 4, max_tokens=n, fp8=fp8, share_store_of=runs[0] if runs else None))
+            seeds = [300 + 10 * i + j // 2 % 3 for j in range(iters)]
+            made = {s: synth.flat_tokens(w, n, s) for s in set(seeds)}
+            made = {s: (bits_to_dev(x, dev), torch.from_numpy(c).to(dev)) for s, (x, c) in made.items()}
+            inputs.append([made[s] for s in seeds])
+            alone.append([torch.empty((n, w.hidden), dtype=torch.bfloat16, device=dev) for _ in seeds])
+            beside.append([torch.empty((n, w.hidden), dtype=torch.bfloat16, device=dev) for _ in seeds])
+        torch.cuda.synchronize(dev)
+
+        def go(i, outs):
+            try:
+                torch.cuda.set_device(dev)
+                for (x, c), out in zip(inputs[i], outs[i]):
+                    runs[i].ctx.denoise_iteration(x.data_ptr(), c.data_ptr(), n, out.data_ptr())
+                runs[i].ctx.synchronize()
+            except Exception as e:                        # (shown by the main thread)
+                errors.append(e)
+
+        for i in range(2):
+            go(i, alone)
+        threads = [threading.Thread(target=go, args=(i, beside)) for i in range(2)]
+        for t in threads:
+            t.start()
+        with torch.cuda.stream(torch.cuda.Stream(dev)):
+            for _ in range(40):
+                a @ a
+        for t in threads:
+            t.join()
+        torch.cuda.synchronize(dev)
+        assert not errors, errors
+        for i in range(2):
+            for x, y in zip(alone[i], beside[i]):
+                assert torch.equal(x.view(torch.int16), y.view(torch.int16))
+    finally:
+        for r in runs:
+            r.close()
