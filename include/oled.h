@@ -386,6 +386,10 @@ void oled_policy_destroy(oled_policy* p);
 int oled_policy_set_policy(oled_policy* p, int32_t policy);
 /* fills_reused counter of the simulator's layer. */
 int oled_policy_fills_reused(oled_policy* p, uint64_t* out);
+/* Token rows per weight tile that a step's FFN over the resident experts starts with, given the tokens of the layer's
+ * previous execution (0: none) and the most rows an expert received in it. */
+int32_t oled_policy_tile_rows(int32_t n_tokens, int32_t top_k, int32_t n_experts, int32_t last_tokens,
+                              int32_t last_max_count);
 /* Layer-adaptive sizing over n simulated layers (one oled_policy each): as oled_adapt_capacity(). */
 int oled_policy_adapt(oled_policy** layers, int32_t n_layers, int32_t total_capacity,
                       int32_t* new_capacity);

@@ -46,6 +46,7 @@ EXPORTS = [
     "oled_adapt_capacity", "oled_get_capacity", "oled_policy_set_policy", "oled_policy_fills_reused",
     "oled_policy_adapt", "oled_clear_status", "oled_policy_time", "oled_expert_blob_bytes",
     "oled_self_check_report", "oled_debug_perm", "oled_policy_create_stack", "oled_debug_timeline",
+    "oled_policy_tile_rows",
 ]
 EXPERTS_BF16, EXPERTS_FP8 = 0, 1
 NOALLOC_MAX_TOKENS = 256
@@ -143,6 +144,7 @@ def load() -> C.CDLL:
     lib.oled_get_capacity.argtypes = [vp, vp]
     lib.oled_policy_set_policy.argtypes = [vp, i32]
     lib.oled_policy_fills_reused.argtypes = [vp, u64p]
+    lib.oled_policy_tile_rows.argtypes = [i32, i32, i32, i32, i32]
     lib.oled_policy_adapt.argtypes = [C.POINTER(vp), i32, i32, vp]
     lib.oled_route_noalloc.argtypes = [vp, vp, vp, vp, i32, i32, i32, i32, vp, vp, vp, vp, vp, vp]
     _lib = lib
@@ -319,7 +321,7 @@ class OledContext:
 def route_noalloc(hidden_ptr, w_router_ptr, bias_ptr, conf_ptr, n_tokens: int, hidden: int,
                   n_experts: int, top_k: int, cuda_stream: int, ids_ptr, gate_ptr, counts_ptr,
                   offsets_ptr, perm_ptr) -> int:
-    """``oled_route_noalloc``: routing of one step with library-internal static scratch; the
+    """``oled_route_noalloc``: routing of one step without scratch of its own; the
     library allocates nothing.  All pointers are device pointers; returns the status code."""
     return load().oled_route_noalloc(hidden_ptr, w_router_ptr, bias_ptr, conf_ptr, n_tokens, hidden,
                                      n_experts, top_k, C.c_void_p(cuda_stream), ids_ptr, gate_ptr,

@@ -23,7 +23,8 @@ namespace {
 struct LayerData {
   LayerCacheState cache;
   int32_t last_active = -1;      // experts activated at the layer's previous execution (-1: none yet)
-  int32_t last_max_count = -1;   // most token rows any expert received then
+  int32_t last_tokens = 0;       // tokens of the layer's previous execution (0: none yet)
+  int32_t last_max_count = 0;    // most token rows any expert received then
   int32_t last_misses = -1;      // its misses
   std::vector<int32_t> last_counts;  // its per-expert row counts
   const uint8_t* host_blob = nullptr;
@@ -889,13 +890,7 @@ static int step_impl(oled_ctx* ctx, int32_t layer, const void* hidden, const flo
       }
       if (pass == 0) grp.n_guess = grp.n;
     }
-    // Token tile of this launch (the counts are not known on the host yet): the most rows an expert received at
-    // the layer's previous execution and an eighth, at most twice the mean load per expert (a few heavily loaded
-    // experts take several tiles).  An expert that receives more rows than the tile holds has its weights
-    // streamed once per tile, a tile that is too large costs pipeline stages.
-    const int mean_load = (int)(((size_t)T * K + E - 1) / E);
-    const int seen = L.last_max_count >= 0 ? L.last_max_count + (L.last_max_count + 7) / 8 : T;
-    const int rc0 = run_ffn_launches(ctx, grp, std::min(T, std::min(seen, std::max(32, 2 * mean_load))), nullptr, nullptr, false,
+    const int rc0 = run_ffn_launches(ctx, grp, resident_tile_rows(T, K, E, L.last_tokens, L.last_max_count), nullptr, nullptr, false,
                                      &ctx->hit_fused, rep);
     if (rc0 != OLED_OK) return rc0;
   }
@@ -1026,6 +1021,7 @@ static int step_impl(oled_ctx* ctx, int32_t layer, const void* hidden, const flo
   L.stats.evictions += (uint64_t)plan.n_evictions;
   L.stats.active_experts += (uint64_t)plan.n_active;
   L.last_active = plan.n_active;
+  L.last_tokens = T;
   L.last_max_count = 0;
   for (int32_t e = 0; e < E; ++e) L.last_max_count = std::max(L.last_max_count, counts[e]);
   L.last_misses = n_miss;
@@ -1467,6 +1463,12 @@ int oled_policy_fills_reused(oled_policy* p, uint64_t* out) {
   if (!p || !out) return OLED_ERR_INVALID_ARG;
   *out = p->fills_reused;
   return OLED_OK;
+}
+
+int32_t oled_policy_tile_rows(int32_t n_tokens, int32_t top_k, int32_t n_experts, int32_t last_tokens,
+                              int32_t last_max_count) {
+  if (n_tokens <= 0 || top_k <= 0 || n_experts <= 0 || last_tokens < 0 || last_max_count < 0) return OLED_ERR_INVALID_ARG;
+  return resident_tile_rows(n_tokens, top_k, n_experts, last_tokens, last_max_count);
 }
 
 int oled_policy_adapt(oled_policy** layers, int32_t n_layers, int32_t total_capacity, int32_t* new_capacity) {

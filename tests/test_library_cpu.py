@@ -175,6 +175,29 @@ def test_small_caller_chosen_staging_raises_the_adaptive_floor(binding):
         assert got["hits"] + got["misses"] == e
 
 
+@pytest.mark.parametrize("top_k,n_experts", [(8, 64), (2, 16), (8, 128), (1, 4), (6, 6)])
+def test_token_tile_follows_the_previous_execution_only_where_it_was_alike(binding, top_k, n_experts):
+    """A step's tile holds the previous execution's fullest expert and an eighth, if that execution had about as many
+    tokens; after a much smaller or larger one it is the tile of a first execution.  Never more than the tokens, never
+    less than the mean load."""
+    rows = lambda t, last_t, last_max: binding.load().oled_policy_tile_rows(t, top_k, n_experts, last_t, last_max)
+    for t in (1, 2, 31, 32, 33, 250, 1000, 4096, 65535):
+        mean = -(-t * top_k // n_experts)
+        first = rows(t, 0, 0)
+        assert first == min(t, max(32, 2 * mean))
+        for most in (mean, 2 * mean, t):
+            assert rows(t, t, most) == min(first, most + -(-most // 8))
+        for last_t in (1, 2, 32, 250, 1000, 4096, 65535):
+            last_mean = -(-last_t * top_k // n_experts)
+            for most in (last_mean, last_t):
+                r = rows(t, last_t, most)
+                assert mean <= r <= first <= t or r == first == t
+                if 4 * t > 5 * last_t or 5 * t < 4 * last_t:
+                    assert r == first
+    assert rows(1000, 900, 1000) >= rows(1000, 900, 500)
+    assert binding.load().oled_policy_tile_rows(0, top_k, n_experts, 0, 0) == binding.ERR_INVALID_ARG
+
+
 def test_misaligned_pointers_are_rejected_before_anything_is_launched(binding):
     """oled_route_noalloc accesses rows and ids with 16-byte vectors: a pointer into the middle of
     such a vector is an argument error (nothing touches the GPU, so this runs without one)."""
