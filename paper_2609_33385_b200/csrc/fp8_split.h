@@ -18,7 +18,9 @@ __device__ __forceinline__ uint32_t token_exponent(uint32_t amax_bits) {
   return min(max((amax_bits >> 23) & 0xffu, 8u), 254u);
 }
 __device__ __forceinline__ float token_scale(uint32_t amax_bits) {
-  return __uint_as_float((261u - token_exponent(amax_bits)) << 23);  // 2^(134 - biased exponent)
+  // (a row with an infinity or a NaN scales by NaN: e4m3 has no infinity, the conversion would saturate it to a finite code)
+  return __uint_as_float(amax_bits >= 0x7f800000u ? 0x7fffffffu
+                                                  : (261u - token_exponent(amax_bits)) << 23);  // 2^(134 - biased exponent)
 }
 __device__ __forceinline__ float token_scale_inverse(uint32_t amax_bits) {
   return __uint_as_float((token_exponent(amax_bits) - 7u) << 23);

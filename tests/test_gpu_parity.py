@@ -997,3 +997,46 @@ def test_contexts_on_streams_of_their_own_run_side_by_side(n, fp8):
     finally:
         for r in runs:
             r.close()
+
+
+@pytest.mark.parametrize("direct", [1, 0], ids=["direct", "widening"])
+@pytest.mark.parametrize("n", [24, 300, 4200])
+def test_fp8_intermediate_rows_that_overflow_give_no_finite_outputs(n, direct):
+    """A token whose SwiGLU product exceeds the largest bf16 in one feature: its intermediate row holds an infinity, so every
+    output the feature has a weight in is not finite, whatever form the codes are read in; the other tokens are unaffected.
+    The down codes are the smallest there are (2^-9): a form that let the infinity saturate to a finite code would give
+    ordinary numbers."""
+    from paper_2609_33385_b200 import binding
+    from paper_2609_33385_b200.runner import bits_to_dev, dev_to_bits
+    w = synth.tiny(n_layers=1, n_experts=4, top_k=1, hidden=1024, intermediate=1024)
+    run = _runner(w, capacity=[4], max_tokens=n, fp8=True)
+    try:
+        run.ctx.set_option(binding.OPT_FP8_DIRECT, direct)
+        h, i, f = w.hidden, w.intermediate, 37
+        for e in range(w.n_experts):
+            blob = run.blobs[0][e]
+            for m in (0, 1):                              # feature f, and no other, sees a row's first element: times 1.0
+                codes = blob[m * i * h:(m + 1) * i * h].reshape(i, h)
+                codes[:, 0] = 0
+                codes[f] = 0
+                codes[f, 0] = 0x38
+            blob[2 * i * h:3 * i * h].reshape(h, i)[:, f] = 0x01
+            scales = blob[3 * h * i:3 * h * i + 4 * (2 * i + h)].view(np.float32)
+            scales[[f, i + f]] = 1.0
+        h_bits, conf = synth.flat_tokens(w, n, 90)
+        h_bits[:, 0] = 0x3F80
+        c = torch.from_numpy(conf).to(run.device)
+        outs = []
+        for first in (0x3F80, 0x6280):                    # 1.0, then 2^70 in row 5: a product of 2^140
+            h_bits[5, 0] = first
+            out = torch.empty((n, h), dtype=torch.bfloat16, device=run.device)
+            run.step(0, bits_to_dev(h_bits, run.device), c, out)
+            run.ctx.synchronize()
+            outs.append(dev_to_bits(out))
+        finite = np.isfinite(synth.bf16_bits_to_f32(outs[1]))
+        assert np.isfinite(synth.bf16_bits_to_f32(outs[0])).all()
+        assert not finite[5].any()
+        others = np.arange(n) != 5
+        assert np.array_equal(outs[0][others], outs[1][others])
+    finally:
+        run.close()
