@@ -788,7 +788,6 @@ static int step_impl(oled_ctx* ctx, int32_t layer, const void* hidden, const flo
     // at most 32 tokens: one copy of the rows serves every expert (the FFN form that can use it takes
     // every launch of such a step, unless fp8 codes are to be widened)
     ctx->scatter.dense = T <= kDenseTokens && (ctx->shape.expert_format != OLED_EXPERTS_FP8 || ctx->step_split) ? 1 : 0;
-    ctx->perm_stale = true;
   }
   const bool scattered = ctx->scatter.cap > 0;
   {
@@ -858,7 +857,6 @@ static int step_impl(oled_ctx* ctx, int32_t layer, const void* hidden, const flo
   if (ctx->self_check && scattered) {
     launch_permute(st, ctx->d_ids, ctx->d_counts, T, E, K, ctx->d_offsets, ctx->d_perm, ctx->d_pos, nullptr, nullptr, H,
                    nullptr);
-    ctx->perm_stale = false;
     launch_scatter_check(st, ctx->d_ids, ctx->d_counts, ctx->d_assignment, ctx->scatter.cap, T, E, K, ctx->d_status);
     ctx->launches += 2;
   }
@@ -902,6 +900,8 @@ static int step_impl(oled_ctx* ctx, int32_t layer, const void* hidden, const flo
   {
     const int rcw = wait_gate_report(ctx);
     if (rcw != OLED_OK) return rcw;
+    // (only now: make_perm() sorts by the reported counts, those of an earlier step could lead it out of its buffers)
+    ctx->perm_stale = scattered && !ctx->self_check;
   }
   const unsigned long long* scores = ctx->host_scores.data();
   const int32_t* counts = ctx->host_counts.data();
