@@ -111,7 +111,10 @@ typedef struct {
  *   cuda_stream     a cudaStream_t (may be 0) on which every step is enqueued; borrowed.
  *   out_ctx         receives the context; the library owns it until oled_destroy().
  * Allocates the slot pool (sum C_l + staging slots, each one expert blob), router weights and
- * scratch in device memory.  Errors: INVALID_ARG, OOM, CUDA. */
+ * scratch in device memory, all at once.  The scratch for token rows is R * (2H + 2I) bytes (fp8 stores: twice
+ * that) with R = max_tokens * top_k, or up to 32768 if E * max_tokens is more than that: few-token steps then give
+ * every expert a region of rows and need no sort.  If only that is too much, R = max_tokens * top_k it is, and those steps
+ * sort.  Errors: INVALID_ARG, OOM, CUDA. */
 int oled_create(const oled_model_shape* shape, const int32_t* cache_capacity, void* cuda_stream,
                 oled_ctx** out_ctx);
 

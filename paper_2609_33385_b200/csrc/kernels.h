@@ -162,7 +162,7 @@ struct TokenSplit {
   uint32_t* amax_mid = nullptr;  // [rows]
   uint8_t* terms_in = nullptr;   // [2][rows][H] e4m3 codes: term 1 of every row, then term 2
   uint8_t* terms_mid = nullptr;  // [2][rows][I]
-  int rows = 0;                  // rows of the buffers above (tokens x top-k of the context)
+  int rows = 0;                  // rows of the buffers above (as many as the context has token rows)
   bool complete() const { return amax_in && amax_mid && terms_in && terms_mid && rows > 0; }
 };
 // Few-token steps: the gate kernel itself brings the token rows to their experts, so that no

@@ -595,41 +595,49 @@ int oled_create(const oled_model_shape* shape, const int32_t* cache_capacity, vo
                     (size_t)kFfnWorkCounters * (E + ctx->ready_words) * sizeof(uint32_t) +
                     (size_t)kPermuteSegments * E * sizeof(int32_t);
   ctx->ctrl_bytes = (ctx->ctrl_bytes + 15) / 16 * 16;
-  DeviceLayout mem;
-  mem.add(&ctx->pool, (size_t)ctx->n_slots * ctx->slot_bytes);
-  mem.add(&ctx->d_ctrl[0], 2 * ctx->ctrl_bytes);
-  mem.add_guarded(ctx->guards, &ctx->d_logits, T * E);
-  mem.add_guarded(ctx->guards, &ctx->d_ids, T * K);
-  mem.add_guarded(ctx->guards, &ctx->d_gate_buf[0], T * K);
-  mem.add_guarded(ctx->guards, &ctx->d_gate_buf[1], T * K);
-  mem.add_guarded(ctx->guards, &ctx->d_offsets, E + 1);
-  mem.add_guarded(ctx->guards, &ctx->d_perm, T * K);
-  mem.add_guarded(ctx->guards, &ctx->d_pos_buf[0], T * K);
-  mem.add_guarded(ctx->guards, &ctx->d_pos_buf[1], T * K);
-  mem.add_guarded(ctx->guards, &ctx->d_xp, ctx->row_buf * H);
-  mem.add_guarded(ctx->guards, &ctx->d_hbuf, ctx->row_buf * I);
-  mem.add(&ctx->d_assignment, ctx->row_buf);
-  if (s.expert_format == OLED_EXPERTS_FP8 && H % 128 == 0 && I % 128 == 0) {
-    mem.add(&ctx->split.amax_in, ctx->row_buf);
-    mem.add(&ctx->split.amax_mid, ctx->row_buf);
-    mem.add(&ctx->split.terms_in, 2 * ctx->row_buf * H);
-    mem.add(&ctx->split.terms_mid, 2 * ctx->row_buf * I);
-    ctx->split.rows = (int)ctx->row_buf;
+  // (where memory is too short for scattered steps' rows, those steps sort theirs)
+  for (;;) {
+    DeviceLayout mem;
+    ctx->guards = GuardList{};
+    mem.add(&ctx->pool, (size_t)ctx->n_slots * ctx->slot_bytes);
+    mem.add(&ctx->d_ctrl[0], 2 * ctx->ctrl_bytes);
+    mem.add_guarded(ctx->guards, &ctx->d_logits, T * E);
+    mem.add_guarded(ctx->guards, &ctx->d_ids, T * K);
+    mem.add_guarded(ctx->guards, &ctx->d_gate_buf[0], T * K);
+    mem.add_guarded(ctx->guards, &ctx->d_gate_buf[1], T * K);
+    mem.add_guarded(ctx->guards, &ctx->d_offsets, E + 1);
+    mem.add_guarded(ctx->guards, &ctx->d_perm, T * K);
+    mem.add_guarded(ctx->guards, &ctx->d_pos_buf[0], T * K);
+    mem.add_guarded(ctx->guards, &ctx->d_pos_buf[1], T * K);
+    mem.add_guarded(ctx->guards, &ctx->d_xp, ctx->row_buf * H);
+    mem.add_guarded(ctx->guards, &ctx->d_hbuf, ctx->row_buf * I);
+    mem.add(&ctx->d_assignment, ctx->row_buf);
+    if (s.expert_format == OLED_EXPERTS_FP8 && H % 128 == 0 && I % 128 == 0) {
+      mem.add(&ctx->split.amax_in, ctx->row_buf);
+      mem.add(&ctx->split.amax_mid, ctx->row_buf);
+      mem.add(&ctx->split.terms_in, 2 * ctx->row_buf * H);
+      mem.add(&ctx->split.terms_mid, 2 * ctx->row_buf * I);
+      ctx->split.rows = (int)ctx->row_buf;
+    }
+    mem.add_guarded(ctx->guards, &ctx->d_y, T * K * H);
+    mem.add(&ctx->d_status, kStatusWords);
+    mem.add(&ctx->d_timeline, (size_t)s.n_layers);
+    mem.add(&ctx->d_hidden_stage, T * H);
+    mem.add(&ctx->d_conf_stage, T);
+    mem.add(&ctx->d_out_stage, T * H);
+    mem.add(&ctx->d_iter[0], T * H);
+    mem.add(&ctx->d_iter[1], T * H);
+    for (int l = 0; l < s.n_layers; ++l) {
+      mem.add(&ctx->layers[l].w_router, E * H);
+      if (s.has_router_bias) mem.add(&ctx->layers[l].bias, E);
+    }
+    mem.add(&ctx->d_counts_copy, E);
+    rc = mem.allocate(ctx);
+    if (rc == OLED_OK) break;
+    if (ctx->row_buf == T * K) return fail(rc);
+    ctx->row_buf = T * K;
   }
-  mem.add_guarded(ctx->guards, &ctx->d_y, T * K * H);
-  mem.add(&ctx->d_status, kStatusWords);
-  mem.add(&ctx->d_timeline, (size_t)s.n_layers);
-  mem.add(&ctx->d_hidden_stage, T * H);
-  mem.add(&ctx->d_conf_stage, T);
-  mem.add(&ctx->d_out_stage, T * H);
-  mem.add(&ctx->d_iter[0], T * H);
-  mem.add(&ctx->d_iter[1], T * H);
-  for (int l = 0; l < s.n_layers; ++l) {
-    mem.add(&ctx->layers[l].w_router, E * H);
-    if (s.has_router_bias) mem.add(&ctx->layers[l].bias, E);
-  }
-  mem.add(&ctx->d_counts_copy, E);
-  if ((rc = mem.allocate(ctx)) != OLED_OK) return fail(rc);
+  ctx->last_cuda_error = 0;
   ctx->d_ctrl[1] = ctx->d_ctrl[0] + ctx->ctrl_bytes;
   select_ctrl(ctx, 0);
   ctx->d_gate = ctx->d_gate_buf[0];

@@ -1040,3 +1040,46 @@ def test_fp8_intermediate_rows_that_overflow_give_no_finite_outputs(n, direct):
         assert np.array_equal(outs[0][others], outs[1][others])
     finally:
         run.close()
+
+
+@pytest.mark.parametrize("fp8", [False, True], ids=["bf16", "fp8"])
+def test_a_context_that_fits_only_without_scatter_rows(fp8):
+    """Device memory short of what few-token steps would like for a region of rows per expert (512 experts, 64 tokens: 32768
+    rows instead of 64): the context is created all the same, its steps sort their rows, with the same outputs."""
+    from paper_2609_33385_b200.runner import bits_to_dev
+    n, e, h = 64, 512, 768
+    w = synth.tiny(n_layers=1, n_experts=e, top_k=1, hidden=h, intermediate=128)
+    dev = torch.device("cuda:0")
+    h_bits, conf = synth.flat_tokens(w, n, 70)
+    x, c = bits_to_dev(h_bits, dev), torch.from_numpy(conf).to(dev)
+    outs = [torch.empty((n, h), dtype=torch.bfloat16, device=dev) for _ in range(2)]
+    roomy = tight = hold = None
+    try:
+        roomy = _runner(w, capacity=[e], max_tokens=n, fp8=fp8)
+        roomy.step(0, x, c, outs[0])
+        roomy.ctx.synchronize()
+        before = torch.cuda.mem_get_info(dev)[0]           # (every kernel module is loaded by now)
+        again = _runner(w, capacity=[e], max_tokens=n, fp8=fp8, share_store_of=roomy)
+        roomy_bytes = before - torch.cuda.mem_get_info(dev)[0]
+        again.close()
+        torch.cuda.empty_cache()
+        surplus = (32768 - n) * (h + 128) * 2 * (2 if fp8 else 1)
+        assert roomy_bytes > surplus
+        keep = roomy_bytes - surplus // 2
+        hold = torch.empty(torch.cuda.mem_get_info(dev)[0] - keep, dtype=torch.uint8, device=dev)
+        tight = _runner(w, capacity=[e], max_tokens=n, fp8=fp8, share_store_of=roomy)
+        assert keep - torch.cuda.mem_get_info(dev)[0] < roomy_bytes - surplus * 3 // 4
+        hold = None
+        torch.cuda.empty_cache()
+        for _ in range(2):                                 # fetched experts, then resident ones
+            tight.step(0, x, c, outs[1])
+            tight.ctx.synchronize()
+            assert torch.equal(outs[0].view(torch.int16), outs[1].view(torch.int16))
+        a, b = roomy.ctx.debug_last(0, n), tight.ctx.debug_last(0, n)
+        assert all(np.array_equal(a[k], b[k]) for k in ("ids", "perm", "counts", "scores"))
+    finally:
+        hold = None
+        torch.cuda.empty_cache()
+        for r in (roomy, tight):
+            if r is not None:
+                r.close()
