@@ -266,8 +266,8 @@ int oled_residual_add(oled_ctx* ctx, const void* x, const void* r, void* y, size
 /* OLED_OPT_GATHER_IN_FFN: 1 (default) = in a many-token step whose FFN launches all run on CTA pairs
  * and whose expert matrices have at least 2^22 elements, each gate/up launch copies its own experts'
  * token rows into sorted order while its first items run (one thread per CTA, bulk copies through
- * shared memory, a counter per token tile that the items wait for); 0 = the permutation kernel
- * copies them, as in every other many-token step. */
+ * shared memory, a counter per token tile that the items wait for); 2 = the same whatever the size of the
+ * matrices; 0 = the permutation kernel copies them, as in every other many-token step. */
 #define OLED_OPT_GATHER_IN_FFN 17
 #define OLED_TIMELINE_SLOTS 12 /* 0 gate, 1 permutation, 2 gather (not recorded),
                                   3..10 the step's FFN launches in order, 11 combine */

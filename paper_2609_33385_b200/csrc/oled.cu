@@ -128,7 +128,7 @@ struct oled_ctx {
   bool timeline_on = false;    // OLED_OPT_TIMELINE
   bool fp8_direct = true;      // OLED_OPT_FP8_DIRECT
   int l2_prefetch = 1;         // OLED_OPT_L2_PREFETCH (2: whatever the length of the expert stream)
-  bool gather_in_ffn = true;   // OLED_OPT_GATHER_IN_FFN
+  int gather_in_ffn = 1;       // OLED_OPT_GATHER_IN_FFN (2: whatever the size of the expert matrices)
   cudaEvent_t ev_layer_done = nullptr;  // recorded behind a layer's last kernel (L2 prefetch of the next layer)
   StepTimeline* d_timeline = nullptr;
   bool y_bf16 = false;         // this step keeps the per-assignment outputs in bf16 (many tokens)
@@ -823,13 +823,13 @@ static int step_impl(oled_ctx* ctx, int32_t layer, const void* hidden, const flo
   }
   // Many rows per expert (every FFN launch of the step on CTA pairs, token tiles of 256 rows): no
   // gather kernel, each gate/up launch copies its experts' token rows while its first items run.
-  const bool gather_in_ffn = !few && ctx->gather_in_ffn && ctx->ffn_impl == 0 &&
+  const bool gather_in_ffn = !few && ctx->gather_in_ffn != 0 && ctx->ffn_impl == 0 &&
                              std::min<size_t>(T, 2 * (((size_t)T * K + E - 1) / E)) > 128 &&
                              (reinterpret_cast<uintptr_t>(hidden) & 15u) == 0 &&  // (bulk copies of whole rows)
                              // (a row's copy - loads, stores, fence and count on one thread - takes as long as 4 M
                              // elements of an expert matrix take the tensor cores; measured with / without: 2 layers
                              // of 2048 tokens, H x I 2 M: 875 / 654 us, one of 4096 tokens, 6 M: 1372 / 1418 us)
-                             (size_t)H * ctx->shape.intermediate >= (size_t)4 << 20 &&
+                             (ctx->gather_in_ffn == 2 || (size_t)H * ctx->shape.intermediate >= (size_t)4 << 20) &&
                              ffn_tc_token_source_usable(ctx->maps, H, ctx->shape.intermediate);
   // Otherwise the permutation kernel, where one runs, copies the rows (a step without per-segment counts but beyond 4096
   // assignments leaves that to a gather kernel).
@@ -1332,7 +1332,7 @@ int oled_set_option(oled_ctx* ctx, int32_t option, int64_t value) {
       ctx->maps.use_pairs = value != 0;
       return OLED_OK;
     case OLED_OPT_GATHER_IN_FFN:
-      ctx->gather_in_ffn = value != 0;
+      ctx->gather_in_ffn = value == 2 ? 2 : value != 0 ? 1 : 0;
       return OLED_OK;
     default:
       return OLED_ERR_INVALID_ARG;

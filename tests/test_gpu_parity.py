@@ -200,6 +200,13 @@ def test_many_tokens_per_expert_multi_tile(n):
         run.close()
 
 
+def _rows_copied_by_the_permutation(run, n):
+    """Did the permutation kernel of the steps since the last reading copy the token rows (by its bytes in the profile)?"""
+    p = run.ctx.profile_read()["permute"]
+    assert p["launches"] > 0
+    return p["bytes"] > p["launches"] * n * run.w.top_k * 12
+
+
 @pytest.mark.parametrize("n", [700, 2100])
 def test_cta_pair_ffn_form_many_tokens(n):
     """Token tiles of 256 rows with hidden a multiple of 512 and intermediate a multiple of 256: the
@@ -229,26 +236,32 @@ def test_cta_pair_ffn_form_many_tokens(n):
             run.ctx.reset_cache()
         assert np.linalg.norm(outs[0] - outs[1]) <= 1e-3 * np.linalg.norm(outs[1])
         assert np.array_equal(outs[0], outs[2])   # the same items in the same arithmetic, one launch or two
-        # token rows gathered by the FFN launch itself (the default where it applies, n = 2100
-        # here) or by a gather kernel in front: the same operands
+        # token rows gathered by the FFN launch itself (forced: the matrices are small; a many-token step, n = 2100)
+        # or by the permutation kernel in front: the same operands
+        run.ctx.set_option(binding.OPT_PROFILE, 1)
         for fuse in (1, 0):
-            run.ctx.set_option(binding.OPT_FFN_PAIRS, 1)
-            run.ctx.set_option(binding.OPT_FUSE_FFN, fuse)
-            run.ctx.set_option(binding.OPT_GATHER_IN_FFN, 0)
-            out = torch.empty((n, w.hidden), dtype=torch.bfloat16, device=run.device)
-            run.step(0, bits_to_dev(h_bits, run.device), c, out)
-            _check_step(run, 0, n, out, ref)
-            assert np.array_equal(outs[0], out.float().cpu().numpy().astype(np.float64))
-            run.ctx.reset_cache()
+            for gather in (2, 0):
+                run.ctx.set_option(binding.OPT_FFN_PAIRS, 1)
+                run.ctx.set_option(binding.OPT_FUSE_FFN, fuse)
+                run.ctx.set_option(binding.OPT_GATHER_IN_FFN, gather)
+                run.step(0, bits_to_dev(h_bits, run.device), c, out)   # (cold: the experts are fetched)
+                _check_step(run, 0, n, out, ref)
+                run.ctx.profile_read()
+                out = torch.empty((n, w.hidden), dtype=torch.bfloat16, device=run.device)
+                run.step(0, bits_to_dev(h_bits, run.device), c, out)
+                if n == 2100:
+                    assert _rows_copied_by_the_permutation(run, n) == (gather == 0)
+                assert np.array_equal(outs[0], out.float().cpu().numpy().astype(np.float64))
+                run.ctx.reset_cache()
     finally:
         run.close()
 
 
 @pytest.mark.parametrize("hidden", [512, 4608])
 def test_gather_in_ffn_with_cache_misses(hidden):
-    """A many-token step with misses: the launches over the fetched experts gather their own token rows
-    as well (token tile 256 whatever their counts), ragged tiles included.  hidden 4608: a row is moved
-    as two pieces (8192 + 1024 bytes)."""
+    """A many-token step with misses whose FFN launches gather their own token rows (forced: the matrices are small): those
+    over the fetched experts as well (token tile 256 whatever their counts), ragged tiles included.  hidden 4608: a
+    row is moved as two pieces (8192 + 1024 bytes)."""
     from paper_2609_33385_b200 import binding
     from paper_2609_33385_b200.runner import bits_to_dev, dev_to_bits
     n = 2100
@@ -258,6 +271,8 @@ def test_gather_in_ffn_with_cache_misses(hidden):
     run = _runner(w, capacity=[2], max_tokens=n)
     ora = _oracle_for(run, [2])
     try:
+        run.ctx.set_option(binding.OPT_GATHER_IN_FFN, 2)
+        run.ctx.set_option(binding.OPT_PROFILE, 1)
         got = []
         for seed in (9, 10):
             h_bits, conf = synth.flat_tokens(w, n, seed)
@@ -267,7 +282,8 @@ def test_gather_in_ffn_with_cache_misses(hidden):
             _check_step(run, 0, n, out, ref)
             got.append(dev_to_bits(out).copy())
         assert run.ctx.stats().misses > 0
-        # the same two steps with a gather kernel in front: the same bits
+        assert not _rows_copied_by_the_permutation(run, n)
+        # the same two steps with the rows copied by the permutation kernel: the same bits
         run.ctx.reset_cache()
         run.ctx.set_option(binding.OPT_GATHER_IN_FFN, 0)
         for i, seed in enumerate((9, 10)):
@@ -275,6 +291,7 @@ def test_gather_in_ffn_with_cache_misses(hidden):
             out = torch.empty((n, w.hidden), dtype=torch.bfloat16, device=run.device)
             run.step(0, bits_to_dev(h_bits, run.device), torch.from_numpy(conf).to(run.device), out)
             assert np.array_equal(got[i], dev_to_bits(out))
+        assert _rows_copied_by_the_permutation(run, n)
     finally:
         run.close()
 
