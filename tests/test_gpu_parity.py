@@ -715,16 +715,20 @@ def test_fp8_expert_store_tiny_stack():
         run.close()
 
 
-@pytest.mark.parametrize("n", [40, 300, 700])
-def test_fp8_expert_store_token_tile_variants(n):
-    """fp8 blobs through every FFN tile form that exists for them: stacked (token tiles up to 32
-    rows) and two accumulators (64 and 128 rows; fp8 stores stop at 128-row tiles, so the
-    700-token case takes several tiles per expert)."""
+@pytest.mark.parametrize("direct", [1, 0], ids=["direct", "widening"])
+@pytest.mark.parametrize("n", [24, 40, 300, 700, 2100])
+def test_fp8_expert_store_token_tile_variants(n, direct):
+    """fp8 blobs through every FFN tile form that exists for them (OLED_OPT_FP8_DIRECT): codes read directly, token tiles
+    of 32, 48 and 128 rows; codes widened, stacked (token tiles up to 32 rows) and two accumulators (64 and 128
+    rows).  700 tokens: several tiles per expert; 2100: more than 4096 assignments, where matrices this small are
+    widened in both settings."""
+    from paper_2609_33385_b200 import binding
     from paper_2609_33385_b200.runner import bits_to_dev
     w = synth.tiny(n_layers=1, n_experts=4, top_k=2, hidden=512, intermediate=256)
     run = _runner(w, capacity=[4], max_tokens=n, fp8=True)
     ora = _oracle_for(run, [4])
     try:
+        run.ctx.set_option(binding.OPT_FP8_DIRECT, direct)
         h_bits, conf = synth.flat_tokens(w, n, 50)
         x, c = bits_to_dev(h_bits, run.device), torch.from_numpy(conf).to(run.device)
         out = torch.empty((n, w.hidden), dtype=torch.bfloat16, device=run.device)
@@ -735,8 +739,8 @@ def test_fp8_expert_store_token_tile_variants(n):
 
 
 def test_fp8_direct_form_agrees_with_widening_form_on_wide_range_rows():
-    """Token tiles of at most 32 rows take the form whose MMAs read the e4m3 codes directly, the
-    token rows entering as two e4m3 terms after a per-row power-of-two scale.  Rows with a wide
+    """The form whose MMAs read the e4m3 codes directly, the token rows entering as two e4m3 terms
+    after a per-row power-of-two scale, on a block of 24 tokens.  Rows with a wide
     dynamic range (elements 2^-12 below the row's maximum), an all-zero row and a row 2^10 larger
     than the rest: same discrete results, outputs within tolerance of the oracle, and the two
     forms (OLED_OPT_FP8_DIRECT 1 / 0) agree far more closely than either has to with the oracle."""
@@ -773,6 +777,57 @@ def test_fp8_direct_form_agrees_with_widening_form_on_wide_range_rows():
                 assert np.linalg.norm(a[t] - ref["out"][t]) / den <= REL_L2, ("direct form against the oracle", t)
                 assert np.linalg.norm(b[t] - ref["out"][t]) / den <= REL_L2, ("widening form against the oracle", t)
                 assert np.linalg.norm(a[t] - b[t]) / den < 3e-3, ("the two forms", t)
+    finally:
+        run.close()
+
+
+@pytest.mark.parametrize("shape,counts,capacity", [((8, 8, 2048, 512), (700, 523), 8), ((8, 8, 2048, 512), (700, 700), 5),
+                                                   ((40, 8, 1024, 1024), (530, 1024), 40)])
+def test_fp8_codes_read_directly_beyond_4096_assignments(shape, counts, capacity):
+    """fp8 steps of more than 4096 assignments with expert matrices of 2^20 elements and more: the segmented permutation
+    makes the rows' e4m3 terms, the FFN reads the codes directly over sorted rows and stores bf16 outputs per
+    assignment.  Every expert takes several tiles, segments and tiles end raggedly, a row has a wide range of
+    magnitudes, one is all zero and one far above the others; capacity 5: fetched experts in launches of their own.
+    Parity with the oracle; the same bits when repeated; and no further from the oracle's 64-bit sums than the
+    widening form (OLED_OPT_FP8_DIRECT 0), which multiplies the rows as they are.  Both are 2.3e-3 to 2.9e-3 away - bf16
+    intermediate rows and outputs, which fall either way in the last place: over 50 shapes and seeds the two errors
+    differed by up to 0.03 % from 100 tokens on."""
+    from paper_2609_33385_b200 import binding
+    from paper_2609_33385_b200.runner import bits_to_dev, dev_to_bits
+    e, k, h, i = shape
+    w = synth.tiny(n_layers=1, n_experts=e, top_k=k, hidden=h, intermediate=i, weight_std=0.02)
+    run = _runner(w, capacity=[capacity], max_tokens=max(counts), fp8=True)
+    ora = _oracle_for(run, [capacity])
+    try:
+        assert h * i >= 1 << 20 and min(counts) * k > 4096
+        run.ctx.set_option(binding.OPT_SELF_CHECK, 1)
+        for rep, n in enumerate(counts):
+            h_bits, conf = synth.flat_tokens(w, n, 600 + rep)
+            f = (h_bits.astype(np.uint32) << 16).view(np.float32).copy()
+            f[1, ::3] *= 2.0 ** -12
+            f[3, :] = 0.0
+            f[5, :] *= 2.0 ** 6
+            h_bits = (f.view(np.uint32) >> 16).astype(np.uint16)
+            x, c = bits_to_dev(h_bits, run.device), torch.from_numpy(conf).to(run.device)
+            outs = []
+            with np.errstate(over="ignore"):
+                ref = ora.denoise_step(0, h_bits, conf)
+            for again, direct in enumerate((1, 1, 0)):
+                run.ctx.set_option(binding.OPT_FP8_DIRECT, direct)
+                out = torch.empty((n, h), dtype=torch.bfloat16, device=run.device)
+                run.step(0, x, c, out)
+                if again == 0:
+                    _check_step(run, 0, n, out, ref, check_out=False)
+                else:
+                    ora.denoise_step(0, h_bits, conf)      # (keeps the oracle's resident set in step)
+                outs.append(dev_to_bits(out))
+            assert np.array_equal(outs[0], outs[1])
+            got = [synth.bf16_bits_to_f32(o).astype(np.float64) for o in outs[1:]]
+            rows = np.arange(n) != 5                       # (row 5 would be the whole norm)
+            err = [np.linalg.norm((g - ref["out"])[rows]) / np.linalg.norm(ref["out"][rows]) for g in got]
+            assert max(err) <= REL_L2 and err[0] <= 1.002 * err[1], err
+            assert np.linalg.norm(got[0][5] - ref["out"][5]) <= REL_L2 * np.linalg.norm(ref["out"][5])
+            assert np.all(got[0][3] == 0.0)
     finally:
         run.close()
 
@@ -835,8 +890,8 @@ def test_one_launch_and_two_launch_ffn_forms_agree_bit_for_bit():
     """OLED_OPT_FUSE_FFN: gate/up + down projection as one launch (down items wait on per-expert
     completion counters) or as two launches.  Which kernel computes an item does not change its
     arithmetic, so the layer outputs must be bit-identical, and both in parity with the oracle;
-    block sizes with one and with two token tiles per expert, cold start so that launches of
-    fetched experts (behind event waits) are covered too."""
+    token tiles of 16 to 128 rows, cold start so that launches of fetched experts (behind event
+    waits) are covered too."""
     from paper_2609_33385_b200 import binding
     from paper_2609_33385_b200.runner import bits_to_dev, dev_to_bits
     w = synth.tiny(n_layers=1, n_experts=6, top_k=3, hidden=512, intermediate=256)
@@ -847,7 +902,7 @@ def test_one_launch_and_two_launch_ffn_forms_agree_bit_for_bit():
         ora = _oracle_for(run, [3])
         try:
             res = []
-            for rep, n in enumerate((7, 33, 60, 150)):      # 150 tokens: 64-row tiles, always two launches
+            for rep, n in enumerate((7, 33, 60, 150)):
                 h_bits, conf = synth.flat_tokens(w, n, 80 + rep)
                 x, c = bits_to_dev(h_bits, run.device), torch.from_numpy(conf).to(run.device)
                 out = torch.empty((n, w.hidden), dtype=torch.bfloat16, device=run.device)
