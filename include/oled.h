@@ -82,8 +82,8 @@ typedef struct {
  *     The tensor cores read the codes as they are; a bf16 token row, scaled by a power of two, enters
  *     as the sum of two e4m3 terms, which represents every element within 2^-14 of the row's
  *     largest magnitude exactly (OLED_OPT_FP8_DIRECT; in steps of more than 4096 token-expert
- *     assignments where hidden * intermediate is at least 2^20).  Otherwise the codes are widened to
- *     bf16 on chip (exactly) and the arithmetic is the bf16 path's. */
+ *     assignments only from 297 tokens and hidden * intermediate = 2^20 on).  Otherwise the codes are widened to
+ *     bf16 on chip (exactly) and the arithmetic is the bf16 path's.  A row with an infinity or a NaN yields NaN. */
 #define OLED_EXPERTS_BF16 0
 #define OLED_EXPERTS_FP8 1
 /* Bytes of one expert blob in the given format. */
@@ -238,8 +238,8 @@ int oled_residual_add(oled_ctx* ctx, const void* x, const void* r, void* y, size
  *   1 (default) or 2 = as ONE launch wherever that form exists: SMs that run out of gate/up items
  *   go on with the down projection of experts that are complete instead of idling until the whole
  *   gate/up launch has ended.
- * OLED_OPT_PDL: programmatic dependent launch between the kernels of a few-token step
- *   (process-wide, not per context). */
+ * OLED_OPT_PDL: programmatic dependent launch between the kernels of a step of up to 16384
+ *   token-expert assignments (process-wide, not per context). */
 #define OLED_OPT_SPLIT_LAST_FILL 9
 #define OLED_OPT_FUSE_COMBINE 10
 #define OLED_OPT_FUSE_FFN 11

@@ -32,8 +32,8 @@
 //
 // With few experts activated (8 at one token) it is bound by the chain of one CTA's item instead.  Hence the
 // roles: one warp loads weights, one loads token rows (each TMA copy is 120 cycles of its thread; with both on one
-// thread that thread was the limit: 8 layers of 1 token 282 us, now 261; 8 layers of 16 similar tokens 421,
-// now 384), one issues MMAs, and the epilogue's warps build the work table while the first item already runs.
+// thread that thread was the limit: 8 layers of 1 token 282 us against 261 when they were parted; 8 layers of 16 similar tokens 421
+// against 384), one issues MMAs, and the epilogue's warps build the work table while the first item already runs.
 //
 // Token rows (FfnRows): dense steps (at most 32 tokens) multiply EVERY expert with all rows of the step,
 // stored once, in token order - the tile costs what a gathered one would (N is 16 or 32 either way) and
@@ -255,7 +255,8 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
     if (spec && elect_one()) {
       for (int i = 0; i < pre1; ++i) load_weights(i, i, false, spec_m, grp.slot[spec_g]);
       // the rest of the item into L2, for steps whose gate kernel is short (8 layers of 16 similar tokens 362 -> 356 us; with
-      // 250 tokens fp8 it took bandwidth from the gate's own loads, 775 -> 789, with 100 tokens still 523 -> 517)
+      // 250 tokens fp8 it took bandwidth from the gate's own loads, 775 -> 789, with 100 tokens still 523 -> 517; where
+      // between those two the line lies was not measured, it is drawn at one gate CTA per SM)
       if (p.rows.cap <= 148)
         for (int a = pre1 * p.k_atoms; a < k_blocks1 * p.k_atoms; ++a)
           few_prefetch_w1(&p.tm_w1, a * kK, spec_m, grp.slot[spec_g], policy);

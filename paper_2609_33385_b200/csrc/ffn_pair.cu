@@ -524,7 +524,7 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant_
     }
   } else if (warp < kPairEpiWarps) {
     // ------------------------------------------------------------ epilogue (both CTAs)
-    // warp w: TMEM lane quarter w mod 4 (32 of the CTA's 128 rows), every fourth 16-column chunk
+    // warp w: TMEM lane quarter w mod 4 (32 of the CTA's 128 rows), every second 16-column chunk
     if (gathers && !grp.withhold_loads) {
       // These warps have nothing to do until the first item's MMAs are through: they copy the token
       // rows of the tiles the first wave of items reads (one row per warp at a time, plain loads and
@@ -575,7 +575,7 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant_
       const int n_mma = max(32, (it.valid + 31) & ~31);
       const int col = it.m0 + (int)rank * (it.kind == 1 ? 128 : 256) + quarter * 32 + lane;  // feature / output row of this thread
       void* const out_y = fused ? sec.out2 : out_ptr;
-      // The warp's chunks (four at most: chunk ci is columns 16 * (4 ci + part) ..).  The accumulators are handed back
+      // The warp's chunks (eight at most: chunk ci is columns 16 * (2 ci + part) ..).  The accumulators are handed back
       // as soon as the LAST chunk has been read, so what stands before that is kept short: the results
       // stay in registers as packed bf16 and are stored afterwards, while the MMAs of the next item already write
       // the columns.  (With every chunk stored before the next was read the MMAs waited 8000 cycles per item, 16 % of a

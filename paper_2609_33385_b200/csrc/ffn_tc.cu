@@ -24,7 +24,7 @@
 //
 // Work items (expert, token tile, weight tile) are drawn from a global counter by each CTA's
 // producer and handed to its other roles through a ring in shared memory (see take_item); a
-// pipeline stage holds one k-block of 64, or two for small token tiles; KIND 2 starts its weight
+// pipeline stage holds one k-block of 64, or two (fp8 stores, one weight tile); KIND 2 starts its weight
 // stream before its predecessor KIND 1 has finished (see the set-up in the kernel).
 //
 // Warp roles (704 threads): warps 0-15 epilogue (TMEM lane quarter = warp id mod 4, the warps of
@@ -147,8 +147,8 @@ __device__ __forceinline__ void decode_item(const SharedCtl* ctl, const FfnGroup
   it.valid = min(n_box, ctl->count[g] - nt * n_box);
 }
 
-// DUAL: two accumulators per item - gate and up (KIND 1, always), or two row blocks of Wd
-// (KIND 2 with the 256-token tile).
+// DUAL: two accumulators per item - gate and up, or two row blocks of Wd (always with bf16 stores, whose tiles here have
+// 256 rows).
 // WIDEN: the slot pool holds fp8 expert blobs (tm_w is a byte map over the e4m3 codes); the MMA's
 // weight operand comes from tensor memory.
 template <int KIND, bool DUAL, bool WIDEN>
@@ -165,7 +165,7 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n_box = grp.n_box;
-  static_assert(DUAL || WIDEN || KIND == 2, "gate/up tiles of bf16 stores have two accumulators");
+  static_assert(DUAL || WIDEN, "tiles of bf16 stores have two accumulators");
   constexpr int kK = kBlockK;  // k-values of a k-block (one 128-byte swizzle atom of weights)
   constexpr bool dual = DUAL;
   constexpr bool stacked = KIND == 1 && !DUAL;  // gate/up items: 64 gate + 64 up rows in one 128-row tile
@@ -718,17 +718,16 @@ struct Rings {
 int epi_warps_for(int kind, int out_bf16, int n_box) {
   return std::min((kind != 2 || out_bf16) ? kEpiWarps : 8, 4 * (n_box / 16));
 }
-// Stage shape and count.  A stage holds two k-blocks where at least four such stages fit (small
-// token tiles, one weight tile) and the contraction has an even number of k-blocks.  bf16 stores:
-// as many stages (weight tile(s) + token tile) as fit in shared memory, ten k-blocks at most
-// (eleven measured slower).  fp8 stores: a stage is a load slot in shared memory plus columns of
+// Stage shape and count.  A stage holds two k-blocks where at least four such stages fit (fp8 stores, one
+// weight tile) and the contraction has an even number of k-blocks.  bf16 stores: as many stages (two weight
+// tiles + token tile) as fit in shared memory.  fp8 stores: a stage is a load slot in shared memory plus columns of
 // tensor memory behind the accumulators (two accumulator stages if at least two weight stages
 // still fit); the depth is a multiple of the number of converter groups (see the kernel).
 Rings rings_for(int kind, bool dual, int n_box, int out_bf16, bool fp8, int k_dim) {
   const uint32_t a = (dual ? 2u : 1u) * kATile, b = (uint32_t)n_box * 128u;
   const uint32_t avail = kSmemMax - kCtlBytes - 1024u;
   const uint32_t atom = (fp8 ? a / 2 : a) + b;  // one k-block in shared memory
-  int kblocks = (int)std::min<uint32_t>((uint32_t)(fp8 ? 2 * kMaxStages : 10), avail / atom);
+  int kblocks = (int)std::min<uint32_t>((uint32_t)(fp8 ? 2 * kMaxStages : kMaxStages), avail / atom);
   if (fp8) {
     const int acc_cols = (dual ? 2 : 1) * n_box, a_cols = dual ? 64 : 32;
     const int free_cols = 512 - 2 * acc_cols >= 2 * a_cols ? 512 - 2 * acc_cols : 512 - acc_cols;
@@ -807,7 +806,7 @@ int ffn_tc_setup(FfnTcMaps* maps, const uint8_t* pool, size_t slot_bytes, int n_
   }
   static bool attr_done = false;
   if (!attr_done) {
-    if (!set_smem_attr<1, true, false>() || !set_smem_attr<2, true, false>() || !set_smem_attr<2, false, false>() ||
+    if (!set_smem_attr<1, true, false>() || !set_smem_attr<2, true, false>() ||
         !set_smem_attr<1, true, true>() || !set_smem_attr<1, false, true>() || !set_smem_attr<2, false, true>())
       return OLED_ERR_CUDA;
     attr_done = true;
@@ -823,7 +822,7 @@ static int box_index(int max_count, int cap) {
 
 // Token tiles of at most kFewMaxRows rows go to ffn_few.cu (4 layers of 64 experts, us, against the two-accumulator
 // tiles here: 300 tokens 635 / 707, 512 tokens 701 / 773; beyond 128 rows the operand traffic of its single weight
-// tile costs more than it saves: 1000 tokens 1035 against 926 on CTA pairs).  Of fp8 stores every tile does, provided
+// tile costs more than it saves: 1000 tokens 1035 here, 926 on CTA pairs when that was measured, 800 now).  Of fp8 stores every tile does, provided
 // the rows' e4m3 terms are at hand (8 layers of 250 tokens: 763 / 1459); otherwise converter warps widen the codes.
 static bool few_form(const FfnTcMaps& maps, int max_count, const TokenSplit* split) {
   if (!maps.few) return false;
@@ -887,7 +886,6 @@ int launch_ffn_tc(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp_in
   const bool early_allowed = kind == 2 && (behind_event_wait || host_counts == nullptr);
   const uint32_t smem1 = kind == 2 ? rings_for(1, !stacked1, grp.n_box, 0, fp8, H).smem : 0u;
   if (kind == 3) return OLED_ERR_INVALID_ARG;  // callers ask ffn_tc_can_fuse() / ffn_pair_can_fuse() first
-  const bool dual2 = grp.n_box == 256;
   auto go = [&](auto kind_c, auto dual_c, auto widen_c, int m_tiles, const CUtensorMap& tw, const CUtensorMap& ta, void* out,
                 int out_bf16) {
     launch_variant<decltype(kind_c)::value, decltype(dual_c)::value, decltype(widen_c)::value>(
@@ -901,9 +899,8 @@ int launch_ffn_tc(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp_in
   if (kind == 1 && stacked1) go(k1, false_type{}, true_type{}, I / (kBlockM / 2), maps.w13_half, maps.xp[ib], hbuf, 0);
   else if (kind == 1 && fp8) go(k1, true_type{}, true_type{}, I / kBlockM, maps.w13, maps.xp[ib], hbuf, 0);
   else if (kind == 1) go(k1, true_type{}, false_type{}, I / kBlockM, maps.w13, maps.xp[ib], hbuf, 0);
-  else if (dual2) go(k2, true_type{}, false_type{}, H / (2 * kBlockM), maps.w2, maps.hbuf[ib], y, y_bf16);
   else if (fp8) go(k2, false_type{}, true_type{}, H / kBlockM, maps.w2, maps.hbuf[ib], y, y_bf16);
-  else go(k2, false_type{}, false_type{}, H / kBlockM, maps.w2, maps.hbuf[ib], y, y_bf16);
+  else go(k2, true_type{}, false_type{}, H / (2 * kBlockM), maps.w2, maps.hbuf[ib], y, y_bf16);  // (256 rows)
   return cudaGetLastError() == cudaSuccess ? OLED_OK : OLED_ERR_CUDA;
 }
 

@@ -156,7 +156,7 @@ constexpr int kPermuteSegments = 16;
 //   amax_in, terms_in:   written by the gate kernel of a scattered step (or the gathering
 //                        permutation kernel), which also zeroes amax_mid
 //   amax_mid:            raised with atomicMax by the gate/up epilogue
-//   terms_mid:           written by the split kernel between the two projections
+//   terms_mid:           written by warps of the one-launch FFN, or the split kernel between its two launches
 struct TokenSplit {
   uint32_t* amax_in = nullptr;   // [rows]
   uint32_t* amax_mid = nullptr;  // [rows]
@@ -272,7 +272,7 @@ struct FfnTcMaps {
 int ffn_tc_setup(FfnTcMaps* maps, const uint8_t* pool, size_t slot_bytes, int n_slots, int H, int I, bool fp8,
                  const uint16_t* xp, const uint16_t* hbuf, int rows, const TokenSplit* split = nullptr);
 // kind 1: gate/up + SwiGLU into hbuf; kind 2: down projection into y; kind 3: both in one launch
-// (bf16 stores and token tiles of at most 32 rows only: ask ffn_tc_can_fuse; `done` then points at
+// (where ffn_tc_can_fuse or ffn_pair_can_fuse says so; `done`, and split_done with fp8 stores, then point at
 // one ZERO word per expert of the group).  One launch each.
 // work_counter: two device words that are ZERO when the kernel starts; its CTAs draw their work items
 // from the first and rows to split from the second (every launch that can be in flight at the same time needs
@@ -281,9 +281,9 @@ int ffn_tc_setup(FfnTcMaps* maps, const uint8_t* pool, size_t slot_bytes, int n_
 // counts and scores to the host.
 // behind_event_wait: the launch follows a cudaStreamWaitEvent (with, for kind 2, at most its own
 // kind 1 launch in between), i.e. everything enqueued before that wait has completed.
-// split (fp8 stores; nullptr: none): the token operands as e4m3 terms.  With them, token tiles of
-// at most 32 rows take the form whose MMAs read the experts' e4m3 codes as they are; a kind 2
-// launch is then preceded by the split kernel (ffn_tc_launches tells how many launches a call makes).
+// split (fp8 stores; nullptr: none): the token operands as e4m3 terms.  With them the MMAs read the experts' e4m3
+// codes as they are, whatever the tile; a kind 2 launch is then preceded by the split kernel (ffn_tc_launches tells
+// how many launches a call makes).
 int launch_ffn_tc(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& grp, int max_count, int kind,
                   const int32_t* host_counts, const FfnRows& rows, uint16_t* hbuf, float* y, int y_bf16, int H,
                   int I, int n_sms, uint32_t* status, uint32_t* work_counter, bool behind_event_wait,

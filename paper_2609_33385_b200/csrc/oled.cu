@@ -22,7 +22,6 @@ namespace {
 
 struct LayerData {
   LayerCacheState cache;
-  int32_t last_active = -1;      // experts activated at the layer's previous execution (-1: none yet)
   int32_t last_tokens = 0;       // tokens of the layer's previous execution (0: none yet)
   int32_t last_max_count = 0;    // most token rows any expert received then
   int32_t last_misses = -1;      // its misses
@@ -94,7 +93,7 @@ struct oled_ctx {
   uint16_t* d_xp = nullptr;    // [row_buf,H]
   uint16_t* d_hbuf = nullptr;  // [row_buf,I]
   TokenSplit split;            // fp8 stores: the FFN's token operands as e4m3 terms (see TokenSplit)
-  const TokenSplit* step_split = nullptr;  // &split in steps whose permutation kernel fills it
+  const TokenSplit* step_split = nullptr;  // &split in steps whose gate or permutation kernel fills it
   float* d_y = nullptr;        // [T*k,H]
   uint32_t* d_status = nullptr;
   uint32_t* d_work = nullptr;         // control block: work-item counters of the step's FFN launches
@@ -105,7 +104,7 @@ struct oled_ctx {
   int32_t* d_seg = nullptr;           // control block, last: [kPermuteSegments][E] per-segment counts of many-token steps
   int work_next = 0;                  // next unused counter of the current layer execution
   bool ctrl_dirty = true;             // both control blocks must be cleared before the next gate launch
-  unsigned int seq = 0;               // step sequence number echoed by the gate kernel
+  unsigned int seq = 0;               // step sequence number echoed by the report
   volatile unsigned long long* h_report = nullptr;  // pinned, mapped: tagged scores [E] | tagged counts [E]
   std::vector<unsigned long long> host_scores;       // decoded copy of the last report
   std::vector<int32_t> host_counts;
@@ -373,8 +372,7 @@ void prof_add_ffn(oled_ctx* ctx, uint64_t n, uint64_t rows, bool fused) {
 }
 
 // The FFN launches over one group: gate/up and down projection, or ONE fused launch where that
-// form exists (bf16 stores, token tiles of at most 32 rows, no event to wait for between the two
-// projections).  host_counts == nullptr: the per-expert counts are not known on the host yet (the
+// form exists (ffn_few.cu, ffn_pair.cu; no event to wait for between the two projections).  host_counts == nullptr: the per-expert counts are not known on the host yet (the
 // group is the resident set and experts without tokens cost nothing).
 // before_down: an event the down projection (and nothing before it) has to wait for, or null.
 // behind_event_wait: the caller has just enqueued a cudaStreamWaitEvent on the stream.
@@ -401,7 +399,7 @@ int run_ffn_launches(oled_ctx* ctx, const FfnGroup& grp, int max_count, const in
                       ctx->d_y, H, I);
     ctx->launches += 2;
   } else {
-    // Token tiles of at most 32 rows, bf16 stores: one launch.  SMs that run out of gate/up items go on with
+    // ffn_few.cu: one launch.  SMs that run out of gate/up items go on with
     // the down projection of experts that are complete (per layer: 8 experts 35 against 39 us as two launches,
     // 20 experts 52 against 56, 63 and 128 experts 133 and 217 us either way).
     // Many-token tiles on CTA pairs: always one launch (a boundary between cluster kernels is a full stop).
@@ -474,7 +472,7 @@ int run_ffn_group(oled_ctx* ctx, LayerData& L, const std::vector<int32_t>& exper
   return rc;
 }
 
-// Blocks until the gate kernel of step `seq` has published counts and scores, and decodes them.
+// Blocks until the counts and scores of step `seq` have been published, and decodes them.
 int wait_gate_report(oled_ctx* ctx) {
   const size_t E = (size_t)ctx->shape.n_experts;
   const unsigned long long tag16 = (unsigned long long)(ctx->seq & 0xffffu);
@@ -743,8 +741,8 @@ static int step_impl(oled_ctx* ctx, int32_t layer, const void* hidden, const flo
   // per-assignment outputs y: fp32 for small steps; bf16 once y's traffic matters (the rounding
   // adds at most 2^-9 relative per term, far inside the output tolerance)
   ctx->y_bf16 = ctx->ffn_impl == 0 && (size_t)T * K > 4096;
-  // 1. gate, counts and reuse-score numerators, permutation; the permutation kernel reports
-  // counts and scores to the host.  This step takes the control block the last step did not use.
+  // 1. gate, counts and reuse-score numerators, permutation (few-token steps: the gate kernel brings the rows to their
+  // experts).  Counts and scores reach the host with the first FFN launch.  This step takes the control block the last step did not use.
   if (ctx->ctrl_dirty) OLED_CUDA(ctx, cudaMemsetAsync(ctx->d_ctrl[0], 0, 2 * ctx->ctrl_bytes, st));
   ctx->ctrl_dirty = true;
   select_ctrl(ctx, ctx->ctrl_sel ^ 1);
@@ -1028,7 +1026,6 @@ static int step_impl(oled_ctx* ctx, int32_t layer, const void* hidden, const flo
   L.stats.bytes_moved += (uint64_t)n_miss * ctx->slot_bytes;
   L.stats.evictions += (uint64_t)plan.n_evictions;
   L.stats.active_experts += (uint64_t)plan.n_active;
-  L.last_active = plan.n_active;
   L.last_tokens = T;
   L.last_max_count = 0;
   for (int32_t e = 0; e < E; ++e) L.last_max_count = std::max(L.last_max_count, counts[e]);

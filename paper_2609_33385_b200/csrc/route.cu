@@ -249,7 +249,7 @@ __device__ __forceinline__ void sort_assignments(const int32_t* ids, int n, int 
 // - the same total order a round-by-round selection walks.
 // One token per CTA while that gives at most one wave of CTAs; two or four beyond (every CTA
 // streams the whole router matrix, so a second wave costs as much as the first).
-// The kernel reports nothing to the host: the permutation kernel, which follows it in every step,
+// The kernel reports nothing to the host: the step's first FFN launch, which starts when it has completed,
 // publishes the finished counts and scores without any ticket or fence.
 template <int TT, int WARPS, int UNROLL, int kEPerWarp>
 __global__ void __launch_bounds__(WARPS * 32, 1)
@@ -650,7 +650,7 @@ route_many_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ w
 // One CTA per expert (blockIdx.x): offset = sum of the counts before it; then a stable scan of the
 // flat assignment list (ascending t*K+j) hands out consecutive sorted rows.
 // If xp != nullptr the expert's CTAs (gridDim.y of them) also copy its token rows into sorted
-// order (xp[r,:] = x[perm[r]/K,:]); used for small steps, larger ones run gather_kernel instead.
+// order (xp[r,:] = x[perm[r]/K,:]); used for small steps and, segment by segment, in many-token steps.
 // Each of those CTAs repeats the scan for itself - a few hundred ids - keeps the token of every
 // sorted row in shared memory (reading the rows' numbers back from global memory would cost a
 // round trip before the first load), and takes every gridDim.y-th batch of RB rows, so that an
@@ -767,7 +767,7 @@ permute_kernel(const int32_t* __restrict__ ids, const int32_t* __restrict__ coun
   }
   if (threadIdx.x < 3 * RB) s_amax[threadIdx.x / RB][threadIdx.x % RB] = 0u;
   __syncthreads();  // the tokens of this expert's rows are in shared memory
-  // eight rows at a time: their token numbers, then their loads, are independent memory
+  // RB rows at a time: their token numbers, then their loads, are independent memory
   // operations in flight together (a row-by-row loop is a chain of dependent round trips)
   // (segmented launches: all rows of the segment are this CTA's)
   const int vec_per_row = H / 8, first = s_base, rows = segmented ? seg_counts[blockIdx.y * E + e] : counts[e];

@@ -88,13 +88,6 @@ __device__ __forceinline__ void tma_load_3d_hint(const CUtensorMap* map, uint32_
 __device__ __forceinline__ void red_release_add(uint32_t* counter, uint32_t n) {
   asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(counter), "r"(n) : "memory");
 }
-__device__ __forceinline__ void tma_load_4d(const CUtensorMap* map, uint32_t dst, uint32_t bar, int c0,
-                                            int c1, int c2, int c3) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
-      ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
-      : "memory");
-}
 __device__ __forceinline__ void tma_load_2d(const CUtensorMap* map, uint32_t dst, uint32_t bar, int c0,
                                             int c1) {
   asm volatile(
@@ -138,20 +131,8 @@ __device__ __forceinline__ void tc_mma_ts_lo(uint32_t d_tmem, uint32_t a_tmem, u
       ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-// The same contraction with BOTH operands e4m3 in shared memory (kind::f8f6f4: K = 32 per
-// instruction, one byte per element, so 32 bytes along K per instruction as in the bf16 form).
-__device__ __forceinline__ void tc_mma_e4m3_lo(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi,
-                                               uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
-      "mov.b64 da, {%1, %3};\n\t"
-      "mov.b64 db, {%2, %3};\n\t"
-      "setp.ne.b32 p, %5, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], da, db, %4, p;\n\t}"
-      ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-// The two forms above with whole descriptors and the accumulate flag fixed at compile time.
+// Both operands in shared memory, with whole descriptors and the accumulate flag fixed at compile time: bf16, or e4m3
+// (kind::f8f6f4: K = 32 per instruction, one byte per element, so 32 bytes along K per instruction as in the bf16 form).
 template <bool E4M3, bool ACCUMULATE>
 __device__ __forceinline__ void tc_mma_desc(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc) {
   if constexpr (E4M3)
@@ -284,18 +265,6 @@ __device__ __forceinline__ uint32_t make_idesc(int n) {
 // Instruction descriptor: D fp32, A/B e4m3 (format code 0 of kind::f8f6f4), both K-major, M = 128, N = n.
 __device__ __forceinline__ uint32_t make_idesc_e4m3(int n) {
   return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-}
-
-// 16 bytes global -> shared, asynchronously; src_bytes = 0 writes zeros instead.
-__device__ __forceinline__ void cp_async_16(uint32_t dst, const void* src, uint32_t src_bytes) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
-}
-// Waits until at most n of the calling thread's committed cp.async groups are still in flight (n <= 3).
-__device__ __forceinline__ void cp_async_wait_groups(int n) {
-  if (n <= 0) asm volatile("cp.async.wait_group 0;" ::: "memory");
-  else if (n == 1) asm volatile("cp.async.wait_group 1;" ::: "memory");
-  else if (n == 2) asm volatile("cp.async.wait_group 2;" ::: "memory");
-  else asm volatile("cp.async.wait_group 3;" ::: "memory");
 }
 
 __device__ __forceinline__ uint4 lds128(uint32_t addr) {
