@@ -346,47 +346,56 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
       item = __shfl_sync(0xffffffffu, item, 0);
       ok = ok && wait_table();
       const int n_first = ctl->n_first, n_items = n_first + (fused ? ctl->n_tiles * m_tiles2 : 0);
+      int steal_c0 = 0;          // guesses to take over: looked through so far, and those of the last 32 that are ours
+      uint32_t steal_mask = 0;
       while (ok) {
-        int g, nt, m;
-        bool down = KIND == 2;
+        int g, nt, m, next = item;
+        bool down = KIND == 2, whole = false;
         if (item >= n_items) {
           publish(kItemNone, 0);
           break;
         }
         if (item >= n_first && !guesses_claimed) {
           // before the CTA's first down item: every guess that turned out right must have a running CTA
-          if (!(ok = warp_wait(smem_u32(&ctl->looked), 0u, abort_flag, p.status))) break;
-          const bool open = *reinterpret_cast<volatile int*>(&ctl->guesses_open) != 0;
-          for (int c0 = 0; ok && open && c0 < n_spec; c0 += 32) {
-            const int c = c0 + lane;
-            const bool needed = c < n_spec && ctl->count[grp.expert[c / m_tiles1]] > 0;
-            uint32_t mine = __ballot_sync(0xffffffffu, needed && atomicExch(p.claims + c, 1u) == 0u);
-            for (; ok && mine != 0u; mine &= mine - 1u) {
-              const int it = c0 + __ffs((int)mine) - 1, ig = it / m_tiles1, im = it - ig * m_tiles1;
-              ok = publish(pack_item(ig, 0, 1, 0), im) && load_item(0, k_blocks1, false, im, grp.slot[ig]);
-            }
+          if (!warp_wait(smem_u32(&ctl->looked), 0u, abort_flag, p.status)) {
+            ok = false;
+            break;
           }
-          guesses_claimed = true;
-          if (!ok) break;
+          if (*reinterpret_cast<volatile int*>(&ctl->guesses_open) != 0)
+            for (; steal_mask == 0u && steal_c0 < n_spec; steal_c0 += 32) {
+              const int c = steal_c0 + lane;
+              const bool needed = c < n_spec && ctl->count[grp.expert[c / m_tiles1]] > 0;
+              steal_mask = __ballot_sync(0xffffffffu, needed && atomicExch(p.claims + c, 1u) == 0u);
+            }
+          guesses_claimed = steal_mask == 0u;
         }
-        if (item < n_first) {
-          while (ctl->item_prefix[g1 + 1] <= item) ++g1;
-          g = g1;
-          int in = item - ctl->item_prefix[g];
-          if (guess && g < p.n_guess) in += min(max((int)gridDim.x - g * m_tiles1, 0), m_tiles1);
-          nt = in / m_tiles1;
-          m = in - nt * m_tiles1;
+        if (fused && !guesses_claimed && steal_mask != 0u) {
+          const int c = steal_c0 - 32 + __ffs((int)steal_mask) - 1;
+          steal_mask &= steal_mask - 1u;
+          g = c / m_tiles1;
+          m = c - g * m_tiles1;
+          nt = 0;
+          whole = true;
         } else {
-          const int q = (item - n_first) / m_tiles2;
-          m = item - n_first - q * m_tiles2;
-          while (ctl->tile_prefix[g2 + 1] <= q) ++g2;
-          g = g2;
-          nt = q - ctl->tile_prefix[g];
-          down = true;
+          if (item < n_first) {
+            while (ctl->item_prefix[g1 + 1] <= item) ++g1;
+            g = g1;
+            int in = item - ctl->item_prefix[g];
+            if (guess && g < p.n_guess) in += min(max((int)gridDim.x - g * m_tiles1, 0), m_tiles1);
+            nt = in / m_tiles1;
+            m = in - nt * m_tiles1;
+          } else {
+            const int q = (item - n_first) / m_tiles2;
+            m = item - n_first - q * m_tiles2;
+            while (ctl->tile_prefix[g2 + 1] <= q) ++g2;
+            g = g2;
+            nt = q - ctl->tile_prefix[g];
+            down = true;
+          }
+          whole = dense && !down;
+          if (lane == 0) next = (int)atomicAdd(p.work_counter, 1u) + counter_base;  // (in flight under this item's loads)
         }
-        int next = 0;
-        if (lane == 0) next = (int)atomicAdd(p.work_counter, 1u) + counter_base;  // (in flight under this item's loads)
-        ok = publish(pack_item(g, down, dense && !down, nt), m) &&
+        ok = publish(pack_item(g, down, whole, nt), m) &&
              load_item(0, down ? k_blocks2 : k_blocks1, down, m, grp.slot[g]);
         item = __shfl_sync(0xffffffffu, next, 0);
       }
@@ -550,6 +559,7 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
         *reinterpret_cast<volatile int*>(&ctl->guess_lost) = lost ? 1 : 0;
         mbar_arrive(smem_u32(&ctl->claimed));
       }
+      __nanosleep(800);  // (looks that find the others' claims on their way cost 0.2 us per layer)
       const unsigned long long t0 = globaltimer();
       bool open = true, late = false;
       while (open && !late) {
