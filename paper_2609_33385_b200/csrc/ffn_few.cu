@@ -34,6 +34,10 @@
 // roles: one warp loads weights, one loads token rows (each TMA copy is 120 cycles of its thread; with both on one
 // thread that thread was the limit: 8 layers of 1 token 282 us against 261 when they were parted; 8 layers of 16 similar tokens 421
 // against 384), one issues MMAs, and the epilogue's warps build the work table while the first item already runs.
+// A stage's token rows are one copy whatever their number (a tensor map per size of the tile, k-blocks as its slowest
+// dimension), and those of a guess are requested as soon as the gate is through, before it is known whether the guess was
+// right: 8 layers of 1 token 241.2 -> 237.4 us, of 16 similar tokens 368.3 -> 365.6, 16 layers of 32 from fp8 stores
+// 1235 -> 1226, 8 layers of 250 from fp8 stores 789 -> 781.
 //
 // Token rows (FfnRows): dense steps (at most 32 tokens) multiply EVERY expert with all rows of the step,
 // stored once, in token order - the tile costs what a gathered one would (N is 16 or 32 either way) and
@@ -106,15 +110,15 @@ constexpr int kItemNone = -1, kItemAbort = -2, kItemDrop = -3;
 // whole: the item multiplies with n_box rows (dense gate/up items, items loaded on a guess), not the fewest that do
 __device__ __forceinline__ int pack_item(int g, int down, int whole, int nt) { return g | down << 9 | whole << 10 | nt << 11; }
 
-// Token rows of an item: 16, 32, 48, 64, 96 or 128, loaded in boxes of 64, 32 and 16 rows (largest first; a box of
-// fp8 terms holds its rows' first terms, then their second ones).
+// Token rows of an item: 16, 32, 48, 64, 96 or 128, and the tensor map whose box is that high.
 __host__ __device__ constexpr int few_size(int rows) { return rows <= 64 ? (rows + 15) & ~15 : (rows + 31) & ~31; }
+__host__ __device__ constexpr int few_map(int size) { return size <= 64 ? size / 16 - 1 : size / 32 + 1; }
 
 struct FewArgs {
   CUtensorMap tm_w1;    // gate/up weights, 5-D (see ffn_few_setup)
   CUtensorMap tm_w2;    // down-projection weights
-  CUtensorMap tm_x[3];  // token rows, boxes of 16, 32 and 64 (fp8: of their terms)
-  CUtensorMap tm_h[3];  // intermediate rows
+  CUtensorMap tm_x[kFewSizes];  // token rows, a box per size (fp8: of their terms)
+  CUtensorMap tm_h[kFewSizes];  // intermediate rows
   FfnGroup grp;
   FfnRows rows;
   uint16_t* hbuf;
@@ -185,8 +189,10 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
   constexpr int kK = FP8 ? 128 : 64;  // k-values of a k-block
   const bool dense = p.rows.dense != 0;
   constexpr uint32_t kRowBytes = FP8 ? 256u : 128u;  // of a token row in a k-block (fp8: two terms)
-  const uint32_t atom_bytes = kFewWTile + (uint32_t)n_box * kRowBytes;
-  const uint32_t stage_bytes = (uint32_t)p.k_atoms * atom_bytes;
+  // a stage: the weight tiles of its k-blocks, then their token rows (k-block by k-block; fp8: the rows' first terms
+  // before the second ones)
+  const uint32_t stage_tokens = (uint32_t)p.k_atoms * kFewWTile;
+  const uint32_t stage_bytes = stage_tokens + (uint32_t)(p.k_atoms * n_box) * kRowBytes;
   const int k_blocks1 = H / (kK * p.k_atoms), k_blocks2 = I / (kK * p.k_atoms);  // stages per item
   const int m_tiles1 = KIND == 2 ? H / 128 : I / 64;  // weight tiles of the first-phase (or only) items
   const int m_tiles2 = H / 128;
@@ -222,7 +228,7 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
     uint32_t dst = tiles_base + (uint32_t)st * stage_bytes;
     mbar_expect_tx(bar, (uint32_t)p.k_atoms * kFewWTile);
     int k0 = kb * p.k_atoms * kK;
-    for (int a = 0; a < p.k_atoms; ++a, k0 += kK, dst += atom_bytes) {
+    for (int a = 0; a < p.k_atoms; ++a, k0 += kK, dst += kFewWTile) {
       if (down) tma_load_3d_hint(&p.tm_w2, dst, bar, k0, m * 128, slot, policy);
       else few_load_w1(&p.tm_w1, dst, bar, k0, m, slot, policy);
     }
@@ -262,6 +268,11 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
           few_prefetch_w1(&p.tm_w1, a * kK, spec_m, grp.slot[spec_g], policy);
     }
     __syncwarp();
+  }
+  if (warp == kFewTokenWarp) {  // the maps of the loads to come (a guess's own map goes with its loads)
+    const int size = few_map(n_box);
+    const CUtensorMap* const map = lane == 0 ? &p.tm_w2 : lane == 1 ? p.tm_x + size : lane == 2 ? p.tm_h + size : p.tm_h;
+    if (lane < 4) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
   }
   if (warp == kFewMmaWarp) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl->tmem_base)),
@@ -410,40 +421,40 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
     int stage = 0, ready_g = -1;
     uint32_t phase = 0;
     bool ok = true;
-    auto load_tokens = [&](int st, int kb, const CUtensorMap* maps, int row0, int n) {  // one elected lane
+    auto load_tokens = [&](int st, int kb, const CUtensorMap* map, int row0, int n) {  // one elected lane
       const uint32_t bar = full0 + (uint32_t)st * 8u;
-      uint32_t dst0 = tiles_base + (uint32_t)st * stage_bytes + kFewWTile;
+      const uint32_t dst = tiles_base + (uint32_t)st * stage_bytes + stage_tokens;
       mbar_expect_tx(bar, (uint32_t)(p.k_atoms * n) * kRowBytes);
-      int k0 = kb * p.k_atoms * kK;
-      for (int a = 0; a < p.k_atoms; ++a, k0 += kK, dst0 += atom_bytes) {
-        uint32_t dst = dst0;
-        for (int r = 0; r < n;) {
-          const int box = n - r >= 64 ? 2 : n - r >= 32 ? 1 : 0;
-          if (FP8) tma_load_3d(maps + box, dst, bar, k0, row0 + r, 0);  // (both terms in one box)
-          else tma_load_2d(maps + box, dst, bar, k0, row0 + r);
-          r += 16 << box;
-          dst += (uint32_t)(16 << box) * kRowBytes;
-        }
-      }
+      if (FP8) tma_load_4d(map, dst, bar, 0, row0, 0, kb * p.k_atoms);
+      else tma_load_3d(map, dst, bar, 0, row0, kb * p.k_atoms);
     };
     griddep_wait();
+    // A guess: the rows that its expert would have are requested at once, before it is known whether there are any (if not,
+    // the stages are completed all the same and released unread).
+    const int guess_row0 = spec && !dense ? grp.expert[spec_g] * p.rows.cap : 0;
+    if (spec) {
+      if (elect_one())
+        for (int i = 0; i < pre1; ++i) load_tokens(i, i, p.tm_x + few_map(n_box), guess_row0, n_box);
+      __syncwarp();
+      stage = pre1 == p.n_stages ? 0 : pre1;
+      phase = pre1 == p.n_stages ? 1u : 0u;
+    }
     for (int seq = 0; ok; ++seq) {
       const int slot = seq % kFewRing;
       if (!warp_wait(smem_u32(&ctl->item_full[slot]), (uint32_t)(seq / kFewRing) & 1u, abort_flag, p.status)) break;
       const int code = __shfl_sync(0xffffffffu, *reinterpret_cast<volatile int*>(&ctl->item_ring[slot]), 0);
       if (lane == 0) mbar_arrive(smem_u32(&ctl->item_empty[slot]));
       if (code == kItemNone) break;
-      int k_blocks = k_blocks1, n = n_box, row0 = 0;
-      const bool drop = code == kItemDrop, down = !drop && (code >> 9) & 1;
-      const bool loaded = seq == 0 && spec;  // (a guess: its weights are there or on their way)
-      if (drop) {  // a wrong guess: its stages are completed all the same (with any rows) and released unread
-        k_blocks = pre1;
-      } else {
+      if (code == kItemDrop) continue;
+      int k_blocks = k_blocks1, n = n_box, row0 = guess_row0, kb = pre1;
+      const bool down = (code >> 9) & 1;
+      if (seq != 0 || !spec) {
         const int g = code & 511, nt = code >> 11, e = grp.expert[g];
-        if (!(loaded && (dense || p.rows.offsets == nullptr)) && !(ok = wait_table())) break;
+        if (!(ok = wait_table())) break;
         n = size_of(code);
         if (down) k_blocks = k_blocks2;
-        row0 = dense && !down ? 0 : (loaded ? e * p.rows.cap : first_row(e)) + nt * n_box;
+        row0 = dense && !down ? 0 : first_row(e) + nt * n_box;
+        kb = 0;
         if (fused && down && g != ready_g) {
           // the intermediate rows of every token tile of this expert (fp8: their terms) must be in memory
           ok = FP8 ? wait_count(p.split_done + g, (uint32_t)ctl->count[e], 0u) : wait_count(p.done + g, done_target(g), 0u);
@@ -455,13 +466,13 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
           asm volatile("fence.proxy.async.global;" ::: "memory");
         }
       }
-      const CUtensorMap* const maps = down ? p.tm_h : p.tm_x;
-      for (int kb = 0; kb < k_blocks; ++kb) {
+      const CUtensorMap* const map = (down ? p.tm_h : p.tm_x) + few_map(n);
+      for (; kb < k_blocks; ++kb) {
         if (!warp_wait(empty0 + (uint32_t)stage * 8u, phase ^ 1u, abort_flag, p.status)) {
           ok = false;
           break;
         }
-        if (elect_one()) load_tokens(stage, kb, maps, row0, n);
+        if (elect_one()) load_tokens(stage, kb, map, row0, n);
         __syncwarp();
         if (++stage == p.n_stages) {
           stage = 0;
@@ -482,8 +493,8 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
     int stage = 0, local = 0;
     uint32_t phase = 0;
     bool ok = true;
-    const uint32_t ring_step = atom_bytes >> 4, stage_step = stage_bytes >> 4;  // descriptor addresses count 16 bytes
-    const uint64_t a_desc0 = make_smem_desc(tiles_base), b_desc0 = make_smem_desc(tiles_base + kFewWTile);
+    const uint32_t stage_step = stage_bytes >> 4;  // descriptor addresses count 16 bytes
+    const uint64_t a_desc0 = make_smem_desc(tiles_base), b_desc0 = make_smem_desc(tiles_base + stage_tokens);
     for (int seq = 0; ok; ++seq) {
       const int slot = seq % kFewRing;
       if (!warp_wait(smem_u32(&ctl->item_full[slot]), (uint32_t)(seq / kFewRing) & 1u, abort_flag, p.status)) break;
@@ -512,6 +523,7 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
       const int n = size_of(code);
       const uint32_t idesc = __shfl_sync(0xffffffffu, FP8 ? make_idesc_e4m3(2 * n) : make_idesc(n), 0);
       const uint32_t d0 = __shfl_sync(0xffffffffu, tmem_base + (uint32_t)(acc * acc_cols), 0);
+      const uint32_t b_step = __shfl_sync(0xffffffffu, ((uint32_t)n * kRowBytes) >> 4, 0);  // to a stage's second k-block
       for (int kb = 0; kb < k_blocks; ++kb) {
         if (!warp_wait(full0 + (uint32_t)stage * 8u, phase, abort_flag, p.status)) {
           ok = false;
@@ -528,7 +540,7 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
           for (int k = 1; k < 4; ++k) tc_mma_desc<FP8, true>(d0, a0 + k * 2, b0 + k * 2, idesc);
           if (p.k_atoms == 2) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) tc_mma_desc<FP8, true>(d0, a0 + ring_step + k * 2, b0 + ring_step + k * 2, idesc);
+            for (int k = 0; k < 4; ++k) tc_mma_desc<FP8, true>(d0, a0 + (kFewWTile >> 4) + k * 2, b0 + b_step + k * 2, idesc);
           }
           tc_commit(empty0 + (uint32_t)stage * 8u);
           if (kb + 1 == k_blocks) tc_commit(smem_u32(&ctl->tmem_full[acc]));
@@ -750,10 +762,7 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
         const bool last = c + step >= n;
         uint32_t ra[16];
         if (c < n) {
-          // (fp8: the columns come box by box, first terms before second ones)
-          const int box = c < (n & ~63) ? 64 : c < (n & ~31) ? 32 : 16;
-          const int col0 = FP8 ? 2 * (c & ~(box - 1)) + (c & (box - 1)) : c;
-          const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * acc_cols + col0);
+          const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * acc_cols + c);
           tmem_ld16(t_row, ra);
           if (!first || !ahead) {
             columns(c, row, dst, inv);
@@ -761,7 +770,7 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
           }
           if (FP8) {  // D = (D1 + D2 / 16) / row scale of the token
             uint32_t rt[16];
-            tmem_ld16(t_row + (uint32_t)box, rt);
+            tmem_ld16(t_row + (uint32_t)n, rt);  // (the second terms' columns lie behind the first ones')
             tmem_ld_wait();
 #pragma unroll
             for (int j = 0; j < 16; ++j)
@@ -905,17 +914,18 @@ int ffn_few_setup(FfnTcMaps* maps, const uint8_t* pool, size_t slot_bytes, int n
     const cuuint32_t box[3] = {k_box, 128, 1};
     if (!encode_tensor_map(&maps->few_w2, 3, pool + (size_t)2 * I * H * esz, dims, strides, box, fp8)) return OLED_ERR_CUDA;
   }
-  for (int i = 0; i < 3; ++i) {  // token rows, intermediate rows (fp8: [term][row][k], a box takes both terms)
-    const cuuint32_t box[3] = {k_box, 16u << i, 2};
-    for (int op = 0; op < 2; ++op) {
-      const cuuint64_t width = (cuuint64_t)(op == 0 ? H : I);
-      const void* base = fp8 ? (const void*)(op == 0 ? split->terms_in : split->terms_mid) : (const void*)(op == 0 ? xp : hbuf);
-      const cuuint64_t dims[3] = {width, (cuuint64_t)rows, 2};
-      const cuuint64_t strides[2] = {width * esz, width * esz * (cuuint64_t)rows};
-      if (!encode_tensor_map(op == 0 ? &maps->few_x[i] : &maps->few_h[i], fp8 ? 3 : 2, base, dims, strides, box, fp8))
-        return OLED_ERR_CUDA;
-    }
-  }
+  for (int atoms = 1; atoms <= 2; ++atoms)  // token rows, intermediate rows: k-blocks as the slowest dimension, so that a
+    for (int size : {16, 32, 48, 64, 96, 128})  // stage's rows are one copy (fp8: [k-block][term][row][k])
+      for (int op = 0; op < 2; ++op) {
+        const cuuint64_t width = (cuuint64_t)(op == 0 ? H : I);
+        const void* base = fp8 ? (const void*)(op == 0 ? split->terms_in : split->terms_mid) : (const void*)(op == 0 ? xp : hbuf);
+        const cuuint64_t k_blocks = width / k_box, term_stride = width * (cuuint64_t)rows;
+        const cuuint64_t dims[4] = {k_box, (cuuint64_t)rows, fp8 ? 2 : k_blocks, k_blocks};
+        const cuuint64_t strides[3] = {width * esz, fp8 ? term_stride : 128, 128};
+        const cuuint32_t box[4] = {k_box, (cuuint32_t)size, fp8 ? 2u : (cuuint32_t)atoms, (cuuint32_t)atoms};
+        CUtensorMap* const m = (op == 0 ? maps->few_x : maps->few_h)[atoms - 1] + few_map(size);
+        if (!encode_tensor_map(m, fp8 ? 4 : 3, base, dims, strides, box, fp8)) return OLED_ERR_CUDA;
+      }
   maps->few = true;
   static const bool attr_ok = [] {
     return cudaFuncSetAttribute(ffn_few_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFewSmemMax) == cudaSuccess &&
@@ -938,14 +948,14 @@ int launch_ffn_few(cudaStream_t st, const FfnTcMaps& maps, const FfnGroup& group
   FewArgs a;
   a.tm_w1 = maps.few_w1;
   a.tm_w2 = maps.few_w2;
-  for (int i = 0; i < 3; ++i) {
-    a.tm_x[i] = maps.few_x[i];
-    a.tm_h[i] = maps.few_h[i];
-  }
   a.grp = group;
   const FfnGroup& grp = a.grp;
   a.grp.n_box = few_size(std::min(max_count, kFewMaxRows));
   const FewRings r = few_rings(grp.n_box, fp8, H, I);
+  for (int i = 0; i < kFewSizes; ++i) {
+    a.tm_x[i] = maps.few_x[r.k_atoms - 1][i];
+    a.tm_h[i] = maps.few_h[r.k_atoms - 1][i];
+  }
   a.y_bf16 = y_bf16;
   a.rows = rows;
   a.hbuf = hbuf;

@@ -243,9 +243,11 @@ void launch_ffn_simple(cudaStream_t st, const FfnGroup& grp, const uint8_t* pool
                        int I);
 
 // ---- ffn_tc.cu (tcgen05 / TMEM / TMA) ------------------------------------------------------
+constexpr int kFewSizes = 6;  // token tiles of ffn_few.cu: 16, 32, 48, 64, 96 or 128 rows
 struct FfnTcMaps {
-  CUtensorMap few_w1, few_w2, few_x[3], few_h[3];  // the maps of ffn_few.cu (fp8 stores: over codes and token terms)
-  bool few = false;                                // ... exist
+  // the maps of ffn_few.cu (fp8 stores: over codes and token terms); token rows by k-blocks of a stage and size of the tile
+  CUtensorMap few_w1, few_w2, few_x[2][kFewSizes], few_h[2][kFewSizes];
+  bool few = false;  // ... exist
   CUtensorMap w13;       // [slots][2I][H] bf16, box {64,128,1}
   CUtensorMap w13_half;  // fp8 stores, widening form: the same, box {64,64,1}
   CUtensorMap w2;        // [slots][H][I]  bf16, box {64,128,1}
