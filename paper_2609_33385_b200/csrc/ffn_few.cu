@@ -260,12 +260,6 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
     __syncwarp();
     if (spec && elect_one()) {
       for (int i = 0; i < pre1; ++i) load_weights(i, i, false, spec_m, grp.slot[spec_g]);
-      // the rest of the item into L2, for steps whose gate kernel is short (8 layers of 16 similar tokens 362 -> 356 us; with
-      // 250 tokens fp8 it took bandwidth from the gate's own loads, 775 -> 789, with 100 tokens still 523 -> 517; where
-      // between those two the line lies was not measured, it is drawn at one gate CTA per SM)
-      if (p.rows.cap <= 148)
-        for (int a = pre1 * p.k_atoms; a < k_blocks1 * p.k_atoms; ++a)
-          few_prefetch_w1(&p.tm_w1, a * kK, spec_m, grp.slot[spec_g], policy);
     }
     __syncwarp();
   }
@@ -311,6 +305,20 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
     int stage = 0, g1 = 0, g2 = 0, seq = 0;
     uint32_t phase = 0;
     bool ok = true;
+    // The rest of the guessed item into L2, for steps whose gate kernel is short (8 layers of 16 similar tokens 362 -> 356 us;
+    // with 250 tokens fp8 it took bandwidth from the gate's own loads, 775 -> 789, with 100 tokens still 523 -> 517; where
+    // between those two the line lies was not measured, it is drawn at one gate CTA per SM).  Paced to a little more than
+    // what HBM delivers (148 CTAs: a k-block each in 0.37 us): all at once they were a queue that the gate's own loads
+    // stood in (pause 0 / 150 / 300 ns: 8 layers of 1 token 240.0 / 235.3 / 232.8 us, of 16 similar tokens 367.2 / 363.2 /
+    // 367.7; 16 layers of 32 from fp8 stores 1231 / 1230 / 1243).  Nothing beyond the item: a line that waits in L2 is read there
+    // twice (64 MB of the following items during the gate 1164 -> 1181 us; the CTA's next item all along the stream -> 1415).
+    if (spec && p.rows.cap <= 148) {
+      for (int a = pre1 * p.k_atoms; a < k_blocks1 * p.k_atoms; ++a) {
+        if (elect_one()) few_prefetch_w1(&p.tm_w1, a * kK, spec_m, grp.slot[spec_g], policy);
+        __nanosleep(150);
+      }
+      __syncwarp();
+    }
     if (!early) griddep_wait();
     if (lane == 0) timeline_start(p.timeline, p.timeline_slot);
     const bool spec_ok = spec && __ldcg(p.rows.counts + grp.expert[spec_g]) > 0;
