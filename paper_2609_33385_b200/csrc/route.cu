@@ -239,6 +239,14 @@ __device__ __forceinline__ void sort_assignments(const int32_t* ids, int n, int 
   }
 }
 
+// The router matrix ahead of the input (staged forms): its first `chunks` * 256 columns go to shared memory, and up to
+// two further chunks of the first pass to registers (one token per CTA: the combine of two has none left).
+// (Routing without a step fetches nothing ahead: the matrix is the caller's, may still be in the making, and with the copies behind
+// the dependency wait a call of 32 tokens took 12.9 us instead of 10.)
+struct RouterAhead {
+  int on = 0;      // the matrix is older than everything that may still run on the stream
+  int chunks = 0;
+};
 // TT tokens per CTA, WARPS warps; each warp owns kEPerWarp experts per pass and all TT tokens.  Small
 // blocks use TT = 1 with 16 warps (one pass covers 64 experts) and keep several 256-wide
 // chunks of loads in flight; the chain order of every logit is the same in all variants.
@@ -258,7 +266,8 @@ route_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ wr,
              int K, float* __restrict__ logits_out, int32_t* __restrict__ ids,
              float* __restrict__ gate, int32_t* __restrict__ counts,
              unsigned long long* __restrict__ scores, CombinePrev prev, StepTimeline* timeline,
-             const __grid_constant__ ScatterRows scatter, const __grid_constant__ RouteFinish finish) {
+             const __grid_constant__ ScatterRows scatter, const __grid_constant__ RouteFinish finish,
+             const __grid_constant__ RouterAhead ahead) {
   extern __shared__ __align__(16) uint8_t s_dyn[];
   float* s_logits = reinterpret_cast<float*>(s_dyn);                       // [TT][E]
   constexpr bool staged = TT <= 4;
@@ -279,27 +288,48 @@ route_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ wr,
   if (threadIdx.x == 0) timeline_entry(timeline, 0);
   constexpr int kRouteWarps = WARPS;
   const int my_tokens = min(TT, T - t0);
-  if (staged && gridDim.x <= 148) {
-    // Small steps: the router weights do not depend on the predecessor (the previous layer's
-    // expert FFN), but the expert weights streamed since their last use have pushed them out of
-    // L2 - so they are called back in while this kernel still waits for its input.
-    for (int eb = warp * kEPerWarp; eb < E; eb += kRouteWarps * kEPerWarp)
+  // The router matrix does not depend on the predecessor (the previous layer's expert FFN, which a CTA of this kernel
+  // usually waits 4 to 8 us for): what fits is fetched now.  What bounds the logits otherwise is one SM's share of L2, 64
+  // bytes a cycle: 64 experts x 2048 took 3.4-3.6 us after the input was there, now 2.6 (one pass' worth from chip: 8 layers
+  // of 1 token 236.3 -> 230.0 us, of 16 similar tokens 361.4 -> 355.1, 16 layers of 32 1994 -> 1985).
+  // [E][chunks * 256], a row's 512 bytes of a chunk are read by a warp at a time
+  uint16_t* const s_w = reinterpret_cast<uint16_t*>(s_key + (size_t)TT * Ep);
+  const int w_cols = staged ? ahead.chunks * 256 : 0, n_chunks = H / 256;
+  constexpr int kTail = TT == 1 ? 2 : 0;
+  const bool tail_ahead = ahead.on && n_chunks - ahead.chunks <= kTail;
+  uint4 w_tail[kTail == 0 ? 1 : kTail][kEPerWarp];
+  if (staged && ahead.on) {
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(s_w);
+    const int pieces = w_cols / 8;  // of 16 bytes, per row
+    for (int e = warp; e < E; e += kRouteWarps)
+      for (int c = lane; c < pieces; c += 32)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + (uint32_t)(e * pieces + c) * 16u),
+                     "l"(wr + (size_t)e * H + c * 8)
+                     : "memory");
+    if (tail_ahead) {
 #pragma unroll
-      for (int b = 0; b < kEPerWarp; ++b) {
-        const int e = min(eb + b, E - 1);
-        for (int off = lane * 64; off < H; off += 32 * 64)  // 128-byte lines of the row
-          asm volatile("prefetch.global.L2 [%0];" ::"l"(wr + (size_t)e * H + off));
-      }
+      for (int i = 0; i < kTail; ++i)
+#pragma unroll
+        for (int b = 0; b < kEPerWarp; ++b)
+          if (w_cols + i * 256 < H)
+            w_tail[i][b] = *reinterpret_cast<const uint4*>(wr + (size_t)min(warp * kEPerWarp + b, E - 1) * H + w_cols + i * 256 + lane * 8);
+    }
+  }
+  if (staged && gridDim.x <= 148 && !tail_ahead) {
+    // the rest into L2, out of which the expert weights streamed since its last use may have pushed it
+    for (int e = warp; e < E; e += kRouteWarps)
+      for (int c = w_cols + lane * 64; c < H; c += 32 * 64)  // 128-byte lines of the row
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(wr + (size_t)e * H + c));
   }
   uint16_t* const dense_rows = staged && scatter.cap > 0 && scatter.dense && scatter.split.amax_in == nullptr ? scatter.xp : nullptr;
   griddep_wait();
   if (threadIdx.x == 0) timeline_start(timeline, 0);
   if (staged) {
     if (prev.y != nullptr) {
+      combine_rows<TT == 1 ? 1 : 2>(prev, t0, my_tokens, H, s_x, dense_rows);
       // CTA 0 also clears the control block the previous step used (its kernels have completed)
       if (blockIdx.x == 0 && prev.zero_words != nullptr)
         for (int i = threadIdx.x; i < prev.n_zero_words; i += blockDim.x) prev.zero_words[i] = 0u;
-      combine_rows<TT == 1 ? 1 : 2>(prev, t0, my_tokens, H, s_x, dense_rows);
     } else {
       for (int c = threadIdx.x; c < my_tokens * (H / 8); c += blockDim.x) {
         const uint4 v = reinterpret_cast<const uint4*>(x + (size_t)t0 * H)[c];
@@ -310,6 +340,7 @@ route_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ wr,
     if ((int)threadIdx.x < my_tokens) s_conf[threadIdx.x] = conf[t0 + threadIdx.x];
     for (int i = threadIdx.x; i < TT * (Ep - E); i += blockDim.x) s_key[(i / (Ep - E)) * Ep + E + i % (Ep - E)] = 0u;
     if (threadIdx.x < kST) s_amax[threadIdx.x] = 0u;
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     if (scatter.split.amax_in != nullptr)
       for (int a = 0; a < my_tokens; ++a) {
@@ -334,31 +365,50 @@ route_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ wr,
     float bias_e[kEPerWarp];  // (requested ahead of the loop, not after it)
 #pragma unroll
     for (int b = 0; b < kEPerWarp; ++b) bias_e[b] = bias != nullptr ? bias[min(eb + b, E - 1)] : 0.0f;
-#pragma unroll UNROLL
-    for (int hc = 0; hc < H; hc += 256) {
+    // one chunk of 256 columns: weights ww, the tokens' rows from shared memory (or global memory)
+    auto chunk = [&](int hc, const uint4 (&ww)[kEPerWarp]) {
       const int h = hc + lane * 8;
-      uint32_t xw[TT][4], ww[kEPerWarp][4];
+      uint4 xw[TT];
 #pragma unroll
-      for (int a = 0; a < TT; ++a) {
-        const int t = min(t0 + a, T - 1);
+      for (int a = 0; a < TT; ++a)
         // (staged rows beyond the step's last token hold stale shared memory: their logits are never used)
-        const uint4 v = staged ? *reinterpret_cast<const uint4*>(s_x + (size_t)a * H + h)
-                               : *reinterpret_cast<const uint4*>(x + (size_t)t * H + h);
-        xw[a][0] = v.x; xw[a][1] = v.y; xw[a][2] = v.z; xw[a][3] = v.w;
-      }
-#pragma unroll
-      for (int b = 0; b < kEPerWarp; ++b) {
-        const int e = min(eb + b, E - 1);
-        const uint4 v = *reinterpret_cast<const uint4*>(wr + (size_t)e * H + h);
-        ww[b][0] = v.x; ww[b][1] = v.y; ww[b][2] = v.z; ww[b][3] = v.w;
-      }
+        xw[a] = staged ? *reinterpret_cast<const uint4*>(s_x + (size_t)a * H + h)
+                       : *reinterpret_cast<const uint4*>(x + (size_t)min(t0 + a, T - 1) * H + h);
       // elements in ascending h: word 0 low half, word 0 high half, word 1 low half, ...
-#pragma unroll
-      for (int wi = 0; wi < 4; ++wi)
+      auto word = [&](auto get) {
 #pragma unroll
         for (int a = 0; a < TT; ++a)
 #pragma unroll
-          for (int b = 0; b < kEPerWarp; ++b) fma_bf16_pair(acc[a][b], xw[a][wi], ww[b][wi]);
+          for (int b = 0; b < kEPerWarp; ++b) fma_bf16_pair(acc[a][b], get(xw[a]), get(ww[b]));
+      };
+      word([](const uint4& v) { return v.x; });
+      word([](const uint4& v) { return v.y; });
+      word([](const uint4& v) { return v.z; });
+      word([](const uint4& v) { return v.w; });
+    };
+    int hc = 0;
+    if (staged) {
+#pragma unroll 2
+      for (; hc < w_cols; hc += 256) {
+        uint4 ww[kEPerWarp];
+#pragma unroll
+        for (int b = 0; b < kEPerWarp; ++b)
+          ww[b] = *reinterpret_cast<const uint4*>(s_w + (size_t)min(eb + b, E - 1) * w_cols + hc + lane * 8);
+        chunk(hc, ww);
+      }
+      if (tail_ahead && eb == warp * kEPerWarp) {
+#pragma unroll
+        for (int i = 0; i < kTail; ++i, hc += 256)
+          if (hc < H) chunk(hc, w_tail[i]);
+      }
+    }
+#pragma unroll UNROLL
+    for (; hc < H; hc += 256) {
+      uint4 ww[kEPerWarp];
+#pragma unroll
+      for (int b = 0; b < kEPerWarp; ++b)
+        ww[b] = *reinterpret_cast<const uint4*>(wr + (size_t)min(eb + b, E - 1) * H + hc + lane * 8);
+      chunk(hc, ww);
     }
 #pragma unroll
     for (int a = 0; a < TT; ++a)
@@ -382,13 +432,20 @@ route_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ wr,
     // top-k by rank: expert e is selected iff fewer than K experts precede it in the order (logit descending,
     // index ascending), and its rank is the number that do.  `parts` neighbouring threads per (token, expert)
     // count a share of the experts each, four keys at a time.  (A warp per expert at a time took 1.4 us for
-    // one token and 64 experts, 6.5 us for two and 128; now 0.5 and 0.9.)
+    // one token and 64 experts, 6.5 us for two and 128; now 0.5 and 0.9.  Divisions by E had doubled that.)
     const int items = my_tokens * E;
-    int parts = 1;
-    while (parts < 32 && items * parts * 2 <= WARPS * 32) parts <<= 1;
+    int parts = 1, parts_log2 = 0;
+    for (; parts < 32 && items * parts * 2 <= WARPS * 32; parts <<= 1) ++parts_log2;
     const int part = threadIdx.x & (parts - 1);
-    for (int i0 = 0; i0 < items; i0 += WARPS * 32 / parts) {
-      const int i = i0 + (int)threadIdx.x / parts, a = min(i, items - 1) / E, e = min(i, items - 1) - a * E;
+    for (int i0 = 0; i0 < items; i0 += (WARPS * 32) >> parts_log2) {
+      const int i = i0 + ((int)threadIdx.x >> parts_log2);
+      int a = 0, e = min(i, items - 1);
+#pragma unroll
+      for (int j = 1; j < TT; ++j)
+        if (e >= E) {
+          e -= E;
+          ++a;
+        }
       const uint32_t ke = s_key[a * Ep + e];
       const uint4* row = reinterpret_cast<const uint4*>(s_key + a * Ep);
       int before = 0;
@@ -451,8 +508,9 @@ route_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ wr,
         }
         for (int j = 0; j < (scatter.dense ? 1 : K); ++j) {
           const size_t row = scatter.dense ? (size_t)(t0 + a) : (size_t)s_r[a * K + j];
-          reinterpret_cast<uint4*>(scatter.xp)[row * vec_per_row + c] = v;
-          if (scatter.split.amax_in != nullptr) {
+          if (scatter.split.amax_in == nullptr) {
+            reinterpret_cast<uint4*>(scatter.xp)[row * vec_per_row + c] = v;
+          } else {  // (the FFN reads the terms only: 8 layers of 250 tokens 748 -> 734 us without the copies)
             reinterpret_cast<uint2*>(scatter.split.terms_in)[row * vec_per_row + c] = t1;
             reinterpret_cast<uint2*>(scatter.split.terms_in)[((size_t)scatter.split.rows + row) * vec_per_row + c] = t2;
           }
@@ -880,12 +938,20 @@ constexpr int kStagedWarps = 16;
 static size_t staged_smem(int tt, int H, int E) {  // logits, rows, keys
   return ((((size_t)tt * E * sizeof(float)) + 15) & ~(size_t)15) + (size_t)tt * H * 2 + (size_t)tt * ((E + 3) & ~3) * 4;
 }
+constexpr size_t kStagedSmem = 224 * 1024;  // (of 227 KB; the rest holds the kernel's static arrays)
+// As many chunks of the router matrix as fit behind the rows.
+static RouterAhead router_ahead(int tt, int H, int E) {
+  RouterAhead r;
+  r.on = 1;
+  r.chunks = (int)std::min<size_t>(H / 256, (kStagedSmem - staged_smem(tt, H, E)) / ((size_t)E * 512));
+  return r;
+}
 static bool staged_attributes() {  // the staged rows: up to 4 x 16 K elements
   static const bool ok = [] {
     const bool done =
-        cudaFuncSetAttribute(route_kernel<1, kStagedWarps, 4, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024) == cudaSuccess &&
-        cudaFuncSetAttribute(route_kernel<2, kStagedWarps, 4, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024) == cudaSuccess &&
-        cudaFuncSetAttribute(route_kernel<4, kStagedWarps, 2, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024) == cudaSuccess;
+        cudaFuncSetAttribute(route_kernel<1, kStagedWarps, 4, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStagedSmem) == cudaSuccess &&
+        cudaFuncSetAttribute(route_kernel<2, kStagedWarps, 4, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStagedSmem) == cudaSuccess &&
+        cudaFuncSetAttribute(route_kernel<4, kStagedWarps, 2, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStagedSmem) == cudaSuccess;
     if (!done) cudaGetLastError();
     return done;
   }();
@@ -900,16 +966,14 @@ void launch_route(cudaStream_t st, const uint16_t* x, const uint16_t* w_router, 
   if (route_staged(T, K)) {
     constexpr int W = kStagedWarps;
     staged_attributes();
-    auto smem = [&](int tt) { return staged_smem(tt, H, E); };
-    if (T <= 148)
-      launch_pdl(route_kernel<1, W, 4, 4>, dim3(T), dim3(W * 32), smem(1), st, x, w_router, bias, conf, T, H, E, K,
-                 logits, ids, gate, counts, scores, prev, timeline, scatter, RouteFinish{});
-    else if (T <= 296)  // (four tokens per CTA measured slower at 256 tokens x 128 experts: 33 against 20 us)
-      launch_pdl(route_kernel<2, W, 4, 4>, dim3((T + 1) / 2), dim3(W * 32), smem(2), st, x, w_router, bias, conf, T, H,
-                 E, K, logits, ids, gate, counts, scores, prev, timeline, scatter, RouteFinish{});
-    else
-      launch_pdl(route_kernel<4, W, 2, 4>, dim3((T + 3) / 4), dim3(W * 32), smem(4), st, x, w_router, bias, conf, T, H,
-                 E, K, logits, ids, gate, counts, scores, prev, timeline, scatter, RouteFinish{});
+    auto go = [&](auto kernel, int tt) {
+      const RouterAhead ahead = router_ahead(tt, H, E);  // (a context's copy of the matrix: its writer has been waited for)
+      launch_pdl(kernel, dim3((T + tt - 1) / tt), dim3(W * 32), staged_smem(tt, H, E) + (size_t)ahead.chunks * E * 512, st, x, w_router,
+                 bias, conf, T, H, E, K, logits, ids, gate, counts, scores, prev, timeline, scatter, RouteFinish{}, ahead);
+    };
+    if (T <= 148) go(route_kernel<1, W, 4, 4>, 1);
+    else if (T <= 296) go(route_kernel<2, W, 4, 4>, 2);  // (four tokens per CTA measured slower at 256 tokens x 128 experts: 33 against 20 us)
+    else go(route_kernel<4, W, 2, 4>, 4);
   } else {
     // (re-tilings of the plain kernel - more tokens or experts per warp, more warps per CTA, deeper
     // unrolling - were all slower at 4096 tokens x 64 experts x 4096)
@@ -1014,17 +1078,12 @@ void launch_route_alone(cudaStream_t st, const uint16_t* x, const uint16_t* w_ro
                         int T, int H, int E, int K, int32_t* ids, float* gate, int32_t* counts, const RouteFinish& finish) {
   const size_t sort_bytes = (size_t)kStagedWarps * E * sizeof(int);
   if (T > 1) launch_pdl(clear_word_kernel, dim3(1), dim3(1), 0, st, finish.offsets + E);
-  if (T <= 148) {
-    const size_t smem = std::max(staged_smem(1, H, E), sort_bytes);
-    launch_pdl(route_kernel<1, kStagedWarps, 4, 4>, dim3(T), dim3(kStagedWarps * 32), smem, st, x, w_router, bias, conf, T, H, E,
-               K, (float*)nullptr, ids, gate, counts, (unsigned long long*)nullptr, CombinePrev{}, (StepTimeline*)nullptr,
-               ScatterRows{}, finish);
-  } else {
-    const size_t smem = std::max(staged_smem(2, H, E), sort_bytes);
-    launch_pdl(route_kernel<2, kStagedWarps, 4, 4>, dim3((T + 1) / 2), dim3(kStagedWarps * 32), smem, st, x, w_router, bias,
-               conf, T, H, E, K, (float*)nullptr, ids, gate, counts, (unsigned long long*)nullptr, CombinePrev{},
-               (StepTimeline*)nullptr, ScatterRows{}, finish);
-  }
+  auto go = [&](auto kernel, int tt) {
+    launch_pdl(kernel, dim3((T + tt - 1) / tt), dim3(kStagedWarps * 32), std::max(staged_smem(tt, H, E), sort_bytes), st, x, w_router, bias, conf, T, H, E, K, (float*)nullptr,
+               ids, gate, counts, (unsigned long long*)nullptr, CombinePrev{}, (StepTimeline*)nullptr, ScatterRows{}, finish, RouterAhead{});
+  };
+  if (T <= 148) go(route_kernel<1, kStagedWarps, 4, 4>, 1);
+  else go(route_kernel<2, kStagedWarps, 4, 4>, 2);
 }
 
 }  // namespace

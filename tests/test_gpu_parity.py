@@ -995,6 +995,42 @@ def test_guess_rows_requested_before_the_counts(n_experts, top_k, hidden, inter,
         run.close()
 
 
+@pytest.mark.parametrize("fp8", [False, True], ids=["bf16", "fp8"])
+@pytest.mark.parametrize("n_experts,top_k,hidden,counts", [(64, 8, 2048, (1, 33, 149)), (3, 2, 256, (1, 149)), (33, 4, 4096, (2, 148)),
+                                                           (8, 2, 16384, (1, 3)), (70, 8, 2048, (1, 150)), (512, 32, 1024, (1, 12)),
+                                                           (16, 2, 768, (5, 600))])
+def test_gate_with_the_router_matrix_fetched_ahead(n_experts, top_k, hidden, counts, fp8):
+    """Few-token gate: the router matrix wholly on chip (shared memory, or with the last one or two chunks in registers), partly
+    or not at all, one and several passes over the experts, one, two and four tokens per CTA; logits, ids, gate scores and order equal
+    the oracle's bit for bit, in a stack iteration (where the combine runs in the same kernel) the same as layer by layer."""
+    from oracle import moe_layer as oracle_moe
+    from paper_2609_33385_b200.runner import bits_to_dev, dev_to_bits
+    w = synth.tiny(n_layers=2, n_experts=n_experts, top_k=top_k, hidden=hidden, intermediate=128)
+    run = _runner(w, capacity=[n_experts] * 2, max_tokens=max(counts), fp8=fp8, distinct_layers=1)
+    try:
+        for n in counts:
+            h_bits, conf = synth.flat_tokens(w, n, 700)
+            x, c = bits_to_dev(h_bits, run.device), torch.from_numpy(conf).to(run.device)
+            out, nxt, both = (torch.empty((n, w.hidden), dtype=torch.bfloat16, device=run.device) for _ in range(3))
+            run.ctx.denoise_iteration(x.data_ptr(), c.data_ptr(), n, both.data_ptr())
+            run.ctx.synchronize()
+            for l in range(2):
+                run.step(l, x, c, out)
+                dbg = run.ctx.debug_last(l, n)
+                logits = oracle_moe.gate_logits(oracle_moe.bf16_to_f32(dev_to_bits(x)),
+                                                oracle_moe.bf16_to_f32(run.router_bits[l]), run.bias[l])
+                ids, gate = oracle_moe.topk_route(logits, top_k)
+                assert np.array_equal(run.ctx.debug_logits(l, n).view(np.uint32), logits.view(np.uint32))
+                assert np.array_equal(dbg["ids"], ids)
+                assert np.array_equal(dbg["gate"].view(np.uint32), gate.view(np.uint32))
+                assert np.array_equal(dbg["perm"], oracle_moe.permutation(ids, n_experts)[2])
+                run.ctx.residual_add(x.data_ptr(), out.data_ptr(), nxt.data_ptr(), x.numel())
+                x, nxt = nxt, torch.empty_like(nxt)
+            assert np.array_equal(dev_to_bits(x), dev_to_bits(both))
+    finally:
+        run.close()
+
+
 @pytest.mark.parametrize("n_experts,top_k,counts", [(16, 16, (297, 1030)), (65, 14, (300, 2072)), (512, 32, (298, 401))])
 def test_gate_sums_of_tokens_in_two_segments(n_experts, top_k, counts):
     """Many-token gate: a CTA's 8 to 14 tokens lie in one segment of the order or in two, segments are 20 tokens at the
