@@ -176,9 +176,8 @@ __device__ __forceinline__ void combine_rows(const CombinePrev& p, int t0, int n
   }
 }
 
-// What the allocation-free routing entry point adds to the gate kernel: the counts, offsets and the stable
-// permutation, made by the CTA that finishes last.  Which one that is the CTAs find out by counting in offsets[E], the
-// call's own output word: ZERO at the start (several CTAs; one CTA needs no count), overwritten by the sort.
+// What the allocation-free routing entry point adds to the gate kernel: the counts, offsets and the stable permutation, by
+// the gate kernel's CTA where there is one, else by a kernel of one CTA behind it (sort_kernel).
 struct RouteFinish {
   int32_t* offsets = nullptr;  // nullptr: a gate kernel of a step
   int32_t* perm = nullptr;
@@ -525,18 +524,9 @@ route_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ wr,
       route_token_tail(s_logits + a * E, t, lane, E, K, conf, ids, gate, counts, scores);
     }
   }
-  if (finish.offsets != nullptr) {
-    // routing without a step: the last CTA to get here sorts the assignments (the ids of the others are visible to it:
-    // every CTA's stores precede its count)
-    __shared__ int s_last;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      __threadfence();
-      s_last = gridDim.x == 1 || atomicAdd(finish.offsets + E, 1) == (int)gridDim.x - 1 ? 1 : 0;
-      __threadfence();
-    }
-    __syncthreads();
-    if (s_last) sort_assignments<WARPS>(ids, T * K, E, counts, finish.offsets, finish.perm, reinterpret_cast<int*>(s_dyn));
+  if (finish.offsets != nullptr && gridDim.x == 1) {
+    __syncthreads();  // (the ids are stored)
+    sort_assignments<WARPS>(ids, T * K, E, counts, finish.offsets, finish.perm, reinterpret_cast<int*>(s_dyn));
   }
   if (threadIdx.x == 0) timeline_end(timeline, 0);
 }
@@ -1060,30 +1050,34 @@ void launch_gather(cudaStream_t st, const uint16_t* x, const int32_t* perm, int 
 // device memory to its own arena at start-up, or a latency-critical decode loop in which the
 // implicit device-wide synchronisation of cudaMalloc / cudaFree is not acceptable.  For them
 // this entry point runs the gate, top-k, gate scores and the token->expert permutation of one
-// step without logits or scores in memory.  Its only scratch is the call's own output word offsets[n_experts], by which
-// the CTA that finishes last knows that it does (it then sorts the assignments), so calls share nothing and may overlap
-// or be replayed in any order.  The word is cleared by a kernel of one thread, under which the gate kernel already
-// starts.  (As three memsets, the gate kernel and the permutation kernel a call of 32 tokens took 16 us, nearly all of
-// it on the host.)
+// step without logits or scores in memory, and without scratch: a kernel of one CTA, which waits beside the gate kernel
+// and starts when that ends, sorts the assignments, so calls share nothing and may overlap or be replayed in any order.  (As
+// three memsets, the gate kernel and the permutation kernel a call of 32 tokens took 16 us, nearly all of it on the host; sorted
+// by the gate kernel's last CTA, found by counting in a word that a kernel in front cleared, 9.8; now 8.9.)
 namespace oled {
 namespace {
 
-__global__ void clear_word_kernel(int32_t* word) {
+__global__ void __launch_bounds__(kStagedWarps * 32)
+sort_kernel(const int32_t* ids, int n, int E, int32_t* counts, int32_t* offsets, int32_t* perm) {
+  extern __shared__ int s_hist[];
   griddep_launch_dependents();
   griddep_wait();
-  *word = 0;
+  sort_assignments<kStagedWarps>(ids, n, E, counts, offsets, perm, s_hist);
 }
 
 void launch_route_alone(cudaStream_t st, const uint16_t* x, const uint16_t* w_router, const float* bias, const float* conf,
                         int T, int H, int E, int K, int32_t* ids, float* gate, int32_t* counts, const RouteFinish& finish) {
   const size_t sort_bytes = (size_t)kStagedWarps * E * sizeof(int);
-  if (T > 1) launch_pdl(clear_word_kernel, dim3(1), dim3(1), 0, st, finish.offsets + E);
   auto go = [&](auto kernel, int tt) {
-    launch_pdl(kernel, dim3((T + tt - 1) / tt), dim3(kStagedWarps * 32), std::max(staged_smem(tt, H, E), sort_bytes), st, x, w_router, bias, conf, T, H, E, K, (float*)nullptr,
-               ids, gate, counts, (unsigned long long*)nullptr, CombinePrev{}, (StepTimeline*)nullptr, ScatterRows{}, finish, RouterAhead{});
+    launch_pdl(kernel, dim3((T + tt - 1) / tt), dim3(kStagedWarps * 32), std::max(staged_smem(tt, H, E), sort_bytes), st, x, w_router,
+               bias, conf, T, H, E, K, (float*)nullptr, ids, gate, counts, (unsigned long long*)nullptr, CombinePrev{},
+               (StepTimeline*)nullptr, ScatterRows{}, finish, RouterAhead{});
   };
   if (T <= 148) go(route_kernel<1, kStagedWarps, 4, 4>, 1);
   else go(route_kernel<2, kStagedWarps, 4, 4>, 2);
+  if (T > 1)
+    launch_pdl(sort_kernel, dim3(1), dim3(kStagedWarps * 32), sort_bytes, st, (const int32_t*)ids, T * K, E, counts, finish.offsets,
+               finish.perm);
 }
 
 }  // namespace
