@@ -51,7 +51,7 @@
 // row's power-of-two scale and applies the weight row's scale.  The input rows' terms come from the gate
 // kernel, those of the intermediate rows from four more warps per CTA (KIND 3) or from split_rows_kernel.  (An M = 128
 // instruction consumes 128 weight rows x 32 bytes whatever the element size; widening the codes to bf16 first
-// makes the thread that issues the MMAs the bound: 8 layers of 250 tokens 1459 us, now 763.)
+// makes the thread that issues the MMAs the bound: 8 layers of 250 tokens 1459 us, now 735.)
 //
 // Warp roles: warps 0-7 the work table, then the epilogue (lane quarter = warp mod 4, interleaved 16-column
 // chunks), warp 8 weights, warp 9 token rows, warp 10 MMA issue; in one
@@ -886,15 +886,16 @@ split_rows_kernel(const __grid_constant__ FfnGroup grp, const __grid_constant__ 
 }
 
 // Stage shape and count: two k-blocks per stage where at least three such stages fit and both contractions
-// have an even number of them (half the waits and commits on the MMA thread); ten bf16 k-blocks in flight
-// at most (eleven measured slower), eight of e4m3 codes (16 tokens, 8 layers: 557 us, with ten 569).
+// have an even number of them (half the waits and commits on the MMA thread); twelve bf16 k-blocks in flight
+// at most (tiles of 16 rows have room for them; with ten 8 layers of 1 token 228.8 us, now 226.9, of 16 similar tokens 359.5 and
+// 358.2), eight of e4m3 codes (16 tokens, 8 layers: 557 us, with ten 569).
 struct FewRings {
   int stages, k_atoms;
   uint32_t smem;
 };
 FewRings few_rings(int n_box, bool fp8, int H, int I) {
   const uint32_t atom = kFewWTile + (uint32_t)n_box * 128u * (fp8 ? 2u : 1u);
-  const int kblocks = (int)std::min<uint32_t>(fp8 ? 8u : 10u, (kFewSmemMax - kFewCtlBytes - 1024u) / atom);
+  const int kblocks = (int)std::min<uint32_t>(fp8 ? 8u : 12u, (kFewSmemMax - kFewCtlBytes - 1024u) / atom);
   const int kk = fp8 ? 128 : 64;
   FewRings r;
   r.k_atoms = kblocks >= 6 && (H / kk) % 2 == 0 && (I / kk) % 2 == 0 ? 2 : 1;

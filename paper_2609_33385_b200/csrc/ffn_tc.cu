@@ -823,7 +823,7 @@ static int box_index(int max_count, int cap) {
 // Token tiles of at most kFewMaxRows rows go to ffn_few.cu (4 layers of 64 experts, us, against the two-accumulator
 // tiles here: 300 tokens 635 / 707, 512 tokens 701 / 773; beyond 128 rows the operand traffic of its single weight
 // tile costs more than it saves: 1000 tokens 1035 here, 926 on CTA pairs when that was measured, 800 now).  Of fp8 stores every tile does, provided
-// the rows' e4m3 terms are at hand (8 layers of 250 tokens: 763 / 1459); otherwise converter warps widen the codes.
+// the rows' e4m3 terms are at hand (8 layers of 250 tokens: 735 / 1459); otherwise converter warps widen the codes.
 static bool few_form(const FfnTcMaps& maps, int max_count, const TokenSplit* split) {
   if (!maps.few) return false;
   return maps.fp8 ? split != nullptr && split->complete() : max_count <= kFewMaxRows;
