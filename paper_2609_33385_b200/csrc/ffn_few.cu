@@ -313,7 +313,7 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
     // 367.7; 16 layers of 32 from fp8 stores 1231 / 1230 / 1243).  Nothing beyond the item: a line that waits in L2 is read there
     // twice (64 MB of the following items during the gate 1164 -> 1181 us; the CTA's next item all along the stream -> 1415).
     if (spec && p.rows.cap <= 148) {
-      for (int a = pre1 * p.k_atoms; a < k_blocks1 * p.k_atoms; ++a) {
+      for (int a = pre1 * p.k_atoms; a < min(k_blocks1, pre1 + 12) * p.k_atoms; ++a) {  // (longer items: no more than the gate lasts)
         if (elect_one()) few_prefetch_w1(&p.tm_w1, a * kK, spec_m, grp.slot[spec_g], policy);
         __nanosleep(150);
       }
