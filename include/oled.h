@@ -353,7 +353,8 @@ int oled_last_cuda_error(oled_ctx* ctx);
  *   or NULL, confidences fp32[n_tokens]: device, read only.
  *   ids int32[n_tokens*top_k], gate fp32[n_tokens*top_k], counts int32[n_experts],
  *   offsets int32[n_experts+1], perm int32[n_tokens*top_k]: device, written; caller-owned.
- *   n_tokens <= OLED_NOALLOC_MAX_TOKENS, else OLED_ERR_TOO_MANY_TOKENS; other limits as above.
+ *   n_tokens <= OLED_NOALLOC_MAX_TOKENS, else OLED_ERR_TOO_MANY_TOKENS; other limits as above (a hidden_dim
+ *   whose rows do not fit a CTA's shared memory is rejected with OLED_ERR_INVALID_ARG before anything is launched).
  *   hidden, w_router and ids must be 16-byte aligned (they are accessed with 16-byte vectors), the
  *   other arrays 4-byte aligned; a misaligned pointer is rejected with OLED_ERR_INVALID_ARG before
  *   anything is launched.

@@ -183,7 +183,7 @@ struct RouteFinish {
   int32_t* perm = nullptr;
 };
 // counts[E], offsets[E + 1] and the stable permutation by expert of n assignments, by one CTA of WARPS warps (E at most
-// one expert per thread).  Every warp counts the experts of a contiguous part of the list, the counts are scanned over
+// one expert per thread; a number that names no expert is passed over).  Every warp counts the experts of a contiguous part of the list, the counts are scanned over
 // (expert, warp), and every warp hands out its part's rows in order.  s_hist: [WARPS][E].
 template <int WARPS>
 __device__ __forceinline__ void sort_assignments(const int32_t* ids, int n, int E, int32_t* __restrict__ counts,
@@ -196,7 +196,8 @@ __device__ __forceinline__ void sort_assignments(const int32_t* ids, int n, int 
   const int part = (n + WARPS * 32 - 1) / (WARPS * 32) * 32, first = warp * part, last = min(n, first + part);
   int* const hist = s_hist + warp * E;
   for (int i0 = first; i0 < last; i0 += 32) {
-    const int id = i0 + lane < last ? __ldcg(ids + i0 + lane) : -1;
+    int id = i0 + lane < last ? __ldcg(ids + i0 + lane) : -1;
+    if ((unsigned)id >= (unsigned)E) id = -1;
     const uint32_t same = __match_any_sync(0xffffffffu, id);
     if (id >= 0 && lane == __ffs((int)same) - 1) hist[id] += __popc(same);
     __syncwarp();
@@ -228,7 +229,8 @@ __device__ __forceinline__ void sort_assignments(const int32_t* ids, int n, int 
   }
   __syncthreads();
   for (int i0 = first; i0 < last; i0 += 32) {
-    const int id = i0 + lane < last ? __ldcg(ids + i0 + lane) : -1;
+    int id = i0 + lane < last ? __ldcg(ids + i0 + lane) : -1;
+    if ((unsigned)id >= (unsigned)E) id = -1;
     const uint32_t same = __match_any_sync(0xffffffffu, id);
     const int rank = __popc(same & ((1u << lane) - 1u));
     if (id >= 0) perm[hist[id] + rank] = i0 + lane;
@@ -1067,19 +1069,23 @@ sort_kernel(const int32_t* ids, int n, int E, int32_t* counts, int32_t* offsets,
   sort_assignments<kStagedWarps>(ids, n, E, counts, offsets, perm, s_hist);
 }
 
-void launch_route_alone(cudaStream_t st, const uint16_t* x, const uint16_t* w_router, const float* bias, const float* conf,
-                        int T, int H, int E, int K, int32_t* ids, float* gate, int32_t* counts, const RouteFinish& finish) {
-  const size_t sort_bytes = (size_t)kStagedWarps * E * sizeof(int);
+// Dynamic shared memory of the gate kernel in this role (the one-token form sorts in it).
+size_t route_alone_smem(int T, int H, int E) {
+  return std::max(staged_smem(T <= 148 ? 1 : 2, H, E), (size_t)kStagedWarps * E * sizeof(int));
+}
+
+// The sort indexes by what the gate kernel has stored: it is launched only behind a gate kernel that was.
+cudaError_t launch_route_alone(cudaStream_t st, const uint16_t* x, const uint16_t* w_router, const float* bias, const float* conf,
+                               int T, int H, int E, int K, int32_t* ids, float* gate, int32_t* counts, const RouteFinish& finish) {
   auto go = [&](auto kernel, int tt) {
-    launch_pdl(kernel, dim3((T + tt - 1) / tt), dim3(kStagedWarps * 32), std::max(staged_smem(tt, H, E), sort_bytes), st, x, w_router,
-               bias, conf, T, H, E, K, (float*)nullptr, ids, gate, counts, (unsigned long long*)nullptr, CombinePrev{},
-               (StepTimeline*)nullptr, ScatterRows{}, finish, RouterAhead{});
+    return launch_pdl(kernel, dim3((T + tt - 1) / tt), dim3(kStagedWarps * 32), route_alone_smem(T, H, E), st, x, w_router,
+                      bias, conf, T, H, E, K, (float*)nullptr, ids, gate, counts, (unsigned long long*)nullptr, CombinePrev{},
+                      (StepTimeline*)nullptr, ScatterRows{}, finish, RouterAhead{});
   };
-  if (T <= 148) go(route_kernel<1, kStagedWarps, 4, 4>, 1);
-  else go(route_kernel<2, kStagedWarps, 4, 4>, 2);
-  if (T > 1)
-    launch_pdl(sort_kernel, dim3(1), dim3(kStagedWarps * 32), sort_bytes, st, (const int32_t*)ids, T * K, E, counts, finish.offsets,
-               finish.perm);
+  const cudaError_t err = T <= 148 ? go(route_kernel<1, kStagedWarps, 4, 4>, 1) : go(route_kernel<2, kStagedWarps, 4, 4>, 2);
+  if (err != cudaSuccess || T == 1) return err;
+  return launch_pdl(sort_kernel, dim3(1), dim3(kStagedWarps * 32), (size_t)kStagedWarps * E * sizeof(int), st, (const int32_t*)ids,
+                    T * K, E, counts, finish.offsets, finish.perm);
 }
 
 }  // namespace
@@ -1112,11 +1118,12 @@ extern "C" int oled_route_noalloc(const void* hidden, const void* w_router, cons
     }
     return OLED_OK;
   }
+  if (route_alone_smem(n_tokens, hidden_dim, n_experts) > kStagedSmem) return OLED_ERR_INVALID_ARG;
   RouteFinish finish;
   if (!staged_attributes()) return OLED_ERR_CUDA;
   finish.offsets = offsets;
   finish.perm = perm;
-  launch_route_alone(st, static_cast<const uint16_t*>(hidden), static_cast<const uint16_t*>(w_router), bias, confidences,
-                     n_tokens, hidden_dim, n_experts, top_k, ids, gate, counts, finish);
-  return cudaGetLastError() == cudaSuccess ? OLED_OK : OLED_ERR_CUDA;
+  const cudaError_t err = launch_route_alone(st, static_cast<const uint16_t*>(hidden), static_cast<const uint16_t*>(w_router), bias,
+                                             confidences, n_tokens, hidden_dim, n_experts, top_k, ids, gate, counts, finish);
+  return cudaGetLastError() == cudaSuccess && err == cudaSuccess ? OLED_OK : OLED_ERR_CUDA;
 }

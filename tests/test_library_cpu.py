@@ -216,6 +216,23 @@ def test_misaligned_pointers_are_rejected_before_anything_is_launched(binding):
     assert call(bias=ok4 + 1) == binding.ERR_INVALID_ARG
 
 
+def test_rows_beyond_shared_memory_are_rejected_before_anything_is_launched(binding):
+    """oled_route_noalloc keeps the rows of its one or two tokens per CTA in shared memory: a hidden size whose rows cannot
+    fit is an argument error, not a launch that is refused in front of one that sorts its results (nothing touches the GPU)."""
+    ok16 = 0x7000_0000_0100
+    a = [ok16 + 0x1000 * i for i in range(8)]
+
+    def call(n, hidden, n_experts=8):
+        return binding.route_noalloc(a[0], a[1], None, a[2], n, hidden, n_experts, 2, 0, *a[3:])
+    for n in (1, 2, 148):                                   # one token per CTA: a row of 224 KB and the logits beside it
+        for hidden in (114688, 1 << 20, 0x7FFFFF00):
+            assert call(n, hidden) == binding.ERR_INVALID_ARG, (n, hidden)
+    for n in (149, 256):                                    # two
+        for hidden in (57344, 114688, 0x7FFFFF00):
+            assert call(n, hidden) == binding.ERR_INVALID_ARG, (n, hidden)
+    assert call(149, 55552, 512) == binding.ERR_INVALID_ARG  # (217 KB of rows, 8 KB of logits and keys)
+
+
 def test_two_e4m3_terms_hold_a_scaled_bf16_row():
     """The arithmetic the direct fp8 tensor-core form rests on (csrc/fp8_split.h), restated in numpy
     with the oracle's decoder: a bf16 row scaled by the power of two that brings its largest
