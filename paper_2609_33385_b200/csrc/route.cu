@@ -240,14 +240,8 @@ __device__ __forceinline__ void sort_assignments(const int32_t* ids, int n, int 
   }
 }
 
-// The router matrix ahead of the input (staged forms): its first `chunks` * 256 columns go to shared memory, and up to
-// two further chunks of the first pass to registers (one token per CTA: the combine of two has none left).
-// (Routing without a step fetches nothing ahead: the matrix is the caller's, may still be in the making, and with the copies behind
-// the dependency wait a call of 32 tokens took 12.9 us instead of 10.)
-struct RouterAhead {
-  int on = 0;      // the matrix is older than everything that may still run on the stream
-  int chunks = 0;
-};
+// Chunks of the router matrix that wait in registers (kAhead; the combine of two tokens has no registers left for them).
+__host__ __device__ constexpr int router_tail(int tt) { return tt == 1 ? 2 : 0; }
 // TT tokens per CTA, WARPS warps; each warp owns kEPerWarp experts per pass and all TT tokens.  Small
 // blocks use TT = 1 with 16 warps (one pass covers 64 experts) and keep several 256-wide
 // chunks of loads in flight; the chain order of every logit is the same in all variants.
@@ -258,17 +252,19 @@ struct RouterAhead {
 // - the same total order a round-by-round selection walks.
 // One token per CTA while that gives at most one wave of CTAs; two or four beyond (every CTA
 // streams the whole router matrix, so a second wave costs as much as the first).
+// kAhead: the router matrix is on chip before the input is there, `ahead` chunks of 256 columns in shared memory and what is
+// left, at most router_tail() chunks, in registers (router_chunks_ahead() says when; never in routing without a step, whose
+// matrix is the caller's and may still be in the making).
 // The kernel reports nothing to the host: the step's first FFN launch, which starts when it has completed,
 // publishes the finished counts and scores without any ticket or fence.
-template <int TT, int WARPS, int UNROLL, int kEPerWarp>
+template <int TT, int WARPS, int UNROLL, int kEPerWarp, bool kAhead = false>
 __global__ void __launch_bounds__(WARPS * 32, 1)
 route_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ wr,
              const float* __restrict__ bias, const float* __restrict__ conf, int T, int H, int E,
              int K, float* __restrict__ logits_out, int32_t* __restrict__ ids,
              float* __restrict__ gate, int32_t* __restrict__ counts,
              unsigned long long* __restrict__ scores, CombinePrev prev, StepTimeline* timeline,
-             const __grid_constant__ ScatterRows scatter, const __grid_constant__ RouteFinish finish,
-             const __grid_constant__ RouterAhead ahead) {
+             const __grid_constant__ ScatterRows scatter, const __grid_constant__ RouteFinish finish, int ahead) {
   extern __shared__ __align__(16) uint8_t s_dyn[];
   float* s_logits = reinterpret_cast<float*>(s_dyn);                       // [TT][E]
   constexpr bool staged = TT <= 4;
@@ -290,16 +286,14 @@ route_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ wr,
   constexpr int kRouteWarps = WARPS;
   const int my_tokens = min(TT, T - t0);
   // The router matrix does not depend on the predecessor (the previous layer's expert FFN, which a CTA of this kernel
-  // usually waits 4 to 8 us for): what fits is fetched now.  What bounds the logits otherwise is one SM's share of L2, 64
-  // bytes a cycle: 64 experts x 2048 took 3.4-3.6 us after the input was there, now 2.6 (one pass' worth from chip: 8 layers
-  // of 1 token 236.3 -> 230.0 us, of 16 similar tokens 361.4 -> 355.1, 16 layers of 32 1994 -> 1985).
-  // [E][chunks * 256], a row's 512 bytes of a chunk are read by a warp at a time
+  // usually waits 4 to 8 us for).  What bounds the logits otherwise is one SM's share of L2, 64 bytes a cycle: 64 experts x
+  // 2048 took 3.4-3.6 us after the input was there, from chip 2.6.
+  // [E][ahead * 256], a row's 512 bytes of a chunk are read by a warp at a time
   uint16_t* const s_w = reinterpret_cast<uint16_t*>(s_key + (size_t)TT * Ep);
-  const int w_cols = staged ? ahead.chunks * 256 : 0, n_chunks = H / 256;
-  constexpr int kTail = TT == 1 ? 2 : 0;
-  const bool tail_ahead = ahead.on && n_chunks - ahead.chunks <= kTail;
+  const int w_cols = ahead * 256;
+  constexpr int kTail = kAhead ? router_tail(TT) : 0;
   uint4 w_tail[kTail == 0 ? 1 : kTail][kEPerWarp];
-  if (staged && ahead.on) {
+  if (kAhead) {
     const uint32_t dst = (uint32_t)__cvta_generic_to_shared(s_w);
     const int pieces = w_cols / 8;  // of 16 bytes, per row
     for (int e = warp; e < E; e += kRouteWarps)
@@ -307,19 +301,16 @@ route_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ wr,
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + (uint32_t)(e * pieces + c) * 16u),
                      "l"(wr + (size_t)e * H + c * 8)
                      : "memory");
-    if (tail_ahead) {
 #pragma unroll
-      for (int i = 0; i < kTail; ++i)
+    for (int i = 0; i < kTail; ++i)
 #pragma unroll
-        for (int b = 0; b < kEPerWarp; ++b)
-          if (w_cols + i * 256 < H)
-            w_tail[i][b] = *reinterpret_cast<const uint4*>(wr + (size_t)min(warp * kEPerWarp + b, E - 1) * H + w_cols + i * 256 + lane * 8);
-    }
-  }
-  if (staged && gridDim.x <= 148 && !tail_ahead) {
-    // the rest into L2, out of which the expert weights streamed since its last use may have pushed it
+      for (int b = 0; b < kEPerWarp; ++b)
+        if (w_cols + i * 256 < H)
+          w_tail[i][b] = *reinterpret_cast<const uint4*>(wr + (size_t)min(warp * kEPerWarp + b, E - 1) * H + w_cols + i * 256 + lane * 8);
+  } else if (staged && gridDim.x <= 148) {
+    // into L2, out of which the expert weights streamed since its last use may have pushed it
     for (int e = warp; e < E; e += kRouteWarps)
-      for (int c = w_cols + lane * 64; c < H; c += 32 * 64)  // 128-byte lines of the row
+      for (int c = lane * 64; c < H; c += 32 * 64)  // 128-byte lines of the row
         asm volatile("prefetch.global.L2 [%0];" ::"l"(wr + (size_t)e * H + c));
   }
   uint16_t* const dense_rows = staged && scatter.cap > 0 && scatter.dense && scatter.split.amax_in == nullptr ? scatter.xp : nullptr;
@@ -341,7 +332,7 @@ route_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ wr,
     if ((int)threadIdx.x < my_tokens) s_conf[threadIdx.x] = conf[t0 + threadIdx.x];
     for (int i = threadIdx.x; i < TT * (Ep - E); i += blockDim.x) s_key[(i / (Ep - E)) * Ep + E + i % (Ep - E)] = 0u;
     if (threadIdx.x < kST) s_amax[threadIdx.x] = 0u;
-    asm volatile("cp.async.wait_all;" ::: "memory");
+    if (kAhead) asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     if (scatter.split.amax_in != nullptr)
       for (int a = 0; a < my_tokens; ++a) {
@@ -387,8 +378,8 @@ route_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ wr,
       word([](const uint4& v) { return v.z; });
       word([](const uint4& v) { return v.w; });
     };
-    int hc = 0;
-    if (staged) {
+    if constexpr (kAhead) {
+      int hc = 0;
 #pragma unroll 2
       for (; hc < w_cols; hc += 256) {
         uint4 ww[kEPerWarp];
@@ -397,19 +388,18 @@ route_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ wr,
           ww[b] = *reinterpret_cast<const uint4*>(s_w + (size_t)min(eb + b, E - 1) * w_cols + hc + lane * 8);
         chunk(hc, ww);
       }
-      if (tail_ahead && eb == warp * kEPerWarp) {
 #pragma unroll
-        for (int i = 0; i < kTail; ++i, hc += 256)
-          if (hc < H) chunk(hc, w_tail[i]);
-      }
-    }
+      for (int i = 0; i < kTail; ++i, hc += 256)  // (there are any only where one pass takes all experts: these are its rows)
+        if (hc < H) chunk(hc, w_tail[i]);
+    } else {
 #pragma unroll UNROLL
-    for (; hc < H; hc += 256) {
-      uint4 ww[kEPerWarp];
+      for (int hc = 0; hc < H; hc += 256) {
+        uint4 ww[kEPerWarp];
 #pragma unroll
-      for (int b = 0; b < kEPerWarp; ++b)
-        ww[b] = *reinterpret_cast<const uint4*>(wr + (size_t)min(eb + b, E - 1) * H + hc + lane * 8);
-      chunk(hc, ww);
+        for (int b = 0; b < kEPerWarp; ++b)
+          ww[b] = *reinterpret_cast<const uint4*>(wr + (size_t)min(eb + b, E - 1) * H + hc + lane * 8);
+        chunk(hc, ww);
+      }
     }
 #pragma unroll
     for (int a = 0; a < TT; ++a)
@@ -931,19 +921,30 @@ static size_t staged_smem(int tt, int H, int E) {  // logits, rows, keys
   return ((((size_t)tt * E * sizeof(float)) + 15) & ~(size_t)15) + (size_t)tt * H * 2 + (size_t)tt * ((E + 3) & ~3) * 4;
 }
 constexpr size_t kStagedSmem = 224 * 1024;  // (of 227 KB; the rest holds the kernel's static arrays)
-// As many chunks of the router matrix as fit behind the rows, where one pass of the warps takes all experts.  (With more experts
-// little of it fits: 7 layers of 9 tokens, 128 experts x 2048, 261 us without and 275 with it; 8 of 2 tokens, 121 x 2560, 252 / 260.)
-static RouterAhead router_ahead(int tt, int H, int E) {
-  RouterAhead r;
-  if (E > kStagedWarps * 4) return r;
-  r.on = 1;
-  r.chunks = (int)std::min<size_t>(H / 256, (kStagedSmem - staged_smem(tt, H, E)) / ((size_t)E * 512));
-  return r;
+// Chunks of the router matrix to fetch into shared memory ahead of the input, 0: none.  Only where
+//  * the whole matrix is on chip then (64 experts of 2048, 128 of 512): a part of it is the same wait for the copies and the
+//    same reads of L2 for the rest (6 chunks of 16 at 64 x 4096 from fp8 stores: a lone step of one token 42.5 us, without them 40.7,
+//    stacks of four such layers 150 / 139); what shared memory has no room for waits in registers where one pass of the warps
+//    takes all experts;
+//  * a CTA has one token or two (four, stacks of 400 tokens at 16 x 512: bf16 / fp8 stores 183.9 / 218.6 us with it, 181.3 / 217.0 without);
+//  * there is an FFN launch to wait for - the kernel carries its combine out -, or the CTAs are so few that the copies are no
+//    queue in front of the logits (lone steps at 64 x 2048 of 1 / 4 / 16 / 32 / 100 tokens: 28.1 / 54.0 / 111.0 / 118.4 / 127.2 us with it,
+//    28.7 / 54.0 / 110.7 / 117.5 / 125.0 without; from fp8 stores 26.1 / 38.5 / 64.5 / 71.6 / 75.2 and 26.8 / 39.0 / 65.0 / 70.6 / 73.4).
+// Stacks of four layers without / with it: 64 x 2048, 1 token 113.4 / 109.6 us, 32 tokens 469.8 / 468.3; 128 x 512, 1 / 16 / 100 tokens
+// 90.8 / 212.9 / 287.7 and 85.7 / 209.0 / 284.9; 160 x 512 from fp8 stores, 32 tokens 151.4 / 149.0; of six layers 16 x 512, 250 tokens (two
+// a CTA) 158.4 / 157.5, from fp8 stores 184.9 / 181.3.
+static int router_chunks_ahead(int T, int H, int E, bool combines) {
+  if (T > 296 || !(combines || T <= 16)) return 0;
+  const int tt = T <= 148 ? 1 : 2;
+  const int chunks = (int)std::min<size_t>(H / 256, (kStagedSmem - staged_smem(tt, H, E)) / ((size_t)E * 512));
+  return H / 256 - chunks <= (E <= kStagedWarps * 4 ? router_tail(tt) : 0) ? chunks : 0;
 }
 static bool staged_attributes() {  // the staged rows: up to 4 x 16 K elements
   static const bool ok = [] {
     const bool done =
         cudaFuncSetAttribute(route_kernel<1, kStagedWarps, 4, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStagedSmem) == cudaSuccess &&
+        cudaFuncSetAttribute(route_kernel<2, kStagedWarps, 4, 4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStagedSmem) == cudaSuccess &&
+        cudaFuncSetAttribute(route_kernel<1, kStagedWarps, 4, 4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStagedSmem) == cudaSuccess &&
         cudaFuncSetAttribute(route_kernel<2, kStagedWarps, 4, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStagedSmem) == cudaSuccess &&
         cudaFuncSetAttribute(route_kernel<4, kStagedWarps, 2, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStagedSmem) == cudaSuccess;
     if (!done) cudaGetLastError();
@@ -960,12 +961,15 @@ void launch_route(cudaStream_t st, const uint16_t* x, const uint16_t* w_router, 
   if (route_staged(T, K)) {
     constexpr int W = kStagedWarps;
     staged_attributes();
+    // (the matrix is the context's copy, whose writer has been waited for: it is older than all that may still run on the stream)
+    const int ahead = router_chunks_ahead(T, H, E, prev.y != nullptr);
     auto go = [&](auto kernel, int tt) {
-      const RouterAhead ahead = router_ahead(tt, H, E);  // (a context's copy of the matrix: its writer has been waited for)
-      launch_pdl(kernel, dim3((T + tt - 1) / tt), dim3(W * 32), staged_smem(tt, H, E) + (size_t)ahead.chunks * E * 512, st, x, w_router,
+      launch_pdl(kernel, dim3((T + tt - 1) / tt), dim3(W * 32), staged_smem(tt, H, E) + (size_t)ahead * E * 512, st, x, w_router,
                  bias, conf, T, H, E, K, logits, ids, gate, counts, scores, prev, timeline, scatter, RouteFinish{}, ahead);
     };
-    if (T <= 148) go(route_kernel<1, W, 4, 4>, 1);
+    if (T <= 148 && ahead > 0) go(route_kernel<1, W, 4, 4, true>, 1);
+    else if (T <= 148) go(route_kernel<1, W, 4, 4>, 1);
+    else if (ahead > 0) go(route_kernel<2, W, 4, 4, true>, 2);
     else if (T <= 296) go(route_kernel<2, W, 4, 4>, 2);  // (four tokens per CTA measured slower at 256 tokens x 128 experts: 33 against 20 us)
     else go(route_kernel<4, W, 2, 4>, 4);
   } else {
@@ -1080,7 +1084,7 @@ cudaError_t launch_route_alone(cudaStream_t st, const uint16_t* x, const uint16_
   auto go = [&](auto kernel, int tt) {
     return launch_pdl(kernel, dim3((T + tt - 1) / tt), dim3(kStagedWarps * 32), route_alone_smem(T, H, E), st, x, w_router,
                       bias, conf, T, H, E, K, (float*)nullptr, ids, gate, counts, (unsigned long long*)nullptr, CombinePrev{},
-                      (StepTimeline*)nullptr, ScatterRows{}, finish, RouterAhead{});
+                      (StepTimeline*)nullptr, ScatterRows{}, finish, 0);
   };
   const cudaError_t err = T <= 148 ? go(route_kernel<1, kStagedWarps, 4, 4>, 1) : go(route_kernel<2, kStagedWarps, 4, 4>, 2);
   if (err != cudaSuccess || T == 1) return err;

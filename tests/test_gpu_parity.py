@@ -998,11 +998,14 @@ def test_guess_rows_requested_before_the_counts(n_experts, top_k, hidden, inter,
 @pytest.mark.parametrize("fp8", [False, True], ids=["bf16", "fp8"])
 @pytest.mark.parametrize("n_experts,top_k,hidden,counts", [(64, 8, 2048, (1, 33, 149)), (3, 2, 256, (1, 149)), (33, 4, 4096, (2, 148)),
                                                            (8, 2, 16384, (1, 3)), (70, 8, 2048, (1, 150)), (512, 32, 1024, (1, 12)),
-                                                           (16, 2, 768, (5, 600))])
+                                                           (16, 2, 768, (5, 600)), (64, 8, 1792, (1, 16, 17, 148)), (70, 8, 1024, (2, 148)),
+                                                           (400, 4, 256, (3, 20)), (32, 4, 1024, (16, 149, 296))])
 def test_gate_with_the_router_matrix_fetched_ahead(n_experts, top_k, hidden, counts, fp8):
-    """Few-token gate: the router matrix wholly on chip (shared memory, or with the last one or two chunks in registers), partly
-    or not at all, one and several passes over the experts, one, two and four tokens per CTA; logits, ids, gate scores and order equal
-    the oracle's bit for bit, in a stack iteration (where the combine runs in the same kernel) the same as layer by layer."""
+    """Few-token gate: the router matrix on chip ahead of the input (in a stack's second layer, up to 16 tokens in the first one
+    and in lone steps too) wholly in shared memory, with its last chunk or the last two in registers, in one and in several passes
+    over the experts, for one and two tokens per CTA; and not fetched ahead, where it does not fit whole or four tokens share a CTA.
+    Logits, ids, gate scores and order equal the oracle's bit for bit, in a stack iteration (where the combine runs in the same
+    kernel) the same as layer by layer."""
     from oracle import moe_layer as oracle_moe
     from paper_2609_33385_b200.runner import bits_to_dev, dev_to_bits
     w = synth.tiny(n_layers=2, n_experts=n_experts, top_k=top_k, hidden=hidden, intermediate=128)
