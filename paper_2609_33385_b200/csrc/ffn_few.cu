@@ -886,16 +886,18 @@ split_rows_kernel(const __grid_constant__ FfnGroup grp, const __grid_constant__ 
 }
 
 // Stage shape and count: two k-blocks per stage where at least three such stages fit and both contractions
-// have an even number of them (half the waits and commits on the MMA thread); twelve bf16 k-blocks in flight
-// at most (tiles of 16 rows have room for them; with ten 8 layers of 1 token 228.8 us, now 226.9, of 16 similar tokens 359.5 and
-// 358.2), eight of e4m3 codes (16 tokens, 8 layers: 557 us, with ten 569).
+// have an even number of them (half the waits and commits on the MMA thread); ten bf16 k-blocks in flight
+// at most, eight of e4m3 codes (16 tokens, 8 layers: 557 us, with ten 569).  Tiles of 16 rows have room for twelve bf16 ones, which
+// gains at hidden 2048 with 64 experts only (layers of 1 token with twelve / ten 26.5 / 26.7 us, of 16 similar tokens 41.4 / 42.1); elsewhere it costs:
+// four layers of 64 experts, 4096 x 768, 1 token 173.2 / 155.8 us, 3072 x 768, 5 tokens 308.5 / 300.6, 768 x 1024, 16 tokens 187.6 / 183.8,
+// of 128 experts, 2048 x 768, 8 tokens 316.1 / 309.9.
 struct FewRings {
   int stages, k_atoms;
   uint32_t smem;
 };
 FewRings few_rings(int n_box, bool fp8, int H, int I) {
   const uint32_t atom = kFewWTile + (uint32_t)n_box * 128u * (fp8 ? 2u : 1u);
-  const int kblocks = (int)std::min<uint32_t>(fp8 ? 8u : 12u, (kFewSmemMax - kFewCtlBytes - 1024u) / atom);
+  const int kblocks = (int)std::min<uint32_t>(fp8 ? 8u : 10u, (kFewSmemMax - kFewCtlBytes - 1024u) / atom);
   const int kk = fp8 ? 128 : 64;
   FewRings r;
   r.k_atoms = kblocks >= 6 && (H / kk) % 2 == 0 && (I / kk) % 2 == 0 ? 2 : 1;
