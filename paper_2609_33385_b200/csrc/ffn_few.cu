@@ -56,6 +56,7 @@
 // Warp roles: warps 0-7 the work table, then the epilogue (lane quarter = warp mod 4, interleaved 16-column
 // chunks), warp 8 weights, warp 9 token rows, warp 10 MMA issue; in one
 // launch warp 11 counts stored items, and with fp8 stores warps 12-15 make the intermediate rows' terms.  Every wait is bounded as in ffn_tc.cu.
+// (Times that stand together in a comment were taken in turn on one machine; machines differ by 5 %, so they do not chain.)
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -92,6 +93,7 @@ struct __align__(16) FewCtl {
   unsigned long long looked;  // ... guesses_open is
   uint32_t tmem_base;
   int abort;
+  int gate_through; // the weight warp is past its dependency wait
   int n_tiles;      // token tiles of the group
   int n_first;      // first-phase (or only) items that are drawn from the counter
   int guess_lost;   // another CTA has taken this one's guess over: its results are not stored
@@ -254,6 +256,7 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
       mbar_init(smem_u32(&ctl->claimed), 1);
       mbar_init(smem_u32(&ctl->looked), 1);
       ctl->abort = 0;
+      ctl->gate_through = 0;
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -300,26 +303,32 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
   };
   auto wait_table = [&]() { return warp_wait(smem_u32(&ctl->table), 0u, abort_flag, p.status); };
 
+  // While the gate kernel runs, a warp with nothing to do before the first item (the counting warp, in two launches the MMA warp)
+  // calls the rest of the guessed item into L2: paced, all at once it was a queue that the gate's own loads stood in, and no
+  // further once the gate is through, when the ring is to have the memory to itself.  (By the weight warp, on a fixed schedule,
+  // it held the first item back: that / this, both with twelve k-blocks in flight, four layers of 64 experts x 2048, 64 tokens 497.6 / 491.8 us,
+  // 100 tokens 508.6 / 496.0, x 4096, 100 tokens from fp8 stores 454.4 / 442.6.)  148 CTAs take a k-block each off HBM in 0.37 us; not
+  // at all / a pause of 75 / 150 / 300 ns (450 as 300): 8 layers of 1 token 226.5 / 222.9 / 220.3 / 215.1 us, of 16 similar tokens 346.1 /
+  // 345.1 / 339.2 / 335.3; 16 layers of 32 tokens 1943 / 1949 / 1939 / 1925, from fp8 stores 1170 / 1175 / 1172 / 1172; 8 layers of 250
+  // from fp8 stores 726 / 733 / 733 / 733.  Nothing beyond the item: a line that waits in L2 is read there twice (16 layers of 32 from fp8
+  // stores, 64 MB of the following items during the gate 1164 -> 1181; the CTA's next item all along the stream -> 1415).
+  auto call_rest_of_guess = [&]() {
+    if (!spec) return;
+    for (int a = pre1 * p.k_atoms; a < k_blocks1 * p.k_atoms; ++a) {
+      if (__any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(&ctl->gate_through) != 0)) break;
+      if (elect_one()) few_prefetch_w1(&p.tm_w1, a * kK, spec_m, grp.slot[spec_g], policy);
+      __nanosleep(300);
+    }
+    __syncwarp();
+  };
+
   if (warp == kFewWeightWarp) {
     // ------------------------------------------------------------ weights (TMA), and who does what
     int stage = 0, g1 = 0, g2 = 0, seq = 0;
     uint32_t phase = 0;
     bool ok = true;
-    // The rest of the guessed item into L2, for steps whose gate kernel is short (8 layers of 16 similar tokens 362 -> 356 us;
-    // with 250 tokens fp8 it took bandwidth from the gate's own loads, 775 -> 789, with 100 tokens still 523 -> 517; where
-    // between those two the line lies was not measured, it is drawn at one gate CTA per SM).  Paced to a little more than
-    // what HBM delivers (148 CTAs: a k-block each in 0.37 us): all at once they were a queue that the gate's own loads
-    // stood in (pause 0 / 150 / 300 ns: 8 layers of 1 token 240.0 / 235.3 / 232.8 us, of 16 similar tokens 367.2 / 363.2 /
-    // 367.7; 16 layers of 32 from fp8 stores 1231 / 1230 / 1243).  Nothing beyond the item: a line that waits in L2 is read there
-    // twice (64 MB of the following items during the gate 1164 -> 1181 us; the CTA's next item all along the stream -> 1415).
-    if (spec && p.rows.cap <= 148) {
-      for (int a = pre1 * p.k_atoms; a < min(k_blocks1, pre1 + 12) * p.k_atoms; ++a) {  // (longer items: no more than the gate lasts)
-        if (elect_one()) few_prefetch_w1(&p.tm_w1, a * kK, spec_m, grp.slot[spec_g], policy);
-        __nanosleep(150);
-      }
-      __syncwarp();
-    }
     if (!early) griddep_wait();
+    if (lane == 0) *reinterpret_cast<volatile int*>(&ctl->gate_through) = 1;
     if (lane == 0) timeline_start(p.timeline, p.timeline_slot);
     const bool spec_ok = spec && __ldcg(p.rows.counts + grp.expert[spec_g]) > 0;
     auto publish = [&](int code, int m) {
@@ -503,6 +512,7 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
     bool ok = true;
     const uint32_t stage_step = stage_bytes >> 4;  // descriptor addresses count 16 bytes
     const uint64_t a_desc0 = make_smem_desc(tiles_base), b_desc0 = make_smem_desc(tiles_base + stage_tokens);
+    if (!fused) call_rest_of_guess();
     for (int seq = 0; ok; ++seq) {
       const int slot = seq % kFewRing;
       if (!warp_wait(smem_u32(&ctl->item_full[slot]), (uint32_t)(seq / kFewRing) & 1u, abort_flag, p.status)) break;
@@ -569,6 +579,7 @@ ffn_few_kernel(const __grid_constant__ FewArgs p) {
     // its first down item cost 0.7 us per layer at one token, 2 us at 32 from fp8 stores).
     bool lost = false;
     if (guess) {
+      call_rest_of_guess();
       griddep_wait();
       if (spec) {
         uint32_t taken = 0;

@@ -996,6 +996,44 @@ def test_guess_rows_requested_before_the_counts(n_experts, top_k, hidden, inter,
 
 
 @pytest.mark.parametrize("fp8", [False, True], ids=["bf16", "fp8"])
+@pytest.mark.parametrize("n", [20, 40, 250])
+def test_the_rest_of_a_guess_called_ahead_changes_nothing(n, fp8):
+    """Items several times longer than the ring, whose rest the counting warp (one launch) or the MMA warp (two) calls into L2
+    until the gate is through - or not at all, where the launch does not start ahead of the gate (OLED_OPT_PDL 0): the same bits in
+    all four forms for right and wrong guesses, and in parity with the oracle."""
+    from paper_2609_33385_b200 import binding
+    from paper_2609_33385_b200.runner import bits_to_dev, dev_to_bits
+    w = synth.tiny(n_layers=1, n_experts=8, top_k=2, hidden=4096, intermediate=128)
+    outs = []
+    for fuse, pdl in ((1, 1), (1, 0), (0, 1), (0, 0)):
+        run = _runner(w, capacity=[8], max_tokens=n, fp8=fp8)
+        run.ctx.set_option(binding.OPT_FUSE_FFN, fuse)
+        run.ctx.set_option(binding.OPT_PDL, pdl)
+        ora = _oracle_for(run, [8])
+        try:
+            for rep in range(4):
+                h_bits, conf = synth.flat_tokens(w, n, 650)
+                if rep == 2:
+                    h_bits[:] = h_bits[0]
+                x, c = bits_to_dev(h_bits, run.device), torch.from_numpy(conf).to(run.device)
+                out = torch.empty((n, w.hidden), dtype=torch.bfloat16, device=run.device)
+                run.step(0, x, c, out)
+                outs.append(dev_to_bits(out).copy())
+                if not outs[4:]:
+                    ref = ora.denoise_step(0, h_bits, conf)
+                    _check_step(run, 0, n, out, ref, check_out=False)
+                    got = synth.bf16_bits_to_f32(outs[-1]).astype(np.float64)
+                    # a rounding to bf16 moves a value by at most 2^-8 of it: the output's own, and those of the intermediate
+                    # rows, whose sum is at most 2^-8 of an output's root mean square in standard deviation (six of them)
+                    assert np.abs(got - ref["out"]).max() <= 2.0 ** -8 * (np.abs(ref["out"]).max() + 6.0 * np.sqrt(np.mean(ref["out"] ** 2)))
+                    assert np.linalg.norm(got - ref["out"]) <= REL_L2 * np.linalg.norm(ref["out"])
+                else:
+                    assert np.array_equal(outs[-1], outs[len(outs) - 5])
+        finally:
+            run.close()
+
+
+@pytest.mark.parametrize("fp8", [False, True], ids=["bf16", "fp8"])
 @pytest.mark.parametrize("n_experts,top_k,hidden,counts", [(64, 8, 2048, (1, 33, 149)), (3, 2, 256, (1, 149)), (33, 4, 4096, (2, 148)),
                                                            (8, 2, 16384, (1, 3)), (70, 8, 2048, (1, 150)), (512, 32, 1024, (1, 12)),
                                                            (16, 2, 768, (5, 600)), (64, 8, 1792, (1, 16, 17, 148)), (70, 8, 1024, (2, 148)),
