@@ -347,8 +347,7 @@ int oled_last_cuda_error(oled_ctx* ctx);
  * hosts that cannot let a library allocate device memory - a server that gives all of it to its
  * own arena at start-up, or a decode loop that cannot afford the device-wide synchronisation
  * hidden in cudaMalloc/cudaFree.  It runs the same gate, top-k and gate-score arithmetic as
- * oled_denoise_step() and the same stable permutation, needs no context and has no scratch but the arrays
- * of the call itself.
+ * oled_denoise_step() and the same stable permutation, and needs neither a context nor scratch.
  *   hidden [n_tokens,hidden_dim] bf16, w_router [n_experts,hidden_dim] bf16, bias fp32[n_experts]
  *   or NULL, confidences fp32[n_tokens]: device, read only.
  *   ids int32[n_tokens*top_k], gate fp32[n_tokens*top_k], counts int32[n_experts],

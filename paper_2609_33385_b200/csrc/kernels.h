@@ -175,8 +175,8 @@ struct ScatterRows {
   int dense = 0;                   // steps of at most kDenseTokens tokens: xp holds the rows once, in token order,
                                    // and the FFN multiplies every expert with all of them (ffn_few.cu)
   int32_t* assignment = nullptr;   // [E * cap] row -> t * K + j
-  uint16_t* xp = nullptr;          // [E * cap][H] copies of the token rows
-  TokenSplit split;                // fp8 stores, direct form: the rows' e4m3 terms and magnitudes as well
+  uint16_t* xp = nullptr;          // [E * cap][H] copies of the token rows - or, fp8 stores, direct form:
+  TokenSplit split;                // their e4m3 terms and magnitudes in place of them (xp is not written)
 };
 void launch_route(cudaStream_t st, const uint16_t* x, const uint16_t* w_router, const float* bias,
                   const float* conf, int T, int H, int E, int K, float* logits, int32_t* ids,

@@ -2,7 +2,7 @@
 
 Some hosts hand all device memory to their own arena, or cannot afford the device-wide
 synchronisation of cudaMalloc inside the decode loop; for them the library offers
-``oled_route_noalloc``, whose only scratch is the call's own output arrays.  The first test calls it
+``oled_route_noalloc``, which has no scratch at all.  The first test calls it
 through the C ABI twice in a row, with different inputs (so stale contents of anything shared
 would show), and checks every output bit for bit against what ``oled_denoise_step`` produced
 for the same inputs and against the CPU oracle's gate, top-k and permutation of the same bits; the
